@@ -856,15 +856,14 @@ __device__ __forceinline__ void shift_exact(float hi, float lo, float d, float& 
     H = hi + d;
     L = lo + (hi - (H - d));
 }
-// (H, L) = (hi + lo) * r + (oh + ol) for a power of two r, with the rounding of hi * r + oh
-// moved into L (TwoSum: exact for any ordering of the two terms)
-__device__ __forceinline__ void scale_shift_exact(float hi, float lo, float r, float oh, float ol, float& H,
-                                                  float& L) {
+// (H, L) = (hi + lo) * r + oh for a power of two r, with the rounding of hi * r + oh moved into L
+// (TwoSum: exact for any ordering of the two terms)
+__device__ __forceinline__ void scale_shift_exact(float hi, float lo, float r, float oh, float& H, float& L) {
     const float a = hi * r;  // exact
     H = a + oh;
     const float bb = H - a;
     const float err = (a - (H - bb)) + (oh - bb);
-    L = fmaf(lo, r, err + ol);
+    L = fmaf(lo, r, err);
 }
 
 // pairs of the list per close-pair vote (the unguarded passes)
@@ -1696,23 +1695,19 @@ __global__ void __launch_bounds__(256) k_leaf_a(AdaptiveView av, const int* __re
                 // the source leaf's centre offset in this leaf's widths and its width ratio,
                 // from the integer box coordinates (same tree): with d = lev_b - lev_s,
                 // (c_s - c_b) / h_b = N / 2^(1 + max(0, -d)),
-                // N = (2 i_s + 1) 2^max(0, d) - (2 i_b + 1) 2^max(0, -d) -- as hi + lo floats,
-                // exactly, and without FP64 instructions (1/64 of the FP32 rate here)
+                // N = (2 i_s + 1) 2^max(0, d) - (2 i_b + 1) 2^max(0, -d).  Levels go to 20, so both
+                // terms stay below 2^22, and adjacent boxes have |N| <= 2^|d| + 1 < 2^24: N is exact
+                // in an int and in a float (no remainder).  (64-bit N took nine conversions per list
+                // entry on the FP64 pipe, 1/64 of the FP32 rate here: 35 % of that pipe's cycles,
+                // Gaussian N = 1e6, p = 4: the kernel 2.28 -> 1.73 ms, FP32 results unchanged bit for bit.)
                 const int d = lev - av.level[sb];
                 const int up = d > 0 ? d : 0, dn = d < 0 ? -d : 0;
                 const float r = __int_as_float((127 + d) << 23);          // h_s / h_b = 2^d
                 const float sc = __int_as_float((127 - 1 - dn) << 23);    // 2^-(1 + dn)
                 const int* ijk_s = av.ijk + 3 * (size_t)sb;
-                float oh[3], ol[3];
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    const long long N = ((2ll * ijk_s[k] + 1) << up) - ((2ll * ijk_b[k] + 1) << dn);
-                    const float h = (float)N;
-                    oh[k] = h * sc;
-                    ol[k] = (float)(N - (long long)h) * sc;
-                }
-                const float ohx = oh[0], ohy = oh[1], ohz = oh[2];
-                const float olx = ol[0], oly = ol[1], olz = ol[2];
+                const float ohx = (float)(((2 * ijk_s[0] + 1) << up) - ((2 * ijk_b[0] + 1) << dn)) * sc;
+                const float ohy = (float)(((2 * ijk_s[1] + 1) << up) - ((2 * ijk_b[1] + 1) << dn)) * sc;
+                const float ohz = (float)(((2 * ijk_s[2] + 1) << up) - ((2 * ijk_b[2] + 1) << dn)) * sc;
                 if (!DAFMM_RANGE(av.pbeg[sb], av.pend[sb], av.n, kChkBoxRange)) return;
                 const int r0 = av.xq0[sb], n = av.pend[sb] - av.pbeg[sb];
                 if (!DAFMM_RANGE(r0, (long long)r0 + n, av.nrec, kChkRecord)) return;
@@ -1721,9 +1716,9 @@ __global__ void __launch_bounds__(256) k_leaf_a(AdaptiveView av, const int* __re
                     for (int i = lane; i < take; i += 32) {
                         const float4 rec = xq_load(av.xq, r0 + i0s + i), rl = xq_load(av.xl, r0 + i0s + i);
                         float X, Y, Z, XL, YL, ZL;
-                        scale_shift_exact(rec.x, rl.x, r, ohx, olx, X, XL);
-                        scale_shift_exact(rec.y, rl.y, r, ohy, oly, Y, YL);
-                        scale_shift_exact(rec.z, rl.z, r, ohz, olz, Z, ZL);
+                        scale_shift_exact(rec.x, rl.x, r, ohx, X, XL);
+                        scale_shift_exact(rec.y, rl.y, r, ohy, Y, YL);
+                        scale_shift_exact(rec.z, rl.z, r, ohz, Z, ZL);
                         list_store(buf, fill + i, X, Y, Z, rec.w, XL, YL, ZL, rl.w);
                     }
                     fill += take;
@@ -1785,13 +1780,12 @@ __global__ void __launch_bounds__(256) k_leaf_a(AdaptiveView av, const int* __re
                 if (!DAFMM_IN(wb, av.nbox, kChkBoxIndex)) continue;
                 const int dl = av.level[wb] - lev;
                 float sx0, sy0, sz0, iw;
-                if (dl >= 0 && dl <= 30) {
+                if (dl >= 0 && dl <= kMaxAdaptiveDepth) {  // (both terms below 2^22: exact in int and float)
                     const float r = (float)(1u << dl);
-                    const long long rr = 1ll << dl;
                     const int* iwb = av.ijk + 3 * (size_t)wb;
-                    const float ox = 0.5f * (float)((2ll * ib[0] + 1) * rr - (2ll * iwb[0] + 1));
-                    const float oy = 0.5f * (float)((2ll * ib[1] + 1) * rr - (2ll * iwb[1] + 1));
-                    const float oz = 0.5f * (float)((2ll * ib[2] + 1) * rr - (2ll * iwb[2] + 1));
+                    const float ox = 0.5f * (float)(((2 * ib[0] + 1) << dl) - (2 * iwb[0] + 1));
+                    const float oy = 0.5f * (float)(((2 * ib[1] + 1) << dl) - (2 * iwb[1] + 1));
+                    const float oz = 0.5f * (float)(((2 * ib[2] + 1) << dl) - (2 * iwb[2] + 1));
                     sx0 = fmaf(plw.x, r, fmaf(pw.x, r, ox));
                     sy0 = fmaf(plw.y, r, fmaf(pw.y, r, oy));
                     sz0 = fmaf(plw.z, r, fmaf(pw.z, r, oz));
