@@ -1343,10 +1343,6 @@ int eval_adaptive(dafmm_tree* t, int order, int precision, double* dphi, double*
                    "M2L (harmonic expansion)");
                 ++launches;
             }
-            for (int l = 2; l <= t->maxlev; ++l) {
-                CK(c, ops->p2l_a(av, precision, t->level_start[l], t->level_start[l + 1], t->aL, s), "P2L");
-                ++launches;
-            }
         } else {
             // FP64: the M2L by rotation (Sec. 3.4), by default from p = 4
             const bool rot = precision == DAFMM_FP64 && (c->m2l_rot > 0 || (c->m2l_rot < 0 && order >= 4));
@@ -1359,9 +1355,12 @@ int eval_adaptive(dafmm_tree* t, int order, int precision, double* dphi, double*
                 CK(c, ops->m2l_a(od, av, precision | rflags, t->grp_tg, t->grp_ptr, l * 8, mx, t->aM,
                                  t->aMf, t->aL, s),
                    "M2L");
-                CK(c, ops->p2l_a(av, precision, t->level_start[l], t->level_start[l + 1], t->aL, s), "P2L");
-                launches += 2;
+                ++launches;
             }
+        }
+        if (t->nx > 0) {  // every level's boxes in one launch (they only add to their own rows)
+            CK(c, ops->p2l_a(av, precision, t->level_start[2], t->nbox, t->aL, s), "P2L");
+            ++launches;
         }
         mark(5);
         for (int l = 2; l < t->maxlev; ++l) {  // parents at level l, children at l + 1

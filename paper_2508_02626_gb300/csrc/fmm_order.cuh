@@ -1514,11 +1514,64 @@ __global__ void __launch_bounds__(256) k_m2l_a(const T* __restrict__ K, Adaptive
     }
 }
 
-// P2L (Eq. 6): particles of the X-list leaves of each box of [lb, le) into its local expansion
+// The steps that restore the coefficients of z exponent >= 2 of a harmonic expansion from its free
+// ones by Laplace's equation (internal.h): V[i] = w1 V[i1] + w2 V[i2], those of z exponent c at
+// [cst[c], cst[c + 1]).
+struct HarmTab {
+    static constexpr int N = NC - nharm_of(P) > 0 ? NC - nharm_of(P) : 1;
+    int cst[P + 3];
+    unsigned short i[N], i1[N], i2[N];
+    float w1[N], w2[N];
+    double d1[N], d2[N];
+};
+constexpr HarmTab make_harm_tab() {
+    HarmTab t{};
+    int k = 0;
+    for (int c = 2; c <= P; ++c) {
+        t.cst[c] = k;
+        for (int n = c; n <= P; ++n)
+            for (int b = 0; b <= n - c; ++b, ++k) {
+                const int a = n - c - b;
+                t.i[k] = (unsigned short)da_index(a, b, c);
+                t.i1[k] = (unsigned short)da_index(a + 2, b, c - 2);
+                t.i2[k] = (unsigned short)da_index(a, b + 2, c - 2);
+                t.d1[k] = -(double)((a + 2) * (a + 1)) / (double)(c * (c - 1));
+                t.d2[k] = -(double)((b + 2) * (b + 1)) / (double)(c * (c - 1));
+                t.w1[k] = (float)t.d1[k];
+                t.w2[k] = (float)t.d2[k];
+            }
+    }
+    for (int c = P < 1 ? 2 : P + 1; c < P + 3; ++c) t.cst[c] = k;
+    return t;
+}
+__device__ const HarmTab harm_tab = make_harm_tab();
+
+__device__ __forceinline__ float harm_step(const float* V, int s) {
+    return fmaf(harm_tab.w1[s], V[harm_tab.i1[s]], harm_tab.w2[s] * V[harm_tab.i2[s]]);
+}
+__device__ __forceinline__ double harm_step(const double* V, int s) {
+    return fma(harm_tab.d1[s], V[harm_tab.i1[s]], harm_tab.d2[s] * V[harm_tab.i2[s]]);
+}
+
+// P2L (Eq. 6): particles of the X-list leaves of each box of [lb, le) into its local expansion,
+// one warp per box, all levels in one launch.
+//   1 / |w + d| = |w|^-1 (1 - 2 s.d + s^2 d^2)^(-1/2) with s = -w / |w|^2, so the P2L of w is the
+// generated P2M (Eq. 2) of s with the charge q / |w|; and since a local expansion is harmonic,
+// only its (p + 1)^2 free coefficients are generated and summed (121 instead of 286 at p = 10),
+// the others restored once per box by Laplace's equation.  The X lists' particles are taken as
+// one sequence -- 32 list entries at a time, prefix sums over the lanes -- so that every lane has
+// a particle whatever the leaves' sizes.  FP32: the source's offset in this box's frame comes
+// from its record (hi + lo) and the exact integer offset of the two boxes, rounded once to FP32,
+// as the FP64 difference was, but without FP64 instructions (they ran at 69 % of the FP64 pipe,
+// 1/64 of the FP32 rate, and bound the kernel).
+// Measured against the full-basis form before (one launch per level, a leaf at a time, FP64
+// differences): 64-problem forest, p = 6 (FP32): 0.913 -> 0.296 ms; Gaussian N = 1e6, p = 4 (FP32):
+// 0.444 -> 0.159 ms; Gaussian N = 1e5, s = 256, p = 8 (FP64): 9.89 -> 2.91 ms.
 template <class T>
-__global__ void k_p2l_a(AdaptiveView av, int lb, int le, double* __restrict__ L) {
+__global__ void __launch_bounds__(128) k_p2l_a(AdaptiveView av, int lb, int le, double* __restrict__ L) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* sm = reinterpret_cast<T*>(smem_raw) + threadIdx.y * (32 * 33);
+    static_assert(NCP <= 32 * 33, "the staging block holds a row");
     const int lane = threadIdx.x;
     const int b = lb + blockIdx.x * blockDim.y + threadIdx.y;
     if (b >= le) return;
@@ -1528,32 +1581,90 @@ __global__ void k_p2l_a(AdaptiveView av, int lb, int le, double* __restrict__ L)
     double cx, cy, cz, h;
     abox_geom(av, b, cx, cy, cz, h);
     const double ih = 1.0 / h;
-    constexpr int NJ = (NC + 31) / 32;
+    const int lev = av.level[b];
+    const int* ib = av.ijk + 3 * (size_t)b;
+    constexpr int NO = nharm_of(P);
+    constexpr int NJ = (NO + 31) / 32;
     T acc[NJ];
 #pragma unroll
     for (int j = 0; j < NJ; ++j) acc[j] = T(0);
-    ChunkSink<T, NJ> sink{sm, lane, acc};
-    for (int xi = x0i; xi < x1i; ++xi) {
-        const int c = av.x_idx[xi];
-        if (!DAFMM_IN(c, av.nbox, kChkBoxIndex) || !DAFMM_RANGE(av.pbeg[c], av.pend[c], av.n, kChkBoxRange)) continue;
-        const int i0 = av.pbeg[c], i1 = av.pend[c];
-        for (int base = i0; base < i1; base += 32) {
-            const int i = base + lane;
-            T X = T(1), Y = T(0), Z = T(0), q = T(0);  // a dummy far point for idle lanes
-            if (i < i1) {
-                X = (T)((cx - av.x[i]) * ih);
-                Y = (T)((cy - av.y[i]) * ih);
-                Z = (T)((cz - av.z[i]) * ih);
-                q = (T)av.q[i];
+    ChunkSink<T, NJ, NO> sink{sm, lane, acc};
+    for (int xg = x0i; xg < x1i; xg += 32) {
+        // one list entry per lane: its particles (FP32: its first record, its centre offset and
+        // width in this box's widths), and the inclusive prefix sum of the counts
+        int cnt = 0, first = 0;
+        float r = 1.f, ox = 0.f, oy = 0.f, oz = 0.f;
+        if (xg + lane < x1i) {
+            const int c = av.x_idx[xg + lane];
+            if (DAFMM_IN(c, av.nbox, kChkBoxIndex) && DAFMM_RANGE(av.pbeg[c], av.pend[c], av.n, kChkBoxRange)) {
+                first = av.pbeg[c];
+                cnt = av.pend[c] - first;
+                if constexpr (sizeof(T) == 4) {
+                    first = av.xq0[c];
+                    if (!DAFMM_RANGE(first, (long long)first + cnt, av.nrec, kChkRecord)) cnt = 0;
+                    const int d = lev - av.level[c];  // > 0: the leaves of an X list are coarser
+                    const int* ic = av.ijk + 3 * (size_t)c;
+                    r = __int_as_float((127 + d) << 23);
+                    ox = 0.5f * (float)(((2 * ic[0] + 1) << d) - (2 * ib[0] + 1));
+                    oy = 0.5f * (float)(((2 * ic[1] + 1) << d) - (2 * ib[1] + 1));
+                    oz = 0.5f * (float)(((2 * ic[2] + 1) << d) - (2 * ib[2] + 1));
+                }
             }
-            gen::GEN(p2l)<T>(X, Y, Z, q, sink);
+        }
+        int incl = cnt;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += v;
+        }
+        const int total = __shfl_sync(0xffffffffu, incl, 31);
+        for (int base = 0; base < total; base += 32) {
+            const int j = base + lane;
+            int e = 0;  // the entry that holds particle j: the first with incl > j
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) {
+                const int v = __shfl_sync(0xffffffffu, incl, e + d - 1);
+                if (v <= j) e += d;
+            }
+            const int i = __shfl_sync(0xffffffffu, first - (incl - cnt), e) + j;
+            T X = T(1), Y = T(0), Z = T(0), q = T(0);  // a dummy far point for idle lanes
+            if constexpr (sizeof(T) == 4) {
+                const float er = __shfl_sync(0xffffffffu, r, e), ex = __shfl_sync(0xffffffffu, ox, e),
+                            ey = __shfl_sync(0xffffffffu, oy, e), ez = __shfl_sync(0xffffffffu, oz, e);
+                if (j < total) {
+                    const float4 rec = xq_load(av.xq, i), rl = xq_load(av.xl, i);
+                    float lx, ly, lz;
+                    scale_shift_exact(rec.x, rl.x, er, ex, X, lx);
+                    scale_shift_exact(rec.y, rl.y, er, ey, Y, ly);
+                    scale_shift_exact(rec.z, rl.z, er, ez, Z, lz);
+                    X += lx;
+                    Y += ly;
+                    Z += lz;
+                    q = rec.w;
+                }
+            } else if (j < total) {
+                X = (av.x[i] - cx) * ih;
+                Y = (av.y[i] - cy) * ih;
+                Z = (av.z[i] - cz) * ih;
+                q = av.q[i];
+            }
+            // w = -(X, Y, Z); s = -w / |w|^2
+            const T ir = dafmm_rsqrt(X * X + Y * Y + Z * Z), rho = ir * ir;
+            gen::GEN(p2mh)<T>(X * rho, Y * rho, Z * rho, q * ir, sink);
         }
     }
+    __syncwarp();
 #pragma unroll
     for (int j = 0; j < NJ; ++j) {
         const int k = lane + 32 * j;
-        if (k < NC) L[(size_t)b * NCP + k] += (double)acc[j] * ih;
+        if (k < NO) sm[harm_full_index(k)] = acc[j];
     }
+    __syncwarp();
+    for (int c = 2; c <= P; ++c) {
+        for (int s = harm_tab.cst[c] + lane; s < harm_tab.cst[c + 1]; s += 32) sm[harm_tab.i[s]] = harm_step(sm, s);
+        __syncwarp();
+    }
+    for (int k = lane; k < NC; k += 32) L[(size_t)b * NCP + k] += (double)sm[k] * ih;
 }
 
 // L2L (Eq. 7) from the parents [lb, le) of one level into their existing children (added to
