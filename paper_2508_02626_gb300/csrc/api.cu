@@ -268,14 +268,28 @@ int ensure_order(dafmm_ctx* c, int p, cudaStream_t s, bool need_k) {
             shift_rp8(t, od.nc, rp8.data());
             if ((rc = upload(c, w == 0 ? &od.m2m_rp8 : &od.l2l_rp8, rp8.data(), rp8.size(), "shift table"))) return rc;
         }
-        {  // the M2M of harmonic multipoles
+        {  // the M2M of harmonic multipoles, its rows and columns by free index
             const HostShiftTable& t = ops->m2mh;
+            const int nh = nharm_of(p);
+            std::vector<int> free_of(od.nc, -1), rp(nh + 1, 0);
+            for (int j = 0; j < nh; ++j) free_of[harm_full_index(j)] = j;
+            std::vector<unsigned short> col(t.nnz), ord(nh);
+            for (int e = 0; e < t.nnz; ++e) col[e] = (unsigned short)free_of[t.col[e]];
+            for (int j = 0; j < nh; ++j) {  // (rows outside the free coefficients are empty)
+                rp[j] = t.rowptr[harm_full_index(j)];
+                ord[j] = (unsigned short)j;
+            }
+            rp[nh] = t.nnz;
+            std::stable_sort(ord.begin(), ord.end(),
+                             [&](int a, int b) { return rp[a + 1] - rp[a] > rp[b + 1] - rp[b]; });
             std::vector<float> vf(t.val, t.val + t.nnz);
-            if ((rc = upload(c, &od.m2mh_rowptr, t.rowptr, (size_t)od.nc + 1, "shift table"))) return rc;
-            if ((rc = upload(c, &od.m2mh_col, t.col, (size_t)t.nnz, "shift table"))) return rc;
+            if ((rc = upload(c, &od.m2mh_rowptr, rp.data(), rp.size(), "shift table"))) return rc;
+            if ((rc = upload(c, &od.m2mh_col, col.data(), col.size(), "shift table"))) return rc;
+            if ((rc = upload(c, &od.m2mh_ord, ord.data(), ord.size(), "shift table"))) return rc;
             if ((rc = upload(c, &od.m2mh_par, t.par, (size_t)t.nnz, "shift table"))) return rc;
             if ((rc = upload(c, &od.m2mh_val, t.val, (size_t)t.nnz, "shift table"))) return rc;
             if ((rc = upload(c, &od.m2mh_valf, vf.data(), (size_t)t.nnz, "shift table"))) return rc;
+            od.m2mh_nnz = t.nnz;
         }
         // DA product table: for each output k, the pairs (i, j) with e_i + e_j = e_k
         std::vector<int> ex(3 * od.nc);
@@ -376,7 +390,8 @@ void free_order(dafmm_ctx* c, OrderData& od) {
     }
     {
         const HostShiftTable& t = ops->m2mh;
-        dev_free(c, od.m2mh_rowptr, od.m2mh_rowptr ? (nc + 1) * sizeof(int) : 0);
+        dev_free(c, od.m2mh_rowptr, od.m2mh_rowptr ? ((size_t)nharm_of(od.p) + 1) * sizeof(int) : 0);
+        dev_free(c, od.m2mh_ord, od.m2mh_ord ? (size_t)nharm_of(od.p) * sizeof(unsigned short) : 0);
         dev_free(c, od.m2mh_col, od.m2mh_col ? t.nnz * sizeof(unsigned short) : 0);
         dev_free(c, od.m2mh_par, od.m2mh_par ? (size_t)t.nnz : 0);
         dev_free(c, od.m2mh_val, od.m2mh_val ? t.nnz * sizeof(double) : 0);
@@ -940,6 +955,8 @@ void free_adaptive(dafmm_ctx* c, dafmm_tree* t) {
     dev_free(c, t->u_ptr, nb1 * 4); dev_free(c, t->w_ptr, nb1 * 4); dev_free(c, t->x_ptr, nb1 * 4);
     dev_free(c, t->u_idx, (size_t)t->nu * 4); dev_free(c, t->w_idx, (size_t)t->nw * 4); dev_free(c, t->x_idx, (size_t)t->nx * 4);
     dev_free(c, t->leaves, (size_t)t->nleaves * 4);
+    dev_free(c, t->parents, t->parent_start.empty() ? 0 : (size_t)t->parent_start.back() * 4);
+    t->parents = nullptr;
     dev_free(c, t->grp_tg, (size_t)t->nbox * 4);
     dev_free(c, t->grp_ptr, ((size_t)(t->maxlev + 1) * 8 + 1) * 4);
     if (t->a_exp_p >= 0) {
@@ -1107,19 +1124,29 @@ int build_adaptive(dafmm_ctx* c, dafmm_tree* t, const double* dxyz, const double
     if ((rc = dev_alloc(c, (void**)&t->a_geom, (size_t)nbox * sizeof(double4), "box geometry"))) return rc;
     e = launch_box_geometry(t->a_root, t->a_level, t->a_ijk, t->d_rootdom, nbox, t->a_geom, s);
     if (e != cudaSuccess) return cuda_fail(c, e, "geometry");
-    // leaves (breadth-first order)
-    if ((rc = scratch.alloc(2 * ((size_t)nbox + 1) * 4, "leaf scratch"))) return rc;
+    // leaves, and the boxes that have children (both in breadth-first order): a leaf's place is the
+    // number of leaves before it, a parent's the rest; the parents of level l are
+    // parents[parent_start[l] .. parent_start[l + 1])
+    const int nlev = t->maxlev + 1;
+    if ((rc = scratch.alloc((2 * ((size_t)nbox + 1) + kMaxAdaptiveDepth + 2) * 4, "leaf scratch"))) return rc;
     int* flags = scratch.as<int>();
     int* foff = flags + nbox + 1;
+    int* pstart = foff + nbox + 1;
+    LevelStarts ls;
+    for (int l = 0; l <= nlev; ++l) ls.v[l] = t->level_start[l];
     e = launch_leaf_flags(t->a_child, nbox, flags, s);
     if (e == cudaSuccess) e = launch_scan(flags, foff, nbox, s);
-    int nl = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&nl, foff + nbox, 4, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = launch_parent_starts(ls, nlev, foff, pstart, s);
+    t->parent_start.assign(nlev + 1, 0);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(t->parent_start.data(), pstart, (nlev + 1) * sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(c, e, "leaves");
+    const int npar = t->parent_start[nlev], nl = nbox - npar;
     t->nleaves = nl;
     if ((rc = dev_alloc(c, (void**)&t->leaves, (size_t)(nl > 0 ? nl : 1) * 4, "leaves"))) return rc;
-    e = launch_scatter_flagged(flags, foff, nbox, t->leaves, s);
+    if ((rc = dev_alloc(c, (void**)&t->parents, (size_t)npar * 4, "parents"))) return rc;
+    e = launch_scatter_flagged(flags, foff, nbox, t->leaves, t->parents, s);
     if (e != cudaSuccess) return cuda_fail(c, e, "leaves");
     // FP32 records: leaves in list order take consecutive even record ranges (at most one
     // padding record per leaf)
@@ -1273,7 +1300,9 @@ int eval_adaptive(dafmm_tree* t, int order, int precision, double* dphi, double*
         ++launches;
         mark(1);
         for (int l = t->maxlev - 1; l >= 2; --l) {
-            CK(c, ops->m2m_a(od, av, prec_m, t->level_start[l], t->level_start[l + 1], t->aM, s), "M2M");
+            CK(c, ops->m2m_a(od, av, prec_m, t->parents + t->parent_start[l],
+                             t->parent_start[l + 1] - t->parent_start[l], t->aM, s),
+               "M2M");
             ++launches;
         }
         if (harm) {
@@ -1364,7 +1393,9 @@ int eval_adaptive(dafmm_tree* t, int order, int precision, double* dphi, double*
         }
         mark(5);
         for (int l = 2; l < t->maxlev; ++l) {  // parents at level l, children at l + 1
-            CK(c, ops->l2l_a(od, av, precision, t->level_start[l], t->level_start[l + 1], t->aL, s), "L2L");
+            CK(c, ops->l2l_a(od, av, precision, t->parents + t->parent_start[l],
+                             t->parent_start[l + 1] - t->parent_start[l], t->aL, s),
+               "L2L");
             ++launches;
         }
         mark(6);
@@ -2333,9 +2364,9 @@ size_t dafmm_footprint(int64_t n, int order, int uniform_depth, int max_leaf, in
     if (uniform_depth < 0) {
         // adaptive: about 16 n / max_leaf boxes; per box its hierarchy record, list entries
         // (U, W and X, about 64 on average), its first FP32 record, a padding record (with its
-        // remainder record) and the expansions
+        // remainder record), its place in the list of parents and the expansions
         const size_t nbox = 2 + (size_t)(16 * n) / (size_t)(max_leaf > 0 ? max_leaf : 1);
-        b += nbox * (kBoxInts * 4 + 64 * 4 + 24 + 32 + ncp * (8 + 8 + 4));
+        b += nbox * (kBoxInts * 4 + 64 * 4 + 24 + 32 + 4 + ncp * (8 + 8 + 4));
         b += (size_t)kNumKeys * nc * ncp * 12;
         b += (size_t)n * 12 + radix_sort_temp_bytes(n) + radix_sort_temp_bytes((int64_t)nbox);
         return b;

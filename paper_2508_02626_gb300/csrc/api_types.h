@@ -97,6 +97,8 @@ struct dafmm_tree {
     int64_t nv = 0;  // M2L (V list) pairs
     int* leaves = nullptr;
     int nleaves = 0;
+    int* parents = nullptr;         // the boxes that have children, breadth-first
+    std::vector<int> parent_start;  // those of level l: [parent_start[l], parent_start[l + 1])
     int* grp_tg = nullptr;          // boxes of levels >= 2 grouped by (level, octant)
     int* grp_ptr = nullptr;         // (maxlev + 1) * 8 + 1 offsets
     std::vector<int> grp_ptr_h;

@@ -9,13 +9,13 @@
 //   P2M  (Eq. 2)  k_p2m       one warp per leaf; each lane runs the generated straight-line
 //                             P2M of one particle, a padded shared-memory transpose sums the
 //                             32 lanes per coefficient
-//   M2M  (Eq. 4)  k_m2m       32 parents per block; the 8 octant maps are one table with sign
+//   M2M  (Eq. 4)  k_m2m       8 parents per block; the 8 octant maps are one table with sign
 //                             flips (Sec. 3.3)
 //   M2L  (Eq. 5)  k_kgen      K^_v for all 316 displacements, FP64 numerical DA products of the
 //                             generated transfer map (one block per v)
 //                 k_m2l       L~_t = (1/h) sum_v K^_v M~_{t-v} over the 189 displacements of
 //                             the target's octant (SIMT, FP64 or FP32)
-//   L2L  (Eq. 7)  k_l2l       32 parents per block, 8 child tables by sign flips
+//   L2L  (Eq. 7)  k_l2l       32 parents and 16 rows per block, 8 child tables by sign flips
 //   L2P + P2P     k_leaf      one warp per target leaf: pairwise sum over the 27 neighbour
 //                             leaves and the generated L2P of the leaf's local expansion
 #include <cuda_fp16.h>
@@ -212,7 +212,6 @@ __device__ __forceinline__ float tab_val<float>(const ShiftTab& t, int e) { retu
 
 constexpr int SH_ROWS = (NC + 7) / 8;  // output rows per warp (8 warps)
 
-// parents at level lc-1; children at level lc stored octant-major
 // Both shifts use the octant structure of Sec. 3.3: the entry (b, a) of the table of child
 // octant c is the octant-0 entry times (-1)^popcount(par & c), par = parity pattern of the
 // entry.  Summing over the 8 octants first -- the Hadamard transform
@@ -234,103 +233,171 @@ __device__ __forceinline__ void hadamard8(T (&m)[8]) {
             }
 }
 
-// parents per thread block of the M2M kernels: 8.  The NC output rows of a parent are then
-// spread over 32 threads (4 lanes in each of the 8 warps), about NC / 32 rows each; a level of
-// 4096 parents spreads over 512 blocks; and the transformed children S[8][8][NCP + 1] (43 KB in
-// FP32 at p = 8) leave room for several blocks per SM
-template <class T>
-constexpr int m2m_parents() {
-    return 8;
+// The parents of one level's shift and where their rows lie.  Uniform trees: parent i of level
+// lc - 1 in the order of its children's octant slabs.  Adaptive trees: box list[i]; only boxes
+// with children are listed (at most one box in about eight has any, so a walk over all boxes
+// left most lanes idle).
+struct ShiftUniform {
+    int lc, n;  // children's level, parents
+    __device__ __forceinline__ int parent(int i) const {
+        const int Pc = 1 << (lc - 1);
+        return octmajor_index(lc - 1, i % Pc, (i / Pc) % Pc, i / (Pc * Pc));
+    }
+    __device__ __forceinline__ int child(int i, int c) const { return c * n + i; }
+};
+struct ShiftAdaptive {
+    AdaptiveView av;
+    const int* list;
+    int n;
+    __device__ __forceinline__ int parent(int i) const { return list[i]; }
+    __device__ __forceinline__ int child(int i, int c) const {
+        const int ch = av.child[8 * list[i] + c];
+        return ch >= 0 && DAFMM_IN(ch, av.nbox, kChkBoxIndex) ? ch : -1;
+    }
+};
+
+// parents per thread block of the M2M kernel: 8.  The output rows of a parent are then spread
+// over 32 threads (4 lanes in each of the 8 warps) and a level of 4096 parents over 512 blocks.
+constexpr int kM2MParents = 8;
+// rows of S: the coefficients staged per box, made odd (bank conflicts)
+template <bool H>
+constexpr int m2m_stride() {
+    return (H ? nharm_of(P) : NC) | 1;
 }
-template <class T>
-constexpr size_t m2m_smem() {
-    return (size_t)8 * m2m_parents<T>() * (NCP + 1) * sizeof(T);
+// the transformed children S [8][kM2MParents][stride], and (harmonic) the table's entries
+template <class T, bool H>
+constexpr size_t m2m_smem(int nnz) {
+    return (size_t)8 * kM2MParents * m2m_stride<H>() * sizeof(T) + (H ? (size_t)nnz * (sizeof(T) + 2) : 0);
 }
 
-// M2M from the children at level lc into the parents at level lc - 1 (uniform tree).  harm:
-// harmonic multipoles -- tab is the harmonic M2M table, which reads and writes only the free
-// coefficients, so only those are staged and computed.
-template <class T>
-__global__ void __launch_bounds__(256) k_m2m(ShiftTab tab, int lc, const double* __restrict__ Mc,
-                                             double* __restrict__ Mp, int rows32, int harm) {
-    constexpr int PP = m2m_parents<T>(), RS = 32 / PP;
+// M2M (Eq. 4) from the children into the parents of one level.  H: harmonic multipoles -- tab is
+// the harmonic M2M table (rows and columns by free index), which reads and writes only the free
+// coefficients.  Its entries are staged in shared memory, the parity and column of an entry as
+// one offset into S: read from global memory they are a chain of dependent loads per entry.  The
+// rows go to the lanes in order of decreasing length (tab.ord), so that the four rows a warp works
+// on at a time end together.  Measured, all levels: clustered N = 4e6, p = 10, FP64: 2.86 -> 0.63
+// ms (mostly the parents' list); uniform N = 1e6, p = 8: FP64 89 -> 78 us, FP32 40 -> 32 us.
+template <class T, bool H, class Fam>
+__global__ void __launch_bounds__(256) k_m2m(ShiftTab tab, const __grid_constant__ Fam fam, const double* Mc,
+                                             double* Mp, int rows32) {
+    constexpr int PP = kM2MParents, RS = 32 / PP, ST = m2m_stride<H>(), NO = H ? nharm_of(P) : NC;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* S = reinterpret_cast<T*>(smem_raw);  // [8][PP][NCP + 1]
-    const int Pc = 1 << (lc - 1);
-    const int nparent = Pc * Pc * Pc;
-    const int lin0 = blockIdx.x * PP;
-    const int NO = harm ? nharm_of(P) : NC;  // coefficients staged and computed per box
+    T* S = reinterpret_cast<T*>(smem_raw);
+    T* tv = S + 8 * PP * ST;
+    unsigned short* tx = reinterpret_cast<unsigned short*>(tv + (H ? tab.nnz : 0));
+    if constexpr (H) {
+        for (int e = threadIdx.x; e < tab.nnz; e += 256) {
+            tv[e] = tab_val<T>(tab, e);
+            tx[e] = (unsigned short)(tab.par[e] * (PP * ST) + tab.col[e]);
+        }
+    }
+    const int i0 = blockIdx.x * PP;
     for (int e = threadIdx.x; e < PP * NO; e += 256) {
         const int r = e / NO, j = e - r * NO;
-        const int k = harm ? harm_full_index(j) : j;
-        const int lin = lin0 + r;
+        const int k = H ? harm_full_index(j) : j;
         T m[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
-            const size_t at = (size_t)(c * nparent + lin) * NCP + k;
-            m[c] = lin >= nparent ? T(0) : rows32 ? (T)reinterpret_cast<const float*>(Mc)[at] : (T)Mc[at];
+            const int ch = i0 + r < fam.n ? fam.child(i0 + r, c) : -1;
+            const size_t at = (size_t)ch * NCP + k;
+            m[c] = ch < 0 ? T(0) : rows32 ? (T)reinterpret_cast<const float*>(Mc)[at] : (T)Mc[at];
         }
         hadamard8(m);
 #pragma unroll
-        for (int q = 0; q < 8; ++q) S[(q * PP + r) * (NCP + 1) + k] = m[q];
+        for (int q = 0; q < 8; ++q) S[(q * PP + r) * ST + j] = m[q];
     }
     __syncthreads();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int r = lane % PP, sub = lane / PP;
-    const int lin = lin0 + r;
-    if (lin >= nparent) return;
-    const int px = lin % Pc, py = (lin / Pc) % Pc, pz = lin / (Pc * Pc);
-    const size_t ob = (size_t)octmajor_index(lc - 1, px, py, pz) * NCP;
-    for (int j = w * RS + sub; j < NO; j += 8 * RS) {
-        const int b = harm ? harm_full_index(j) : j;
+    if (i0 + r >= fam.n) return;
+    const size_t ob = (size_t)fam.parent(i0 + r) * NCP;
+    const T* Sr = S + r * ST;
+    for (int jj = w * RS + sub; jj < NO; jj += 8 * RS) {
+        const int j = tab.ord ? tab.ord[jj] : jj;
         T acc = T(0);
-        for (int e = tab.rowptr[b]; e < tab.rowptr[b + 1]; ++e)
-            acc += tab_val<T>(tab, e) * S[(tab.par[e] * PP + r) * (NCP + 1) + tab.col[e]];
-        if (rows32) reinterpret_cast<float*>(Mp)[ob + b] = (float)acc;
-        else Mp[ob + b] = (double)acc;
-    }
-}
-
-// the 8 partial sums R_m of row b of the L2L table applied to a local expansion in `src`
-template <class T>
-__device__ __forceinline__ void l2l_row(const ShiftTab& tab, int b, const T* src, T (&R)[8]) {
-#pragma unroll
-    for (int m = 0; m < 8; ++m) {
-        T s = T(0);
-        for (int e = tab.rp8[8 * b + m]; e < tab.rp8[8 * b + m + 1]; ++e) s += tab_val<T>(tab, e) * src[tab.col[e]];
-        R[m] = s;
-    }
-    hadamard8(R);  // R[c] = what child octant c receives
-}
-
-// children at level lc receive L2L of their parent (added to what M2L wrote)
-template <class T>
-__global__ void __launch_bounds__(256) k_l2l(ShiftTab tab, int lc, const double* __restrict__ Lp,
-                                             double* __restrict__ Lc) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* src = reinterpret_cast<T*>(smem_raw);  // [32][NCP + 1]
-    const int Pc = 1 << (lc - 1);
-    const int nparent = Pc * Pc * Pc;
-    const int lin0 = blockIdx.x * 32;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int e = threadIdx.x; e < 32 * NC; e += 256) {
-        const int r = e / NC, k = e - r * NC;
-        const int lin = lin0 + r;
-        T v = T(0);
-        if (lin < nparent) {
-            const int px = lin % Pc, py = (lin / Pc) % Pc, pz = lin / (Pc * Pc);
-            v = (T)Lp[(size_t)octmajor_index(lc - 1, px, py, pz) * NCP + k];
+        if constexpr (H) {
+#pragma unroll 4
+            for (int e = tab.rowptr[j]; e < tab.rowptr[j + 1]; ++e) acc += tv[e] * Sr[tx[e]];
+        } else {
+            for (int e = tab.rowptr[j]; e < tab.rowptr[j + 1]; ++e)
+                acc += tab_val<T>(tab, e) * Sr[tab.par[e] * (PP * ST) + tab.col[e]];
         }
-        src[r * (NCP + 1) + k] = v;
+        const size_t at = ob + (H ? harm_full_index(j) : j);
+        if (rows32) reinterpret_cast<float*>(Mp)[at] = (float)acc;
+        else Mp[at] = (double)acc;
+    }
+}
+
+// L2L (Eq. 7): the children of one level's parents receive the parents' locals (added to what
+// M2L and P2L wrote).  A block takes 32 parents (one per lane) and 16 rows of the table (one per
+// warp), so that even a level of 64 parents spreads over ncoef / 16 blocks; the parents' columns
+// and the rows' table entries are staged in shared memory, and the 8 children's results pass
+// through it so that their rows are updated in whole 128-byte (FP64) segments.  The form before
+// (8 warps walking all rows, entries read from global memory one dependent load after another,
+// strided updates) took about 170 us per level whatever its size.  Measured, all levels: uniform
+// N = 1e6, p = 8, FP64: 509 -> 125 us; clustered N = 4e6, p = 10, FP64: 4.35 -> 1.83 ms; 64-problem
+// forest, p = 6, FP32: 235 -> 57 us.
+constexpr int kL2LRows = 16;
+template <class T>
+constexpr size_t l2l_smem(int maxe) {
+    return ((size_t)32 * (NCP + 1) + (size_t)8 * 32 * (kL2LRows + 1) + maxe) * sizeof(T) + (size_t)maxe * 2;
+}
+
+template <class T, class Fam>
+__global__ void __launch_bounds__(32 * kL2LRows) k_l2l(ShiftTab tab, const __grid_constant__ Fam fam, int maxe,
+                                                       const double* Lp, double* Lc) {
+    constexpr int ST = NCP + 1, OR = kL2LRows + 1;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T* src = reinterpret_cast<T*>(smem_raw);  // [32][ST]
+    T* out = src + 32 * ST;                   // [8][32][OR]
+    T* tv = out + 8 * 32 * OR;                // the rows' entries
+    unsigned short* tc = reinterpret_cast<unsigned short*>(tv + maxe);
+    const int b0 = blockIdx.y * kL2LRows, nb = min(kL2LRows, NC - b0);
+    const int i0 = blockIdx.x * 32;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int e0 = tab.rowptr[b0], e1 = tab.rowptr[b0 + nb];
+    for (int e = e0 + (int)threadIdx.x; e < e1; e += 32 * kL2LRows) {
+        tv[e - e0] = tab_val<T>(tab, e);
+        tc[e - e0] = tab.col[e];
+    }
+    // row b reads columns a >= b componentwise only, which have indices >= b
+    for (int r = w; r < 32; r += kL2LRows) {
+        if (i0 + r >= fam.n) break;
+        const double* row = Lp + (size_t)fam.parent(i0 + r) * NCP;
+        for (int k = b0 + lane; k < NC; k += 32) src[r * ST + k] = (T)row[k];
     }
     __syncthreads();
-    const int lin = lin0 + lane;
-    if (lin >= nparent) return;
-    for (int b = w; b < NC; b += 8) {
+    if (w < nb && i0 + lane < fam.n) {
+        const T* srow = src + lane * ST;
+        const int* rp = tab.rp8 + 8 * (b0 + w);
         T R[8];
-        l2l_row(tab, b, src + lane * (NCP + 1), R);
+        int nm = 0;  // parity classes with entries, class 0 aside
 #pragma unroll
-        for (int c = 0; c < 8; ++c) Lc[(size_t)(c * nparent + lin) * NCP + b] += (double)R[c];
+        for (int m = 0; m < 8; ++m) {
+            T s = T(0);
+            const int ea = rp[m] - e0, ez = rp[m + 1] - e0;
+#pragma unroll 4
+            for (int e = ea; e < ez; ++e) s += tv[e] * srow[tc[e]];
+            R[m] = s;
+            nm += m > 0 && ez > ea;
+        }
+        if (nm > 0) {
+            hadamard8(R);  // R[c] = what child octant c receives
+        } else {
+#pragma unroll
+            for (int c = 1; c < 8; ++c) R[c] = R[0];  // (the top degree's rows: one entry)
+        }
+#pragma unroll
+        for (int c = 0; c < 8; ++c) out[(c * 32 + lane) * OR + w] = R[c];
+    }
+    __syncthreads();
+    const int i = threadIdx.x % kL2LRows;
+    if (i >= nb) return;
+    for (int g = threadIdx.x / kL2LRows; g < 8 * 32; g += 32) {
+        const int r = g & 31, c = g >> 5;
+        if (i0 + r >= fam.n) continue;
+        const int ch = fam.child(i0 + r, c);
+        if (ch >= 0) Lc[(size_t)ch * NCP + b0 + i] += (double)out[g * OR + i];
     }
 }
 
@@ -1341,13 +1408,6 @@ __device__ __forceinline__ void abox_geom(const AdaptiveView& av, int b, double&
     h = g.w;
 }
 
-__device__ __forceinline__ bool abox_is_leaf(const AdaptiveView& av, int b) {
-    const int4 c0 = *reinterpret_cast<const int4*>(av.child + 8 * b);
-    const int4 c1 = *reinterpret_cast<const int4*>(av.child + 8 * b + 4);
-    return (c0.x & c0.y & c0.z & c0.w & c1.x & c1.y & c1.z & c1.w) < 0 &&
-           c0.x < 0 && c0.y < 0 && c0.z < 0 && c0.w < 0 && c1.x < 0 && c1.y < 0 && c1.z < 0 && c1.w < 0;
-}
-
 // P2M (Eq. 2) at the leaves listed in `leaves`: one warp per leaf, as in k_p2m (H: the
 // harmonic basis's free coefficients only, written at their layout positions)
 template <class T, bool H = false>
@@ -1400,46 +1460,6 @@ __global__ void k_p2m_a(AdaptiveView av, const int* __restrict__ leaves, int nle
     for (int j = 0; j < NJ; ++j) {
         const int k = lane + 32 * j;
         if (k < NO) M[(size_t)b * NCP + (H ? harm_full_index(k) : k)] = (double)acc[j];
-    }
-}
-
-// M2M (Eq. 4) into the non-leaf boxes [lb, le) of one level, from their existing children
-// (missing children count as zero; leaves keep their P2M result).  harm: harmonic multipoles,
-// tab the harmonic M2M table -- free coefficients only, as in k_m2m.
-template <class T>
-__global__ void __launch_bounds__(256) k_m2m_a(ShiftTab tab, AdaptiveView av, int lb, int le, double* __restrict__ M,
-                                               int harm) {
-    constexpr int PP = m2m_parents<T>(), RS = 32 / PP;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* S = reinterpret_cast<T*>(smem_raw);  // [8][PP][NCP + 1]
-    const int b0 = lb + blockIdx.x * PP;
-    const int NO = harm ? nharm_of(P) : NC;
-    for (int e = threadIdx.x; e < PP * NO; e += 256) {
-        const int r = e / NO, j = e - r * NO;
-        const int k = harm ? harm_full_index(j) : j;
-        const int bx = b0 + r;
-        T m[8];
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const int ch = bx < le ? av.child[8 * bx + c] : -1;
-            m[c] = ch >= 0 && DAFMM_IN(ch, av.nbox, kChkBoxIndex) ? (T)M[(size_t)ch * NCP + k] : T(0);
-        }
-        hadamard8(m);
-#pragma unroll
-        for (int q = 0; q < 8; ++q) S[(q * PP + r) * (NCP + 1) + k] = m[q];
-    }
-    __syncthreads();
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int r = lane % PP, sub = lane / PP;
-    const int bx = b0 + r;
-    if (bx >= le || abox_is_leaf(av, bx)) return;
-    double* out = M + (size_t)bx * NCP;
-    for (int j = w * RS + sub; j < NO; j += 8 * RS) {
-        const int b = harm ? harm_full_index(j) : j;
-        T acc = T(0);
-        for (int e = tab.rowptr[b]; e < tab.rowptr[b + 1]; ++e)
-            acc += tab_val<T>(tab, e) * S[(tab.par[e] * PP + r) * (NCP + 1) + tab.col[e]];
-        out[b] = (double)acc;
     }
 }
 
@@ -1665,57 +1685,6 @@ __global__ void __launch_bounds__(128) k_p2l_a(AdaptiveView av, int lb, int le, 
         __syncwarp();
     }
     for (int k = lane; k < NC; k += 32) L[(size_t)b * NCP + k] += (double)sm[k] * ih;
-}
-
-// L2L (Eq. 7) from the parents [lb, le) of one level into their existing children (added to
-// what M2L and P2L wrote)
-template <class T>
-__global__ void __launch_bounds__(256) k_l2l_a(ShiftTab tab, AdaptiveView av, int lb, int le, double* __restrict__ L) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* src = reinterpret_cast<T*>(smem_raw);  // [32][NCP + 1]
-    const int b0 = lb + blockIdx.x * 32;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int e = threadIdx.x; e < 32 * NC; e += 256) {
-        const int r = e / NC, k = e - r * NC;
-        const int P = b0 + r;
-        src[r * (NCP + 1) + k] = P < le ? (T)L[(size_t)P * NCP + k] : T(0);
-    }
-    __syncthreads();
-    if constexpr (sizeof(T) == 8) {
-        // FP64 (bound by the FP64 pipe): lane = parent, every lane on the same row b
-        const int P = b0 + lane;
-        if (P >= le || abox_is_leaf(av, P)) return;
-        int ch[8];
-#pragma unroll
-        for (int c = 0; c < 8; ++c) ch[c] = av.child[8 * P + c];
-        for (int b = w; b < NC; b += 8) {
-            T R[8];
-            l2l_row(tab, b, src + lane * (NCP + 1), R);
-#pragma unroll
-            for (int c = 0; c < 8; ++c)
-                if (ch[c] >= 0 && DAFMM_IN(ch[c], av.nbox, kChkBoxIndex)) L[(size_t)ch[c] * NCP + b] += (double)R[c];
-        }
-        return;
-    }
-    // FP32: warp w takes parents w, w + 8, ...; its lanes take consecutive rows b, so that the
-    // read-modify-write of each child's row is one coalesced access per warp instead of 32
-    // scattered ones (an ncu capture of the lane-per-parent form: long-scoreboard stalls 14 per
-    // issue, the L2 hit rate 45 %; clustered N = 4e6, p = 10: L2L 3.69 -> 3.26 ms)
-    for (int r = w; r < 32; r += 8) {
-        const int P = b0 + r;
-        if (P >= le || abox_is_leaf(av, P)) continue;
-        int ch[8];
-#pragma unroll
-        for (int c = 0; c < 8; ++c) ch[c] = av.child[8 * P + c];
-        const T* srow = src + r * (NCP + 1);
-        for (int b = lane; b < NC; b += 32) {
-            T R[8];
-            l2l_row(tab, b, srow, R);
-#pragma unroll
-            for (int c = 0; c < 8; ++c)
-                if (ch[c] >= 0 && DAFMM_IN(ch[c], av.nbox, kChkBoxIndex)) L[(size_t)ch[c] * NCP + b] += (double)R[c];
-        }
-    }
 }
 
 // leaves: P2P over the U list, M2P over the W list, L2P of the leaf's local expansion
@@ -2045,45 +2014,61 @@ static cudaError_t p2m_launch(const TreeView& tv, int prec, double* M, const F16
     return cudaGetLastError();
 }
 
-static cudaError_t m2m_launch(const OrderData& od, int prec, int lc, const double* Mc, double* Mp,
-                              cudaStream_t s) {
+template <class T, bool H, class Fam>
+static cudaError_t m2m_run(const ShiftTab& tab, const Fam& fam, const double* Mc, double* Mp, int rows32,
+                           cudaStream_t s) {
+    const size_t smem = m2m_smem<T, H>(H ? tab.nnz : 0);
+    const cudaError_t e = set_smem(k_m2m<T, H, Fam>, smem);
+    if (e != cudaSuccess) return e;
+    k_m2m<T, H, Fam><<<(fam.n + kM2MParents - 1) / kM2MParents, 256, smem, s>>>(tab, fam, Mc, Mp, rows32);
+    return cudaGetLastError();
+}
+
+template <class Fam>
+static cudaError_t m2m_any(const OrderData& od, int prec, const Fam& fam, const double* Mc, double* Mp,
+                           cudaStream_t s) {
     const int rows32 = (prec & kRowsF32) ? 1 : 0;
-    const int harm = (prec & kRowsHarm) ? 1 : 0;
+    const bool harm = (prec & kRowsHarm) != 0;
     prec &= ~(kRowsF32 | kRowsHarm);
     if (harm && (prec == DAFMM_FP64 || prec == DAFMM_FF || !od.m2mh_rowptr)) return cudaErrorInvalidValue;
-    const int Pc = 1 << (lc - 1);
-    const int nparent = Pc * Pc * Pc;
-    const bool f32 = prec == DAFMM_FP32;
-    const ShiftTab tab = harm ? od.m2mh() : od.m2m();
-    cudaError_t e;
-    if (!f32) {
-        constexpr int PP = m2m_parents<double>();
-        if ((e = set_smem(k_m2m<double>, m2m_smem<double>())) != cudaSuccess) return e;
-        k_m2m<double><<<(nparent + PP - 1) / PP, 256, m2m_smem<double>(), s>>>(tab, lc, Mc, Mp, 0, harm);
-    } else {
-        constexpr int PP = m2m_parents<float>();
-        if ((e = set_smem(k_m2m<float>, m2m_smem<float>())) != cudaSuccess) return e;
-        k_m2m<float><<<(nparent + PP - 1) / PP, 256, m2m_smem<float>(), s>>>(tab, lc, Mc, Mp, rows32, harm);
+    if (prec != DAFMM_FP32)
+        return harm ? m2m_run<double, true>(od.m2mh(), fam, Mc, Mp, 0, s)
+                    : m2m_run<double, false>(od.m2m(), fam, Mc, Mp, 0, s);
+    return harm ? m2m_run<float, true>(od.m2mh(), fam, Mc, Mp, rows32, s)
+                : m2m_run<float, false>(od.m2m(), fam, Mc, Mp, rows32, s);
+}
+
+static cudaError_t m2m_launch(const OrderData& od, int prec, int lc, const double* Mc, double* Mp,
+                              cudaStream_t s) {
+    return m2m_any(od, prec, ShiftUniform{lc, 1 << (3 * (lc - 1))}, Mc, Mp, s);
+}
+
+// most table entries in one block's rows of the L2L
+static int l2l_max_entries() {
+    int mx = 1;
+    for (int b = 0; b < NC; b += kL2LRows) {
+        const int e = b + kL2LRows < NC ? b + kL2LRows : NC;
+        const int n = gen::GENT(l2l, _rowptr)[e] - gen::GENT(l2l, _rowptr)[b];
+        if (n > mx) mx = n;
     }
+    return mx;
+}
+
+template <class T, class Fam>
+static cudaError_t l2l_run(const ShiftTab& tab, const Fam& fam, const double* Lp, double* Lc, cudaStream_t s) {
+    static const int maxe = (l2l_max_entries() + 3) & ~3;
+    const size_t smem = l2l_smem<T>(maxe);
+    const cudaError_t e = set_smem(k_l2l<T, Fam>, smem);
+    if (e != cudaSuccess) return e;
+    const dim3 grd((fam.n + 31) / 32, (NC + kL2LRows - 1) / kL2LRows);
+    k_l2l<T, Fam><<<grd, 32 * kL2LRows, smem, s>>>(tab, fam, maxe, Lp, Lc);
     return cudaGetLastError();
 }
 
 static cudaError_t l2l_launch(const OrderData& od, int prec, int lc, const double* Lp, double* Lc,
                               cudaStream_t s) {
-    const int Pc = 1 << (lc - 1);
-    const int nparent = Pc * Pc * Pc;
-    const bool f32 = prec == DAFMM_FP32;
-    const size_t smem = (size_t)32 * (NCP + 1) * (f32 ? 4 : 8);
-    cudaError_t e;
-    dim3 grd((nparent + 31) / 32);
-    if (!f32) {
-        if ((e = set_smem(k_l2l<double>, smem)) != cudaSuccess) return e;
-        k_l2l<double><<<grd, 256, smem, s>>>(od.l2l(), lc, Lp, Lc);
-    } else {
-        if ((e = set_smem(k_l2l<float>, smem)) != cudaSuccess) return e;
-        k_l2l<float><<<grd, 256, smem, s>>>(od.l2l(), lc, Lp, Lc);
-    }
-    return cudaGetLastError();
+    const ShiftUniform fam{lc, 1 << (3 * (lc - 1))};
+    return prec == DAFMM_FP32 ? l2l_run<float>(od.l2l(), fam, Lp, Lc, s) : l2l_run<double>(od.l2l(), fam, Lp, Lc, s);
 }
 
 static cudaError_t m2l_launch(const OrderData& od, int prec, int l, const double* M, const float* Mf,
@@ -2219,25 +2204,10 @@ static cudaError_t p2m_a_launch(const AdaptiveView& av, const int* leaves, int n
     return cudaGetLastError();
 }
 
-static cudaError_t m2m_a_launch(const OrderData& od, const AdaptiveView& av, int prec, int lb, int le, double* M,
-                                cudaStream_t s) {
-    if (le <= lb) return cudaSuccess;
-    const int harm = (prec & kRowsHarm) ? 1 : 0;
-    prec &= ~kRowsHarm;
-    if (harm && (prec == DAFMM_FP64 || prec == DAFMM_FF || !od.m2mh_rowptr)) return cudaErrorInvalidValue;
-    const bool f32 = prec == DAFMM_FP32;
-    const ShiftTab tab = harm ? od.m2mh() : od.m2m();
-    cudaError_t e;
-    if (!f32) {
-        constexpr int PP = m2m_parents<double>();
-        if ((e = set_smem(k_m2m_a<double>, m2m_smem<double>())) != cudaSuccess) return e;
-        k_m2m_a<double><<<(le - lb + PP - 1) / PP, 256, m2m_smem<double>(), s>>>(tab, av, lb, le, M, harm);
-    } else {
-        constexpr int PP = m2m_parents<float>();
-        if ((e = set_smem(k_m2m_a<float>, m2m_smem<float>())) != cudaSuccess) return e;
-        k_m2m_a<float><<<(le - lb + PP - 1) / PP, 256, m2m_smem<float>(), s>>>(tab, av, lb, le, M, harm);
-    }
-    return cudaGetLastError();
+static cudaError_t m2m_a_launch(const OrderData& od, const AdaptiveView& av, int prec, const int* parents, int np,
+                                double* M, cudaStream_t s) {
+    if (np <= 0) return cudaSuccess;
+    return m2m_any(od, prec, ShiftAdaptive{av, parents, np}, M, M, s);
 }
 
 static cudaError_t m2l_a_launch(const OrderData& od, const AdaptiveView& av, int prec, const int* tg,
@@ -2290,21 +2260,11 @@ static cudaError_t p2l_a_launch(const AdaptiveView& av, int prec, int lb, int le
     return cudaGetLastError();
 }
 
-static cudaError_t l2l_a_launch(const OrderData& od, const AdaptiveView& av, int prec, int lb, int le, double* L,
-                                cudaStream_t s) {
-    if (le <= lb) return cudaSuccess;
-    const bool f32 = prec == DAFMM_FP32;
-    const size_t smem = (size_t)32 * (NCP + 1) * (f32 ? 4 : 8);
-    dim3 grd((le - lb + 31) / 32);
-    cudaError_t e;
-    if (!f32) {
-        if ((e = set_smem(k_l2l_a<double>, smem)) != cudaSuccess) return e;
-        k_l2l_a<double><<<grd, 256, smem, s>>>(od.l2l(), av, lb, le, L);
-    } else {
-        if ((e = set_smem(k_l2l_a<float>, smem)) != cudaSuccess) return e;
-        k_l2l_a<float><<<grd, 256, smem, s>>>(od.l2l(), av, lb, le, L);
-    }
-    return cudaGetLastError();
+static cudaError_t l2l_a_launch(const OrderData& od, const AdaptiveView& av, int prec, const int* parents, int np,
+                                double* L, cudaStream_t s) {
+    if (np <= 0) return cudaSuccess;
+    const ShiftAdaptive fam{av, parents, np};
+    return prec == DAFMM_FP32 ? l2l_run<float>(od.l2l(), fam, L, L, s) : l2l_run<double>(od.l2l(), fam, L, L, s);
 }
 
 static cudaError_t leaf_a_launch(const AdaptiveView& av, const int* leaves, int nleaves, int prec, const double* L,

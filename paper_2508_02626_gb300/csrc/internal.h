@@ -65,6 +65,8 @@ struct ShiftTab {                 // compressed rows of a level-independent M2M 
     const double* val;
     const float* valf;
     const int* rp8;               // [nc * 8 + 1]: start of the entries of (row, parity class)
+    const unsigned short* ord = nullptr;  // the rows by decreasing length (null: as they are)
+    int nnz = 0;                  // (harmonic M2M table only)
 };
 
 struct MulTab {                   // DA product table for the K generation
@@ -84,7 +86,10 @@ struct OrderData {
     double* l2l_val = nullptr; float* l2l_valf = nullptr;
     int* m2m_rp8 = nullptr; int* l2l_rp8 = nullptr;
     // the M2M of harmonic multipoles (free rows composed with the expansion from the free
-    // coefficients; no rp8 runs)
+    // coefficients; rows and columns by free index; no rp8 runs; m2mh_ord: rows by decreasing
+    // length)
+    unsigned short* m2mh_ord = nullptr;
+    int m2mh_nnz = 0;
     int* m2mh_rowptr = nullptr; unsigned short* m2mh_col = nullptr; unsigned char* m2mh_par = nullptr;
     double* m2mh_val = nullptr; float* m2mh_valf = nullptr;
     // F16 splits of the M2L matrices with their power-of-two row and matrix factors
@@ -138,7 +143,7 @@ struct OrderData {
     float2* ax_valf = nullptr;
     ShiftTab m2m() const { return ShiftTab{m2m_rowptr, m2m_col, m2m_par, m2m_val, m2m_valf, m2m_rp8}; }
     ShiftTab l2l() const { return ShiftTab{l2l_rowptr, l2l_col, l2l_par, l2l_val, l2l_valf, l2l_rp8}; }
-    ShiftTab m2mh() const { return ShiftTab{m2mh_rowptr, m2mh_col, m2mh_par, m2mh_val, m2mh_valf, nullptr}; }
+    ShiftTab m2mh() const { return ShiftTab{m2mh_rowptr, m2mh_col, m2mh_par, m2mh_val, m2mh_valf, nullptr, m2mh_ord, m2mh_nnz}; }
     MulTab mul() const { return MulTab{mul_rowptr, mul_pairs, mul_minus}; }
 };
 
@@ -215,12 +220,15 @@ struct OrderOps {
                             const double* in, double* out, cudaStream_t);
     // adaptive trees
     cudaError_t (*p2m_a)(const AdaptiveView&, const int* leaves, int nleaves, int prec, double* M, cudaStream_t);
-    cudaError_t (*m2m_a)(const OrderData&, const AdaptiveView&, int prec, int lb, int le, double* M, cudaStream_t);
+    // parents: the np boxes of one level that have children
+    cudaError_t (*m2m_a)(const OrderData&, const AdaptiveView&, int prec, const int* parents, int np, double* M,
+                         cudaStream_t);
     cudaError_t (*m2l_a)(const OrderData&, const AdaptiveView&, int prec, const int* tg, const int* grp_ptr, int grp0,
                          int max_group, const double* M, const float* Mf, double* L, cudaStream_t);
     cudaError_t (*p2l_a)(const AdaptiveView&, int prec, int lb, int le, double* L, cudaStream_t);
-    // L2L from the parents [lb, le) of one level into their children
-    cudaError_t (*l2l_a)(const OrderData&, const AdaptiveView&, int prec, int lb, int le, double* L, cudaStream_t);
+    // L2L from the parents of one level into their children
+    cudaError_t (*l2l_a)(const OrderData&, const AdaptiveView&, int prec, const int* parents, int np, double* L,
+                         cudaStream_t);
     cudaError_t (*leaf_a)(const AdaptiveView&, const int* leaves, int nleaves, int prec, const double* L,
                           const double* M, const float* Mf, double* phi, double* field, int warps, cudaStream_t);
     // the M2L by rotation of a uniform tree's level in float-float (DAFMM_FF; tables rot_Tf,

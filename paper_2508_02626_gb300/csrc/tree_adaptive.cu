@@ -545,9 +545,22 @@ __global__ void k_leaf_flags(const int* __restrict__ child, int nbox, int* flags
     flags[b] = leaf ? 1 : 0;
 }
 
-__global__ void k_scatter_flagged(const int* __restrict__ flags, const int* __restrict__ offs, int nbox, int* out) {
+__global__ void k_scatter_flagged(const int* __restrict__ flags, const int* __restrict__ offs, int nbox, int* out,
+                                  int* rest) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < nbox && flags[b]) out[offs[b]] = b;
+    if (b >= nbox) return;
+    if (flags[b]) out[offs[b]] = b;
+    else rest[b - offs[b]] = b;
+}
+
+__global__ void k_parent_starts(LevelStarts ls, int nlev, const int* __restrict__ offs, int* out) {
+    const int l = threadIdx.x;
+    if (l <= nlev) out[l] = ls.v[l] - offs[ls.v[l]];
+}
+
+cudaError_t launch_parent_starts(const LevelStarts& ls, int nlev, const int* offs, int* out, cudaStream_t s) {
+    k_parent_starts<<<1, 32, 0, s>>>(ls, nlev, offs, out);
+    return cudaGetLastError();
 }
 
 // group key (level, octant) of the boxes of levels >= 2; other boxes sort last
@@ -579,9 +592,9 @@ cudaError_t launch_leaf_flags(const int* child, int nbox, int* flags, cudaStream
     return cudaGetLastError();
 }
 
-cudaError_t launch_scatter_flagged(const int* flags, const int* offs, int nbox, int* out, cudaStream_t s) {
+cudaError_t launch_scatter_flagged(const int* flags, const int* offs, int nbox, int* out, int* rest, cudaStream_t s) {
     if (nbox == 0) return cudaSuccess;
-    k_scatter_flagged<<<(nbox + 255) / 256, 256, 0, s>>>(flags, offs, nbox, out);
+    k_scatter_flagged<<<(nbox + 255) / 256, 256, 0, s>>>(flags, offs, nbox, out, rest);
     return cudaGetLastError();
 }
 

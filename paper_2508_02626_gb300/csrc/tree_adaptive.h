@@ -87,7 +87,14 @@ cudaError_t launch_gather_adaptive(const double* xyz, const double* q, const int
                                    double* y, double* z, double* qs, float4* xq, size_t xq_n4, int64_t n, cudaStream_t s);
 
 cudaError_t launch_leaf_flags(const int* child, int nbox, int* flags, cudaStream_t s);
-cudaError_t launch_scatter_flagged(const int* flags, const int* offs, int nbox, int* out, cudaStream_t s);
+// box b of flag 1 to out[offs[b]], of flag 0 to rest[b - offs[b]] (offs: exclusive scan of flags)
+cudaError_t launch_scatter_flagged(const int* flags, const int* offs, int nbox, int* out, int* rest, cudaStream_t s);
+// first box of each level, plus the end
+struct LevelStarts {
+    int v[kMaxAdaptiveDepth + 2];
+};
+// out[l] = boxes with children before level l, l = 0 .. nlev (offs: leaves before each box)
+cudaError_t launch_parent_starts(const LevelStarts& ls, int nlev, const int* offs, int* out, cudaStream_t s);
 cudaError_t launch_group_keys(const int* level, const int* ijk, int nbox, uint64_t* keys, int* vals, cudaStream_t s);
 cudaError_t launch_group_ptr(const uint64_t* keys, int n, int ngroups, int* ptr, cudaStream_t s);
 
