@@ -104,12 +104,6 @@ __device__ __forceinline__ void warp_row_to_f32(const double* __restrict__ row, 
     for (int k = lane; k < NC; k += 32) buf[k] = (float)row[k];
     __syncwarp();
 }
-// ... or an FP32 row
-__device__ __forceinline__ void warp_row_f32(const float* __restrict__ row, float* buf, int lane) {
-    __syncwarp();
-    for (int k = lane; k < NC; k += 32) buf[k] = row[k];
-    __syncwarp();
-}
 
 // ---- P2M ---------------------------------------------------------------------------------
 // rows32: the multipole rows are FP32 (NCP floats per leaf) instead of FP64.  The FP32 kernel
@@ -895,33 +889,19 @@ __device__ __forceinline__ float rsqrt_or_zero(float x) {
     return x >= 1.17549435e-38f ? y : 0.f;
 }
 
-// Shared-memory source list of the near field, in the target leaf's frame: pair p of the list
-// (records 2p and 2p + 1) occupies four float4s from buf[4p]:
-//   (X, X', Y, Y')  (Z, Z', Q, Q')      offsets and charges rounded to FP32
-//   (x, x', y, y')  (z, z', q, q')      their FP32 remainders
-__device__ __forceinline__ void list_store(float4* buf, int j, float X, float Y, float Z, float Q, float xl,
-                                           float yl, float zl, float ql) {
-    float* f = reinterpret_cast<float*>(buf) + 16 * (j >> 1) + (j & 1);
-    f[0] = X;
-    f[2] = Y;
-    f[4] = Z;
-    f[6] = Q;
-    f[8] = xl;
-    f[10] = yl;
-    f[12] = zl;
-    f[14] = ql;
-}
-// a record that adds exactly nothing (q = 0, far from every target: finite 1/r, no guard needed)
-__device__ __forceinline__ void list_store_null(float4* buf, int j) {
-    list_store(buf, j, 4096.f, 4096.f, 4096.f, 0.f, 0.f, 0.f, 0.f, 0.f);
-}
+// Shared-memory source list of the near field, one segment of kSegPairs pairs of records per
+// warp, in the target leaf's frame and negated (a difference is then one addition), as four
+// planes of float4 so that a warp stores 32 pairs without bank conflicts:
+//   plane 0 (-X, -X', -Y, -Y')  1 (-Z, -Z', Q, Q')    offsets and charges rounded to FP32
+//         2 (-x, -x', -y, -y')  3 (-z, -z', q, q')    their FP32 remainders
+constexpr int kSegPairs = 64;
 
-// (H, L) = hi + lo shifted by d with the rounding of hi + d moved into L (Fast2Sum: exact when
+// (H, L) = -(hi + lo + d) with the rounding of hi + d moved into L (Fast2Sum: exact when
 // |d| >= |hi| or d = 0, which holds for the integer leaf offsets d in {-1, 0, 1} of a uniform
 // tree and |hi| <= 1/2)
-__device__ __forceinline__ void shift_exact(float hi, float lo, float d, float& H, float& L) {
-    H = hi + d;
-    L = lo + (hi - (H - d));
+__device__ __forceinline__ void shift_neg(float hi, float lo, float d, float& H, float& L) {
+    H = -hi - d;
+    L = (-hi - (H + d)) - lo;
 }
 // (H, L) = (hi + lo) * r + oh for a power of two r, with the rounding of hi * r + oh moved into L
 // (TwoSum: exact for any ordering of the two terms)
@@ -933,134 +913,191 @@ __device__ __forceinline__ void scale_shift_exact(float hi, float lo, float r, f
     L = fmaf(lo, r, err);
 }
 
-// pairs of the list per close-pair vote (the unguarded passes)
-#ifndef DAFMM_P2P_GROUP
-#define DAFMM_P2P_GROUP 2
-#endif
+// pair `pair` of the records into slot j of the segment, scaled by r and shifted by (ox, oy, oz)
+// (UNIT: r = 1 and integer offsets -- the leaves of a uniform tree)
+template <bool UNIT>
+__device__ __forceinline__ void stage_pair(float4* buf, int j, const float4* __restrict__ xq,
+                                           const float4* __restrict__ xl, int pair, float r, float ox, float oy,
+                                           float oz) {
+    const float4 a = xq[2 * pair], b = xq[2 * pair + 1], c = xl[2 * pair], d = xl[2 * pair + 1];
+    float4 A, B, C, D;
+    if constexpr (UNIT) {
+        shift_neg(a.x, c.x, ox, A.x, C.x);
+        shift_neg(a.y, c.y, ox, A.y, C.y);
+        shift_neg(a.z, c.z, oy, A.z, C.z);
+        shift_neg(a.w, c.w, oy, A.w, C.w);
+        shift_neg(b.x, d.x, oz, B.x, D.x);
+        shift_neg(b.y, d.y, oz, B.y, D.y);
+    } else {
+        scale_shift_exact(-a.x, -c.x, r, -ox, A.x, C.x);
+        scale_shift_exact(-a.y, -c.y, r, -ox, A.y, C.y);
+        scale_shift_exact(-a.z, -c.z, r, -oy, A.z, C.z);
+        scale_shift_exact(-a.w, -c.w, r, -oy, A.w, C.w);
+        scale_shift_exact(-b.x, -d.x, r, -oz, B.x, D.x);
+        scale_shift_exact(-b.y, -d.y, r, -oz, B.y, D.y);
+    }
+    B.z = b.z;
+    B.w = b.w;
+    D.z = d.z;
+    D.w = d.w;
+    buf[j] = A;
+    buf[kSegPairs + j] = B;
+    buf[2 * kSegPairs + j] = C;
+    buf[3 * kSegPairs + j] = D;
+}
+
+// the pairs of up to 32 source leaves (lane e: np pairs from pair0, their scale and shift), end to
+// end, segment by segment: the warp stages each segment -- every lane finds the leaf of its pair
+// in the prefix sums, so that leaves of any size fill the lanes -- and body(first pair, pairs)
+// works on it
+template <bool UNIT, class Body>
+__device__ __forceinline__ void near_segments(float4* buf, const float4* __restrict__ xq,
+                                              const float4* __restrict__ xl, int np, int pair0, float r, float ox,
+                                              float oy, float oz, int lane, Body&& body) {
+    int incl = np;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += v;
+    }
+    const int total = __shfl_sync(0xffffffffu, incl, 31), at0 = pair0 - (incl - np);
+    for (int seg0 = 0; seg0 < total; seg0 += kSegPairs) {
+        const int segn = min(kSegPairs, total - seg0);
+        __syncwarp();  // the previous segment is no longer read
+#pragma unroll
+        for (int k = 0; k < kSegPairs; k += 32) {
+            const int j = seg0 + k + lane;
+            int e = 0;  // the first leaf with incl > j
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) {
+                const int v = __shfl_sync(0xffffffffu, incl, e + d - 1);
+                if (v <= j) e += d;
+            }
+            const int pair = __shfl_sync(0xffffffffu, at0, e) + j;
+            const float er = UNIT ? 1.f : __shfl_sync(0xffffffffu, r, e);
+            const float ex = __shfl_sync(0xffffffffu, ox, e), ey = __shfl_sync(0xffffffffu, oy, e),
+                        ez = __shfl_sync(0xffffffffu, oz, e);
+            if (k + lane < segn) stage_pair<UNIT>(buf, k + lane, xq, xl, pair, er, ex, ey, ez);
+        }
+        __syncwarp();
+        body(seg0, segn);
+    }
+}
 
 // a pair closer than this (in leaf widths of the target's leaf) takes the remainders of its
 // offsets into its difference: beyond it, T - S alone is within a few FP32 roundings of the
 // difference's own size (the remainders are below 2^-23 leaf widths)
 constexpr float kCloseR2 = 0.01f;
 
-// list pairs [p0, p1) acting on the target t = T + tl (T: rounded offsets, tl: remainders,
-// in the list's frame), both halves of every step in one packed FP32x2 instruction: per half
-//   e = T - S  (+ (tl - sl) when |e| < 0.1),  r2 = fma(ex, ex, fma(ey, ey, ez ez)),
-//   qr = q / r,  qr3 = qr / r^2,
-// and the halves accumulate separately in P (potential) and X, Y, Z (field without its sign
-// convention).  e carries the difference of the two particles to a few FP32 roundings of
-// itself however close they are: pairs closer than 0.1 leaf widths -- rare, so the remainders
-// are loaded and added only in an iteration where a lane of the warp has one -- take the
-// remainders.  GUARD (the target's own leaf, which holds the target and any coincident
-// particles) always takes them and gives r = 0 no contribution; without it r2 starts from the
-// smallest normal float, so distinct particles -- which never coincide across leaves --
-// always give a finite 1/r.
-// one pair of the list: its difference e (T - S, plus the remainders for the target's own
-// leaf) and r^2
-template <bool GUARD>
-__device__ __forceinline__ void p2p_diff(const float4* __restrict__ buf, int p, float2 tx, float2 ty, float2 tz,
-                                         float2 lx, float2 ly, float2 lz, float2& ex, float2& ey, float2& ez,
-                                         float2& r2, float2& q) {
-    const float2 m1 = make_float2(-1.f, -1.f);
-    const float4 A = buf[4 * p], B = buf[4 * p + 1];
-    ex = __ffma2_rn(make_float2(A.x, A.y), m1, tx);
-    ey = __ffma2_rn(make_float2(A.z, A.w), m1, ty);
-    ez = __ffma2_rn(make_float2(B.x, B.y), m1, tz);
-    q = make_float2(B.z, B.w);
-    if (GUARD) {
-        const float4 C = buf[4 * p + 2], D = buf[4 * p + 3];
-        ex = __fadd2_rn(ex, __ffma2_rn(make_float2(C.x, C.y), m1, lx));
-        ey = __fadd2_rn(ey, __ffma2_rn(make_float2(C.z, C.w), m1, ly));
-        ez = __fadd2_rn(ez, __ffma2_rn(make_float2(D.x, D.y), m1, lz));
-        r2 = __fmul2_rn(ez, ez);
-    } else {
-        r2 = __ffma2_rn(ez, ez, make_float2(1.17549435e-38f, 1.17549435e-38f));
-    }
-    r2 = __ffma2_rn(ey, ey, r2);
-    r2 = __ffma2_rn(ex, ex, r2);
+// a target: its offset in the leaf's frame (splat for the packed instructions) and the remainders
+struct NearTarget {
+    float2 tx, ty, tz;
+    float lx, ly, lz;
+};
+__device__ __forceinline__ NearTarget near_target(const float4* __restrict__ xq, const float4* __restrict__ xl, int r) {
+    const float4 t = xq_load(xq, r), l = xq_load(xl, r);
+    return NearTarget{make_float2(t.x, t.x), make_float2(t.y, t.y), make_float2(t.z, t.z), l.x, l.y, l.z};
+}
+
+// running sums of one target: potential and field (without its sign convention), the two
+// sources of a packed instruction separately
+struct NearSums {
+    float2 P, X, Y, Z;
+};
+
+__device__ __forceinline__ float2 splat2(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 norm2(float2 ex, float2 ey, float2 ez, float2 r0) {
+    return __ffma2_rn(ex, ex, __ffma2_rn(ey, ey, __ffma2_rn(ez, ez, r0)));
+}
+
+// the remainders of list pair p in the difference of target t
+__device__ __forceinline__ void near_rest(const float4* buf, int p, const NearTarget& t, float2 ex, float2 ey,
+                                          float2 ez, float2& fx, float2& fy, float2& fz) {
+    const float4 C = buf[2 * kSegPairs + p], D = buf[3 * kSegPairs + p];
+    fx = __fadd2_rn(ex, __fadd2_rn(splat2(t.lx), make_float2(C.x, C.y)));
+    fy = __fadd2_rn(ey, __fadd2_rn(splat2(t.ly), make_float2(C.z, C.w)));
+    fz = __fadd2_rn(ez, __fadd2_rn(splat2(t.lz), make_float2(D.x, D.y)));
 }
 
 // a pair closer than 0.1 leaf widths takes the remainders into its difference (halves whose
 // r^2 is below kCloseR2; the others keep T - S)
-__device__ __forceinline__ void p2p_close(const float4* __restrict__ buf, int p, float2 lx, float2 ly, float2 lz,
-                                          float2& ex, float2& ey, float2& ez, float2& r2) {
-    const float2 m1 = make_float2(-1.f, -1.f);
-    const bool cx = r2.x < kCloseR2, cy = r2.y < kCloseR2;
-    const float4 C = buf[4 * p + 2], D = buf[4 * p + 3];
-    const float2 fx = __fadd2_rn(ex, __ffma2_rn(make_float2(C.x, C.y), m1, lx));
-    const float2 fy = __fadd2_rn(ey, __ffma2_rn(make_float2(C.z, C.w), m1, ly));
-    const float2 fz = __fadd2_rn(ez, __ffma2_rn(make_float2(D.x, D.y), m1, lz));
-    if (cx) {
+__device__ __forceinline__ void near_close(const float4* buf, int p, const NearTarget& t, float2& ex, float2& ey,
+                                           float2& ez, float2& r2) {
+    float2 fx, fy, fz;
+    near_rest(buf, p, t, ex, ey, ez, fx, fy, fz);
+    if (r2.x < kCloseR2) {
         ex.x = fx.x;
         ey.x = fy.x;
         ez.x = fz.x;
     }
-    if (cy) {
+    if (r2.y < kCloseR2) {
         ex.y = fx.y;
         ey.y = fy.y;
         ez.y = fz.y;
     }
-    r2 = __ffma2_rn(ez, ez, make_float2(1.17549435e-38f, 1.17549435e-38f));
-    r2 = __ffma2_rn(ey, ey, r2);
-    r2 = __ffma2_rn(ex, ex, r2);
+    r2 = norm2(ex, ey, ez, splat2(1.17549435e-38f));
 }
 
 // the pair's terms into the sums
 template <bool GUARD>
-__device__ __forceinline__ void p2p_acc(float2 ex, float2 ey, float2 ez, float2 r2, float2 q, float2& P, float2& X,
-                                        float2& Y, float2& Z) {
+__device__ __forceinline__ void near_add(float2 ex, float2 ey, float2 ez, float2 r2, float2 q, NearSums& s) {
     const float2 ir = GUARD ? make_float2(rsqrt_or_zero(r2.x), rsqrt_or_zero(r2.y))
                             : make_float2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
     const float2 qr = __fmul2_rn(q, ir);
     const float2 qr3 = __fmul2_rn(qr, __fmul2_rn(ir, ir));
-    P = __fadd2_rn(P, qr);
-    X = __ffma2_rn(qr3, ex, X);
-    Y = __ffma2_rn(qr3, ey, Y);
-    Z = __ffma2_rn(qr3, ez, Z);
+    s.P = __fadd2_rn(s.P, qr);
+    s.X = __ffma2_rn(qr3, ex, s.X);
+    s.Y = __ffma2_rn(qr3, ey, s.Y);
+    s.Z = __ffma2_rn(qr3, ez, s.Z);
 }
 
-// list pairs [p0, p1) acting on the target t = T + tl (T: rounded offsets, tl: remainders,
-// in the list's frame), both halves of every step in one packed FP32x2 instruction: per half
+// List pairs [p0, p1) of the segment acting on this lane's two targets, both sources of a pair in
+// one packed FP32x2 instruction: per source
 //   e = T - S  (+ (tl - sl) when |e| < 0.1),  r2 = fma(ex, ex, fma(ey, ey, ez ez)),
-//   qr = q / r,  qr3 = qr / r^2,
-// and the halves accumulate separately in P (potential) and X, Y, Z (field without its sign
-// convention).  e carries the difference of the two particles to a few FP32 roundings of
-// itself however close they are: pairs closer than 0.1 leaf widths -- rare -- take the
-// remainders, loaded and added only for a group of four pairs in which a lane of the warp has
-// one (one vote per group keeps the group's arithmetic in one stretch of code).  GUARD
-// (the target's own leaf, which holds the target and any coincident particles) always takes
-// them and gives r = 0 no contribution; without it r2 starts from the smallest normal float,
-// so distinct particles -- which never coincide across leaves -- always give a finite 1/r.
+//   qr = q / r,  qr3 = qr / r^2.
+// e carries the difference of the two particles to a few FP32 roundings of itself however close
+// they are: pairs closer than 0.1 leaf widths -- rare -- take the remainders, loaded and added only
+// in an iteration where a lane of the warp has one.  GUARD (the target's own leaf, which holds the
+// target and any coincident particles) always takes them and gives r = 0 no contribution; without
+// it r2 starts from the smallest normal float, so distinct particles -- which never coincide
+// across leaves -- always give a finite 1/r.  (A null record -- q = 0 at its leaf's centre -- adds
+// exactly nothing either way.)
+// Two targets per lane: the FP32 pipe needs 26 cycles per packed pair and target, and the two
+// 16-byte broadcast loads of a pair return 1 KB to the registers, 8 cycles of the SM's L1 -- 32
+// for its four partitions.  With one target per lane the L1 was the bound (ncu: L1 80 % busy, the
+// FMA pipe 48 %); two targets halve the loads per interaction.  With the conflict-free staging:
+// uniform N = 1e6, p = 8: the kernel 0.80 -> 0.63 ms (5 or 6 blocks per SM; 4: 0.68); clustered
+// N = 4e6, p = 10: 10.5 -> 8.1 ms; 64-problem forest, p = 6: 2.74 -> 2.06 ms.
 template <bool GUARD>
-__device__ __forceinline__ void p2p_pairs(const float4* __restrict__ buf, int p0, int p1, float2 tx, float2 ty,
-                                          float2 tz, float2 lx, float2 ly, float2 lz, float2& P, float2& X,
-                                          float2& Y, float2& Z) {
-    int p = p0;
-    if (!GUARD) {
-        constexpr int G = DAFMM_P2P_GROUP;
-        for (; p + G <= p1; p += G) {
-            float2 ex[G], ey[G], ez[G], r2[G], q[G];
-            float rmin = 3.0e38f;
+__device__ __forceinline__ void near_pairs(const float4* buf, int p0, int p1, const NearTarget (&t)[2],
+                                           NearSums (&s)[2]) {
+#pragma unroll 2
+    for (int p = p0; p < p1; ++p) {
+        const float4 A = buf[p], B = buf[kSegPairs + p];
+        const float2 sx = make_float2(A.x, A.y), sy = make_float2(A.z, A.w), sz = make_float2(B.x, B.y),
+                     q = make_float2(B.z, B.w);
+        float2 ex[2], ey[2], ez[2], r2[2];
 #pragma unroll
-            for (int k = 0; k < G; ++k) {
-                p2p_diff<false>(buf, p + k, tx, ty, tz, lx, ly, lz, ex[k], ey[k], ez[k], r2[k], q[k]);
-                rmin = fminf(rmin, fminf(r2[k].x, r2[k].y));
+        for (int u = 0; u < 2; ++u) {
+            ex[u] = __fadd2_rn(t[u].tx, sx);
+            ey[u] = __fadd2_rn(t[u].ty, sy);
+            ez[u] = __fadd2_rn(t[u].tz, sz);
+            if (GUARD) {
+                near_rest(buf, p, t[u], ex[u], ey[u], ez[u], ex[u], ey[u], ez[u]);
+                r2[u] = __ffma2_rn(ex[u], ex[u], __ffma2_rn(ey[u], ey[u], __fmul2_rn(ez[u], ez[u])));
+            } else {
+                r2[u] = norm2(ex[u], ey[u], ez[u], splat2(1.17549435e-38f));
             }
+        }
+        if (!GUARD) {
+            const float rmin = fminf(fminf(r2[0].x, r2[0].y), fminf(r2[1].x, r2[1].y));
             if (__any_sync(__activemask(), rmin < kCloseR2)) {
 #pragma unroll
-                for (int k = 0; k < G; ++k) p2p_close(buf, p + k, lx, ly, lz, ex[k], ey[k], ez[k], r2[k]);
+                for (int u = 0; u < 2; ++u) near_close(buf, p, t[u], ex[u], ey[u], ez[u], r2[u]);
             }
-#pragma unroll
-            for (int k = 0; k < G; ++k) p2p_acc<false>(ex[k], ey[k], ez[k], r2[k], q[k], P, X, Y, Z);
         }
-    }
-#pragma unroll 4
-    for (; p < p1; ++p) {
-        float2 ex, ey, ez, r2, q;
-        p2p_diff<GUARD>(buf, p, tx, ty, tz, lx, ly, lz, ex, ey, ez, r2, q);
-        if (!GUARD && __any_sync(__activemask(), r2.x < kCloseR2 || r2.y < kCloseR2))
-            p2p_close(buf, p, lx, ly, lz, ex, ey, ez, r2);
-        p2p_acc<GUARD>(ex, ey, ez, r2, q, P, X, Y, Z);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) near_add<GUARD>(ex[u], ey[u], ez[u], r2[u], q, s[u]);
     }
 }
 
@@ -1071,12 +1108,58 @@ __device__ __forceinline__ void two_sum_add(float& hi, float& lo, float v) {
     hi = s;
 }
 
-// compensated (hi, lo) sums of the near field: FP32 partial sums over at most 128 sources are
-// folded into them, so that long neighbour lists keep FP32-level error
+// compensated (hi, lo) sums of the near field: FP32 partial sums over at most 128 sources (one
+// segment) are folded into them, so that long neighbour lists keep FP32-level error
 struct CompSums {
     float ph = 0.f, pl = 0.f, xh = 0.f, xl = 0.f, yh = 0.f, yl = 0.f, zh = 0.f, zl = 0.f;
 };
 
+// The lanes of a pass over m <= 32 targets: groups of W lanes, lane l of a group with the targets
+// l and l + W, the groups sharing out the sources.  W = 16, 8 or 4, so that a pass costs about
+// m / 32 of a full one.
+__device__ __forceinline__ int near_width(int m) { return m > 16 ? 16 : (m > 8 ? 8 : 4); }
+
+// the pairwise sums of one segment of n pairs, the first `own` of the target's own leaf (guarded)
+__device__ __forceinline__ void near_segment(const float4* buf, int n, int own, int W, int lane,
+                                             const NearTarget (&t)[2], CompSums (&cs)[2]) {
+    own = max(0, min(own, n));
+    const int lg = __ffs(32 / W) - 1, g = lane / W;  // 2^lg groups
+    NearSums s[2] = {};
+    if (own > 0) {
+        const int h = (own + (1 << lg) - 1) >> lg, pa = min(g * h, own);
+        near_pairs<true>(buf, pa, min(pa + h, own), t, s);
+    }
+    const int h = (n - own + (1 << lg) - 1) >> lg, pa = min(own + g * h, n);
+    near_pairs<false>(buf, pa, min(pa + h, n), t, s);
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        two_sum_add(cs[u].ph, cs[u].pl, s[u].P.x + s[u].P.y);
+        two_sum_add(cs[u].xh, cs[u].xl, s[u].X.x + s[u].X.y);
+        two_sum_add(cs[u].yh, cs[u].yl, s[u].Y.x + s[u].Y.y);
+        two_sum_add(cs[u].zh, cs[u].zl, s[u].Z.x + s[u].Z.y);
+    }
+}
+
+// the groups' sums together: afterwards lane l < 2 W holds target l of the pass (the upper copies
+// hold the same)
+__device__ __forceinline__ CompSums near_join(const CompSums (&cs)[2], int W, int lane) {
+    const bool second = (lane & W) != 0;  // this lane's group keeps the targets l + W
+    const CompSums &keep = second ? cs[1] : cs[0], &give = second ? cs[0] : cs[1];
+    float k[8] = {keep.ph, keep.pl, keep.xh, keep.xl, keep.yh, keep.yl, keep.zh, keep.zl};
+    float v[8] = {give.ph, give.pl, give.xh, give.xl, give.yh, give.yl, give.zh, give.zl};
+    for (int d = W; d < 32; d <<= 1) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = __shfl_xor_sync(0xffffffffu, d == W ? v[j] : k[j], d);
+#pragma unroll
+        for (int j = 0; j < 8; j += 2) {
+            two_sum_add(k[j], k[j + 1], v[j]);
+            k[j + 1] += v[j + 1];
+        }
+    }
+    CompSums r;
+    r.ph = k[0]; r.pl = k[1]; r.xh = k[2]; r.xl = k[3]; r.yh = k[4]; r.yl = k[5]; r.zh = k[6]; r.zl = k[7];
+    return r;
+}
 
 // ---- float-float near field (the DAFMM_FF mode) ----
 // a cascaded float-float sum (as Ogita, Rump and Oishi's Sum2): the high parts through TwoSum,
@@ -1096,9 +1179,10 @@ struct FFSums {
 
 // the difference (T + tl) - (S + sl) in float-float: TwoSum of the rounded parts (exact), the
 // remainders' difference (below 2^-23 leaf widths, one FP32 rounding) added, renormalised
-__device__ __forceinline__ ff ff_diff(float T, float tl, float S, float sl) {
-    const ff d = two_sum(T, -S);
-    return two_sum(d.hi, d.lo + (tl - sl));
+// (the list holds -S and -sl)
+__device__ __forceinline__ ff ff_diff(float T, float tl, float nS, float nsl) {
+    const ff d = two_sum(T, nS);
+    return two_sum(d.hi, d.lo + (tl + nsl));
 }
 
 // list records [2 pa, 2 pe) acting on the target t = T + tl, every step in float-float (about
@@ -1110,7 +1194,7 @@ __device__ __forceinline__ void p2p_segment_ff(const float4* __restrict__ buf, i
                                                float ty, float tz, float tlx, float tly, float tlz, FFSums& acc) {
 #pragma unroll 1
     for (int p = pa; p < pe; ++p) {
-        const float4 A = buf[4 * p], B = buf[4 * p + 1], C = buf[4 * p + 2], D = buf[4 * p + 3];
+        const float4 A = buf[p], B = buf[kSegPairs + p], C = buf[2 * kSegPairs + p], D = buf[3 * kSegPairs + p];
         const bool own = p < pown;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -1135,53 +1219,10 @@ __device__ __forceinline__ ff ff_shfl_down(ff v, int d) {
     return ff(__shfl_down_sync(0xffffffffu, v.hi, d), __shfl_down_sync(0xffffffffu, v.lo, d));
 }
 
-// records per shared-memory segment of the neighbour list (per warp; 32 bytes each)
-#ifndef DAFMM_LEAF_SEG
-#define DAFMM_LEAF_SEG 128
-#endif
-constexpr int kLeafSeg = DAFMM_LEAF_SEG;
 // blocks per SM the uniform FP32 leaf kernel is compiled for (its register budget)
 #ifndef DAFMM_LEAF_MINB
-#define DAFMM_LEAF_MINB 8
+#define DAFMM_LEAF_MINB 5
 #endif
-
-// list pairs (two sources each) per FP32 partial sum of the near field: 64 pairs, 128 sources
-// (64 in each packed half) -- one fold per list segment of kLeafSeg = 128 records
-constexpr int kFoldPairs = 64;
-
-// the pairwise sums of one segment of the list: pairs [pa, pe) for this lane's target, those
-// below pown from the target's own leaf (guarded), FP32 partial sums over at most kFoldPairs
-// pairs folded into the compensated sums
-__device__ __forceinline__ void p2p_segment(const float4* __restrict__ buf, int pa, int pe, int pown, float2 tx,
-                                            float2 ty, float2 tz, float2 lx, float2 ly, float2 lz, CompSums& cs) {
-    for (int pb = pa; pb < pe; pb += kFoldPairs) {
-        const int pc = min(pe, pb + kFoldPairs);
-        const int pm = max(pb, min(pc, pown));
-        float2 P = make_float2(0.f, 0.f), X = P, Y = P, Z = P;
-        if (pb < pm) p2p_pairs<true>(buf, pb, pm, tx, ty, tz, lx, ly, lz, P, X, Y, Z);
-        if (pm < pc) p2p_pairs<false>(buf, pm, pc, tx, ty, tz, lx, ly, lz, P, X, Y, Z);
-        two_sum_add(cs.ph, cs.pl, P.x + P.y);
-        two_sum_add(cs.xh, cs.xl, X.x + X.y);
-        two_sum_add(cs.yh, cs.yl, Y.x + Y.y);
-        two_sum_add(cs.zh, cs.zl, Z.x + Z.y);
-    }
-}
-
-// the upper half-warp's sums join the lower one's (passes whose sources were split between
-// the half-warps)
-__device__ __forceinline__ void join_halves(CompSums& cs) {
-    float v[8] = {cs.ph, cs.pl, cs.xh, cs.xl, cs.yh, cs.yl, cs.zh, cs.zl};
-#pragma unroll
-    for (int j = 0; j < 8; ++j) v[j] = __shfl_down_sync(0xffffffffu, v[j], 16);
-    two_sum_add(cs.ph, cs.pl, v[0]);
-    cs.pl += v[1];
-    two_sum_add(cs.xh, cs.xl, v[2]);
-    cs.xl += v[3];
-    two_sum_add(cs.yh, cs.yl, v[4]);
-    cs.yl += v[5];
-    two_sum_add(cs.zh, cs.zl, v[6]);
-    cs.zl += v[7];
-}
 
 // the neighbour slot (0..26, slot 13 = the leaf itself) held by lane k of the list: the leaf
 // itself first, so that its records -- the only ones that can coincide with a target -- form
@@ -1225,49 +1266,40 @@ k_leaf(TreeView tv, const double* __restrict__ Lleaf,
             }
         }
     }
-    // FP32: the 27 neighbour leaves' particle ranges, one per lane (empty outside the domain),
-    // and the first FP32 record of each, laid end to end as one list: the leaf's own records
-    // first (lane 0), completed to an even count by a null record; lane k's neighbour starts
-    // at nb_off (exclusive scan of the counts over the lanes), nb_tot records in all, the
-    // first own_pairs pairs the leaf's own
-    int nb_n = 0, nb_r0 = 0, nb_off = 0, nb_tot = 0, n_own = 0, own_pad = 0, own_pairs = 0;
+    // FP32: the 27 neighbour leaves, one per lane (none outside the domain): their pairs of
+    // records -- an odd leaf's last pair ends in its null record -- and their offsets in leaf
+    // widths; the leaf itself first (lane 0), its pairs the guarded head of the list
+    int nb_np = 0, nb_pair = 0, own_pairs = 0;
+    float nb_x = 0.f, nb_y = 0.f, nb_z = 0.f;
     if constexpr (!std::is_same<T, double>::value) {
-        int nb_s0 = 0, nb_s1 = 0;
         if (lane < 27) {
             const int slot = own_first_slot(lane);
             const int dx = slot % 3 - 1, dy = (slot / 3) % 3 - 1, dz = slot / 9 - 1;
             const int na = a + dx, nb = b + dy, nc2 = c + dz;
             if (na >= 0 && nb >= 0 && nc2 >= 0 && na < nside && nb < nside && nc2 < nside) {
                 const int nl = octmajor_index(tv.depth, na, nb, nc2);
-                nb_s0 = tv.leaf_start[nl];
-                nb_s1 = tv.leaf_start[nl + 1];
+                int nb_s0 = tv.leaf_start[nl], nb_s1 = tv.leaf_start[nl + 1];
                 if (!DAFMM_RANGE(nb_s0, nb_s1, tv.n, kChkLeafRange)) nb_s0 = nb_s1 = 0;
-                nb_r0 = xq_base(nb_s0, nl);
+                nb_pair = xq_base(nb_s0, nl) >> 1;
+                nb_np = (nb_s1 - nb_s0 + 1) >> 1;
+                nb_x = (float)dx;
+                nb_y = (float)dy;
+                nb_z = (float)dz;
             }
         }
-        nb_n = nb_s1 - nb_s0;
-        nb_off = nb_n;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, nb_off, d);
-            if (lane >= d) nb_off += v;
-        }
-        n_own = __shfl_sync(0xffffffffu, nb_n, 0);
-        own_pad = n_own & 1;
-        nb_tot = __shfl_sync(0xffffffffu, nb_off, 31) + own_pad;
-        nb_off -= nb_n;
-        if (lane > 0) nb_off += own_pad;
-        own_pairs = (n_own + 1) >> 1;
+        own_pairs = __shfl_sync(0xffffffffu, nb_np, 0);
     }
     const int r_own = xq_base(i0, leaf) - i0;  // record of sorted position t: t + r_own
     for (int base = i0; base < i1; base += 32) {
-        // FP32: a pass of at most 16 targets splits the sources between the two half-warps,
-        // lane l and lane l + 16 taking the same target
         const int m = min(32, i1 - base);
-        const bool split = !std::is_same<T, double>::value && m <= 16;
-        const int tl = split ? (lane & 15) : lane;
+        // float-float: a pass of at most 16 targets splits the sources between the two half-warps,
+        // lane l and lane l + 16 taking the same target; FP32: see near_width
+        const bool split = std::is_same<T, ff>::value && m <= 16;
+        const int W = near_width(m);
+        const int per = std::is_same<T, float>::value ? 2 * W : (split ? 16 : 32);
+        const int tl = lane & (per - 1);
         const int t = base + tl;
-        const bool valid = tl < m && (!split || lane < 16);  // the lanes that write
+        const bool valid = tl < m && lane < per;  // the lanes that write
         const int tt = tl < m ? t : i0;
         double fphi = 0.0, fx = 0.0, fy = 0.0, fz = 0.0;  // near field, physical units
         if constexpr (std::is_same<T, double>::value) {
@@ -1294,62 +1326,33 @@ k_leaf(TreeView tv, const double* __restrict__ Lleaf,
                     }
         } else {
             const float4* xl = tv.xq + xq_records(tv.n, tv.nleaf);  // the remainder records
-            const float4 pt = xq_load(tv.xq, tt + r_own), pl = xq_load(xl, tt + r_own);
-            CompSums cs;
-            FFSums fs;
             // The neighbours' records are copied into one shared-memory list, shifted into this
             // leaf's frame (source + neighbour offset, in leaf widths, exactly: the rounding of
-            // the shift joins the remainder), in segments of up to kLeafSeg records; the pairwise
-            // sum then runs over the whole list.  A pass of at most 16 targets gives each
-            // half-warp half of the pairs.
-            __shared__ __align__(16) float4 s_list[4][2 * kLeafSeg];
+            // the shift joins the remainder); the pairwise sum runs over each segment of it.
+            __shared__ __align__(16) float4 s_list[4][4 * kSegPairs];
             float4* buf = s_list[threadIdx.y];
-            const int g = split ? lane >> 4 : 0;
-            const float2 tx2 = make_float2(pt.x, pt.x), ty2 = make_float2(pt.y, pt.y),
-                         tz2 = make_float2(pt.z, pt.z);
-            const float2 lx2 = make_float2(pl.x, pl.x), ly2 = make_float2(pl.y, pl.y),
-                         lz2 = make_float2(pl.z, pl.z);
-            for (int seg0 = 0; seg0 < nb_tot; seg0 += kLeafSeg) {
-                const int segn = min(kLeafSeg, nb_tot - seg0), seg1 = seg0 + segn;
-                __syncwarp();  // the previous segment is no longer read
-                // the neighbours whose records fall into this segment
-                unsigned ov = __ballot_sync(0xffffffffu, lane < 27 && nb_n > 0 && nb_off < seg1 && nb_off + nb_n > seg0);
-                while (ov) {
-                    const int k = __ffs(ov) - 1;
-                    ov &= ov - 1;
-                    const int o = __shfl_sync(0xffffffffu, nb_off, k), n = __shfl_sync(0xffffffffu, nb_n, k);
-                    const int r0 = __shfl_sync(0xffffffffu, nb_r0, k);
-                    const int slot = own_first_slot(k);
-                    const int lo = max(o, seg0), hi = min(o + n, seg1);
-                    const float dx = (float)(slot % 3 - 1), dy = (float)((slot / 3) % 3 - 1), dz = (float)(slot / 9 - 1);
-                    for (int i = lo + lane; i < hi; i += 32) {
-                        const float4 rec = xq_load(tv.xq, r0 + (i - o)), rl = xq_load(xl, r0 + (i - o));
-                        float X, Y, Z, XL, YL, ZL;
-                        shift_exact(rec.x, rl.x, dx, X, XL);
-                        shift_exact(rec.y, rl.y, dy, Y, YL);
-                        shift_exact(rec.z, rl.z, dz, Z, ZL);
-                        list_store(buf, i - seg0, X, Y, Z, rec.w, XL, YL, ZL, rl.w);
-                    }
-                }
-                if (lane == 0) {
-                    if (own_pad && n_own >= seg0 && n_own < seg1) list_store_null(buf, n_own - seg0);
-                    if (segn & 1) list_store_null(buf, segn);  // completes the last pair
-                }
-                __syncwarp();
-                const int np = (segn + 1) >> 1, h = split ? (np + 1) >> 1 : np;
-                const int pa = g ? h : 0, pe = g ? np : h;
-                if constexpr (std::is_same<T, float>::value)
-                    p2p_segment(buf, pa, pe, own_pairs - (seg0 >> 1), tx2, ty2, tz2, lx2, ly2, lz2, cs);
-                else
-                    p2p_segment_ff(buf, pa, pe, own_pairs - (seg0 >> 1), pt.x, pt.y, pt.z, pl.x, pl.y, pl.z, fs);
+            CompSums cs[2], sum;
+            FFSums fs;
+            if constexpr (std::is_same<T, float>::value) {
+                const int l0 = lane & (W - 1);
+                const NearTarget nt[2] = {near_target(tv.xq, xl, (l0 < m ? base + l0 : i0) + r_own),
+                                          near_target(tv.xq, xl, (l0 + W < m ? base + l0 + W : i0) + r_own)};
+                near_segments<true>(buf, tv.xq, xl, nb_np, nb_pair, 1.f, nb_x, nb_y, nb_z, lane,
+                                    [&](int seg0, int n) { near_segment(buf, n, own_pairs - seg0, W, lane, nt, cs); });
+                sum = near_join(cs, W, lane);
+            } else {
+                const float4 pt = xq_load(tv.xq, tt + r_own), pl = xq_load(xl, tt + r_own);
+                near_segments<true>(buf, tv.xq, xl, nb_np, nb_pair, 1.f, nb_x, nb_y, nb_z, lane, [&](int seg0, int n) {
+                    const int h = split ? (n + 1) >> 1 : n, g = split ? lane >> 4 : 0;
+                    p2p_segment_ff(buf, g ? h : 0, g ? n : h, own_pairs - seg0, pt.x, pt.y, pt.z, pl.x, pl.y, pl.z, fs);
+                });
             }
             const double ih = tv.inv_h_leaf, ih2 = ih * ih;
             if constexpr (std::is_same<T, float>::value) {
-                if (split) join_halves(cs);
-                fphi = ((double)cs.ph + (double)cs.pl) * ih;
-                fx = ((double)cs.xh + (double)cs.xl) * ih2;
-                fy = ((double)cs.yh + (double)cs.yl) * ih2;
-                fz = ((double)cs.zh + (double)cs.zl) * ih2;
+                fphi = ((double)sum.ph + (double)sum.pl) * ih;
+                fx = ((double)sum.xh + (double)sum.xl) * ih2;
+                fy = ((double)sum.yh + (double)sum.yl) * ih2;
+                fz = ((double)sum.zh + (double)sum.zl) * ih2;
             } else {
                 ff sp = fs.p.get(), sx = fs.x.get(), sy = fs.y.get(), sz = fs.z.get();
                 if (split) {  // the upper half-warp's sums join the lower one's
@@ -1687,19 +1690,23 @@ __global__ void __launch_bounds__(128) k_p2l_a(AdaptiveView av, int lb, int le, 
     for (int k = lane; k < NC; k += 32) L[(size_t)b * NCP + k] += (double)sm[k] * ih;
 }
 
+// per warp of the FP32 adaptive leaf kernel: the source list's segment (the M2P stages up to two
+// W boxes' multipoles in it afterwards), then the leaf's locals in FP32
+constexpr size_t kLeafWarpSmem = 4 * kSegPairs * sizeof(float4) + NCP * sizeof(float);
+static_assert(2 * NCP * sizeof(float) <= 4 * kSegPairs * sizeof(float4), "two rows fit the segment");
+
 // leaves: P2P over the U list, M2P over the W list, L2P of the leaf's local expansion
 template <class T>
-__global__ void __launch_bounds__(256) k_leaf_a(AdaptiveView av, const int* __restrict__ leaves, int nleaves,
-                                                const double* __restrict__ L, const double* __restrict__ M,
-                                                const float* __restrict__ Mf, double* __restrict__ phi,
-                                                double* __restrict__ field) {
-    __shared__ float s_rows[8][2][NCP];  // per warp: the W box's multipoles and the leaf's locals, FP32
-    extern __shared__ __align__(16) float4 s_list_a[];  // FP32: per warp kLeafSeg records (2 float4s each)
+__global__ void __launch_bounds__(256, 2) k_leaf_a(AdaptiveView av, const int* __restrict__ leaves, int nleaves,
+                                                   const double* __restrict__ L, const double* __restrict__ M,
+                                                   const float* __restrict__ Mf, double* __restrict__ phi,
+                                                   double* __restrict__ field) {
+    extern __shared__ __align__(16) unsigned char s_leaf[];
     const int lane = threadIdx.x;
     const int li = blockIdx.x * blockDim.y + threadIdx.y;
     if (li >= nleaves) return;
-    float* mrow = s_rows[threadIdx.y][0];
-    float* lrow = s_rows[threadIdx.y][1];
+    float4* buf = reinterpret_cast<float4*>(s_leaf + threadIdx.y * kLeafWarpSmem);
+    float* lrow = reinterpret_cast<float*>(buf + 4 * kSegPairs);
     const int b = leaves[li];
     if (!DAFMM_IN(b, av.nbox, kChkBoxIndex)) return;
     double cx, cy, cz, h;
@@ -1719,13 +1726,12 @@ __global__ void __launch_bounds__(256) k_leaf_a(AdaptiveView av, const int* __re
     if (!DAFMM_RANGE(u0, u1, av.nu, kChkListPtr)) u0 = u1 = 0;
     if (!DAFMM_RANGE(w0, w1, av.nw, kChkListPtr)) w0 = w1 = 0;
     for (int base = i0; base < i1; base += 32) {
-        // FP32: a pass of at most 16 targets splits the sources between the two half-warps,
-        // lane l and lane l + 16 taking the same target
         const int m = min(32, i1 - base);
-        const bool split = sizeof(T) == 4 && m <= 16;
-        const int tl = split ? (lane & 15) : lane;
+        const int W = near_width(m);  // FP32: the lanes' split, see near_width
+        const int per = sizeof(T) == 4 ? 2 * W : 32;
+        const int tl = lane & (per - 1);
         const int t = base + tl;
-        const bool valid = tl < m && (!split || lane < 16);  // the lanes that write
+        const bool valid = tl < m && lane < per;  // the lanes that write
         const int tt = tl < m ? t : i0;
         double fphi = 0.0, fx = 0.0, fy = 0.0, fz = 0.0;
         if constexpr (sizeof(T) == 8) {
@@ -1747,85 +1753,51 @@ __global__ void __launch_bounds__(256) k_leaf_a(AdaptiveView av, const int* __re
                 }
             }
         } else {
-            const float4 pt = xq_load(av.xq, av.xq0[b] + (tt - i0)), pl = xq_load(av.xl, av.xq0[b] + (tt - i0));
-            CompSums acc;  // in leaf widths of this leaf
             // The U-list leaves' records are copied into one shared-memory list in this leaf's
             // frame (source x h_s / h + centre offset / h, exactly: h_s / h is a power of two and
-            // the rounding of the sum joins the remainder), the leaf's own records first, in
-            // segments of up to kLeafSeg records; the pairwise sum runs over each segment.
-            float4* buf = s_list_a + (size_t)threadIdx.y * 2 * kLeafSeg;
-            const int g = split ? lane >> 4 : 0;
-            const float2 tx2 = make_float2(pt.x, pt.x), ty2 = make_float2(pt.y, pt.y),
-                         tz2 = make_float2(pt.z, pt.z);
-            const float2 lx2 = make_float2(pl.x, pl.x), ly2 = make_float2(pl.y, pl.y),
-                         lz2 = make_float2(pl.z, pl.z);
-            int fill = 0, done = 0, own_end = 0;  // records in the segment, before it, of the own leaf
-            auto flush = [&]() {
-                if ((fill & 1) && lane == 0) list_store_null(buf, fill);  // completes the last pair
-                __syncwarp();
-                const int np = (fill + 1) >> 1, hp = split ? (np + 1) >> 1 : np;
-                const int pa = g ? hp : 0, pe = g ? np : hp;
-                p2p_segment(buf, pa, pe, (own_end - done) >> 1, tx2, ty2, tz2, lx2, ly2, lz2, acc);
-                __syncwarp();  // the segment is no longer read
-                done += fill;
-                fill = 0;
-            };
+            // the rounding of the sum joins the remainder), 32 leaves at a time; the list begins
+            // with the leaf itself (the only records that can coincide with a target).
+            const int l0 = lane & (W - 1), rb = av.xq0[b] - i0;
+            const NearTarget nt[2] = {near_target(av.xq, av.xl, (l0 < m ? base + l0 : i0) + rb),
+                                      near_target(av.xq, av.xl, (l0 + W < m ? base + l0 + W : i0) + rb)};
+            CompSums cs[2];  // in leaf widths of this leaf
             const int* ijk_b = av.ijk + 3 * (size_t)b;
-            auto add_leaf = [&](int sb) {
-                // the source leaf's centre offset in this leaf's widths and its width ratio,
-                // from the integer box coordinates (same tree): with d = lev_b - lev_s,
-                // (c_s - c_b) / h_b = N / 2^(1 + max(0, -d)),
-                // N = (2 i_s + 1) 2^max(0, d) - (2 i_b + 1) 2^max(0, -d).  Levels go to 20, so both
-                // terms stay below 2^22, and adjacent boxes have |N| <= 2^|d| + 1 < 2^24: N is exact
-                // in an int and in a float (no remainder).  (64-bit N took nine conversions per list
-                // entry on the FP64 pipe, 1/64 of the FP32 rate here: 35 % of that pipe's cycles,
-                // Gaussian N = 1e6, p = 4: the kernel 2.28 -> 1.73 ms, FP32 results unchanged bit for bit.)
-                const int d = lev - av.level[sb];
-                const int up = d > 0 ? d : 0, dn = d < 0 ? -d : 0;
-                const float r = __int_as_float((127 + d) << 23);          // h_s / h_b = 2^d
-                const float sc = __int_as_float((127 - 1 - dn) << 23);    // 2^-(1 + dn)
-                const int* ijk_s = av.ijk + 3 * (size_t)sb;
-                const float ohx = (float)(((2 * ijk_s[0] + 1) << up) - ((2 * ijk_b[0] + 1) << dn)) * sc;
-                const float ohy = (float)(((2 * ijk_s[1] + 1) << up) - ((2 * ijk_b[1] + 1) << dn)) * sc;
-                const float ohz = (float)(((2 * ijk_s[2] + 1) << up) - ((2 * ijk_b[2] + 1) << dn)) * sc;
-                if (!DAFMM_RANGE(av.pbeg[sb], av.pend[sb], av.n, kChkBoxRange)) return;
-                const int r0 = av.xq0[sb], n = av.pend[sb] - av.pbeg[sb];
-                if (!DAFMM_RANGE(r0, (long long)r0 + n, av.nrec, kChkRecord)) return;
-                for (int i0s = 0; i0s < n;) {
-                    const int take = min(n - i0s, kLeafSeg - fill);
-                    for (int i = lane; i < take; i += 32) {
-                        const float4 rec = xq_load(av.xq, r0 + i0s + i), rl = xq_load(av.xl, r0 + i0s + i);
-                        float X, Y, Z, XL, YL, ZL;
-                        scale_shift_exact(rec.x, rl.x, r, ohx, X, XL);
-                        scale_shift_exact(rec.y, rl.y, r, ohy, Y, YL);
-                        scale_shift_exact(rec.z, rl.z, r, ohz, Z, ZL);
-                        list_store(buf, fill + i, X, Y, Z, rec.w, XL, YL, ZL, rl.w);
-                    }
-                    fill += take;
-                    i0s += take;
-                    if (fill == kLeafSeg) flush();
+            for (int ug = u0; ug < u1; ug += 32) {
+                int np = 0, pair = 0;
+                float r = 1.f, ox = 0.f, oy = 0.f, oz = 0.f;
+                const int sb = ug + lane < u1 ? av.u_idx[ug + lane] : -1;
+                if (sb >= 0 && DAFMM_IN(sb, av.nbox, kChkBoxIndex) &&
+                    DAFMM_RANGE(av.pbeg[sb], av.pend[sb], av.n, kChkBoxRange) &&
+                    DAFMM_RANGE(av.xq0[sb], (long long)av.xq0[sb] + (av.pend[sb] - av.pbeg[sb]), av.nrec, kChkRecord)) {
+                    pair = av.xq0[sb] >> 1;
+                    np = (av.pend[sb] - av.pbeg[sb] + 1) >> 1;
+                    // the source leaf's centre offset in this leaf's widths and its width ratio,
+                    // from the integer box coordinates (same tree): with d = lev_b - lev_s,
+                    // (c_s - c_b) / h_b = N / 2^(1 + max(0, -d)),
+                    // N = (2 i_s + 1) 2^max(0, d) - (2 i_b + 1) 2^max(0, -d).  Levels go to 20, so
+                    // both terms stay below 2^22, and adjacent boxes have |N| <= 2^|d| + 1 < 2^24:
+                    // N is exact in an int and in a float.  (64-bit N took nine conversions per
+                    // list entry on the FP64 pipe, 1/64 of the FP32 rate here: 35 % of that
+                    // pipe's cycles, Gaussian N = 1e6, p = 4: the kernel 2.28 -> 1.73 ms, FP32
+                    // results unchanged bit for bit.)
+                    const int d = lev - av.level[sb];
+                    const int up = d > 0 ? d : 0, dn = d < 0 ? -d : 0;
+                    r = __int_as_float((127 + d) << 23);                      // h_s / h_b = 2^d
+                    const float sc = __int_as_float((127 - 1 - dn) << 23);    // 2^-(1 + dn)
+                    const int* ijk_s = av.ijk + 3 * (size_t)sb;
+                    ox = (float)(((2 * ijk_s[0] + 1) << up) - ((2 * ijk_b[0] + 1) << dn)) * sc;
+                    oy = (float)(((2 * ijk_s[1] + 1) << up) - ((2 * ijk_b[1] + 1) << dn)) * sc;
+                    oz = (float)(((2 * ijk_s[2] + 1) << up) - ((2 * ijk_b[2] + 1) << dn)) * sc;
                 }
-            };
-            // the leaf itself (the only records that can coincide with a target), completed to
-            // an even count by a null record, then the other U-list leaves
-            const int n_own = i1 - i0;
-            own_end = n_own + (n_own & 1);  // (set first: a long own leaf flushes segments)
-            add_leaf(b);
-            if (n_own & 1) {
-                if (lane == 0) list_store_null(buf, fill);  // fill < kLeafSeg here
-                ++fill;
-                if (fill == kLeafSeg) flush();
+                const int own = ug == u0 ? (i1 - i0 + 1) >> 1 : 0;
+                near_segments<false>(buf, av.xq, av.xl, np, pair, r, ox, oy, oz, lane,
+                                     [&](int seg0, int n) { near_segment(buf, n, own - seg0, W, lane, nt, cs); });
             }
-            for (int ui = u0; ui < u1; ++ui) {
-                const int sb = av.u_idx[ui];
-                if (sb != b && DAFMM_IN(sb, av.nbox, kChkBoxIndex)) add_leaf(sb);
-            }
-            if (fill > 0) flush();
-            if (split) join_halves(acc);
-            fphi = ((double)acc.ph + (double)acc.pl) * ih;
-            fx = ((double)acc.xh + (double)acc.xl) * ih * ih;
-            fy = ((double)acc.yh + (double)acc.yl) * ih * ih;
-            fz = ((double)acc.zh + (double)acc.zl) * ih * ih;
+            const CompSums sum = near_join(cs, W, lane);
+            fphi = ((double)sum.ph + (double)sum.pl) * ih;
+            fx = ((double)sum.xh + (double)sum.xl) * ih * ih;
+            fy = ((double)sum.yh + (double)sum.yl) * ih * ih;
+            fz = ((double)sum.zh + (double)sum.zl) * ih * ih;
         }
         // M2P from the W list (Sec. 3.2): phi = F/h_w, E = -grad_s F / h_w^2
         if constexpr (sizeof(T) == 8) {
@@ -1855,32 +1827,32 @@ __global__ void __launch_bounds__(256) k_leaf_a(AdaptiveView av, const int* __re
             const float ihf = (float)ih;
             float wphi = 0.f, wfx = 0.f, wfy = 0.f, wfz = 0.f;
             const int* ib = av.ijk + 3 * (size_t)b;
-            for (int wi = w0; wi < w1; ++wi) {
-                const int wb = av.w_idx[wi];
-                if (!DAFMM_IN(wb, av.nbox, kChkBoxIndex)) continue;
-                const int dl = av.level[wb] - lev;
-                float sx0, sy0, sz0, iw;
-                if (dl >= 0 && dl <= kMaxAdaptiveDepth) {  // (both terms below 2^22: exact in int and float)
-                    const float r = (float)(1u << dl);
-                    const int* iwb = av.ijk + 3 * (size_t)wb;
-                    const float ox = 0.5f * (float)(((2 * ib[0] + 1) << dl) - (2 * iwb[0] + 1));
-                    const float oy = 0.5f * (float)(((2 * ib[1] + 1) << dl) - (2 * iwb[1] + 1));
-                    const float oz = 0.5f * (float)(((2 * ib[2] + 1) << dl) - (2 * iwb[2] + 1));
-                    sx0 = fmaf(plw.x, r, fmaf(pw.x, r, ox));
-                    sy0 = fmaf(plw.y, r, fmaf(pw.y, r, oy));
-                    sz0 = fmaf(plw.z, r, fmaf(pw.z, r, oz));
-                    iw = ihf * r;
-                } else {  // (not a W-list shape; kept general)
-                    double wx, wy, wz, wh;
-                    abox_geom(av, wb, wx, wy, wz, wh);
-                    const double iwh = 1.0 / wh;
-                    sx0 = (float)((av.x[tt] - wx) * iwh);
-                    sy0 = (float)((av.y[tt] - wy) * iwh);
-                    sz0 = (float)((av.z[tt] - wz) * iwh);
-                    iw = (float)iwh;
+            // a pass of at most 16 targets works on two W boxes at a time
+            const int two = per < 32 ? 2 : 1, rep = two == 2 ? (lane / per) & 1 : 0;
+            float* mrow = reinterpret_cast<float*>(buf) + rep * NCP;
+            for (int wi = w0; wi < w1; wi += two) {
+                __syncwarp();  // the list and the previous boxes are no longer read
+                for (int e = 0; e < two; ++e) {
+                    const int eb = wi + e < w1 ? av.w_idx[wi + e] : -1;
+                    if (eb < 0 || !DAFMM_IN(eb, av.nbox, kChkBoxIndex)) continue;
+                    float* row = reinterpret_cast<float*>(buf) + e * NCP;
+                    for (int k = lane; k < NC; k += 32)
+                        row[k] = Mf ? Mf[(size_t)eb * NCP + k] : (float)M[(size_t)eb * NCP + k];
                 }
-                if (Mf) warp_row_f32(Mf + (size_t)wb * NCP, mrow, lane);
-                else warp_row_to_f32(M + (size_t)wb * NCP, mrow, lane);
+                __syncwarp();
+                const int wb = wi + rep < w1 ? av.w_idx[wi + rep] : -1;
+                if (wb < 0 || !DAFMM_IN(wb, av.nbox, kChkBoxIndex)) continue;
+                const int dl = av.level[wb] - lev;
+                // (finer boxes of the same tree, levels up to 20: both terms below 2^22, exact)
+                const float r = __int_as_float((127 + dl) << 23);
+                const int* iwb = av.ijk + 3 * (size_t)wb;
+                const float ox = 0.5f * (float)(((2 * ib[0] + 1) << dl) - (2 * iwb[0] + 1));
+                const float oy = 0.5f * (float)(((2 * ib[1] + 1) << dl) - (2 * iwb[1] + 1));
+                const float oz = 0.5f * (float)(((2 * ib[2] + 1) << dl) - (2 * iwb[2] + 1));
+                const float sx0 = fmaf(plw.x, r, fmaf(pw.x, r, ox));
+                const float sy0 = fmaf(plw.y, r, fmaf(pw.y, r, oy));
+                const float sz0 = fmaf(plw.z, r, fmaf(pw.z, r, oz));
+                const float iw = ihf * r;
                 T F, g0, g1, g2;
                 gen::GEN(m2p)<T>(SmemRowF{mrow}, sx0, sy0, sz0, F, g0, g1, g2);
                 wphi = fmaf(F, iw, wphi);
@@ -1888,6 +1860,13 @@ __global__ void __launch_bounds__(256) k_leaf_a(AdaptiveView av, const int* __re
                 wfx = fmaf(-g0, iw2, wfx);
                 wfy = fmaf(-g1, iw2, wfy);
                 wfz = fmaf(-g2, iw2, wfz);
+            }
+            if (two == 2) {
+                __syncwarp();
+                wphi += __shfl_xor_sync(0xffffffffu, wphi, per);
+                wfx += __shfl_xor_sync(0xffffffffu, wfx, per);
+                wfy += __shfl_xor_sync(0xffffffffu, wfy, per);
+                wfz += __shfl_xor_sync(0xffffffffu, wfz, per);
             }
             fphi += (double)wphi;
             fx += (double)wfx;
@@ -2276,7 +2255,7 @@ static cudaError_t leaf_a_launch(const AdaptiveView& av, const int* leaves, int 
     if (prec == DAFMM_FP64) {
         k_leaf_a<double><<<grd, blk, 0, s>>>(av, leaves, nleaves, L, M, nullptr, phi, field);
     } else {
-        const size_t smem = (size_t)warps * 2 * kLeafSeg * sizeof(float4);
+        const size_t smem = (size_t)warps * kLeafWarpSmem;
         cudaError_t e = cudaFuncSetAttribute(k_leaf_a<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         k_leaf_a<float><<<grd, blk, smem, s>>>(av, leaves, nleaves, L, M, Mf, phi, field);
