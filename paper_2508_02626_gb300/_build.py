@@ -62,7 +62,7 @@ def _sources():
 
 
 def _extra_flags():
-    """Extra nvcc flags from DAFMM_NVCC_FLAGS (e.g. -DDAFMM_LEAF_MINB=6 for a tuning build)."""
+    """Extra nvcc flags from DAFMM_NVCC_FLAGS (e.g. -DNAME=VALUE for a tuning build)."""
     return os.environ.get("DAFMM_NVCC_FLAGS", "").split()
 
 

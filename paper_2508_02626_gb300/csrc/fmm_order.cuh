@@ -1067,11 +1067,12 @@ __device__ __forceinline__ void near_add(float2 ex, float2 ey, float2 ez, float2
 // for its four partitions.  With one target per lane the L1 was the bound (ncu: L1 80 % busy, the
 // FMA pipe 48 %); two targets halve the loads per interaction.  With the conflict-free staging:
 // uniform N = 1e6, p = 8: the kernel 0.80 -> 0.63 ms (5 or 6 blocks per SM; 4: 0.68); clustered
-// N = 4e6, p = 10: 10.5 -> 8.1 ms; 64-problem forest, p = 6: 2.74 -> 2.06 ms.
+// N = 4e6, p = 10: 10.5 -> 8.1 ms; 64-problem forest, p = 6: 2.74 -> 2.06 ms.  (The adaptive kernel
+// compiled for 24 warps per SM instead of 16: 7.4 and 2.04 ms.)
 template <bool GUARD>
 __device__ __forceinline__ void near_pairs(const float4* buf, int p0, int p1, const NearTarget (&t)[2],
                                            NearSums (&s)[2]) {
-#pragma unroll 2
+#pragma unroll 1
     for (int p = p0; p < p1; ++p) {
         const float4 A = buf[p], B = buf[kSegPairs + p];
         const float2 sx = make_float2(A.x, A.y), sy = make_float2(A.z, A.w), sz = make_float2(B.x, B.y),
@@ -1109,10 +1110,14 @@ __device__ __forceinline__ void two_sum_add(float& hi, float& lo, float v) {
 }
 
 // compensated (hi, lo) sums of the near field: FP32 partial sums over at most 128 sources (one
-// segment) are folded into them, so that long neighbour lists keep FP32-level error
+// segment) are folded into them, so that long neighbour lists keep FP32-level error.  Each lane's
+// sums for its two targets live in shared memory behind the segment (float [u][8][32]): they are
+// touched once per segment, and 16 registers fewer let more warps hide the pair loop's latencies.
 struct CompSums {
     float ph = 0.f, pl = 0.f, xh = 0.f, xl = 0.f, yh = 0.f, yl = 0.f, zh = 0.f, zl = 0.f;
 };
+constexpr int kNearSmem = 4 * kSegPairs + 2 * 8 * 32 / 4;  // float4s per warp: the segment and the sums
+__device__ __forceinline__ float* near_acc(float4* buf) { return reinterpret_cast<float*>(buf + 4 * kSegPairs); }
 
 // The lanes of a pass over m <= 32 targets: groups of W lanes, lane l of a group with the targets
 // l and l + W, the groups sharing out the sources.  W = 16, 8 or 4, so that a pass costs about
@@ -1120,8 +1125,7 @@ struct CompSums {
 __device__ __forceinline__ int near_width(int m) { return m > 16 ? 16 : (m > 8 ? 8 : 4); }
 
 // the pairwise sums of one segment of n pairs, the first `own` of the target's own leaf (guarded)
-__device__ __forceinline__ void near_segment(const float4* buf, int n, int own, int W, int lane,
-                                             const NearTarget (&t)[2], CompSums (&cs)[2]) {
+__device__ __forceinline__ void near_segment(float4* buf, int n, int own, int W, int lane, const NearTarget (&t)[2]) {
     own = max(0, min(own, n));
     const int lg = __ffs(32 / W) - 1, g = lane / W;  // 2^lg groups
     NearSums s[2] = {};
@@ -1131,29 +1135,38 @@ __device__ __forceinline__ void near_segment(const float4* buf, int n, int own, 
     }
     const int h = (n - own + (1 << lg) - 1) >> lg, pa = min(own + g * h, n);
     near_pairs<false>(buf, pa, min(pa + h, n), t, s);
+    float* acc = near_acc(buf) + lane;
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-        two_sum_add(cs[u].ph, cs[u].pl, s[u].P.x + s[u].P.y);
-        two_sum_add(cs[u].xh, cs[u].xl, s[u].X.x + s[u].X.y);
-        two_sum_add(cs[u].yh, cs[u].yl, s[u].Y.x + s[u].Y.y);
-        two_sum_add(cs[u].zh, cs[u].zl, s[u].Z.x + s[u].Z.y);
+        const float v[4] = {s[u].P.x + s[u].P.y, s[u].X.x + s[u].X.y, s[u].Y.x + s[u].Y.y, s[u].Z.x + s[u].Z.y};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            float hi = acc[(u * 8 + 2 * j) * 32], lo = acc[(u * 8 + 2 * j + 1) * 32];
+            two_sum_add(hi, lo, v[j]);
+            acc[(u * 8 + 2 * j) * 32] = hi;
+            acc[(u * 8 + 2 * j + 1) * 32] = lo;
+        }
     }
 }
 
-// the groups' sums together: afterwards lane l < 2 W holds target l of the pass (the upper copies
-// hold the same)
-__device__ __forceinline__ CompSums near_join(const CompSums (&cs)[2], int W, int lane) {
-    const bool second = (lane & W) != 0;  // this lane's group keeps the targets l + W
-    const CompSums &keep = second ? cs[1] : cs[0], &give = second ? cs[0] : cs[1];
-    float k[8] = {keep.ph, keep.pl, keep.xh, keep.xl, keep.yh, keep.yl, keep.zh, keep.zl};
-    float v[8] = {give.ph, give.pl, give.xh, give.xl, give.yh, give.yl, give.zh, give.zl};
-    for (int d = W; d < 32; d <<= 1) {
+__device__ __forceinline__ void near_zero(float4* buf, int lane) {
+    float* acc = near_acc(buf) + lane;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) v[j] = __shfl_xor_sync(0xffffffffu, d == W ? v[j] : k[j], d);
+    for (int j = 0; j < 16; ++j) acc[j * 32] = 0.f;
+}
+
+// the groups' sums of target tl < 2 W of the pass, in the order of the groups
+__device__ __forceinline__ CompSums near_join(float4* buf, int W, int tl) {
+    __syncwarp();
+    const float* acc = near_acc(buf) + (tl >= W ? 8 * 32 : 0) + (tl & (W - 1));
+    float k[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) k[j] = acc[j * 32];
+    for (int d = W; d < 32; d += W) {
 #pragma unroll
         for (int j = 0; j < 8; j += 2) {
-            two_sum_add(k[j], k[j + 1], v[j]);
-            k[j + 1] += v[j + 1];
+            two_sum_add(k[j], k[j + 1], acc[j * 32 + d]);
+            k[j + 1] += acc[(j + 1) * 32 + d];
         }
     }
     CompSums r;
@@ -1219,10 +1232,14 @@ __device__ __forceinline__ ff ff_shfl_down(ff v, int d) {
     return ff(__shfl_down_sync(0xffffffffu, v.hi, d), __shfl_down_sync(0xffffffffu, v.lo, d));
 }
 
-// blocks per SM the uniform FP32 leaf kernel is compiled for (its register budget)
-#ifndef DAFMM_LEAF_MINB
-#define DAFMM_LEAF_MINB 5
-#endif
+// Leaves (one warp each) per thread block of the uniform leaf kernel: one, since a block of four
+// holds its registers until its longest leaf is done; and the warps per SM its FP32 form is
+// compiled for.  N = 1e6, p = 8: 0.63 ms with four leaves per block at 20 warps per SM, 0.61 with
+// one, 0.60 with the sums in shared memory at 28 warps.  (More warps or independent pairs in
+// flight do not help further, nor do scalar field sums, although a packed FMA of three distinct
+// registers takes 3.9 cycles in a loop of its own and two scalar ones 2.3: 0.61-0.62 ms.)
+constexpr int kLeafWarps = 1;
+constexpr int kLeafMinWarps = 28;
 
 // the neighbour slot (0..26, slot 13 = the leaf itself) held by lane k of the list: the leaf
 // itself first, so that its records -- the only ones that can coincide with a target -- form
@@ -1230,7 +1247,7 @@ __device__ __forceinline__ ff ff_shfl_down(ff v, int d) {
 __device__ __forceinline__ int own_first_slot(int k) { return k == 0 ? 13 : (k <= 13 ? k - 1 : k); }
 
 template <class T>
-__global__ void __launch_bounds__(128, std::is_same<T, float>::value ? DAFMM_LEAF_MINB : (std::is_same<T, ff>::value ? 4 : 8))
+__global__ void __launch_bounds__(32 * kLeafWarps, (std::is_same<T, float>::value ? kLeafMinWarps : (std::is_same<T, ff>::value ? 16 : 32)) / kLeafWarps)
 k_leaf(TreeView tv, const double* __restrict__ Lleaf,
                                               double* __restrict__ phi, double* __restrict__ field) {
     const int lane = threadIdx.x;
@@ -1245,8 +1262,8 @@ k_leaf(TreeView tv, const double* __restrict__ Lleaf,
     const double cy = tv.y0 + ((double)b + 0.5) * tv.h_leaf;
     const double cz = tv.z0 + ((double)c + 0.5) * tv.h_leaf;
     const double* Lrow = Lleaf ? Lleaf + (size_t)leaf * NCP : nullptr;
-    __shared__ float s_lrow[4][NCP];  // per warp: the leaf's local expansion in FP32
-    __shared__ ff s_lrow_ff[std::is_same<T, ff>::value ? 4 : 1][std::is_same<T, ff>::value ? NCP : 1];
+    __shared__ float s_lrow[kLeafWarps][NCP];  // per warp: the leaf's local expansion in FP32
+    __shared__ ff s_lrow_ff[std::is_same<T, ff>::value ? kLeafWarps : 1][std::is_same<T, ff>::value ? NCP : 1];
     if constexpr (std::is_same<T, ff>::value) {  // ... or in float-float
         if (Lrow) {
             __syncwarp();
@@ -1329,17 +1346,18 @@ k_leaf(TreeView tv, const double* __restrict__ Lleaf,
             // The neighbours' records are copied into one shared-memory list, shifted into this
             // leaf's frame (source + neighbour offset, in leaf widths, exactly: the rounding of
             // the shift joins the remainder); the pairwise sum runs over each segment of it.
-            __shared__ __align__(16) float4 s_list[4][4 * kSegPairs];
+            __shared__ __align__(16) float4 s_list[kLeafWarps][kNearSmem];
             float4* buf = s_list[threadIdx.y];
-            CompSums cs[2], sum;
+            CompSums sum;
             FFSums fs;
             if constexpr (std::is_same<T, float>::value) {
+                near_zero(buf, lane);
                 const int l0 = lane & (W - 1);
                 const NearTarget nt[2] = {near_target(tv.xq, xl, (l0 < m ? base + l0 : i0) + r_own),
                                           near_target(tv.xq, xl, (l0 + W < m ? base + l0 + W : i0) + r_own)};
                 near_segments<true>(buf, tv.xq, xl, nb_np, nb_pair, 1.f, nb_x, nb_y, nb_z, lane,
-                                    [&](int seg0, int n) { near_segment(buf, n, own_pairs - seg0, W, lane, nt, cs); });
-                sum = near_join(cs, W, lane);
+                                    [&](int seg0, int n) { near_segment(buf, n, own_pairs - seg0, W, lane, nt); });
+                sum = near_join(buf, W, tl);
             } else {
                 const float4 pt = xq_load(tv.xq, tt + r_own), pl = xq_load(xl, tt + r_own);
                 near_segments<true>(buf, tv.xq, xl, nb_np, nb_pair, 1.f, nb_x, nb_y, nb_z, lane, [&](int seg0, int n) {
@@ -1692,12 +1710,12 @@ __global__ void __launch_bounds__(128) k_p2l_a(AdaptiveView av, int lb, int le, 
 
 // per warp of the FP32 adaptive leaf kernel: the source list's segment (the M2P stages up to two
 // W boxes' multipoles in it afterwards), then the leaf's locals in FP32
-constexpr size_t kLeafWarpSmem = 4 * kSegPairs * sizeof(float4) + NCP * sizeof(float);
+constexpr size_t kLeafWarpSmem = kNearSmem * sizeof(float4) + NCP * sizeof(float);
 static_assert(2 * NCP * sizeof(float) <= 4 * kSegPairs * sizeof(float4), "two rows fit the segment");
 
 // leaves: P2P over the U list, M2P over the W list, L2P of the leaf's local expansion
 template <class T>
-__global__ void __launch_bounds__(256, 2) k_leaf_a(AdaptiveView av, const int* __restrict__ leaves, int nleaves,
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_leaf_a(AdaptiveView av, const int* __restrict__ leaves, int nleaves,
                                                    const double* __restrict__ L, const double* __restrict__ M,
                                                    const float* __restrict__ Mf, double* __restrict__ phi,
                                                    double* __restrict__ field) {
@@ -1706,7 +1724,7 @@ __global__ void __launch_bounds__(256, 2) k_leaf_a(AdaptiveView av, const int* _
     const int li = blockIdx.x * blockDim.y + threadIdx.y;
     if (li >= nleaves) return;
     float4* buf = reinterpret_cast<float4*>(s_leaf + threadIdx.y * kLeafWarpSmem);
-    float* lrow = reinterpret_cast<float*>(buf + 4 * kSegPairs);
+    float* lrow = reinterpret_cast<float*>(buf + kNearSmem);
     const int b = leaves[li];
     if (!DAFMM_IN(b, av.nbox, kChkBoxIndex)) return;
     double cx, cy, cz, h;
@@ -1760,7 +1778,7 @@ __global__ void __launch_bounds__(256, 2) k_leaf_a(AdaptiveView av, const int* _
             const int l0 = lane & (W - 1), rb = av.xq0[b] - i0;
             const NearTarget nt[2] = {near_target(av.xq, av.xl, (l0 < m ? base + l0 : i0) + rb),
                                       near_target(av.xq, av.xl, (l0 + W < m ? base + l0 + W : i0) + rb)};
-            CompSums cs[2];  // in leaf widths of this leaf
+            near_zero(buf, lane);  // sums in leaf widths of this leaf
             const int* ijk_b = av.ijk + 3 * (size_t)b;
             for (int ug = u0; ug < u1; ug += 32) {
                 int np = 0, pair = 0;
@@ -1791,9 +1809,9 @@ __global__ void __launch_bounds__(256, 2) k_leaf_a(AdaptiveView av, const int* _
                 }
                 const int own = ug == u0 ? (i1 - i0 + 1) >> 1 : 0;
                 near_segments<false>(buf, av.xq, av.xl, np, pair, r, ox, oy, oz, lane,
-                                     [&](int seg0, int n) { near_segment(buf, n, own - seg0, W, lane, nt, cs); });
+                                     [&](int seg0, int n) { near_segment(buf, n, own - seg0, W, lane, nt); });
             }
-            const CompSums sum = near_join(cs, W, lane);
+            const CompSums sum = near_join(buf, W, tl);
             fphi = ((double)sum.ph + (double)sum.pl) * ih;
             fx = ((double)sum.xh + (double)sum.xl) * ih * ih;
             fy = ((double)sum.yh + (double)sum.yl) * ih * ih;
@@ -2071,7 +2089,7 @@ static cudaError_t m2l_launch(const OrderData& od, int prec, int l, const double
 static cudaError_t leaf_launch(const TreeView& tv, int prec, const double* Lleaf, double* phi, double* field,
                                cudaStream_t s) {
     if (tv.nleaf == 0) return cudaSuccess;
-    dim3 blk(32, 4), grd((tv.nleaf + 3) / 4);
+    dim3 blk(32, kLeafWarps), grd((tv.nleaf + kLeafWarps - 1) / kLeafWarps);
     if (prec == DAFMM_FP64) k_leaf<double><<<grd, blk, 0, s>>>(tv, Lleaf, phi, field);
     else if (prec == DAFMM_FF) k_leaf<ff><<<grd, blk, 0, s>>>(tv, Lleaf, phi, field);
     else k_leaf<float><<<grd, blk, 0, s>>>(tv, Lleaf, phi, field);
