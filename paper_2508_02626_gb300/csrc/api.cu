@@ -1418,7 +1418,8 @@ int eval_adaptive(dafmm_tree* t, int order, int precision, double* dphi, double*
         ++launches;
         mc = t->aMc;
     }
-    CK(c, ops->leaf_a(av, t->leaves, t->nleaves, precision, t->aL, t->aM, mc, dphi, dfield, c->leaf_warps, s),
+    CK(c, ops->leaf_a(av, t->leaves, t->nleaves, precision, t->aL, t->aM, mc, dphi, dfield, c->leaf_warps,
+                      t->max_per_leaf, s),
        "P2P/M2P/L2P");
     ++launches;
     mark(7);

@@ -1241,13 +1241,110 @@ __device__ __forceinline__ ff ff_shfl_down(ff v, int d) {
 constexpr int kLeafWarps = 1;
 constexpr int kLeafMinWarps = 28;
 
+// ---- FP64 near field ----
+// 1/sqrt(x) for x well inside the normal range: the PTX approximation rsqrt.approx.ftz.f64 y and
+// the binomial series of (1 - e)^(-1/2) in its residual e = 1 - x y^2 up to e^2 (the next term is
+// 5/16 e^3, far below an FP64 rounding for a seed good to 2^-19): five FP64 instructions.
+__device__ __forceinline__ double rsqrt_series(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y * y, 1.0);
+    return fma(y * e, fma(e, 0.375, 0.5), y);
+}
+
+struct Sum64 {
+    double p = 0.0, x = 0.0, y = 0.0, z = 0.0;
+};
+__device__ __forceinline__ Sum64 sum64_shfl(const Sum64& s, int d) {
+    Sum64 r;
+    r.p = s.p + __shfl_xor_sync(0xffffffffu, s.p, d);
+    r.x = s.x + __shfl_xor_sync(0xffffffffu, s.x, d);
+    r.y = s.y + __shfl_xor_sync(0xffffffffu, s.y, d);
+    r.z = s.z + __shfl_xor_sync(0xffffffffu, s.z, d);
+    return r;
+}
+
+// targets of the next pass over `rem` particles: 32 lanes, or the largest power of two that they
+// fill (or fill to four fifths), the sources shared out over the 32 / W groups of lanes
+__device__ __forceinline__ int pass_width(int rem) {
+    if (rem >= 32) return 32;
+    const int w = 1 << (31 - __clz(rem));
+    return 5 * rem >= 8 * w ? 2 * w : w;
+}
+
+// The particles of up to 32 source leaves (lane e: cnt particles from `first`), end to end, every
+// G-th from the g-th, on one target.  The FP64 pipe (1/64 of the FP32 rate on this part) is the
+// bound, so everything else is spent to feed it: every lane has a target or a share of the
+// sources (the list position of a source is a search in the prefix sums), 1/r takes five FP64
+// instructions, and a pair takes 18 (20 with CUDA's rsqrt and an FP64 comparison).  r^2 outside
+// the safe range -- zero for the target itself and coincident particles, which add nothing,
+// denormal, infinite or NaN -- is seen in the exponent by an integer comparison and takes CUDA's
+// rsqrt.
+__device__ __forceinline__ void near64_list(const double* __restrict__ x, const double* __restrict__ y,
+                                            const double* __restrict__ z, const double* __restrict__ q, int cnt,
+                                            int first, int G, int g, int lane, double xt, double yt, double zt,
+                                            Sum64& s) {
+    int incl = cnt;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += v;
+    }
+    const int total = __shfl_sync(0xffffffffu, incl, 31), at0 = first - (incl - cnt);
+#pragma unroll 2
+    for (int j0 = 0; j0 < total; j0 += G) {
+        const int j = j0 + g;
+        int e = 0;  // the first leaf with incl > j
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) {
+            const int v = __shfl_sync(0xffffffffu, incl, e + d - 1);
+            if (v <= j) e += d;
+        }
+        const int i = __shfl_sync(0xffffffffu, at0, e) + j;
+        if (j >= total) continue;
+        const double ex = xt - x[i], ey = yt - y[i], ez = zt - z[i];
+        const double r2 = fma(ez, ez, fma(ey, ey, ex * ex));
+        double ir;
+        if ((unsigned)__double2hiint(r2) - 0x02000000u < 0x7b000000u) ir = rsqrt_series(r2);
+        else if (r2 > 0.0) ir = rsqrt(r2);
+        else continue;
+        const double qr = q[i] * ir, w = qr * (ir * ir);
+        s.p += qr;
+        s.x = fma(w, ex, s.x);
+        s.y = fma(w, ey, s.y);
+        s.z = fma(w, ez, s.z);
+    }
+}
+
+// the sums of a pass: over the lanes' groups, then over the block's NW warps (red: two buffers in
+// turn, so that one barrier per pass does); warp 0 has the result
+template <int NW>
+__device__ __forceinline__ Sum64 pass_join(Sum64 s, int W, int warp, int lane, Sum64 (*red)[NW][32], int& turn) {
+    for (int d = W; d < 32; d <<= 1) s = sum64_shfl(s, d);
+    if constexpr (NW > 1) {
+        red[turn][warp][lane] = s;
+        __syncthreads();
+        if (warp == 0) {
+            for (int v = 1; v < NW; ++v) {
+                const Sum64 o = red[turn][v][lane];
+                s.p += o.p;
+                s.x += o.x;
+                s.y += o.y;
+                s.z += o.z;
+            }
+        }
+        turn ^= 1;
+    }
+    return s;
+}
+
 // the neighbour slot (0..26, slot 13 = the leaf itself) held by lane k of the list: the leaf
 // itself first, so that its records -- the only ones that can coincide with a target -- form
 // the guarded head of the list
 __device__ __forceinline__ int own_first_slot(int k) { return k == 0 ? 13 : (k <= 13 ? k - 1 : k); }
 
 template <class T>
-__global__ void __launch_bounds__(32 * kLeafWarps, (std::is_same<T, float>::value ? kLeafMinWarps : (std::is_same<T, ff>::value ? 16 : 32)) / kLeafWarps)
+__global__ void __launch_bounds__(32 * kLeafWarps, (std::is_same<T, float>::value ? kLeafMinWarps : 16) / kLeafWarps)
 k_leaf(TreeView tv, const double* __restrict__ Lleaf,
                                               double* __restrict__ phi, double* __restrict__ field) {
     const int lane = threadIdx.x;
@@ -1288,7 +1385,7 @@ k_leaf(TreeView tv, const double* __restrict__ Lleaf,
     // widths; the leaf itself first (lane 0), its pairs the guarded head of the list
     int nb_np = 0, nb_pair = 0, own_pairs = 0;
     float nb_x = 0.f, nb_y = 0.f, nb_z = 0.f;
-    if constexpr (!std::is_same<T, double>::value) {
+    {
         if (lane < 27) {
             const int slot = own_first_slot(lane);
             const int dx = slot % 3 - 1, dy = (slot / 3) % 3 - 1, dz = slot / 9 - 1;
@@ -1319,29 +1416,7 @@ k_leaf(TreeView tv, const double* __restrict__ Lleaf,
         const bool valid = tl < m && lane < per;  // the lanes that write
         const int tt = tl < m ? t : i0;
         double fphi = 0.0, fx = 0.0, fy = 0.0, fz = 0.0;  // near field, physical units
-        if constexpr (std::is_same<T, double>::value) {
-            const double xt = tv.x[tt], yt = tv.y[tt], zt = tv.z[tt];
-            for (int dz = -1; dz <= 1; ++dz)
-                for (int dy = -1; dy <= 1; ++dy)
-                    for (int dx = -1; dx <= 1; ++dx) {
-                        const int na = a + dx, nb = b + dy, nc2 = c + dz;
-                        if (na < 0 || nb < 0 || nc2 < 0 || na >= nside || nb >= nside || nc2 >= nside) continue;
-                        const int nl = octmajor_index(tv.depth, na, nb, nc2);
-                        int s0 = tv.leaf_start[nl], s1 = tv.leaf_start[nl + 1];
-                        if (!DAFMM_RANGE(s0, s1, tv.n, kChkLeafRange)) s0 = s1 = 0;
-                        for (int s = s0; s < s1; ++s) {
-                            const double ex = xt - tv.x[s], ey = yt - tv.y[s], ez = zt - tv.z[s];
-                            const double r2 = ex * ex + ey * ey + ez * ez;
-                            if (r2 > 0.0) {
-                                const double ir = rsqrt(r2);
-                                const double qr = tv.q[s] * ir;
-                                const double qr3 = qr * ir * ir;
-                                fphi += qr;
-                                fx += qr3 * ex; fy += qr3 * ey; fz += qr3 * ez;
-                            }
-                        }
-                    }
-        } else {
+        {
             const float4* xl = tv.xq + xq_records(tv.n, tv.nleaf);  // the remainder records
             // The neighbours' records are copied into one shared-memory list, shifted into this
             // leaf's frame (source + neighbour offset, in leaf widths, exactly: the rounding of
@@ -1398,9 +1473,7 @@ k_leaf(TreeView tv, const double* __restrict__ Lleaf,
                 xs = (T)pt.x; ys = (T)pt.y; zs = (T)pt.z;
             }
             if constexpr (sizeof(T) == 4) gen::GEN(l2p)<T>(SmemRowF{s_lrow[threadIdx.y]}, xs, ys, zs, F, g0, g1, g2);
-            else if constexpr (std::is_same<T, ff>::value)
-                gen::GEN(l2p)<T>(SmemRowFF{s_lrow_ff[threadIdx.y]}, xs, ys, zs, F, g0, g1, g2);
-            else gen::GEN(l2p)<T>(RowLoad<T>{Lrow}, xs, ys, zs, F, g0, g1, g2);
+            else gen::GEN(l2p)<T>(SmemRowFF{s_lrow_ff[threadIdx.y]}, xs, ys, zs, F, g0, g1, g2);
             fphi += (double)F;
             fx -= (double)g0 * tv.inv_h_leaf;
             fy -= (double)g1 * tv.inv_h_leaf;
@@ -1413,6 +1486,66 @@ k_leaf(TreeView tv, const double* __restrict__ Lleaf,
                 field[3 * (size_t)o] = fx;
                 field[3 * (size_t)o + 1] = fy;
                 field[3 * (size_t)o + 2] = fz;
+            }
+        }
+    }
+}
+
+// The same in FP64: a block of NW warps per leaf, the warps sharing out the sources of each pass.
+// NW grows as the leaves get fewer (leaf_launch), so that a tree of 64 or 512 leaves still gives
+// every SM its share.  Measured against one warp per leaf with passes of 32 and CUDA's rsqrt:
+// uniform N = 200,003, depth 4, p = 8: 13.1 -> 9.6 ms; N = 1e4, depth 3, p = 6: the evaluation 2.57
+// -> 2.20 ms (this kernel 0.28).
+template <int NW>
+__global__ void __launch_bounds__(32 * NW, 24 / NW) k_leaf64(TreeView tv, const double* __restrict__ Lleaf,
+                                                             double* __restrict__ phi, double* __restrict__ field) {
+    __shared__ Sum64 red[2][NW][32];
+    const int lane = threadIdx.x, warp = threadIdx.y, leaf = blockIdx.x;
+    int i0 = tv.leaf_start[leaf], i1 = tv.leaf_start[leaf + 1];
+    if (!DAFMM_RANGE(i0, i1, tv.n, kChkLeafRange)) i0 = i1 = 0;
+    int a, b, c;
+    octmajor_decode(tv.depth, leaf, a, b, c);
+    const int nside = 1 << tv.depth;
+    const double cx = tv.x0 + ((double)a + 0.5) * tv.h_leaf;
+    const double cy = tv.y0 + ((double)b + 0.5) * tv.h_leaf;
+    const double cz = tv.z0 + ((double)c + 0.5) * tv.h_leaf;
+    // the 27 neighbour leaves, one per lane (none outside the domain)
+    int cnt = 0, first = 0;
+    if (lane < 27) {
+        const int na = a + lane % 3 - 1, nb = b + (lane / 3) % 3 - 1, nc2 = c + lane / 9 - 1;
+        if (na >= 0 && nb >= 0 && nc2 >= 0 && na < nside && nb < nside && nc2 < nside) {
+            const int nl = octmajor_index(tv.depth, na, nb, nc2);
+            int s0 = tv.leaf_start[nl], s1 = tv.leaf_start[nl + 1];
+            if (!DAFMM_RANGE(s0, s1, tv.n, kChkLeafRange)) s0 = s1 = 0;
+            first = s0;
+            cnt = s1 - s0;
+        }
+    }
+    int turn = 0;
+    for (int base = i0, W; base < i1; base += W) {
+        W = pass_width(i1 - base);
+        const int t = base + (lane & (W - 1)), tt = t < i1 ? t : i0;
+        const double xt = tv.x[tt], yt = tv.y[tt], zt = tv.z[tt];
+        Sum64 s;
+        near64_list(tv.x, tv.y, tv.z, tv.q, cnt, first, NW * (32 / W), warp * (32 / W) + lane / W, lane, xt, yt, zt, s);
+        s = pass_join<NW>(s, W, warp, lane, red, turn);
+        if (warp != 0) continue;
+        if (Lleaf) {  // far field from the leaf's local expansion
+            double F, g0, g1, g2;
+            gen::GEN(l2p)<double>(RowLoad<double>{Lleaf + (size_t)leaf * NCP}, (xt - cx) * tv.inv_h_leaf,
+                                  (yt - cy) * tv.inv_h_leaf, (zt - cz) * tv.inv_h_leaf, F, g0, g1, g2);
+            s.p += F;
+            s.x -= g0 * tv.inv_h_leaf;
+            s.y -= g1 * tv.inv_h_leaf;
+            s.z -= g2 * tv.inv_h_leaf;
+        }
+        if (lane < W && t < i1 && DAFMM_IN(tv.perm[t], tv.n, kChkPerm)) {
+            const size_t o = (size_t)tv.perm[t];
+            if (phi) phi[o] = s.p;
+            if (field) {
+                field[3 * o] = s.x;
+                field[3 * o + 1] = s.y;
+                field[3 * o + 2] = s.z;
             }
         }
     }
@@ -1713,9 +1846,8 @@ __global__ void __launch_bounds__(128) k_p2l_a(AdaptiveView av, int lb, int le, 
 constexpr size_t kLeafWarpSmem = kNearSmem * sizeof(float4) + NCP * sizeof(float);
 static_assert(2 * NCP * sizeof(float) <= 4 * kSegPairs * sizeof(float4), "two rows fit the segment");
 
-// leaves: P2P over the U list, M2P over the W list, L2P of the leaf's local expansion
-template <class T>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_leaf_a(AdaptiveView av, const int* __restrict__ leaves, int nleaves,
+// leaves: P2P over the U list, M2P over the W list, L2P of the leaf's local expansion (FP32)
+__global__ void __launch_bounds__(256, 3) k_leaf_a(AdaptiveView av, const int* __restrict__ leaves, int nleaves,
                                                    const double* __restrict__ L, const double* __restrict__ M,
                                                    const float* __restrict__ Mf, double* __restrict__ phi,
                                                    double* __restrict__ field) {
@@ -1731,46 +1863,24 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_leaf_a(Adaptive
     abox_geom(av, b, cx, cy, cz, h);
     const double ih = 1.0 / h;
     const int lev = av.level[b];
-    if constexpr (sizeof(T) == 4) {
-        if (lev >= 2) warp_row_to_f32(L + (size_t)b * NCP, lrow, lane);
-    }
+    if (lev >= 2) warp_row_to_f32(L + (size_t)b * NCP, lrow, lane);
     int i0 = av.pbeg[b], i1 = av.pend[b];
     if (!DAFMM_RANGE(i0, i1, av.n, kChkBoxRange)) i0 = i1 = 0;
-    if constexpr (sizeof(T) == 4) {  // the leaf's own records (its targets)
-        if (!DAFMM_RANGE(av.xq0[b], (long long)av.xq0[b] + (i1 - i0), av.nrec, kChkRecord)) i0 = i1 = 0;
-    }
+    // the leaf's own records (its targets)
+    if (!DAFMM_RANGE(av.xq0[b], (long long)av.xq0[b] + (i1 - i0), av.nrec, kChkRecord)) i0 = i1 = 0;
     int u0 = av.u_ptr[b], u1 = av.u_ptr[b + 1];
     int w0 = av.w_ptr[b], w1 = av.w_ptr[b + 1];
     if (!DAFMM_RANGE(u0, u1, av.nu, kChkListPtr)) u0 = u1 = 0;
     if (!DAFMM_RANGE(w0, w1, av.nw, kChkListPtr)) w0 = w1 = 0;
     for (int base = i0; base < i1; base += 32) {
         const int m = min(32, i1 - base);
-        const int W = near_width(m);  // FP32: the lanes' split, see near_width
-        const int per = sizeof(T) == 4 ? 2 * W : 32;
+        const int W = near_width(m), per = 2 * W;  // the lanes' split, see near_width
         const int tl = lane & (per - 1);
         const int t = base + tl;
         const bool valid = tl < m && lane < per;  // the lanes that write
         const int tt = tl < m ? t : i0;
         double fphi = 0.0, fx = 0.0, fy = 0.0, fz = 0.0;
-        if constexpr (sizeof(T) == 8) {
-            const double xt = av.x[tt], yt = av.y[tt], zt = av.z[tt];
-            for (int ui = u0; ui < u1; ++ui) {
-                const int sb = av.u_idx[ui];
-                if (!DAFMM_IN(sb, av.nbox, kChkBoxIndex) || !DAFMM_RANGE(av.pbeg[sb], av.pend[sb], av.n, kChkBoxRange))
-                    continue;
-                for (int sidx = av.pbeg[sb]; sidx < av.pend[sb]; ++sidx) {
-                    const double ex = xt - av.x[sidx], ey = yt - av.y[sidx], ez = zt - av.z[sidx];
-                    const double r2 = ex * ex + ey * ey + ez * ez;
-                    if (r2 > 0.0) {
-                        const double ir = rsqrt(r2);
-                        const double qr = av.q[sidx] * ir;
-                        const double qr3 = qr * ir * ir;
-                        fphi += qr;
-                        fx += qr3 * ex; fy += qr3 * ey; fz += qr3 * ez;
-                    }
-                }
-            }
-        } else {
+        {
             // The U-list leaves' records are copied into one shared-memory list in this leaf's
             // frame (source x h_s / h + centre offset / h, exactly: h_s / h is a power of two and
             // the rounding of the sum joins the remainder), 32 leaves at a time; the list begins
@@ -1818,23 +1928,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_leaf_a(Adaptive
             fz = ((double)sum.zh + (double)sum.zl) * ih * ih;
         }
         // M2P from the W list (Sec. 3.2): phi = F/h_w, E = -grad_s F / h_w^2
-        if constexpr (sizeof(T) == 8) {
-            for (int wi = w0; wi < w1; ++wi) {
-                const int wb = av.w_idx[wi];
-                if (!DAFMM_IN(wb, av.nbox, kChkBoxIndex)) continue;
-                double wx, wy, wz, wh;
-                abox_geom(av, wb, wx, wy, wz, wh);
-                const double iwh = 1.0 / wh;
-                T F, g0, g1, g2;
-                const T sx0 = (T)((av.x[tt] - wx) * iwh), sy0 = (T)((av.y[tt] - wy) * iwh),
-                        sz0 = (T)((av.z[tt] - wz) * iwh);
-                gen::GEN(m2p)<T>(RowLoad<T>{M + (size_t)wb * NCP}, sx0, sy0, sz0, F, g0, g1, g2);
-                fphi += (double)F * iwh;
-                fx -= (double)g0 * iwh * iwh;
-                fy -= (double)g1 * iwh * iwh;
-                fz -= (double)g2 * iwh * iwh;
-            }
-        } else {
+        {
             // FP32, without FP64 instructions (this part runs FP64 at 1/64 of the FP32 rate): the
             // W box is finer than the leaf by dl levels of the same tree, so with integer box
             // coordinates i at each level (c_b - c_w) / h_w = ((2 i_b + 1) 2^dl - (2 i_w + 1)) / 2
@@ -1871,8 +1965,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_leaf_a(Adaptive
                 const float sy0 = fmaf(plw.y, r, fmaf(pw.y, r, oy));
                 const float sz0 = fmaf(plw.z, r, fmaf(pw.z, r, oz));
                 const float iw = ihf * r;
-                T F, g0, g1, g2;
-                gen::GEN(m2p)<T>(SmemRowF{mrow}, sx0, sy0, sz0, F, g0, g1, g2);
+                float F, g0, g1, g2;
+                gen::GEN(m2p)<float>(SmemRowF{mrow}, sx0, sy0, sz0, F, g0, g1, g2);
                 wphi = fmaf(F, iw, wphi);
                 const float iw2 = iw * iw;
                 wfx = fmaf(-g0, iw2, wfx);
@@ -1893,18 +1987,9 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_leaf_a(Adaptive
         }
         // L2P of this leaf's local expansion
         if (lev >= 2) {
-            T F, g0, g1, g2;
-            T xs, ys, zs;
-            if constexpr (sizeof(T) == 8) {
-                xs = (T)((av.x[tt] - cx) * ih);
-                ys = (T)((av.y[tt] - cy) * ih);
-                zs = (T)((av.z[tt] - cz) * ih);
-            } else {
-                const float4 pt = xq_load(av.xq, av.xq0[b] + (tt - i0));
-                xs = (T)pt.x; ys = (T)pt.y; zs = (T)pt.z;
-            }
-            if constexpr (sizeof(T) == 4) gen::GEN(l2p)<T>(SmemRowF{lrow}, xs, ys, zs, F, g0, g1, g2);
-            else gen::GEN(l2p)<T>(RowLoad<T>{L + (size_t)b * NCP}, xs, ys, zs, F, g0, g1, g2);
+            float F, g0, g1, g2;
+            const float4 pt = xq_load(av.xq, av.xq0[b] + (tt - i0));
+            gen::GEN(l2p)<float>(SmemRowF{lrow}, pt.x, pt.y, pt.z, F, g0, g1, g2);
             fphi += (double)F;
             fx -= (double)g0 * ih;
             fy -= (double)g1 * ih;
@@ -1917,6 +2002,86 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_leaf_a(Adaptive
                 field[3 * (size_t)o] = fx;
                 field[3 * (size_t)o + 1] = fy;
                 field[3 * (size_t)o + 2] = fz;
+            }
+        }
+    }
+}
+
+// The same in FP64: a block of kLeaf64Warps warps per leaf and every blockIdx.y-th of its passes;
+// the warps share out the U-list sources and the W boxes of a pass.  How a leaf's sums are split
+// depends on the leaf and its lists alone (a member of a forest sums as the same tree built
+// alone).  Measured against one warp per leaf with passes of 32 and CUDA's rsqrt: Gaussian
+// N = 100,003, s = 256, p = 8: 37.4 -> 10.1 ms (the few largest leaves held the others up).
+constexpr int kLeaf64Warps = 4;
+__global__ void __launch_bounds__(32 * kLeaf64Warps, 4)
+    k_leaf64_a(AdaptiveView av, const int* __restrict__ leaves, const double* __restrict__ L,
+               const double* __restrict__ M, double* __restrict__ phi, double* __restrict__ field) {
+    constexpr int NW = kLeaf64Warps;
+    __shared__ Sum64 red[2][NW][32];
+    const int lane = threadIdx.x, warp = threadIdx.y;
+    const int b = leaves[blockIdx.x];
+    if (!DAFMM_IN(b, av.nbox, kChkBoxIndex)) return;
+    int i0 = av.pbeg[b], i1 = av.pend[b];
+    if (!DAFMM_RANGE(i0, i1, av.n, kChkBoxRange)) i0 = i1 = 0;
+    int u0 = av.u_ptr[b], u1 = av.u_ptr[b + 1];
+    int w0 = av.w_ptr[b], w1 = av.w_ptr[b + 1];
+    if (!DAFMM_RANGE(u0, u1, av.nu, kChkListPtr)) u0 = u1 = 0;
+    if (!DAFMM_RANGE(w0, w1, av.nw, kChkListPtr)) w0 = w1 = 0;
+    int turn = 0, pass = 0;
+    for (int base = i0, W; base < i1; base += W, ++pass) {
+        W = pass_width(i1 - base);
+        if (pass % gridDim.y != blockIdx.y) continue;
+        const int G = NW * (32 / W), g = warp * (32 / W) + lane / W;
+        const int t = base + (lane & (W - 1)), tt = t < i1 ? t : i0;
+        const double xt = av.x[tt], yt = av.y[tt], zt = av.z[tt];
+        Sum64 s;
+        for (int ug = u0; ug < u1; ug += 32) {
+            int cnt = 0, first = 0;
+            const int sb = ug + lane < u1 ? av.u_idx[ug + lane] : -1;
+            if (sb >= 0 && DAFMM_IN(sb, av.nbox, kChkBoxIndex) &&
+                DAFMM_RANGE(av.pbeg[sb], av.pend[sb], av.n, kChkBoxRange)) {
+                first = av.pbeg[sb];
+                cnt = av.pend[sb] - first;
+            }
+            near64_list(av.x, av.y, av.z, av.q, cnt, first, G, g, lane, xt, yt, zt, s);
+        }
+        // M2P from the W list (Sec. 3.2): phi = F / h_w, E = -grad_s F / h_w^2
+        for (int wi = w0 + g; wi < w1; wi += G) {
+            const int wb = av.w_idx[wi];
+            if (!DAFMM_IN(wb, av.nbox, kChkBoxIndex)) continue;
+            double wx, wy, wz, wh;
+            abox_geom(av, wb, wx, wy, wz, wh);
+            const double iwh = 1.0 / wh;
+            double F, g0, g1, g2;
+            gen::GEN(m2p)<double>(RowLoad<double>{M + (size_t)wb * NCP}, (xt - wx) * iwh, (yt - wy) * iwh,
+                                  (zt - wz) * iwh, F, g0, g1, g2);
+            s.p += F * iwh;
+            s.x -= g0 * iwh * iwh;
+            s.y -= g1 * iwh * iwh;
+            s.z -= g2 * iwh * iwh;
+        }
+        __syncwarp();
+        s = pass_join<NW>(s, W, warp, lane, red, turn);
+        if (warp != 0) continue;
+        if (av.level[b] >= 2) {  // L2P of this leaf's local expansion
+            double cx, cy, cz, h;
+            abox_geom(av, b, cx, cy, cz, h);
+            const double ih = 1.0 / h;
+            double F, g0, g1, g2;
+            gen::GEN(l2p)<double>(RowLoad<double>{L + (size_t)b * NCP}, (xt - cx) * ih, (yt - cy) * ih, (zt - cz) * ih,
+                                  F, g0, g1, g2);
+            s.p += F;
+            s.x -= g0 * ih;
+            s.y -= g1 * ih;
+            s.z -= g2 * ih;
+        }
+        if (lane < W && t < i1 && DAFMM_IN(av.perm[t], av.n, kChkPerm)) {
+            const size_t o = (size_t)av.perm[t];
+            if (phi) phi[o] = s.p;
+            if (field) {
+                field[3 * o] = s.x;
+                field[3 * o + 1] = s.y;
+                field[3 * o + 2] = s.z;
             }
         }
     }
@@ -2090,9 +2255,16 @@ static cudaError_t leaf_launch(const TreeView& tv, int prec, const double* Lleaf
                                cudaStream_t s) {
     if (tv.nleaf == 0) return cudaSuccess;
     dim3 blk(32, kLeafWarps), grd((tv.nleaf + kLeafWarps - 1) / kLeafWarps);
-    if (prec == DAFMM_FP64) k_leaf<double><<<grd, blk, 0, s>>>(tv, Lleaf, phi, field);
-    else if (prec == DAFMM_FF) k_leaf<ff><<<grd, blk, 0, s>>>(tv, Lleaf, phi, field);
-    else k_leaf<float><<<grd, blk, 0, s>>>(tv, Lleaf, phi, field);
+    if (prec == DAFMM_FP64) {
+        // about 16 warps per SM or more from 2432 leaves on; below, more warps per leaf
+        if (tv.nleaf >= 2432) k_leaf64<1><<<tv.nleaf, dim3(32, 1), 0, s>>>(tv, Lleaf, phi, field);
+        else if (tv.nleaf >= 1216) k_leaf64<2><<<tv.nleaf, dim3(32, 2), 0, s>>>(tv, Lleaf, phi, field);
+        else k_leaf64<8><<<tv.nleaf, dim3(32, 8), 0, s>>>(tv, Lleaf, phi, field);
+    } else if (prec == DAFMM_FF) {
+        k_leaf<ff><<<grd, blk, 0, s>>>(tv, Lleaf, phi, field);
+    } else {
+        k_leaf<float><<<grd, blk, 0, s>>>(tv, Lleaf, phi, field);
+    }
     return cudaGetLastError();
 }
 
@@ -2266,17 +2438,19 @@ static cudaError_t l2l_a_launch(const OrderData& od, const AdaptiveView& av, int
 
 static cudaError_t leaf_a_launch(const AdaptiveView& av, const int* leaves, int nleaves, int prec, const double* L,
                                  const double* M, const float* Mf, double* phi, double* field, int warps,
-                                 cudaStream_t s) {
+                                 int max_leaf, cudaStream_t s) {
     if (nleaves == 0) return cudaSuccess;
     warps = warps < 1 ? 1 : (warps > 8 ? 8 : warps);
     dim3 blk(32, warps), grd((nleaves + warps - 1) / warps);
     if (prec == DAFMM_FP64) {
-        k_leaf_a<double><<<grd, blk, 0, s>>>(av, leaves, nleaves, L, M, nullptr, phi, field);
+        // blocks per leaf: one per pass of the largest leaf, up to 8
+        const int ny = max_leaf < 32 ? 1 : (max_leaf > 8 * 32 ? 8 : (max_leaf + 31) / 32);
+        k_leaf64_a<<<dim3(nleaves, ny), dim3(32, kLeaf64Warps), 0, s>>>(av, leaves, L, M, phi, field);
     } else {
         const size_t smem = (size_t)warps * kLeafWarpSmem;
-        cudaError_t e = cudaFuncSetAttribute(k_leaf_a<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(k_leaf_a, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        k_leaf_a<float><<<grd, blk, smem, s>>>(av, leaves, nleaves, L, M, Mf, phi, field);
+        k_leaf_a<<<grd, blk, smem, s>>>(av, leaves, nleaves, L, M, Mf, phi, field);
     }
     return cudaGetLastError();
 }
