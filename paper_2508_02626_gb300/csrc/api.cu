@@ -1013,7 +1013,9 @@ int forest_domains(dafmm_ctx* c, const double* dxyz, const std::vector<int>& off
     int rc = bb.alloc((size_t)nroots * 6 * 8, "bbox");
     if (rc) return rc;
     std::vector<unsigned long long> h(6 * (size_t)nroots);
-    cudaError_t e = launch_bbox_roots(dxyz, d_offs, nroots, bb.as<unsigned long long>(), s);
+    int max_n = 0;
+    for (int r = 0; r < nroots; ++r) max_n = std::max(max_n, offs[r + 1] - offs[r]);
+    cudaError_t e = launch_bbox_roots(dxyz, d_offs, nroots, max_n, bb.as<unsigned long long>(), s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h.data(), bb.p, h.size() * 8, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(c, e, "bounding boxes");
@@ -1095,15 +1097,20 @@ int build_adaptive(dafmm_ctx* c, dafmm_tree* t, const double* dxyz, const double
         CK(c, cudaStreamSynchronize(s), "roots");
     }
     t->level_start.assign({0, nroots});
+    Scratch scan_tmp(c);  // (grown with the number of boxes)
+    auto scan_room = [&](int64_t cnt) {
+        return scan_tmp.bytes >= scan_temp_ints(cnt) * 4 ? DAFMM_OK : scan_tmp.alloc(scan_temp_ints(2 * cnt) * 4, "scan scratch");
+    };
     for (int l = 0; l < max_depth; ++l) {
         const int lb = t->level_start[l], le = t->level_start[l + 1];
         const int nl = le - lb;
         if (scratch.bytes < 2 * ((size_t)nl + 1) * 4 && (rc = scratch.alloc(2 * ((size_t)nl + 1) * 4, "split scratch")))
             return rc;
+        if ((rc = scan_room(nl))) return rc;
         int* cnt = scratch.as<int>();
         int* off = cnt + nl + 1;
         e = launch_split(abuild(t, keys.as<uint64_t>()), lb, le, l, max_leaf, max_depth, cnt, s);
-        if (e == cudaSuccess) e = launch_scan(cnt, off, nl, s);
+        if (e == cudaSuccess) e = launch_scan(cnt, off, nl, scan_tmp.as<int>(), s);
         int total = 0;
         if (e == cudaSuccess) e = cudaMemcpyAsync(&total, off + nl, 4, cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -1134,8 +1141,9 @@ int build_adaptive(dafmm_ctx* c, dafmm_tree* t, const double* dxyz, const double
     int* pstart = foff + nbox + 1;
     LevelStarts ls;
     for (int l = 0; l <= nlev; ++l) ls.v[l] = t->level_start[l];
+    if ((rc = scan_room(nbox))) return rc;
     e = launch_leaf_flags(t->a_child, nbox, flags, s);
-    if (e == cudaSuccess) e = launch_scan(flags, foff, nbox, s);
+    if (e == cudaSuccess) e = launch_scan(flags, foff, nbox, scan_tmp.as<int>(), s);
     if (e == cudaSuccess) e = launch_parent_starts(ls, nlev, foff, pstart, s);
     t->parent_start.assign(nlev + 1, 0);
     if (e == cudaSuccess)
@@ -1159,7 +1167,7 @@ int build_adaptive(dafmm_ctx* c, dafmm_tree* t, const double* dxyz, const double
     }
     if ((rc = dev_alloc(c, (void**)&t->a_xq0, (size_t)nbox * sizeof(int), "leaf records"))) return rc;
     CK(c, cudaMemsetAsync(t->a_xq0, 0, (size_t)nbox * sizeof(int), s), "memset");
-    e = launch_leaf_records(t->leaves, nl, t->a_pbeg, t->a_pend, flags, foff, t->a_xq0, s);
+    e = launch_leaf_records(t->leaves, nl, t->a_pbeg, t->a_pend, flags, foff, scan_tmp.as<int>(), t->a_xq0, s);
     if (e == cudaSuccess)
         e = launch_gather_adaptive(dxyz, dq, t->perm, abuild(t, keys.as<uint64_t>()), t->leaves, nl, t->a_geom,
                                    t->a_xq0, t->x, t->y, t->z, t->q, t->xq, t->xq_n4, t->n, s);
@@ -1178,9 +1186,8 @@ int build_adaptive(dafmm_ctx* c, dafmm_tree* t, const double* dxyz, const double
         return rc;
     CK(c, cudaMemsetAsync(nv, 0, 16, s), "counter");  // the V-pair counter and lflag
     e = launch_list_count(abuild(t, keys.as<uint64_t>()), nbox, cu, cu + nb1, cu + 2 * nb1, nv, lflag, s);
-    if (e == cudaSuccess) e = launch_scan(cu, t->u_ptr, nbox, s);
-    if (e == cudaSuccess) e = launch_scan(cu + nb1, t->w_ptr, nbox, s);
-    if (e == cudaSuccess) e = launch_scan(cu + 2 * nb1, t->x_ptr, nbox, s);
+    const ScanJobs lists = {{cu, cu + nb1, cu + 2 * nb1}, {t->u_ptr, t->w_ptr, t->x_ptr}};
+    if (e == cudaSuccess) e = launch_scans(lists, 3, nbox, scan_tmp.as<int>(), s);
     int tot[3] = {0, 0, 0};
     unsigned long long nvh = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&tot[0], t->u_ptr + nbox, 4, cudaMemcpyDeviceToHost, s);

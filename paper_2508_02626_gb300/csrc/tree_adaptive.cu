@@ -111,10 +111,13 @@ __device__ inline unsigned long long ordered_bits(double v) {
 
 __global__ void __launch_bounds__(256) k_bbox_roots(const double* __restrict__ xyz, const int* __restrict__ offs,
                                                     unsigned long long* bb) {
+    // blocks (r, 0 ..) of problem r stride over its particles: one block per problem took 2.2 ms on
+    // a problem of 1e6 particles beside small ones, many blocks 20 us
     const int r = blockIdx.x;
     const int b = offs[r], e = offs[r + 1];
+    if (b + (int)(blockIdx.y * blockDim.x) >= e) return;
     unsigned long long mn[3] = {~0ull, ~0ull, ~0ull}, mx[3] = {0ull, 0ull, 0ull};
-    for (int i = b + threadIdx.x; i < e; i += blockDim.x)
+    for (int i = b + blockIdx.y * blockDim.x + threadIdx.x; i < e; i += gridDim.y * blockDim.x)
         for (int d = 0; d < 3; ++d) {
             const unsigned long long u = ordered_bits(xyz[3 * (size_t)i + d]);
             mn[d] = u < mn[d] ? u : mn[d];
@@ -139,10 +142,12 @@ __global__ void k_bbox_init(unsigned long long* bb, int nroots) {
     if (i < 6 * nroots) bb[i] = (i % 6) < 3 ? ~0ull : 0ull;
 }
 
-cudaError_t launch_bbox_roots(const double* xyz, const int* offs, int nroots, unsigned long long* bb, cudaStream_t s) {
+cudaError_t launch_bbox_roots(const double* xyz, const int* offs, int nroots, int max_n, unsigned long long* bb,
+                              cudaStream_t s) {
     if (nroots == 0) return cudaSuccess;
     k_bbox_init<<<(6 * nroots + 255) / 256, 256, 0, s>>>(bb, nroots);
-    k_bbox_roots<<<nroots, 256, 0, s>>>(xyz, offs, bb);
+    const int per = (max_n + 2047) / 2048;  // blocks of the largest problem: 8 particles per thread
+    k_bbox_roots<<<dim3(nroots, per < 1 ? 1 : (per > 608 ? 608 : per)), 256, 0, s>>>(xyz, offs, bb);
     return cudaGetLastError();
 }
 
@@ -174,36 +179,38 @@ __device__ inline int first_digit_ge(const uint64_t* keys, int b, int e, int shi
     return b;
 }
 
+// Children of the boxes of level l: eight lanes per box, lane c searching the end of child c's
+// particles (one thread per box ran the eight searches, some 20 dependent loads each, one after
+// another).  [s, e): child c's particles, empty when the box does not split.
+__device__ inline void child_range(const AdaptiveBuild& ab, int b, int level, bool split, int c, int& s, int& e) {
+    const int pb = ab.pbeg[b], pe = ab.pend[b];
+    e = split ? first_digit_ge(ab.keys, pb, pe, 3 * (kQBits - level - 1), c + 1) : pb;
+    s = __shfl_up_sync(0xffffffffu, e, 1, 8);
+    if (c == 0) s = pb;
+}
+
 // per box of level l: number of non-empty children when it splits
 __global__ void k_split_count(AdaptiveBuild ab, int lb, int le, int level, int max_leaf, int max_depth, int* nch) {
-    const int b = lb + blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= le) return;
-    const int pb = ab.pbeg[b], pe = ab.pend[b];
-    int cnt = 0;
-    if (pe - pb > max_leaf && level < max_depth) {
-        const int shift = 3 * (kQBits - level - 1);
-        int s = pb;
-        for (int c = 0; c < 8; ++c) {
-            const int e = first_digit_ge(ab.keys, s, pe, shift, c + 1);
-            cnt += e > s;
-            s = e;
-        }
-    }
-    nch[b - lb] = cnt;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, c = i & 7;
+    const int b = min(lb + (i >> 3), le - 1);
+    int s, e;
+    child_range(ab, b, level, ab.pend[b] - ab.pbeg[b] > max_leaf && level < max_depth, c, s, e);
+    const unsigned any = __ballot_sync(0xffffffffu, e > s);
+    if (c == 0 && lb + (i >> 3) < le) nch[b - lb] = __popc((any >> (threadIdx.x & 24)) & 0xffu);
 }
 
 __global__ void k_split_fill(AdaptiveBuild ab, int lb, int le, int level, const int* offs, int first_new) {
-    const int b = lb + blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= le) return;
-    for (int c = 0; c < 8; ++c) ab.child[8 * b + c] = -1;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, c = i & 7;
+    const int b = min(lb + (i >> 3), le - 1);
     const int k0 = offs[b - lb], k1 = offs[b - lb + 1];
-    if (k0 == k1) return;
-    const int pb = ab.pbeg[b], pe = ab.pend[b];
-    const int shift = 3 * (kQBits - level - 1);
-    int s = pb, k = first_new + k0;
-    for (int c = 0; c < 8; ++c) {
-        const int e = first_digit_ge(ab.keys, s, pe, shift, c + 1);
-        if (e > s && DAFMM_IN(k, ab.cap, kChkSplitChild)) {
+    int s, e;
+    child_range(ab, b, level, k1 > k0, c, s, e);
+    const unsigned any = (__ballot_sync(0xffffffffu, e > s) >> (threadIdx.x & 24)) & 0xffu;
+    if (lb + (i >> 3) >= le) return;
+    int k = -1;
+    if (e > s) {
+        k = first_new + k0 + __popc(any & ((1u << c) - 1u));
+        if (DAFMM_IN(k, ab.cap, kChkSplitChild)) {
             ab.root[k] = ab.root[b];
             ab.level[k] = level + 1;
             ab.ijk[3 * k] = 2 * ab.ijk[3 * b] + (c & 1);
@@ -212,11 +219,11 @@ __global__ void k_split_fill(AdaptiveBuild ab, int lb, int le, int level, const 
             ab.parent[k] = b;
             ab.pbeg[k] = s;
             ab.pend[k] = e;
-            ab.child[8 * b + c] = k;
-            ++k;
+        } else {
+            k = -1;
         }
-        s = e;
     }
+    ab.child[8 * b + c] = k;
 }
 
 __global__ void k_leaf_children_init(int* child, int b0, int b1) {
@@ -229,7 +236,7 @@ cudaError_t launch_split(AdaptiveBuild ab, int lb, int le, int level, int max_le
                          cudaStream_t s) {
     const int n = le - lb;
     if (n == 0) return cudaSuccess;
-    k_split_count<<<(n + 127) / 128, 128, 0, s>>>(ab, lb, le, level, max_leaf, max_depth, nch);
+    k_split_count<<<(n + 15) / 16, 128, 0, s>>>(ab, lb, le, level, max_leaf, max_depth, nch);
     return cudaGetLastError();
 }
 
@@ -237,7 +244,7 @@ cudaError_t launch_split_fill(AdaptiveBuild ab, int lb, int le, int level, const
                               cudaStream_t s) {
     const int n = le - lb;
     if (n == 0) return cudaSuccess;
-    k_split_fill<<<(n + 127) / 128, 128, 0, s>>>(ab, lb, le, level, offs, first_new);
+    k_split_fill<<<(n + 15) / 16, 128, 0, s>>>(ab, lb, le, level, offs, first_new);
     return cudaGetLastError();
 }
 
@@ -247,37 +254,77 @@ cudaError_t launch_children_init(int* child, int b0, int b1, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// exclusive scan of n ints by one block (n up to a few million; used at build time only); in
-// and out are distinct, so the loads of a chunk need not wait for its stores
-__global__ void __launch_bounds__(1024) k_scan_excl(const int* __restrict__ in, int* __restrict__ out, int n) {
-    __shared__ int sums[1024];
-    const int t = threadIdx.x;
-    const int chunk = (n + 1023) / 1024;
-    const int b = t * chunk, e = min(b + chunk, n);
-    int s = 0;
-#pragma unroll 8
-    for (int i = b; i < e; ++i) s += in[i];
-    sums[t] = s;
+// Exclusive scans of n ints (out[n] = total), in tiles of 2048 per block: the tiles' sums first,
+// then every block adds the sums of the tiles before its own and scans it.  One block walking the
+// whole array, each thread a chunk of its own, took about 20 us at any size.
+constexpr int kScanTile = 2048;
+
+__device__ inline int block_sum_256(int v, int* sh) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
     __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {
-        int v = t >= off ? sums[t - off] : 0;
-        __syncthreads();
-        sums[t] += v;
-        __syncthreads();
-    }
-    int run = t ? sums[t - 1] : 0;
-#pragma unroll 8
-    for (int i = b; i < e; ++i) {
-        const int v = in[i];
-        out[i] = run;
-        run += v;
-    }
-    if (t == 1023) out[n] = sums[1023];
+    int t = 0;
+    for (int w = 0; w < 8; ++w) t += sh[w];
+    __syncthreads();
+    return t;
 }
 
-cudaError_t launch_scan(const int* in, int* out, int n, cudaStream_t s) {
-    k_scan_excl<<<1, 1024, 0, s>>>(in, out, n);
+__global__ void __launch_bounds__(256) k_tile_sums(ScanJobs jobs, int n, int* __restrict__ sums, int ntile) {
+    __shared__ int sh[8];
+    const int* in = jobs.in[blockIdx.y];
+    const int base = blockIdx.x * kScanTile;
+    int v = 0;
+    for (int i = base + threadIdx.x; i < min(base + kScanTile, n); i += 256) v += in[i];
+    v = block_sum_256(v, sh);
+    if (threadIdx.x == 0) sums[blockIdx.y * ntile + blockIdx.x] = v;
+}
+
+__global__ void __launch_bounds__(256) k_tile_scan(ScanJobs jobs, int n, const int* __restrict__ sums, int ntile) {
+    __shared__ int sh[8];
+    const int* in = jobs.in[blockIdx.y];
+    int* out = jobs.out[blockIdx.y];
+    const int base = blockIdx.x * kScanTile;
+    int before = 0;
+    for (int t = threadIdx.x; t < (int)blockIdx.x; t += 256) before += sums[blockIdx.y * ntile + t];
+    int run = block_sum_256(before, sh);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int i0 = base; i0 < min(base + kScanTile, n); i0 += 256) {
+        const int i = i0 + threadIdx.x;
+        const int v = i < n ? in[i] : 0;
+        int incl = v;
+        for (int d = 1; d < 32; d <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += u;
+        }
+        if (lane == 31) sh[w] = incl;
+        __syncthreads();
+        int pre = 0, tot = 0;
+        for (int k = 0; k < 8; ++k) {
+            pre += k < w ? sh[k] : 0;
+            tot += sh[k];
+        }
+        __syncthreads();
+        if (i < n) out[i] = run + pre + incl - v;
+        run += tot;
+    }
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = run;
+}
+
+size_t scan_temp_ints(int64_t n) { return 3 * (size_t)(n / kScanTile + 2); }
+
+cudaError_t launch_scans(const ScanJobs& jobs, int njobs, int n, int* temp, cudaStream_t s) {
+    const int ntile = n > 0 ? (n + kScanTile - 1) / kScanTile : 1;
+    const dim3 grd(ntile, njobs);
+    if (ntile > 1) k_tile_sums<<<grd, 256, 0, s>>>(jobs, n, temp, ntile);
+    k_tile_scan<<<grd, 256, 0, s>>>(jobs, n, temp, ntile);
     return cudaGetLastError();
+}
+
+cudaError_t launch_scan(const int* in, int* out, int n, int* temp, cudaStream_t s) {
+    ScanJobs j;
+    j.in[0] = in;
+    j.out[0] = out;
+    return launch_scans(j, 1, n, temp, s);
 }
 
 // ---- colleagues ---------------------------------------------------------------------------
@@ -301,32 +348,27 @@ __device__ inline bool touch(const AdaptiveBuild& ab, int a, int b) {
     return true;
 }
 
+// Colleague k of box b, at relative position (dx, dy, dz): one thread each.  Its parent is the
+// colleague of b's parent at offset floor((i_b + d) / 2) - floor(i_b / 2), its octant the parity.
+// (One thread per box tested all children of the parent's colleagues.)
 __global__ void k_colleagues(AdaptiveBuild ab, int lb, int le) {
-    const int b = lb + blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int b = lb + i / 27, k = i % 27;
     if (b >= le) return;
-    int* col = ab.colleague + 27 * b;
-    for (int k = 0; k < 27; ++k) col[k] = -1;
-    col[13] = b;
+    int c = k == 13 ? b : -1;
     const int P = ab.parent[b];
-    if (P < 0) return;
-    const int* pc = ab.colleague + 27 * P;
-    for (int k = 0; k < 27; ++k) {
-        const int Q = pc[k];
-        if (Q < 0) continue;
-        for (int c = 0; c < 8; ++c) {
-            const int ch = ab.child[8 * Q + c];
-            if (ch < 0 || ch == b) continue;
-            if (!same_level_adjacent(ab.ijk, ch, b)) continue;
-            const int dx = ab.ijk[3 * ch] - ab.ijk[3 * b], dy = ab.ijk[3 * ch + 1] - ab.ijk[3 * b + 1],
-                      dz = ab.ijk[3 * ch + 2] - ab.ijk[3 * b + 2];
-            col[(dx + 1) * 9 + (dy + 1) * 3 + (dz + 1)] = ch;
-        }
+    if (P >= 0 && k != 13) {
+        const int nx = (ab.ijk[3 * b] & 1) + k / 9 - 1, ny = (ab.ijk[3 * b + 1] & 1) + (k / 3) % 3 - 1,
+                  nz = (ab.ijk[3 * b + 2] & 1) + k % 3 - 1;  // in [-1, 2]: parent offset n >> 1, parity n & 1
+        const int Q = ab.colleague[27 * (size_t)P + ((nx >> 1) + 1) * 9 + ((ny >> 1) + 1) * 3 + ((nz >> 1) + 1)];
+        if (Q >= 0) c = ab.child[8 * (size_t)Q + ((nx & 1) | ((ny & 1) << 1) | ((nz & 1) << 2))];
     }
+    ab.colleague[27 * (size_t)b + k] = c;
 }
 
 cudaError_t launch_colleagues(AdaptiveBuild ab, int lb, int le, cudaStream_t s) {
     if (le <= lb) return cudaSuccess;
-    k_colleagues<<<(le - lb + 127) / 128, 128, 0, s>>>(ab, lb, le);
+    k_colleagues<<<(unsigned)(((size_t)(le - lb) * 27 + 255) / 256), 256, 0, s>>>(ab, lb, le);
     return cudaGetLastError();
 }
 
@@ -515,10 +557,10 @@ __global__ void k_leaf_xq0(const int* __restrict__ leaves, int nl, const int* __
 }
 
 cudaError_t launch_leaf_records(const int* leaves, int nl, const int* pbeg, const int* pend, int* cnt, int* off,
-                                int* xq0, cudaStream_t s) {
+                                int* temp, int* xq0, cudaStream_t s) {
     if (nl == 0) return cudaSuccess;
     k_leaf_pairs<<<(nl + 255) / 256, 256, 0, s>>>(leaves, nl, pbeg, pend, cnt);
-    cudaError_t e = launch_scan(cnt, off, nl, s);
+    cudaError_t e = launch_scan(cnt, off, nl, temp, s);
     if (e != cudaSuccess) return e;
     k_leaf_xq0<<<(nl + 255) / 256, 256, 0, s>>>(leaves, nl, off, xq0);
     return cudaGetLastError();

@@ -63,8 +63,9 @@ cudaError_t launch_tree_keys(const int* perm, int64_t n, const int* offs, int nr
                              cudaStream_t s);
 cudaError_t launch_apply_order(const int* pos, int64_t n, const int* perm_in, const uint64_t* keys_in, int* perm_out,
                                uint64_t* keys_out, cudaStream_t s);
-// per-tree bounding boxes as ordered-integer min/max (6 per tree), one CTA per tree
-cudaError_t launch_bbox_roots(const double* xyz, const int* offs, int nroots, unsigned long long* bb, cudaStream_t s);
+// per-tree bounding boxes as ordered-integer min/max (6 per tree); max_n: particles of the largest
+cudaError_t launch_bbox_roots(const double* xyz, const int* offs, int nroots, int max_n, unsigned long long* bb,
+                              cudaStream_t s);
 cudaError_t launch_box_geometry(const int* root, const int* level, const int* ijk, const double* rootdom, int nbox,
                                 double4* geom, cudaStream_t s);
 cudaError_t launch_split(AdaptiveBuild ab, int lb, int le, int level, int max_leaf, int max_depth, int* nch,
@@ -72,7 +73,14 @@ cudaError_t launch_split(AdaptiveBuild ab, int lb, int le, int level, int max_le
 cudaError_t launch_split_fill(AdaptiveBuild ab, int lb, int le, int level, const int* offs, int first_new,
                               cudaStream_t s);
 cudaError_t launch_children_init(int* child, int b0, int b1, cudaStream_t s);
-cudaError_t launch_scan(const int* in, int* out, int n, cudaStream_t s);  // out[n] = total
+// exclusive scans (out[n] = total) of up to three arrays of n ints; temp: scan_temp_ints(n) ints
+struct ScanJobs {
+    const int* in[3];
+    int* out[3];
+};
+size_t scan_temp_ints(int64_t n);
+cudaError_t launch_scans(const ScanJobs& jobs, int njobs, int n, int* temp, cudaStream_t s);
+cudaError_t launch_scan(const int* in, int* out, int n, int* temp, cudaStream_t s);
 cudaError_t launch_colleagues(AdaptiveBuild ab, int lb, int le, cudaStream_t s);
 cudaError_t launch_list_count(AdaptiveBuild ab, int nbox, int* cu, int* cw, int* cx, unsigned long long* nv, int* err,
                               cudaStream_t s);
@@ -81,7 +89,7 @@ cudaError_t launch_list_fill(AdaptiveBuild ab, int nbox, const int* pu, const in
 // first FP32 record of every leaf box (xq0[b], even): the leaves of the list take consecutive
 // record ranges of 2 ceil(n / 2) records; cnt and off are scratch of nl and nl + 1 ints
 cudaError_t launch_leaf_records(const int* leaves, int nl, const int* pbeg, const int* pend, int* cnt, int* off,
-                                int* xq0, cudaStream_t s);
+                                int* temp, int* xq0, cudaStream_t s);
 cudaError_t launch_gather_adaptive(const double* xyz, const double* q, const int* perm, AdaptiveBuild ab,
                                    const int* leaves, int nleaves, const double4* geom, const int* xq0, double* x,
                                    double* y, double* z, double* qs, float4* xq, size_t xq_n4, int64_t n, cudaStream_t s);
