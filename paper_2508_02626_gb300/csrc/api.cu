@@ -375,6 +375,17 @@ int ensure_order(dafmm_ctx* c, int p, cudaStream_t s, bool need_k) {
     return DAFMM_OK;
 }
 
+void free_rot_form(dafmm_ctx* c, const OrderData& od, RotForm& f) {
+    const size_t ni = (size_t)32 * (f.lx + f.lz + f.la), nv = (size_t)kNumKeys * 64 * (f.lx + f.lz),
+                 na = (size_t)od.n_rho * 32 * f.la;
+    dev_free(c, f.idx, ni * sizeof(unsigned));
+    dev_free(c, f.val, nv * sizeof(double));
+    dev_free(c, f.ax, na * sizeof(double));
+    dev_free(c, f.valf, nv * sizeof(float2));
+    dev_free(c, f.axf, na * sizeof(float2));
+    f = RotForm();
+}
+
 void free_order(dafmm_ctx* c, OrderData& od) {
     const int nc = od.nc;
     const OrderOps* ops = od.p >= 0 ? order_ops(od.p) : nullptr;
@@ -438,17 +449,7 @@ void free_order(dafmm_ctx* c, OrderData& od) {
         dev_free(c, od.ax_rowptr, ((size_t)nc + 1) * sizeof(int));
         dev_free(c, od.ax_col, (size_t)od.ax_nnz * sizeof(unsigned short));
         dev_free(c, od.ax_val, (size_t)od.n_rho * od.ax_nnz * sizeof(double));
-        dev_free(c, od.rot_lx, (size_t)od.rot_len[0] * 32 * sizeof(uint2));
-        dev_free(c, od.rot_lz, (size_t)od.rot_len[1] * 32 * sizeof(uint2));
-        dev_free(c, od.rot_la, (size_t)od.rot_len[2] * 32 * sizeof(uint2));
-        dev_free(c, od.rot_lxh, (size_t)od.rot_lenh[0] * 32 * sizeof(uint2));
-        dev_free(c, od.rot_lzh, (size_t)od.rot_lenh[1] * 32 * sizeof(uint2));
-        dev_free(c, od.rot_lah, (size_t)od.rot_lenh[2] * 32 * sizeof(uint2));
-        const size_t nhs = std::max<size_t>((size_t)(ncoef_of(od.p) - nharm_of(od.p)), 1);
-        dev_free(c, od.hxr_step, nhs * sizeof(int4));
-        dev_free(c, od.hxr_w, nhs * sizeof(double2));
-        dev_free(c, od.rot_Tf, (size_t)kNumKeys * 4 * ops->rot_tsz * sizeof(float2));
-        dev_free(c, od.ax_valf, (size_t)od.n_rho * od.ax_nnz * sizeof(float2));
+        for (RotForm& f : od.rot) free_rot_form(c, od, f);
     }
     od = OrderData();
 }
@@ -607,20 +608,36 @@ int ensure_k16h(dafmm_ctx* c, int p, cudaStream_t s) {
     return DAFMM_OK;
 }
 
+// device scratch that is returned to the context when it goes out of scope
+struct Scratch {
+    dafmm_ctx* c;
+    void* p = nullptr;
+    size_t bytes = 0;
+    explicit Scratch(dafmm_ctx* ctx) : c(ctx) {}
+    int alloc(size_t b, const char* what) {
+        release();
+        bytes = b;
+        return dev_alloc(c, &p, b, what);
+    }
+    void release() {
+        dev_free(c, p, bytes);
+        p = nullptr;
+        bytes = 0;
+    }
+    template <class T>
+    T* as() const { return static_cast<T*>(p); }
+    ~Scratch() { release(); }
+};
+
 // tables of the M2L by rotation (Sec. 3.4) of an order (made once, on first use): the four
 // substitution tables of every displacement key, and the axial matrices of the distinct
 // lengths |v| as their structural non-zeros (row b, column a: b_y >= a_y, b_z >= a_z, both
 // differences even), the values taken from the K generation along the x axis
-int ensure_rotation(dafmm_ctx* c, int p, cudaStream_t s) {
+int ensure_rotation_tables(dafmm_ctx* c, int p, const RotStructure& rs, cudaStream_t s) {
     OrderData& od = c->ord[p];
     if (od.rot_T) return DAFMM_OK;
     const OrderOps* ops = order_ops(p);
-    const int nc = ncoef_of(p), ncp = ncp_of(p);
-    // the axial matrices' structure and the kernel's task lists (rot_lists.h)
-    const RotStructure rs = rot_structure(p);
-    const std::vector<int>& rowptr = rs.rowptr;
-    const std::vector<unsigned short>& col = rs.col;
-    const int nnz = (int)col.size();
+    const int nc = ncoef_of(p), ncp = ncp_of(p), nnz = (int)rs.col.size();
     std::vector<int> rho_of(kNumKeys, 0), len2;
     for (int key = 0; key < kNumKeys; ++key) {
         const int vx = key / 49 - 3, vy = (key / 7) % 7 - 3, vz = key % 7 - 3;
@@ -631,38 +648,16 @@ int ensure_rotation(dafmm_ctx* c, int p, cudaStream_t s) {
         if (it == len2.end()) len2.push_back(r2);
     }
     const int nrho = (int)len2.size();
-    static_assert(sizeof(RotTask) == sizeof(uint2), "task layout");
-    const std::vector<RotTask>& lx = rs.lx;
-    const std::vector<RotTask>& lz = rs.lz;
-    const std::vector<RotTask>& la = rs.la;
-    const int len_x = rs.len[0], len_z = rs.len[1], len_a = rs.len[2];
-    // the harmonic form: lists of the free outputs, and the steps restoring the others
-    const RotStructure rsh = rot_structure(p, true);
-    std::vector<int4> hstep;
-    std::vector<double2> hw;
-    int hcst[kMaxOrder + 3];
-    harm_steps(p, hstep, hw, hcst);
-    const size_t nhstep = std::max<size_t>(hstep.size(), 1);
     std::vector<double> r0s(3 * (size_t)nrho, 0.0);
     for (int r = 0; r < nrho; ++r) r0s[3 * r] = std::sqrt((double)len2[r]);
     const size_t tbytes = (size_t)kNumKeys * 4 * ops->rot_tsz * sizeof(double);
     const size_t kbytes = (size_t)nrho * nc * ncp * sizeof(double);
-    double *T = nullptr, *val = nullptr, *d_r0s = nullptr, *Ks = nullptr;
+    double *T = nullptr, *val = nullptr;
     int *rho = nullptr, *rp = nullptr;
     unsigned short* cl = nullptr;
-    uint2 *dlx = nullptr, *dlz = nullptr, *dla = nullptr, *dlxh = nullptr, *dlzh = nullptr, *dlah = nullptr;
-    int4* dhs = nullptr;
-    double2* dhw = nullptr;
+    Scratch d_r0s(c), Ks(c);
     int rc;
     auto release = [&]() {
-        dev_free(c, dlx, lx.size() * sizeof(uint2));
-        dev_free(c, dlz, lz.size() * sizeof(uint2));
-        dev_free(c, dla, la.size() * sizeof(uint2));
-        dev_free(c, dlxh, dlxh ? rsh.lx.size() * sizeof(uint2) : 0);
-        dev_free(c, dlzh, dlzh ? rsh.lz.size() * sizeof(uint2) : 0);
-        dev_free(c, dlah, dlah ? rsh.la.size() * sizeof(uint2) : 0);
-        dev_free(c, dhs, dhs ? nhstep * sizeof(int4) : 0);
-        dev_free(c, dhw, dhw ? nhstep * sizeof(double2) : 0);
         dev_free(c, T, tbytes);
         dev_free(c, val, (size_t)nrho * nnz * sizeof(double));
         dev_free(c, rho, (size_t)kNumKeys * sizeof(int));
@@ -674,85 +669,89 @@ int ensure_rotation(dafmm_ctx* c, int p, cudaStream_t s) {
         (rc = dev_alloc(c, (void**)&rho, (size_t)kNumKeys * sizeof(int), "rotation tables")) ||
         (rc = dev_alloc(c, (void**)&rp, ((size_t)nc + 1) * sizeof(int), "axial M2L matrices")) ||
         (rc = dev_alloc(c, (void**)&cl, (size_t)nnz * sizeof(unsigned short), "axial M2L matrices")) ||
-        (rc = dev_alloc(c, (void**)&dlx, lx.size() * sizeof(uint2), "rotation task lists")) ||
-        (rc = dev_alloc(c, (void**)&dlz, lz.size() * sizeof(uint2), "rotation task lists")) ||
-        (rc = dev_alloc(c, (void**)&dla, la.size() * sizeof(uint2), "rotation task lists")) ||
-        (rc = dev_alloc(c, (void**)&dlxh, rsh.lx.size() * sizeof(uint2), "rotation task lists")) ||
-        (rc = dev_alloc(c, (void**)&dlzh, rsh.lz.size() * sizeof(uint2), "rotation task lists")) ||
-        (rc = dev_alloc(c, (void**)&dlah, rsh.la.size() * sizeof(uint2), "rotation task lists")) ||
-        (rc = dev_alloc(c, (void**)&dhs, nhstep * sizeof(int4), "harmonic expansion")) ||
-        (rc = dev_alloc(c, (void**)&dhw, nhstep * sizeof(double2), "harmonic expansion"))) {
-        release();
-        return rc;
-    }
-    if ((rc = dev_alloc(c, (void**)&d_r0s, r0s.size() * sizeof(double), "rotation scratch")) ||
-        (rc = dev_alloc(c, (void**)&Ks, kbytes, "rotation scratch"))) {
-        dev_free(c, d_r0s, r0s.size() * sizeof(double));
+        (rc = d_r0s.alloc(r0s.size() * sizeof(double), "rotation scratch")) ||
+        (rc = Ks.alloc(kbytes, "rotation scratch"))) {
         release();
         return rc;
     }
     od.rot_T = T; od.rot_rho = rho; od.ax_rowptr = rp; od.ax_col = cl; od.ax_val = val;
     od.ax_nnz = nnz; od.n_rho = nrho;
-    od.rot_lx = dlx; od.rot_lz = dlz; od.rot_la = dla;
-    od.rot_len[0] = len_x; od.rot_len[1] = len_z; od.rot_len[2] = len_a;
-    od.rot_lxh = dlxh; od.rot_lzh = dlzh; od.rot_lah = dlah;
-    od.rot_lenh[0] = rsh.len[0]; od.rot_lenh[1] = rsh.len[1]; od.rot_lenh[2] = rsh.len[2];
-    od.hxr_step = dhs; od.hxr_w = dhw;
-    for (int k = 0; k < kMaxOrder + 3; ++k) od.hxr_cst[k] = hcst[k];
     cudaError_t e = cudaMemcpyAsync(rho, rho_of.data(), rho_of.size() * sizeof(int), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(dlxh, rsh.lx.data(), rsh.lx.size() * sizeof(uint2), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(dlzh, rsh.lz.data(), rsh.lz.size() * sizeof(uint2), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(dlah, rsh.la.data(), rsh.la.size() * sizeof(uint2), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess && !hstep.empty())
-        e = cudaMemcpyAsync(dhs, hstep.data(), hstep.size() * sizeof(int4), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess && !hw.empty())
-        e = cudaMemcpyAsync(dhw, hw.data(), hw.size() * sizeof(double2), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(rp, rowptr.data(), rowptr.size() * sizeof(int), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(cl, col.data(), col.size() * sizeof(unsigned short), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(d_r0s, r0s.data(), r0s.size() * sizeof(double), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(dlx, lx.data(), lx.size() * sizeof(uint2), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(dlz, lz.data(), lz.size() * sizeof(uint2), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(dla, la.data(), la.size() * sizeof(uint2), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = ops->rot_setup(od, d_r0s, nrho, Ks, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // shared by every later evaluation, on any stream
-    dev_free(c, d_r0s, r0s.size() * sizeof(double));
-    dev_free(c, Ks, kbytes);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(rp, rs.rowptr.data(), rs.rowptr.size() * sizeof(int), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(cl, rs.col.data(), rs.col.size() * sizeof(unsigned short), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(d_r0s.p, r0s.data(), r0s.size() * sizeof(double), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = ops->rot_setup(od, d_r0s.as<double>(), nrho, Ks.as<double>(), s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // the host vectors die with this call
     if (e != cudaSuccess) {
         release();
         od.rot_T = nullptr; od.rot_rho = nullptr; od.ax_rowptr = nullptr; od.ax_col = nullptr; od.ax_val = nullptr;
-        od.rot_lx = od.rot_lz = od.rot_la = nullptr;
-        od.rot_lxh = od.rot_lzh = od.rot_lah = nullptr;
-        od.hxr_step = nullptr;
-        od.hxr_w = nullptr;
         return cuda_fail(c, e, "rotation tables");
     }
     return DAFMM_OK;
 }
 
-// float-float copies of the rotation tables and axial values (the DAFMM_FF mode's M2L)
-int ensure_rotation_ff(dafmm_ctx* c, int p, cudaStream_t s) {
-    int rc;
-    if ((rc = ensure_rotation(c, p, s))) return rc;
+// ... and, per form (all coefficients, or the harmonic one), the kernel's task words and its
+// table values in reading order (rot_lists.h; fmm_order.cuh: RotStream)
+int ensure_rotation(dafmm_ctx* c, int p, bool harm, cudaStream_t s) {
     OrderData& od = c->ord[p];
-    if (od.rot_Tf) return DAFMM_OK;
+    if (od.rot[harm].idx) return DAFMM_OK;
+    static_assert(sizeof(RotTask) == sizeof(uint2), "task layout");
+    static_assert(ncoef_of(kMaxOrder) < 512, "nine bits per index in a task word");
+    const RotStructure rs = rot_structure(p, harm);
+    int rc;
+    if ((rc = ensure_rotation_tables(c, p, rs, s))) return rc;
+    std::vector<RotTask> tasks;
+    for (const std::vector<RotTask>* l : {&rs.lx, &rs.lz, &rs.la}) tasks.insert(tasks.end(), l->begin(), l->end());
+    std::vector<unsigned> idx;
+    for (const RotTask& t : tasks) idx.push_back((t.y & 0xffffu) | (t.y >> 16) << 9 | (t.x & 0x80000000u));
+    RotForm f;
+    f.lx = rs.len[0]; f.lz = rs.len[1]; f.la = rs.len[2];
+    Scratch d_tasks(c);
+    if ((rc = dev_alloc(c, (void**)&f.idx, idx.size() * sizeof(unsigned), "rotation task lists")) ||
+        (rc = dev_alloc(c, (void**)&f.val, (size_t)kNumKeys * 64 * (f.lx + f.lz) * sizeof(double), "rotation tables")) ||
+        (rc = dev_alloc(c, (void**)&f.ax, (size_t)od.n_rho * 32 * f.la * sizeof(double), "axial M2L matrices")) ||
+        (rc = d_tasks.alloc(tasks.size() * sizeof(uint2), "rotation scratch"))) {
+        free_rot_form(c, od, f);
+        return rc;
+    }
+    cudaError_t e = cudaMemcpyAsync(f.idx, idx.data(), idx.size() * sizeof(unsigned), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(d_tasks.p, tasks.data(), tasks.size() * sizeof(uint2), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = order_ops(p)->rot_pack(od, f, d_tasks.as<uint2>(), s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // shared by every later evaluation, on any stream
+    if (e != cudaSuccess) {
+        free_rot_form(c, od, f);
+        return cuda_fail(c, e, "rotation tables");
+    }
+    od.rot[harm] = f;
+    return DAFMM_OK;
+}
+
+// float-float copies of a form's tables (the DAFMM_FF mode's M2L)
+int ensure_rotation_ff(dafmm_ctx* c, int p, bool harm, cudaStream_t s) {
+    int rc;
+    if ((rc = ensure_rotation(c, p, harm, s))) return rc;
+    OrderData& od = c->ord[p];
+    RotForm& f = od.rot[harm];
+    if (f.valf) return DAFMM_OK;
     const OrderOps* ops = order_ops(p);
-    const size_t nt = (size_t)kNumKeys * 4 * ops->rot_tsz, na = (size_t)od.n_rho * od.ax_nnz;
+    const size_t nt = (size_t)kNumKeys * 64 * (f.lx + f.lz), na = (size_t)od.n_rho * 32 * f.la;
     float2 *T = nullptr, *A = nullptr;
     if ((rc = dev_alloc(c, (void**)&T, nt * sizeof(float2), "rotation tables (float-float)"))) return rc;
     if ((rc = dev_alloc(c, (void**)&A, na * sizeof(float2), "axial M2L matrices (float-float)"))) {
         dev_free(c, T, nt * sizeof(float2));
         return rc;
     }
-    cudaError_t e = ops->to_ff(od.rot_T, T, nt, s);
-    if (e == cudaSuccess) e = ops->to_ff(od.ax_val, A, na, s);
+    cudaError_t e = ops->to_ff(f.val, T, nt, s);
+    if (e == cudaSuccess) e = ops->to_ff(f.ax, A, na, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // shared by every later evaluation, on any stream
     if (e != cudaSuccess) {
         dev_free(c, T, nt * sizeof(float2));
         dev_free(c, A, na * sizeof(float2));
         return cuda_fail(c, e, "rotation tables (float-float)");
     }
-    od.rot_Tf = T;
-    od.ax_valf = A;
+    f.valf = T;
+    f.axf = A;
     return DAFMM_OK;
 }
 
@@ -972,27 +971,6 @@ void free_adaptive(dafmm_ctx* c, dafmm_tree* t) {
     t->aMf = nullptr;
     t->a_exp_p = -1;
 }
-
-// device scratch that is returned to the context when it goes out of scope
-struct Scratch {
-    dafmm_ctx* c;
-    void* p = nullptr;
-    size_t bytes = 0;
-    explicit Scratch(dafmm_ctx* ctx) : c(ctx) {}
-    int alloc(size_t b, const char* what) {
-        release();
-        bytes = b;
-        return dev_alloc(c, &p, b, what);
-    }
-    void release() {
-        dev_free(c, p, bytes);
-        p = nullptr;
-        bytes = 0;
-    }
-    template <class T>
-    T* as() const { return static_cast<T*>(p); }
-    ~Scratch() { release(); }
-};
 
 // root cubes of the trees: given, or the smallest cube around each tree's points, enlarged by
 // 1e-12 of its size (the same rule as for a single tree)
@@ -1382,14 +1360,19 @@ int eval_adaptive(dafmm_tree* t, int order, int precision, double* dphi, double*
         } else {
             // FP64: the M2L by rotation (Sec. 3.4), by default from p = 4
             const bool rot = precision == DAFMM_FP64 && (c->m2l_rot > 0 || (c->m2l_rot < 0 && order >= 4));
-            if (rot && (rc = ensure_rotation(c, order, s))) return rc;
+            if (rot && (rc = ensure_rotation(c, order, c->m2l_harm != 0, s))) return rc;
             const int rflags = rot ? kM2LRot | (c->m2l_harm ? kM2LHarm : 0) : 0;
-            for (int l = 2; l <= t->maxlev; ++l) {
-                if (l == t->maxlev) mark(4);
+            auto largest = [&](int l0, int l1) {  // the largest (level, octant) group of levels [l0, l1]
                 int mx = 0;
-                for (int o = 0; o < 8; ++o) mx = std::max(mx, t->grp_ptr_h[l * 8 + o + 1] - t->grp_ptr_h[l * 8 + o]);
-                CK(c, ops->m2l_a(od, av, precision | rflags, t->grp_tg, t->grp_ptr, l * 8, mx, t->aM,
-                                 t->aMf, t->aL, s),
+                for (int g = l0 * 8; g < (l1 + 1) * 8; ++g) mx = std::max(mx, t->grp_ptr_h[g + 1] - t->grp_ptr_h[g]);
+                return mx;
+            };
+            // by rotation: every level in one launch; dense: level by level
+            for (int l = 2; l <= t->maxlev; l = rot ? t->maxlev + 1 : l + 1) {
+                if (rot || l == t->maxlev) mark(4);
+                const int le = rot ? t->maxlev : l;
+                CK(c, ops->m2l_a(od, av, precision | rflags, t->grp_tg, t->grp_ptr, l * 8, (le - l + 1) * 8,
+                                 largest(l, le), t->aM, t->aMf, t->aL, s),
                    "M2L");
                 ++launches;
             }
@@ -2113,8 +2096,8 @@ int dafmm_eval(dafmm_tree* t, int order, double theta, int precision, double* ph
             // and from p = 2 in float-float
             const bool rot = precision == DAFMM_FP64 && (c->m2l_rot > 0 || (c->m2l_rot < 0 && order >= 4));
             const bool rot_ff = fff && order >= 2;
-            if (rot && (rc = ensure_rotation(c, order, s))) return rc;
-            if (rot_ff && (rc = ensure_rotation_ff(c, order, s))) return rc;
+            if (rot && (rc = ensure_rotation(c, order, c->m2l_harm != 0, s))) return rc;
+            if (rot_ff && (rc = ensure_rotation_ff(c, order, c->m2l_harm != 0, s))) return rc;
             for (int l = 2; l <= L; ++l) {
                 if (l == L) mark(4);
                 const double inv_h = 1.0 / ldexp(t->dom[3], -l);

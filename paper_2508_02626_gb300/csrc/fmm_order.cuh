@@ -569,6 +569,60 @@ __global__ void __launch_bounds__(256) k_m2l(const T* __restrict__ K, int l, con
     }
 }
 
+// The steps that restore the coefficients of z exponent >= 2 of a harmonic expansion from its free
+// ones by Laplace's equation (internal.h): V[i] = w1 V[i1] + w2 V[i2], those of z exponent c at
+// [cst[c], cst[c + 1]).
+struct HarmTab {
+    static constexpr int N = NC - nharm_of(P) > 0 ? NC - nharm_of(P) : 1;
+    int cst[P + 3];
+    unsigned short i[N], i1[N], i2[N];
+    float w1[N], w2[N], w1l[N], w2l[N];  // FP32, and its remainder (float-float)
+    double d1[N], d2[N];
+};
+constexpr HarmTab make_harm_tab() {
+    HarmTab t{};
+    int k = 0;
+    for (int c = 2; c <= P; ++c) {
+        t.cst[c] = k;
+        for (int n = c; n <= P; ++n)
+            for (int b = 0; b <= n - c; ++b, ++k) {
+                const int a = n - c - b;
+                t.i[k] = (unsigned short)da_index(a, b, c);
+                t.i1[k] = (unsigned short)da_index(a + 2, b, c - 2);
+                t.i2[k] = (unsigned short)da_index(a, b + 2, c - 2);
+                t.d1[k] = -(double)((a + 2) * (a + 1)) / (double)(c * (c - 1));
+                t.d2[k] = -(double)((b + 2) * (b + 1)) / (double)(c * (c - 1));
+                t.w1[k] = (float)t.d1[k];
+                t.w2[k] = (float)t.d2[k];
+                t.w1l[k] = (float)(t.d1[k] - (double)t.w1[k]);
+                t.w2l[k] = (float)(t.d2[k] - (double)t.w2[k]);
+            }
+    }
+    for (int c = P < 1 ? 2 : P + 1; c < P + 3; ++c) t.cst[c] = k;
+    return t;
+}
+__device__ const HarmTab harm_tab = make_harm_tab();
+
+__device__ __forceinline__ float harm_step(const float* V, int s) {
+    return fmaf(harm_tab.w1[s], V[harm_tab.i1[s]], harm_tab.w2[s] * V[harm_tab.i2[s]]);
+}
+__device__ __forceinline__ double harm_step(const double* V, int s) {
+    return fma(harm_tab.d1[s], V[harm_tab.i1[s]], harm_tab.d2[s] * V[harm_tab.i2[s]]);
+}
+__device__ __forceinline__ ff harm_step(const ff* V, int s) {
+    return ff_add(ff_mul(ff(harm_tab.w1[s], harm_tab.w1l[s]), V[harm_tab.i1[s]]),
+                  ff_mul(ff(harm_tab.w2[s], harm_tab.w2l[s]), V[harm_tab.i2[s]]));
+}
+// the warp restores V's coefficients of z exponent >= 2, exponent by exponent
+template <class R>
+__device__ __forceinline__ void harm_expand_warp(R* V, int lane) {
+#pragma unroll 1
+    for (int c = 2; c <= P; ++c) {
+        for (int s = harm_tab.cst[c] + lane; s < harm_tab.cst[c + 1]; s += 32) V[harm_tab.i[s]] = harm_step(V, s);
+        __syncwarp();
+    }
+}
+
 // ---- M2L by rotation (Sec. 3.4), FP64 -------------------------------------------------------
 // K^_v = B_v A_|v| F_v: F_v rotates the source expansion so that v lies on the positive x axis
 // (M^(u) = M(Q^T u), Q = Rz(phi) Rx(theta) with theta = atan2(vz, vy), phi = atan2(sqrt(vy^2 +
@@ -626,13 +680,6 @@ __global__ void k_axial_gather(const double* __restrict__ K, const int* __restri
             val[(size_t)r * nnz + e] = K[((size_t)r * NC + b) * NCP + col[e]];
 }
 
-// One step of the rotation M2L for the warp: out[k] (=, or += with ACC) sum over the tasks of
-// k of tab[offset] * in[index].  Each lane runs its own list of tasks (a precomputed,
-// load-balanced share of the step's multiply-adds, whole outputs per lane, padded to a common
-// length with tasks that read the zero at in[NC]); task t of lane l is list[32 t + l]:
-// x = table offset | last-of-output << 31, y = input index | output index << 16.  Lanes with
-// outputs of very different lengths would otherwise run every loop to the longest one, and
-// FP64 instructions are this kernel's bound.
 // the arithmetic of the rotation M2L: FP64, or float-float (the DAFMM_FF mode)
 __device__ __forceinline__ double rot_add(double a, double b) { return a + b; }
 __device__ __forceinline__ ff rot_add(ff a, ff b) { return ff_acc(a, b); }
@@ -677,139 +724,229 @@ struct RotAcc<ff> {
     using type = RotAccF;
 };
 
-template <bool ACC, class R>
-__device__ __forceinline__ void rot_step(const uint2* __restrict__ list, int len, const R* __restrict__ tab,
-                                         const R* in, R* out, int lane) {
-    typename RotAcc<R>::type s;
+// The tables of the rotation M2L in the order in which the kernel reads them.  Each of the five
+// steps of a pair runs, per lane, a list of multiply-adds out[k] += tab * in[i] (a precomputed,
+// load-balanced share of the step, whole outputs per lane, padded to a common length with tasks
+// that read the zero at in[NC]; lanes with outputs of very different lengths would otherwise run
+// every loop to the longest one).  Task t of lane l: the word idx[32 t + l] = input index | output
+// index << 9 | last-of-output << 31, the same for every displacement, and its table value at
+// val[32 t + l] -- per key the four substitutions' values one after another (forward x, forward
+// z, back z, back x), the axial values per distinct length.  A warp's reads are then whole
+// 128-byte lines; gathered from the packed matrices, 32 lanes read 32 scattered values and the L1
+// held the kernel below the FP64 rate, and far below the FP32 rate in float-float.
+struct RotStream {
+    const unsigned* idx;  // x-step, z-step, axial: [lx + lz + la][32]
+    int lx, lz, la;
+    const int* krho;      // per key, the index of its length
+};
+
+template <bool ACC, int NV, class R>
+__device__ __forceinline__ void rot_step(const unsigned* __restrict__ idx, int len, const R* __restrict__ val,
+                                         R* const (&in)[NV], R* const (&out)[NV], int lane) {
+    typename RotAcc<R>::type s[NV];
 #pragma unroll 4
     for (int t = 0; t < len; ++t) {
-        const uint2 w = list[32 * t + lane];
-        if (DAFMM_IN(w.y & 0xffffu, NC + 1, kChkRotTask)) s.madd(tab[w.x & 0x7fffffffu], in[w.y & 0xffffu]);
-        if (w.x >> 31) {
-            const int k = (int)(w.y >> 16);
-            if (DAFMM_IN(k, NC, kChkRotTask)) {
-                if (ACC) out[k] = rot_add(out[k], s.get());
-                else out[k] = s.get();
+        const unsigned w = idx[32 * t + lane];
+        const R v = val[32 * t + lane];
+        const int i = (int)(w & 511u), k = (int)((w >> 9) & 511u);
+        if (DAFMM_IN(i, NC + 1, kChkRotTask)) {
+#pragma unroll
+            for (int u = 0; u < NV; ++u) s[u].madd(v, in[u][i]);
+        }
+        if (w >> 31) {
+#pragma unroll
+            for (int u = 0; u < NV; ++u) {
+                if (DAFMM_IN(k, NC, kChkRotTask)) {
+                    if (ACC) out[u][k] = rot_add(out[u][k], s[u].get());
+                    else out[u][k] = s[u].get();
+                }
+                s[u] = typename RotAcc<R>::type();
             }
-            s = typename RotAcc<R>::type();
         }
     }
 }
 
-// task lists of the rotation M2L: x-step (substitution about x), z-step, axial matrix
-struct RotLists {
-    const uint2* x;
-    const uint2* z;
-    const uint2* a;
-    int lx, lz, la;
+// the multipole rows: FP64, or (float-float) their FP32 high and low parts, split once per
+// evaluation
+struct RotRows {
+    const double* M;
+    const float *Mh, *Ml;
 };
-
-// the harmonic form of the rotation (harmonic task lists): the steps that restore a vector's
-// coefficients of z exponent >= 2 from its free ones by Laplace's equation (step s sets
-// V[i] = w1 V[i1] + w2 V[i2]; those of z exponent c at [cst[c], cst[c + 1]))
-struct RotHarm {
-    const int4* step;
-    const double2* w;
-    int cst[kMaxOrder + 3];
-};
-
-__device__ __forceinline__ double rot_axpby(double w1, double a, double w2, double b) { return fma(w1, a, w2 * b); }
-__device__ __forceinline__ ff rot_axpby(double w1, ff a, double w2, ff b) {
-    return ff_add(ff_mul(ff(w1), a), ff_mul(ff(w2), b));
+__device__ __forceinline__ void rot_load(double* X, const RotRows& m, size_t row, int lane) {
+    for (int k = lane; k < NC; k += 32) X[k] = m.M[row + k];
+}
+__device__ __forceinline__ void rot_load(ff* X, const RotRows& m, size_t row, int lane) {
+    for (int k = lane; k < NC; k += 32) X[k] = ff(m.Mh[row + k], m.Ml[row + k]);
 }
 
-// the warp restores V's coefficients of z exponent >= 2, level by level
-template <class R>
-__device__ __forceinline__ void rot_expand(R* V, const RotHarm& hm, int lane) {
-#pragma unroll 1
-    for (int c = 2; c <= P; ++c) {
-        for (int s = hm.cst[c] + lane; s < hm.cst[c + 1]; s += 32) {
-            const int4 st = hm.step[s];
-            const double2 w = hm.w[s];
-            V[st.x] = rot_axpby(w.x, V[st.y], w.y, V[st.z]);
-        }
-        __syncwarp();
+// NV well-separated pairs of one displacement key for the warp: S[u] += B_v A_|v| F_v M_src[u]
+// (X, Y: work vectors with X[NC] = Y[NC] = 0).  HARM: harmonic task lists (free outputs only),
+// the vector restored before the last x-step
+template <bool HARM, int NV, class R>
+__device__ __forceinline__ void rot_pairs(const RotStream& rs, const R* __restrict__ val, const R* __restrict__ ax,
+                                          const RotRows& m, const int (&src)[NV], R* const (&X)[NV],
+                                          R* const (&Y)[NV], R* const (&S)[NV], int lane) {
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < NV; ++u) rot_load(X[u], m, (size_t)src[u] * NCP, lane);
+    __syncwarp();
+    const unsigned *iz = rs.idx + 32 * rs.lx, *ia = iz + 32 * rs.lz;
+    rot_step<false, NV>(rs.idx, rs.lx, val, X, Y, lane);  // forward, about x
+    __syncwarp();
+    rot_step<false, NV>(iz, rs.lz, val + 32 * rs.lx, Y, X, lane);  // forward, about z
+    __syncwarp();
+    rot_step<false, NV>(ia, rs.la, ax, X, Y, lane);  // Eq. 5 on the axis
+    __syncwarp();
+    rot_step<false, NV>(iz, rs.lz, val + 32 * (rs.lx + rs.lz), Y, X, lane);  // back, about z
+    __syncwarp();
+    if constexpr (HARM) {  // the x-step reads every z exponent
+#pragma unroll
+        for (int u = 0; u < NV; ++u) harm_expand_warp(X[u], lane);
     }
+    rot_step<true, NV>(rs.idx, rs.lx, val + 32 * (rs.lx + 2 * rs.lz), X, S, lane);  // back, about x, into the sums
 }
 
-// a source row into the work vector: FP64 rows, or (float-float) the rows' FP32 high and low
-// parts, split once per evaluation
-__device__ __forceinline__ void rot_load(double* X, const double* M, const float*, const float*, size_t row, int lane) {
-    for (int k = lane; k < NC; k += 32) X[k] = M[row + k];
-}
-__device__ __forceinline__ void rot_load(ff* X, const double*, const float* Mh, const float* Ml, size_t row, int lane) {
-    for (int k = lane; k < NC; k += 32) X[k] = ff(Mh[row + k], Ml[row + k]);
-}
-
-// one well-separated pair for the warp: S += B_v A_|v| F_v Ms (T: the key's four substitution
-// tables, av: the axial matrix of its length; X, Y: work vectors with X[NC] = Y[NC] = 0; the
-// source row at `row` of M, or of Mh / Ml in float-float)
-// HARM: harmonic task lists (free outputs only), the vector restored before the last x-step
-template <class R, bool HARM>
-__device__ __forceinline__ void rot_pair(const R* __restrict__ T, const R* __restrict__ av, const RotLists& rl,
-                                         const double* __restrict__ M, const float* __restrict__ Mh,
-                                         const float* __restrict__ Ml, size_t row, R* X, R* Y, R* S, int lane,
-                                         const RotHarm& hm) {
-    __syncwarp();
-    rot_load(X, M, Mh, Ml, row, lane);
-    __syncwarp();
-    rot_step<false>(rl.x, rl.lx, T, X, Y, lane);  // forward, about x
-    __syncwarp();
-    rot_step<false>(rl.z, rl.lz, T + ROT_TSZ, Y, X, lane);  // forward, about z
-    __syncwarp();
-    rot_step<false>(rl.a, rl.la, av, X, Y, lane);  // Eq. 5 on the axis
-    __syncwarp();
-    rot_step<false>(rl.z, rl.lz, T + 2 * ROT_TSZ, Y, X, lane);  // back, about z
-    __syncwarp();
-    if constexpr (HARM) rot_expand<R>(X, hm, lane);  // the x-step reads every z exponent
-    rot_step<true>(rl.x, rl.lx, T + 3 * ROT_TSZ, X, S, lane);  // back, about x, into the sums
-}
-
-// the per-warp work vectors of k_m2l_rot
-template <class R>
-struct RotBuf {
-    R v[3][NCP + 1];
+// Where the targets of one octant lie and their sources.  Uniform trees: octant oct of level l.
+// Adaptive trees: the group of one (level, octant); the source of displacement v is child sc of
+// the parent's colleague at offset a (o - v = 2a + sc).
+struct RotUniform {
+    int l;
+    double inv_h;
+    __device__ __forceinline__ int target(int oct, int i) const {
+        const int P3 = 1 << (3 * (l - 1));
+        return i < P3 ? oct * P3 + i : -1;
+    }
+    __device__ __forceinline__ int source(int t, int oct, const int (&v)[3]) const {
+        const int Pp = 1 << (l - 1), lin = t & ((1 << (3 * (l - 1))) - 1), n = 1 << l;
+        const int x = 2 * (lin & (Pp - 1)) + (oct & 1) - v[0], y = 2 * ((lin >> (l - 1)) & (Pp - 1)) + ((oct >> 1) & 1) - v[1],
+                  z = 2 * (lin >> (2 * (l - 1))) + ((oct >> 2) & 1) - v[2];
+        return x >= 0 && y >= 0 && z >= 0 && x < n && y < n && z < n ? octmajor_index(l, x, y, z) : -1;
+    }
+    __device__ __forceinline__ double scale(int) const { return inv_h; }
+};
+struct RotAdaptive {
+    AdaptiveView av;
+    const int *tg, *grp_ptr;
+    int grp0;
+    __device__ __forceinline__ int target(int g, int i) const {
+        const int g0 = grp_ptr[grp0 + g], g1 = grp_ptr[grp0 + g + 1];
+        if (!DAFMM_RANGE(g0, g1, av.nbox, kChkListPtr) || i >= g1 - g0) return -1;
+        const int t = tg[g0 + i];
+        return DAFMM_IN(t, av.nbox, kChkBoxIndex) && DAFMM_IN(av.parent[t], av.nbox, kChkBoxIndex) ? t : -1;
+    }
+    __device__ __forceinline__ int source(int t, int g, const int (&v)[3]) const {
+        const int dx = (g & 1) - v[0], dy = ((g >> 1) & 1) - v[1], dz = ((g >> 2) & 1) - v[2];
+        const int Q = av.colleague[27 * (size_t)av.parent[t] + ((dx >> 1) + 1) * 9 + ((dy >> 1) + 1) * 3 + (dz >> 1) + 1];
+        if (Q < 0 || !DAFMM_IN(Q, av.nbox, kChkBoxIndex)) return -1;
+        const int sb = av.child[8 * (size_t)Q + ((dx & 1) | ((dy & 1) << 1) | ((dz & 1) << 2))];
+        return sb >= 0 && DAFMM_IN(sb, av.nbox, kChkBoxIndex) ? sb : -1;
+    }
+    __device__ __forceinline__ double scale(int t) const { return 1.0 / av.geom[t].w; }  // (each tree has its own)
 };
 
-// R = double: FP64.  R = ff: float-float, the source rows from their FP32 split parts.  The work
-// vectors are in shared memory; the task lists (the same for every pair) are read through the
-// L1 cache (copies of them in shared memory cost the float-float kernel a quarter of its
-// resident warps and gained nothing: measured 73.7 -> 75.5 ms at level 5, N = 1e6, p = 8).
-template <class R, bool HARM>
-__global__ void __launch_bounds__(256, 2) k_m2l_rot(const R* __restrict__ Ttab, const int* __restrict__ krho,
-                                                    RotLists rl, const R* __restrict__ aval, int annz, int l,
-                                                    const double* __restrict__ M, const float* __restrict__ Mh,
-                                                    const float* __restrict__ Ml, double* __restrict__ L,
-                                                    double inv_h, const __grid_constant__ RotHarm hm) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    __shared__ RotBuf<R> bufs[8];
-    const int Pp = 1 << (l - 1), P3 = Pp * Pp * Pp, n_side = 1 << l;
-    const int t = blockIdx.x * 8 + w;  // target box, octant-major
-    if (t >= 8 * P3) return;
-    const int oct = t / P3, lin = t - oct * P3;
+template <class R>
+constexpr size_t rot_smem(int nt) {
+    return (size_t)8 * nt * 3 * (NCP + 1) * sizeof(R);
+}
+
+// L~ = (1/h) sum_v B_v A_|v| F_v M~ for the targets of one octant (blockIdx.y).  A warp takes NT
+// targets -- two pairs of one displacement share the table reads and give two chains -- and KS of
+// a block's 8 warps share out the displacements of the same targets (every KS-th each, the sums
+// joined in that order), so that a level of few boxes still fills the SMs.  The block's warps walk
+// the displacements together (a barrier every fourth one), so that the tables of a key, read by
+// one of them, serve the others from the L1.
+// Measured against one warp per target reading the packed matrices: uniform N = 200,003, depth 4,
+// p = 8: FP64 9.7 -> 7.1 ms, float-float 9.7 -> 5.9 ms; N = 1e4, depth 3, p = 6, FP64: 1.84 -> 0.81
+// ms; Gaussian N = 100,003, p = 8, FP64 (all levels in one launch): 8.4 -> 2.8 ms.
+template <class R, bool HARM, int NT, class Fam>
+__global__ void __launch_bounds__(256, 2) k_m2l_rot(RotStream rs, const R* __restrict__ val, const R* __restrict__ ax,
+                                                    const __grid_constant__ Fam fam, RotRows m, double* __restrict__ L,
+                                                    int KS) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, sub = w % KS, oct = blockIdx.y;  // (adaptive: 8 (level - 2) + octant)
+    if (fam.target(oct, (int)blockIdx.x * (8 / KS) * NT) < 0) return;  // beyond this group
+    R* base = reinterpret_cast<R*>(smem_raw) + (size_t)w * NT * 3 * (NCP + 1);
+    R *X[NT], *Y[NT], *S[NT];
+    int t[NT];
+#pragma unroll
+    for (int u = 0; u < NT; ++u) {
+        X[u] = base + u * 3 * (NCP + 1);
+        Y[u] = X[u] + NCP + 1;
+        S[u] = Y[u] + NCP + 1;
+        t[u] = fam.target(oct, ((int)blockIdx.x * (8 / KS) + w / KS) * NT + u);
+        for (int k = lane; k <= NCP; k += 32) {
+            X[u][k] = rot_zero<R>();  // X[NC], Y[NC]: the zero that padding tasks read
+            Y[u][k] = rot_zero<R>();
+            S[u][k] = rot_zero<R>();
+        }
+    }
     const int ox = oct & 1, oy = (oct >> 1) & 1, oz = (oct >> 2) & 1;
-    const int tx = 2 * (lin % Pp) + ox, ty = 2 * ((lin / Pp) % Pp) + oy, tz = 2 * (lin / (Pp * Pp)) + oz;
-    R* X = bufs[w].v[0];
-    R* Y = bufs[w].v[1];
-    R* S = bufs[w].v[2];
-    for (int k = lane; k <= NCP; k += 32) {
-        X[k] = rot_zero<R>();  // X[NC], Y[NC]: the zero that padding tasks read
-        Y[k] = rot_zero<R>();
-        S[k] = rot_zero<R>();
-    }
+    const size_t kstride = (size_t)64 * (rs.lx + rs.lz), astride = (size_t)32 * rs.la;
+    int d = 0;
     for (int vx = -3 + ox; vx <= 2 + ox; ++vx)
         for (int vy = -3 + oy; vy <= 2 + oy; ++vy)
             for (int vz = -3 + oz; vz <= 2 + oz; ++vz) {
                 if (abs(vx) <= 1 && abs(vy) <= 1 && abs(vz) <= 1) continue;
-                const int sx = tx - vx, sy = ty - vy, sz = tz - vz;
-                if (sx < 0 || sy < 0 || sz < 0 || sx >= n_side || sy >= n_side || sz >= n_side) continue;
+                const int mine = d++;
+                if ((mine & 3) == 0) __syncthreads();
+                if (mine % KS != sub) continue;
+                const int v[3] = {vx, vy, vz};
                 const int key = (vx + 3) * 49 + (vy + 3) * 7 + (vz + 3);
-                rot_pair<R, HARM>(Ttab + (size_t)key * 4 * ROT_TSZ, aval + (size_t)krho[key] * annz, rl, M, Mh, Ml,
-                                  (size_t)octmajor_index(l, sx, sy, sz) * NCP, X, Y, S, lane, hm);
+                const R *kv = val + key * kstride, *ka = ax + rs.krho[key] * astride;
+                int src[NT], nv = 0;
+#pragma unroll
+                for (int u = 0; u < NT; ++u) {
+                    src[u] = t[u] >= 0 ? fam.source(t[u], oct, v) : -1;
+                    nv += src[u] >= 0;
+                }
+                if (nv == NT) {
+                    rot_pairs<HARM, NT, R>(rs, kv, ka, m, src, X, Y, S, lane);
+                } else if (nv > 0) {
+                    const bool second = src[0] < 0;
+                    const int s1[1] = {second ? src[NT - 1] : src[0]};
+                    R *const x1[1] = {second ? X[NT - 1] : X[0]}, *const y1[1] = {second ? Y[NT - 1] : Y[0]},
+                      *const z1[1] = {second ? S[NT - 1] : S[0]};
+                    rot_pairs<HARM, 1, R>(rs, kv, ka, m, s1, x1, y1, z1, lane);
+                }
             }
-    __syncwarp();
-    if constexpr (HARM) rot_expand<R>(S, hm, lane);  // the sums' coefficients of z exponent >= 2
-    for (int k = lane; k < NC; k += 32) L[(size_t)t * NCP + k] = rot_to_double(S[k]) * inv_h;
+    __syncthreads();
+    if (sub != 0) return;
+#pragma unroll
+    for (int u = 0; u < NT; ++u) {
+        if (t[u] < 0) continue;
+        const size_t step = (size_t)NT * 3 * (NCP + 1);
+        for (int o = 1; o < KS; ++o)
+            for (int k = lane; k < NC; k += 32) S[u][k] = rot_add(S[u][k], S[u][k + o * step]);
+        __syncwarp();
+        if constexpr (HARM) harm_expand_warp(S[u], lane);  // the sums' coefficients of z exponent >= 2
+        const double sc = fam.scale(t[u]);
+        for (int k = lane; k < NC; k += 32) L[(size_t)t[u] * NCP + k] = rot_to_double(S[u][k]) * sc;
+    }
+}
+
+// the kernel's table order from the packed matrices: the substitutions' values of every key
+// (tasks: x-step then z-step lists, x = offset | last << 31) ...
+__global__ void k_rot_pack(const double* __restrict__ T, const uint2* __restrict__ tasks, int lx, int lz,
+                           double* __restrict__ val) {
+    const int key = blockIdx.x, nx = 32 * lx, nz = 32 * lz;
+    const double* Tk = T + (size_t)key * 4 * ROT_TSZ;
+    double* out = val + (size_t)key * 2 * (nx + nz);
+    for (int e = threadIdx.x; e < nx + nz; e += blockDim.x) {
+        const unsigned off = tasks[e].x & 0x7fffffffu;
+        if (e < nx) {
+            out[e] = Tk[off];
+            out[nx + 2 * nz + e] = Tk[3 * ROT_TSZ + off];
+        } else {
+            out[e] = Tk[ROT_TSZ + off];
+            out[nz + e] = Tk[2 * ROT_TSZ + off];
+        }
+    }
+}
+// ... and the axial values of every length
+__global__ void k_axial_pack(const double* __restrict__ aval, int nnz, const uint2* __restrict__ tasks, int n,
+                             double* __restrict__ ax) {
+    for (int e = threadIdx.x; e < n; e += blockDim.x)
+        ax[(size_t)blockIdx.x * n + e] = aval[(size_t)blockIdx.x * nnz + (tasks[e].x & 0x7fffffffu)];
 }
 
 // the float-float split of FP64 rows (n values): hi = fl32(v), lo = fl32(v - hi)
@@ -819,53 +956,6 @@ __global__ void k_split_ff(const double* __restrict__ a, float* __restrict__ hi,
         hi[i] = v.hi;
         lo[i] = v.lo;
     }
-}
-
-// the same for the targets tg[g0 .. g1) of one (level, octant) group of an adaptive tree (V-list
-// sources through the parent's colleagues, as in k_m2l_a); one warp per target
-template <bool HARM>
-__global__ void __launch_bounds__(256, 2) k_m2l_rot_a(const double* __restrict__ Ttab, const int* __restrict__ krho,
-                                                      RotLists rl, const double* __restrict__ aval, int annz,
-                                                      AdaptiveView av, const int* __restrict__ tg,
-                                                      const int* __restrict__ grp_ptr, int grp0,
-                                                      const double* __restrict__ M, double* __restrict__ L,
-                                                      const __grid_constant__ RotHarm hm) {
-    __shared__ double sbuf[8][3][NCP + 1];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int oct = blockIdx.y;
-    const int g0 = grp_ptr[grp0 + oct], g1 = grp_ptr[grp0 + oct + 1];
-    const int ti = g0 + blockIdx.x * 8 + w;
-    if (ti >= g1 || !DAFMM_RANGE(g0, g1, av.nbox, kChkListPtr)) return;
-    if (!DAFMM_IN(tg[ti], av.nbox, kChkBoxIndex) || !DAFMM_IN(av.parent[tg[ti]], av.nbox, kChkBoxIndex)) return;
-    const int t = tg[ti], P = av.parent[t];
-    const int ox = oct & 1, oy = (oct >> 1) & 1, oz = (oct >> 2) & 1;
-    double* X = sbuf[w][0];
-    double* Y = sbuf[w][1];
-    double* S = sbuf[w][2];
-    for (int k = lane; k <= NCP; k += 32) {
-        X[k] = 0.0;
-        Y[k] = 0.0;
-        S[k] = 0.0;
-    }
-    for (int vx = -3 + ox; vx <= 2 + ox; ++vx)
-        for (int vy = -3 + oy; vy <= 2 + oy; ++vy)
-            for (int vz = -3 + oz; vz <= 2 + oz; ++vz) {
-                if (abs(vx) <= 1 && abs(vy) <= 1 && abs(vz) <= 1) continue;
-                const int dx = ox - vx, dy = oy - vy, dz = oz - vz;  // = 2a + sc
-                const int scx = dx & 1, scy = dy & 1, scz = dz & 1;
-                const int ax = (dx - scx) >> 1, ay = (dy - scy) >> 1, az = (dz - scz) >> 1;
-                const int Q = av.colleague[27 * P + (ax + 1) * 9 + (ay + 1) * 3 + (az + 1)];
-                if (Q < 0 || !DAFMM_IN(Q, av.nbox, kChkBoxIndex)) continue;
-                const int sb = av.child[8 * Q + (scx | (scy << 1) | (scz << 2))];
-                if (sb < 0 || !DAFMM_IN(sb, av.nbox, kChkBoxIndex)) continue;
-                const int key = (vx + 3) * 49 + (vy + 3) * 7 + (vz + 3);
-                rot_pair<double, HARM>(Ttab + (size_t)key * 4 * ROT_TSZ, aval + (size_t)krho[key] * annz, rl, M,
-                                       nullptr, nullptr, (size_t)sb * NCP, X, Y, S, lane, hm);
-            }
-    __syncwarp();
-    if constexpr (HARM) rot_expand<double>(S, hm, lane);  // the sums' coefficients of z exponent >= 2
-    const double inv_h = 1.0 / av.geom[t].w;  // the target box's width (each tree has its own)
-    for (int k = lane; k < NC; k += 32) L[(size_t)t * NCP + k] = S[k] * inv_h;
 }
 
 // float-float copies of the rotation tables and axial values (n doubles each)
@@ -1688,45 +1778,6 @@ __global__ void __launch_bounds__(256) k_m2l_a(const T* __restrict__ K, Adaptive
     }
 }
 
-// The steps that restore the coefficients of z exponent >= 2 of a harmonic expansion from its free
-// ones by Laplace's equation (internal.h): V[i] = w1 V[i1] + w2 V[i2], those of z exponent c at
-// [cst[c], cst[c + 1]).
-struct HarmTab {
-    static constexpr int N = NC - nharm_of(P) > 0 ? NC - nharm_of(P) : 1;
-    int cst[P + 3];
-    unsigned short i[N], i1[N], i2[N];
-    float w1[N], w2[N];
-    double d1[N], d2[N];
-};
-constexpr HarmTab make_harm_tab() {
-    HarmTab t{};
-    int k = 0;
-    for (int c = 2; c <= P; ++c) {
-        t.cst[c] = k;
-        for (int n = c; n <= P; ++n)
-            for (int b = 0; b <= n - c; ++b, ++k) {
-                const int a = n - c - b;
-                t.i[k] = (unsigned short)da_index(a, b, c);
-                t.i1[k] = (unsigned short)da_index(a + 2, b, c - 2);
-                t.i2[k] = (unsigned short)da_index(a, b + 2, c - 2);
-                t.d1[k] = -(double)((a + 2) * (a + 1)) / (double)(c * (c - 1));
-                t.d2[k] = -(double)((b + 2) * (b + 1)) / (double)(c * (c - 1));
-                t.w1[k] = (float)t.d1[k];
-                t.w2[k] = (float)t.d2[k];
-            }
-    }
-    for (int c = P < 1 ? 2 : P + 1; c < P + 3; ++c) t.cst[c] = k;
-    return t;
-}
-__device__ const HarmTab harm_tab = make_harm_tab();
-
-__device__ __forceinline__ float harm_step(const float* V, int s) {
-    return fmaf(harm_tab.w1[s], V[harm_tab.i1[s]], harm_tab.w2[s] * V[harm_tab.i2[s]]);
-}
-__device__ __forceinline__ double harm_step(const double* V, int s) {
-    return fma(harm_tab.d1[s], V[harm_tab.i1[s]], harm_tab.d2[s] * V[harm_tab.i2[s]]);
-}
-
 // P2L (Eq. 6): particles of the X-list leaves of each box of [lb, le) into its local expansion,
 // one warp per box, all levels in one launch.
 //   1 / |w + d| = |w|^-1 (1 - 2 s.d + s^2 d^2)^(-1/2) with s = -w / |w|^2, so the P2L of w is the
@@ -1834,10 +1885,7 @@ __global__ void __launch_bounds__(128) k_p2l_a(AdaptiveView av, int lb, int le, 
         if (k < NO) sm[harm_full_index(k)] = acc[j];
     }
     __syncwarp();
-    for (int c = 2; c <= P; ++c) {
-        for (int s = harm_tab.cst[c] + lane; s < harm_tab.cst[c + 1]; s += 32) sm[harm_tab.i[s]] = harm_step(sm, s);
-        __syncwarp();
-    }
+    harm_expand_warp(sm, lane);
     for (int k = lane; k < NC; k += 32) L[(size_t)b * NCP + k] += (double)sm[k] * ih;
 }
 
@@ -2268,51 +2316,55 @@ static cudaError_t leaf_launch(const TreeView& tv, int prec, const double* Lleaf
     return cudaGetLastError();
 }
 
-// M2L by rotation at level l (FP64, uniform trees): L~ = (1/h) sum_v B_v A_|v| F_v M~
-// the task lists and expansion steps of the rotation: harmonic (free outputs only) or full
-static RotLists rot_lists(const OrderData& od, bool harm) {
-    if (harm) return RotLists{od.rot_lxh, od.rot_lzh, od.rot_lah, od.rot_lenh[0], od.rot_lenh[1], od.rot_lenh[2]};
-    return RotLists{od.rot_lx, od.rot_lz, od.rot_la, od.rot_len[0], od.rot_len[1], od.rot_len[2]};
+// M2L by rotation: the tables of a form, harmonic (free outputs only) or full
+static RotStream rot_stream(const OrderData& od, bool harm) {
+    const RotForm& f = od.rot[harm];
+    return RotStream{f.idx, f.lx, f.lz, f.la, od.rot_rho};
 }
-static RotHarm rot_harm(const OrderData& od) {
-    RotHarm hm;
-    hm.step = od.hxr_step;
-    hm.w = od.hxr_w;
-    for (int k = 0; k < kMaxOrder + 3; ++k) hm.cst[k] = od.hxr_cst[k];
-    return hm;
+
+// targets: the most in one group (octant); groups: blockIdx.y
+template <class R, bool HARM, int NT, class Fam>
+static cudaError_t rot_run(const OrderData& od, const R* val, const R* ax, const Fam& fam, const RotRows& m, double* L,
+                           int targets, int groups, int KS, cudaStream_t s) {
+    const size_t smem = rot_smem<R>(NT);
+    const cudaError_t e = set_smem(k_m2l_rot<R, HARM, NT, Fam>, smem);
+    if (e != cudaSuccess) return e;
+    const int per = NT * (8 / KS);
+    k_m2l_rot<R, HARM, NT, Fam><<<dim3((targets + per - 1) / per, groups), 256, smem, s>>>(rot_stream(od, HARM), val, ax,
+                                                                                           fam, m, L, KS);
+    return cudaGetLastError();
+}
+
+// a uniform level: two targets per warp from 4864 boxes on (16 warps per SM), displacements shared
+// out over up to 8 warps while there are fewer than 2432 warps
+template <class R>
+static cudaError_t rot_uniform(const OrderData& od, const R* val, const R* ax, int l, const RotRows& m, double* L,
+                               double inv_h, bool harm, cudaStream_t s) {
+    const int nbox = 1 << (3 * l), per = nbox / 8;
+    const RotUniform fam{l, inv_h};
+    int KS = 1;
+    while (KS < 8 && nbox * KS < 2432) KS *= 2;
+    if (!harm) return rot_run<R, false, 1>(od, val, ax, fam, m, L, per, 8, KS, s);
+    if (nbox >= 4864) return rot_run<R, true, 2>(od, val, ax, fam, m, L, per, 8, 1, s);
+    return rot_run<R, true, 1>(od, val, ax, fam, m, L, per, 8, KS, s);
 }
 
 static cudaError_t m2l_rot_launch(const OrderData& od, int l, const double* M, double* L, double inv_h, bool harm,
                                   cudaStream_t s) {
-    const int nbox = 1 << (3 * l);
-    harm = harm && od.rot_lxh;
-    const RotLists rl = rot_lists(od, harm);
-    const RotHarm hm = rot_harm(od);
-    if (harm)
-        k_m2l_rot<double, true><<<(nbox + 7) / 8, 256, 0, s>>>(od.rot_T, od.rot_rho, rl, od.ax_val, od.ax_nnz, l, M,
-                                                                nullptr, nullptr, L, inv_h, hm);
-    else
-        k_m2l_rot<double, false><<<(nbox + 7) / 8, 256, 0, s>>>(od.rot_T, od.rot_rho, rl, od.ax_val, od.ax_nnz, l, M,
-                                                                 nullptr, nullptr, L, inv_h, hm);
-    return cudaGetLastError();
+    return rot_uniform<double>(od, od.rot[harm].val, od.rot[harm].ax, l, RotRows{M, nullptr, nullptr}, L, inv_h, harm, s);
 }
 
-// the same in float-float (DAFMM_FF): tables od.rot_Tf, od.ax_valf; the source rows' FP32 parts
-// Mh, Ml (k_split_ff); the task lists staged in shared memory
+// the same in float-float (DAFMM_FF): the source rows' FP32 parts Mh, Ml (k_split_ff)
 static cudaError_t m2l_rot_ff_launch(const OrderData& od, int l, const float* Mh, const float* Ml, double* L,
                                      double inv_h, bool harm, cudaStream_t s) {
-    const int nbox = 1 << (3 * l);
-    harm = harm && od.rot_lxh;
-    const RotLists rl = rot_lists(od, harm);
-    const RotHarm hm = rot_harm(od);
-    const ff* T = reinterpret_cast<const ff*>(od.rot_Tf);
-    const ff* av = reinterpret_cast<const ff*>(od.ax_valf);
-    if (harm)
-        k_m2l_rot<ff, true><<<(nbox + 7) / 8, 256, 0, s>>>(T, od.rot_rho, rl, av, od.ax_nnz, l, nullptr, Mh, Ml, L,
-                                                            inv_h, hm);
-    else
-        k_m2l_rot<ff, false><<<(nbox + 7) / 8, 256, 0, s>>>(T, od.rot_rho, rl, av, od.ax_nnz, l, nullptr, Mh, Ml, L,
-                                                             inv_h, hm);
+    return rot_uniform<ff>(od, reinterpret_cast<const ff*>(od.rot[harm].valf), reinterpret_cast<const ff*>(od.rot[harm].axf),
+                           l, RotRows{nullptr, Mh, Ml}, L, inv_h, harm, s);
+}
+
+// the kernel's tables of a form; tasks: its x-step, z-step and axial lists end to end
+static cudaError_t rot_pack_launch(const OrderData& od, const RotForm& f, const uint2* tasks, cudaStream_t s) {
+    k_rot_pack<<<kNumKeys, 128, 0, s>>>(od.rot_T, tasks, f.lx, f.lz, f.val);
+    k_axial_pack<<<od.n_rho, 128, 0, s>>>(od.ax_val, od.ax_nnz, tasks + 32 * (f.lx + f.lz), 32 * f.la, f.ax);
     return cudaGetLastError();
 }
 
@@ -2380,21 +2432,17 @@ static cudaError_t m2m_a_launch(const OrderData& od, const AdaptiveView& av, int
 }
 
 static cudaError_t m2l_a_launch(const OrderData& od, const AdaptiveView& av, int prec, const int* tg,
-                                const int* grp_ptr, int grp0, int max_group, const double* M, const float* Mf,
-                                double* L, cudaStream_t s) {
+                                const int* grp_ptr, int grp0, int ngrp, int max_group, const double* M,
+                                const float* Mf, double* L, cudaStream_t s) {
     if (max_group == 0) return cudaSuccess;
-    if (prec & kM2LRot) {  // FP64 by rotation (Sec. 3.4)
-        const bool harm = (prec & kM2LHarm) && od.rot_lxh;
-        const RotLists rl = rot_lists(od, harm);
-        const RotHarm hm = rot_harm(od);
-        const dim3 grd((max_group + 7) / 8, 8);
-        if (harm)
-            k_m2l_rot_a<true><<<grd, 256, 0, s>>>(od.rot_T, od.rot_rho, rl, od.ax_val, od.ax_nnz, av, tg, grp_ptr, grp0,
-                                                  M, L, hm);
-        else
-            k_m2l_rot_a<false><<<grd, 256, 0, s>>>(od.rot_T, od.rot_rho, rl, od.ax_val, od.ax_nnz, av, tg, grp_ptr,
-                                                   grp0, M, L, hm);
-        return cudaGetLastError();
+    if (prec & kM2LRot) {  // FP64 by rotation (Sec. 3.4), ngrp groups from grp0 in one launch
+        // (two warps per pair of targets whatever their number: a member of a forest sums as alone)
+        const bool harm = (prec & kM2LHarm) != 0;
+        const RotAdaptive fam{av, tg, grp_ptr, grp0};
+        const RotRows m{M, nullptr, nullptr};
+        const RotForm& f = od.rot[harm];
+        if (harm) return rot_run<double, true, 2>(od, f.val, f.ax, fam, m, L, max_group, ngrp, 2, s);
+        return rot_run<double, false, 1>(od, f.val, f.ax, fam, m, L, max_group, ngrp, 2, s);
     }
     dim3 grd((max_group + 31) / 32, 8);
     cudaError_t e;
@@ -2503,7 +2551,7 @@ const OrderOps* DAFMM_CAT(order_ops_p, DAFMM_P)() {
         HostShiftTable{gen::GENT(m2mh, _nnz), gen::GENT(m2mh, _rowptr), gen::GENT(m2mh, _col), gen::GENT(m2mh, _par),
                        gen::GENT(m2mh, _val)},
         p2m_launch, m2m_launch, l2l_launch, m2l_launch, leaf_launch, kgen_launch, m2l_rot_launch, rot_setup_launch,
-        ROT_TSZ,
+        rot_pack_launch, ROT_TSZ,
         op_p2m, op_p2l, op_l2p, op_m2p, op_shift,
         p2m_a_launch, m2m_a_launch, m2l_a_launch, p2l_a_launch, l2l_a_launch, leaf_a_launch,
         m2l_rot_ff_launch, to_ff_launch, split_ff_launch};

@@ -78,6 +78,16 @@ struct MulTab {                   // DA product table for the K generation
 struct AdaptiveView;
 
 // ---- per-order operator tables and launchers ------------------------------------------
+// one form of the M2L by rotation: task words and table values in the kernel's reading order
+// (fmm_order.cuh: RotStream), made on first use
+struct RotForm {
+    unsigned* idx = nullptr;     // [lx + lz + la][32]
+    int lx = 0, lz = 0, la = 0;
+    double* val = nullptr;       // [343][2 (lx + lz)][32]
+    double* ax = nullptr;        // [n_rho][la][32]
+    float2 *valf = nullptr, *axf = nullptr;  // float-float copies (the DAFMM_FF mode)
+};
+
 struct OrderData {
     int p = -1, nc = 0, ncp = 0;
     int* m2m_rowptr = nullptr; unsigned short* m2m_col = nullptr; unsigned char* m2m_par = nullptr;
@@ -124,23 +134,7 @@ struct OrderData {
     unsigned short* ax_col = nullptr;
     double* ax_val = nullptr;
     int ax_nnz = 0, n_rho = 0;
-    // the kernel's load-balanced task lists (x-step, z-step, axial), [length][32] each
-    uint2* rot_lx = nullptr;
-    uint2* rot_lz = nullptr;
-    uint2* rot_la = nullptr;
-    int rot_len[3] = {0, 0, 0};
-    // the same lists in the harmonic form (outputs of z exponent <= 1 only) and the steps that
-    // restore the other coefficients (FP64 weights; harm_steps in api.cu)
-    uint2* rot_lxh = nullptr;
-    uint2* rot_lzh = nullptr;
-    uint2* rot_lah = nullptr;
-    int rot_lenh[3] = {0, 0, 0};
-    int4* hxr_step = nullptr;
-    double2* hxr_w = nullptr;
-    int hxr_cst[kMaxOrder + 3] = {};
-    // float-float copies of rot_T and ax_val (the DAFMM_FF mode's M2L), made on first use
-    float2* rot_Tf = nullptr;
-    float2* ax_valf = nullptr;
+    RotForm rot[2];  // the kernel's tables: all coefficients, or the harmonic form (free outputs only)
     ShiftTab m2m() const { return ShiftTab{m2m_rowptr, m2m_col, m2m_par, m2m_val, m2m_valf, m2m_rp8}; }
     ShiftTab l2l() const { return ShiftTab{l2l_rowptr, l2l_col, l2l_par, l2l_val, l2l_valf, l2l_rp8}; }
     ShiftTab m2mh() const { return ShiftTab{m2mh_rowptr, m2mh_col, m2mh_par, m2mh_val, m2mh_valf, nullptr, m2mh_ord, m2mh_nnz}; }
@@ -211,6 +205,7 @@ struct OrderOps {
     cudaError_t (*m2l_rot)(const OrderData&, int level, const double* M, double* L, double inv_h, bool harm,
                            cudaStream_t);
     cudaError_t (*rot_setup)(OrderData&, const double* r0s, int nrho, double* Kscratch, cudaStream_t);
+    cudaError_t (*rot_pack)(const OrderData&, const RotForm&, const uint2* tasks, cudaStream_t);
     int rot_tsz;  // doubles per substitution table (sum over m <= p of (m+1)^2)
     cudaError_t (*op_p2m)(int prec, int64_t n, const double* s, const double* q, double* out, cudaStream_t);
     cudaError_t (*op_p2l)(int prec, int64_t n, const double* w, const double* q, double* out, cudaStream_t);
@@ -224,7 +219,7 @@ struct OrderOps {
     cudaError_t (*m2m_a)(const OrderData&, const AdaptiveView&, int prec, const int* parents, int np, double* M,
                          cudaStream_t);
     cudaError_t (*m2l_a)(const OrderData&, const AdaptiveView&, int prec, const int* tg, const int* grp_ptr, int grp0,
-                         int max_group, const double* M, const float* Mf, double* L, cudaStream_t);
+                         int ngrp, int max_group, const double* M, const float* Mf, double* L, cudaStream_t);
     cudaError_t (*p2l_a)(const AdaptiveView&, int prec, int lb, int le, double* L, cudaStream_t);
     // L2L from the parents of one level into their children
     cudaError_t (*l2l_a)(const OrderData&, const AdaptiveView&, int prec, const int* parents, int np, double* L,
@@ -232,9 +227,8 @@ struct OrderOps {
     cudaError_t (*leaf_a)(const AdaptiveView&, const int* leaves, int nleaves, int prec, const double* L,
                           const double* M, const float* Mf, double* phi, double* field, int warps, int max_leaf,
                           cudaStream_t);  // max_leaf: particles of the largest leaf
-    // the M2L by rotation of a uniform tree's level in float-float (DAFMM_FF; tables rot_Tf,
-    // ax_valf; source rows as FP32 high and low parts), and the conversion of n doubles into
-    // float-float pairs
+    // the M2L by rotation of a uniform tree's level in float-float (DAFMM_FF; source rows as FP32
+    // high and low parts), and the conversion of n doubles into float-float pairs
     cudaError_t (*m2l_rot_ff)(const OrderData&, int level, const float* Mh, const float* Ml, double* L, double inv_h,
                               bool harm, cudaStream_t);
     cudaError_t (*to_ff)(const double* a, float2* b, size_t n, cudaStream_t);
