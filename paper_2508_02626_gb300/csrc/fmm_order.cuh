@@ -1039,11 +1039,11 @@ __device__ __forceinline__ void stage_pair(float4* buf, int j, const float4* __r
 // the pairs of up to 32 source leaves (lane e: np pairs from pair0, their scale and shift), end to
 // end, segment by segment: the warp stages each segment -- every lane finds the leaf of its pair
 // in the prefix sums, so that leaves of any size fill the lanes -- and body(first pair, pairs)
-// works on it
-template <bool UNIT, class Body>
+// works on it; of NW warps that share a leaf, warp w takes every NW-th segment from the w-th
+template <bool UNIT, int NW, class Body>
 __device__ __forceinline__ void near_segments(float4* buf, const float4* __restrict__ xq,
                                               const float4* __restrict__ xl, int np, int pair0, float r, float ox,
-                                              float oy, float oz, int lane, Body&& body) {
+                                              float oy, float oz, int lane, int warp, Body&& body) {
     int incl = np;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
@@ -1051,7 +1051,7 @@ __device__ __forceinline__ void near_segments(float4* buf, const float4* __restr
         if (lane >= d) incl += v;
     }
     const int total = __shfl_sync(0xffffffffu, incl, 31), at0 = pair0 - (incl - np);
-    for (int seg0 = 0; seg0 < total; seg0 += kSegPairs) {
+    for (int seg0 = warp * kSegPairs; seg0 < total; seg0 += NW * kSegPairs) {
         const int segn = min(kSegPairs, total - seg0);
         __syncwarp();  // the previous segment is no longer read
 #pragma unroll
@@ -1245,20 +1245,25 @@ __device__ __forceinline__ void near_zero(float4* buf, int lane) {
     for (int j = 0; j < 16; ++j) acc[j * 32] = 0.f;
 }
 
-// the groups' sums of target tl < 2 W of the pass, in the order of the groups
+// the sums of target tl < 2 W of the pass over the groups of NW warps (their segments follow one
+// another from buf on), in that order
+template <int NW>
 __device__ __forceinline__ CompSums near_join(float4* buf, int W, int tl) {
-    __syncwarp();
-    const float* acc = near_acc(buf) + (tl >= W ? 8 * 32 : 0) + (tl & (W - 1));
-    float k[8];
+    if constexpr (NW > 1) __syncthreads();
+    else __syncwarp();
+    float k[8] = {};
+#pragma unroll 1
+    for (int w = 0; w < NW; ++w) {
+        const float* acc = near_acc(buf + w * kNearSmem) + (tl >= W ? 8 * 32 : 0) + (tl & (W - 1));
+        for (int d = 0; d < 32; d += W) {
 #pragma unroll
-    for (int j = 0; j < 8; ++j) k[j] = acc[j * 32];
-    for (int d = W; d < 32; d += W) {
-#pragma unroll
-        for (int j = 0; j < 8; j += 2) {
-            two_sum_add(k[j], k[j + 1], acc[j * 32 + d]);
-            k[j + 1] += acc[(j + 1) * 32 + d];
+            for (int j = 0; j < 8; j += 2) {
+                two_sum_add(k[j], k[j + 1], acc[j * 32 + d]);
+                k[j + 1] += acc[(j + 1) * 32 + d];
+            }
         }
     }
+    if constexpr (NW > 1) __syncthreads();  // before the next pass starts from zero
     CompSums r;
     r.ph = k[0]; r.pl = k[1]; r.xh = k[2]; r.xl = k[3]; r.yh = k[4]; r.yl = k[5]; r.zh = k[6]; r.zl = k[7];
     return r;
@@ -1322,13 +1327,13 @@ __device__ __forceinline__ ff ff_shfl_down(ff v, int d) {
     return ff(__shfl_down_sync(0xffffffffu, v.hi, d), __shfl_down_sync(0xffffffffu, v.lo, d));
 }
 
-// Leaves (one warp each) per thread block of the uniform leaf kernel: one, since a block of four
-// holds its registers until its longest leaf is done; and the warps per SM its FP32 form is
-// compiled for.  N = 1e6, p = 8: 0.63 ms with four leaves per block at 20 warps per SM, 0.61 with
-// one, 0.60 with the sums in shared memory at 28 warps.  (More warps or independent pairs in
-// flight do not help further, nor do scalar field sums, although a packed FMA of three distinct
-// registers takes 3.9 cycles in a loop of its own and two scalar ones 2.3: 0.61-0.62 ms.)
-constexpr int kLeafWarps = 1;
+// The uniform FP32 leaf kernel: a block per leaf -- a block of four leaves holds its registers until
+// its longest leaf is done -- compiled for 28 warps per SM.  N = 1e6, p = 8: 0.63 ms with four
+// leaves per block at 20 warps per SM, 0.61 with one, 0.60 with the sums in shared memory at 28
+// warps.  (More warps or independent pairs in flight do not help further, nor do scalar field
+// sums, although a packed FMA of three distinct registers takes 3.9 cycles in a loop of its own
+// and two scalar ones 2.3: 0.61-0.62 ms.)  A tree of few leaves gives each NW warps, which share
+// out the segments of its source list (leaf_launch): 64 leaves, N = 3001, p = 4: 91 -> 24 us.
 constexpr int kLeafMinWarps = 28;
 
 // ---- FP64 near field ----
@@ -1433,13 +1438,19 @@ __device__ __forceinline__ Sum64 pass_join(Sum64 s, int W, int warp, int lane, S
 // the guarded head of the list
 __device__ __forceinline__ int own_first_slot(int k) { return k == 0 ? 13 : (k <= 13 ? k - 1 : k); }
 
-template <class T>
-__global__ void __launch_bounds__(32 * kLeafWarps, (std::is_same<T, float>::value ? kLeafMinWarps : 16) / kLeafWarps)
-k_leaf(TreeView tv, const double* __restrict__ Lleaf,
-                                              double* __restrict__ phi, double* __restrict__ field) {
-    const int lane = threadIdx.x;
-    const int leaf = blockIdx.x * blockDim.y + threadIdx.y;
-    if (leaf >= tv.nleaf) return;
+template <class T, int NW>
+constexpr size_t leaf_smem() {  // the warps' segments and sums, and the leaf's local expansion
+    return (size_t)NW * kNearSmem * sizeof(float4) + NCP * sizeof(T);
+}
+
+template <class T, int NW>
+__global__ void __launch_bounds__(32 * NW, (std::is_same<T, float>::value ? kLeafMinWarps : 16) / NW)
+    k_leaf(TreeView tv, const double* __restrict__ Lleaf, double* __restrict__ phi, double* __restrict__ field) {
+    static_assert(NW == 1 || std::is_same<T, float>::value, "float-float: one warp per leaf");
+    extern __shared__ __align__(16) float4 s_near[];
+    T* lrow = reinterpret_cast<T*>(s_near + NW * kNearSmem);
+    const int lane = threadIdx.x, warp = NW > 1 ? threadIdx.y : 0, leaf = blockIdx.x;
+    float4* buf = s_near + warp * kNearSmem;
     int i0 = tv.leaf_start[leaf], i1 = tv.leaf_start[leaf + 1];
     if (!DAFMM_RANGE(i0, i1, tv.n, kChkLeafRange)) i0 = i1 = 0;
     int a, b, c;
@@ -1449,26 +1460,13 @@ k_leaf(TreeView tv, const double* __restrict__ Lleaf,
     const double cy = tv.y0 + ((double)b + 0.5) * tv.h_leaf;
     const double cz = tv.z0 + ((double)c + 0.5) * tv.h_leaf;
     const double* Lrow = Lleaf ? Lleaf + (size_t)leaf * NCP : nullptr;
-    __shared__ float s_lrow[kLeafWarps][NCP];  // per warp: the leaf's local expansion in FP32
-    __shared__ ff s_lrow_ff[std::is_same<T, ff>::value ? kLeafWarps : 1][std::is_same<T, ff>::value ? NCP : 1];
-    if constexpr (std::is_same<T, ff>::value) {  // ... or in float-float
-        if (Lrow) {
-            __syncwarp();
-            for (int k = lane; k < NC; k += 32) s_lrow_ff[threadIdx.y][k] = ff(Lrow[k]);
-            __syncwarp();
+    if (Lrow && warp == 0) {  // the leaf's local expansion, in T (FP32 rows: NCP floats per leaf)
+        const float* Lf = reinterpret_cast<const float*>(Lleaf) + (size_t)leaf * NCP;
+        for (int k = lane; k < NC; k += 32) {
+            if constexpr (std::is_same<T, float>::value) lrow[k] = tv.locals_f32 ? Lf[k] : (float)Lrow[k];
+            else lrow[k] = ff(Lrow[k]);
         }
-    }
-    if constexpr (sizeof(T) == 4) {
-        if (Lrow) {
-            if (tv.locals_f32) {  // the row is FP32 already (NCP floats per leaf)
-                const float* Lf = reinterpret_cast<const float*>(Lleaf) + (size_t)leaf * NCP;
-                __syncwarp();
-                for (int k = lane; k < NC; k += 32) s_lrow[threadIdx.y][k] = Lf[k];
-                __syncwarp();
-            } else {
-                warp_row_to_f32(Lrow, s_lrow[threadIdx.y], lane);
-            }
-        }
+        __syncwarp();
     }
     // FP32: the 27 neighbour leaves, one per lane (none outside the domain): their pairs of
     // records -- an odd leaf's last pair ends in its null record -- and their offsets in leaf
@@ -1511,8 +1509,6 @@ k_leaf(TreeView tv, const double* __restrict__ Lleaf,
             // The neighbours' records are copied into one shared-memory list, shifted into this
             // leaf's frame (source + neighbour offset, in leaf widths, exactly: the rounding of
             // the shift joins the remainder); the pairwise sum runs over each segment of it.
-            __shared__ __align__(16) float4 s_list[kLeafWarps][kNearSmem];
-            float4* buf = s_list[threadIdx.y];
             CompSums sum;
             FFSums fs;
             if constexpr (std::is_same<T, float>::value) {
@@ -1520,12 +1516,13 @@ k_leaf(TreeView tv, const double* __restrict__ Lleaf,
                 const int l0 = lane & (W - 1);
                 const NearTarget nt[2] = {near_target(tv.xq, xl, (l0 < m ? base + l0 : i0) + r_own),
                                           near_target(tv.xq, xl, (l0 + W < m ? base + l0 + W : i0) + r_own)};
-                near_segments<true>(buf, tv.xq, xl, nb_np, nb_pair, 1.f, nb_x, nb_y, nb_z, lane,
-                                    [&](int seg0, int n) { near_segment(buf, n, own_pairs - seg0, W, lane, nt); });
-                sum = near_join(buf, W, tl);
+                near_segments<true, NW>(buf, tv.xq, xl, nb_np, nb_pair, 1.f, nb_x, nb_y, nb_z, lane, warp,
+                                        [&](int seg0, int n) { near_segment(buf, n, own_pairs - seg0, W, lane, nt); });
+                sum = near_join<NW>(s_near, W, tl);
+                if (warp != 0) continue;
             } else {
                 const float4 pt = xq_load(tv.xq, tt + r_own), pl = xq_load(xl, tt + r_own);
-                near_segments<true>(buf, tv.xq, xl, nb_np, nb_pair, 1.f, nb_x, nb_y, nb_z, lane, [&](int seg0, int n) {
+                near_segments<true, 1>(buf, tv.xq, xl, nb_np, nb_pair, 1.f, nb_x, nb_y, nb_z, lane, 0, [&](int seg0, int n) {
                     const int h = split ? (n + 1) >> 1 : n, g = split ? lane >> 4 : 0;
                     p2p_segment_ff(buf, g ? h : 0, g ? n : h, own_pairs - seg0, pt.x, pt.y, pt.z, pl.x, pl.y, pl.z, fs);
                 });
@@ -1562,8 +1559,8 @@ k_leaf(TreeView tv, const double* __restrict__ Lleaf,
                 const float4 pt = xq_load(tv.xq, tt + r_own);
                 xs = (T)pt.x; ys = (T)pt.y; zs = (T)pt.z;
             }
-            if constexpr (sizeof(T) == 4) gen::GEN(l2p)<T>(SmemRowF{s_lrow[threadIdx.y]}, xs, ys, zs, F, g0, g1, g2);
-            else gen::GEN(l2p)<T>(SmemRowFF{s_lrow_ff[threadIdx.y]}, xs, ys, zs, F, g0, g1, g2);
+            if constexpr (sizeof(T) == 4) gen::GEN(l2p)<T>(SmemRowF{lrow}, xs, ys, zs, F, g0, g1, g2);
+            else gen::GEN(l2p)<T>(SmemRowFF{lrow}, xs, ys, zs, F, g0, g1, g2);
             fphi += (double)F;
             fx -= (double)g0 * tv.inv_h_leaf;
             fy -= (double)g1 * tv.inv_h_leaf;
@@ -1966,10 +1963,10 @@ __global__ void __launch_bounds__(256, 3) k_leaf_a(AdaptiveView av, const int* _
                     oz = (float)(((2 * ijk_s[2] + 1) << up) - ((2 * ijk_b[2] + 1) << dn)) * sc;
                 }
                 const int own = ug == u0 ? (i1 - i0 + 1) >> 1 : 0;
-                near_segments<false>(buf, av.xq, av.xl, np, pair, r, ox, oy, oz, lane,
-                                     [&](int seg0, int n) { near_segment(buf, n, own - seg0, W, lane, nt); });
+                near_segments<false, 1>(buf, av.xq, av.xl, np, pair, r, ox, oy, oz, lane, 0,
+                                        [&](int seg0, int n) { near_segment(buf, n, own - seg0, W, lane, nt); });
             }
-            const CompSums sum = near_join(buf, W, tl);
+            const CompSums sum = near_join<1>(buf, W, tl);
             fphi = ((double)sum.ph + (double)sum.pl) * ih;
             fx = ((double)sum.xh + (double)sum.xl) * ih * ih;
             fy = ((double)sum.yh + (double)sum.yl) * ih * ih;
@@ -2299,19 +2296,27 @@ static cudaError_t m2l_launch(const OrderData& od, int prec, int l, const double
     return cudaGetLastError();
 }
 
+template <class T, int NW>
+static cudaError_t leaf_run(const TreeView& tv, const double* Lleaf, double* phi, double* field, cudaStream_t s) {
+    const cudaError_t e = set_smem(k_leaf<T, NW>, leaf_smem<T, NW>());
+    if (e != cudaSuccess) return e;
+    k_leaf<T, NW><<<tv.nleaf, dim3(32, NW), leaf_smem<T, NW>(), s>>>(tv, Lleaf, phi, field);
+    return cudaGetLastError();
+}
+
 static cudaError_t leaf_launch(const TreeView& tv, int prec, const double* Lleaf, double* phi, double* field,
                                cudaStream_t s) {
     if (tv.nleaf == 0) return cudaSuccess;
-    dim3 blk(32, kLeafWarps), grd((tv.nleaf + kLeafWarps - 1) / kLeafWarps);
     if (prec == DAFMM_FP64) {
         // about 16 warps per SM or more from 2432 leaves on; below, more warps per leaf
         if (tv.nleaf >= 2432) k_leaf64<1><<<tv.nleaf, dim3(32, 1), 0, s>>>(tv, Lleaf, phi, field);
         else if (tv.nleaf >= 1216) k_leaf64<2><<<tv.nleaf, dim3(32, 2), 0, s>>>(tv, Lleaf, phi, field);
         else k_leaf64<8><<<tv.nleaf, dim3(32, 8), 0, s>>>(tv, Lleaf, phi, field);
     } else if (prec == DAFMM_FF) {
-        k_leaf<ff><<<grd, blk, 0, s>>>(tv, Lleaf, phi, field);
-    } else {
-        k_leaf<float><<<grd, blk, 0, s>>>(tv, Lleaf, phi, field);
+        return leaf_run<ff, 1>(tv, Lleaf, phi, field, s);
+    } else {  // one wave of warps needs 4256 leaves
+        if (tv.nleaf >= 2432) return leaf_run<float, 1>(tv, Lleaf, phi, field, s);
+        return tv.nleaf >= 608 ? leaf_run<float, 4>(tv, Lleaf, phi, field, s) : leaf_run<float, 8>(tv, Lleaf, phi, field, s);
     }
     return cudaGetLastError();
 }
@@ -2335,17 +2340,18 @@ static cudaError_t rot_run(const OrderData& od, const R* val, const R* ax, const
     return cudaGetLastError();
 }
 
-// a uniform level: two targets per warp from 4864 boxes on (16 warps per SM), displacements shared
-// out over up to 8 warps while there are fewer than 2432 warps
+// a uniform level: two targets per warp from 512 boxes on, the displacements shared out over up to
+// 8 warps while there are fewer than 2432 warps (16 per SM).  N = 200,003, depth 4, p = 8, against
+// one target per warp: FP64 7.1 -> 6.8 ms, float-float 5.9 -> 4.6 ms; N = 1e4, p = 6: 0.81 -> 0.78 ms.
 template <class R>
 static cudaError_t rot_uniform(const OrderData& od, const R* val, const R* ax, int l, const RotRows& m, double* L,
                                double inv_h, bool harm, cudaStream_t s) {
-    const int nbox = 1 << (3 * l), per = nbox / 8;
+    const int nbox = 1 << (3 * l), per = nbox / 8, nt = harm && nbox >= 512 ? 2 : 1;
     const RotUniform fam{l, inv_h};
     int KS = 1;
-    while (KS < 8 && nbox * KS < 2432) KS *= 2;
+    while (KS < 8 && nbox / nt * KS < 2432) KS *= 2;
     if (!harm) return rot_run<R, false, 1>(od, val, ax, fam, m, L, per, 8, KS, s);
-    if (nbox >= 4864) return rot_run<R, true, 2>(od, val, ax, fam, m, L, per, 8, 1, s);
+    if (nt == 2) return rot_run<R, true, 2>(od, val, ax, fam, m, L, per, 8, KS, s);
     return rot_run<R, true, 1>(od, val, ax, fam, m, L, per, 8, KS, s);
 }
 
