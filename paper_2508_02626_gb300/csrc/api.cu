@@ -774,7 +774,7 @@ void free_expansions(dafmm_tree* t) {
         dev_free(c, e.Mh16[l], c16);
         dev_free(c, e.Ml16[l], c16);
         dev_free(c, e.Minv[l], level_boxes(l) * sizeof(float));
-        dev_free(c, e.Lh[l], e.Lh[l] ? level_boxes(l) * harm_row(e.p) * sizeof(float) : 0);
+        dev_free(c, e.Lh[l], e.Lh[l] ? level_boxes(l) * harm_row(e.p) * sizeof(float) * e.lh_split : 0);
     }
     e = Expansions();
 }
@@ -827,10 +827,12 @@ int ensure_f16_levels(dafmm_tree* t, cudaStream_t s) {
 int ensure_lh_levels(dafmm_tree* t) {
     dafmm_ctx* c = t->ctx;
     Expansions& e = t->ex;
+    e.lh_split = tc_m2l_split(e.depth, c->num_sms);
     for (int l = 2; l <= e.depth; ++l) {
         int rc;
         if (!e.Lh[l] &&
-            (rc = dev_alloc(c, (void**)&e.Lh[l], level_boxes(l) * harm_row(e.p) * sizeof(float), "locals (harmonic)")))
+            (rc = dev_alloc(c, (void**)&e.Lh[l], level_boxes(l) * harm_row(e.p) * sizeof(float) * e.lh_split,
+                            "locals (harmonic)")))
             return rc;
     }
     return DAFMM_OK;
@@ -1353,7 +1355,7 @@ int eval_adaptive(dafmm_tree* t, int order, int precision, double* dphi, double*
                 void* full = t->aL + (size_t)b0 * od.ncp;
                 const int nrows = t->nbox - b0;
                 CK(c, tc_harm_expand(order, 1, &red, &full, nullptr, nullptr, &nrows, false, od.hx_step, od.hx_w,
-                                     od.hx_cst, s),
+                                     od.hx_cst, 1, s),
                    "M2L (harmonic expansion)");
                 ++launches;
             }
@@ -2071,6 +2073,7 @@ int dafmm_eval(dafmm_tree* t, int order, double theta, int precision, double* ph
             a.inv_r = harm ? od.k16h_inv_r : od.k16_inv_r;
             a.inv_c = harm ? od.k16h_inv_c : od.k16_inv_c;
             a.nkey = kNumKeys;
+            a.nsplit = harm ? ex.lh_split : 1;
             CK(c, tc_launch(order, a, s), "M2L (tensor cores)");
             ++launches;
             if (harm) {
@@ -2087,7 +2090,8 @@ int dafmm_eval(dafmm_tree* t, int order, double theta, int precision, double* ph
                     ls[l - 2] = tc_l2l && l == 2 ? ex.Llo[l] : nullptr;
                     nrows[l - 2] = (int)level_boxes(l);
                 }
-                CK(c, tc_harm_expand(order, L - 1, red, full, hs, ls, nrows, f32_locals, od.hx_step, od.hx_w, od.hx_cst, s),
+                CK(c, tc_harm_expand(order, L - 1, red, full, hs, ls, nrows, f32_locals, od.hx_step, od.hx_w, od.hx_cst,
+                                     ex.lh_split, s),
                    "M2L (harmonic expansion)");
                 ++launches;
             }

@@ -55,6 +55,7 @@ struct Expansions {
     float* Minv[dafmm::kMaxUniformDepth + 1] = {};
     // the harmonic-basis M2L's output rows (free coefficients, FP32, nharm rounded up to 8)
     float* Lh[dafmm::kMaxUniformDepth + 1] = {};
+    int lh_split = 1;  // blocks of rows in each Lh (tc_m2l_split)
     bool L_f32 = false;  // the last evaluation left FP32 rows (ncp floats per box) in L
     bool M_f32 = false;  // ... and in M
     bool M_harm = false;  // ... and harmonic-basis multipoles (free coefficients only) in M

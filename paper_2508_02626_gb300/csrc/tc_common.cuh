@@ -91,16 +91,30 @@ __device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
 
-// shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 bytes apart
-__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((addr >> 4) & 0x3FFFu);        // start address
-    d |= (uint64_t)1 << 16;                         // leading byte offset (unused for swizzled K-major)
-    d |= (uint64_t)(1024 >> 4) << 32;               // stride byte offset: next 8-row group
-    d |= (uint64_t)1 << 46;                         // descriptor version for tcgen05
-    d |= (uint64_t)2 << 61;                         // swizzle mode: 128-byte
-    return d;
+// Shared-memory matrix descriptor: K-major, 128-byte swizzle.  Low word: start address / 16 and the
+// leading byte offset (unused for swizzled K-major); high word: 8-row groups 1024 bytes apart,
+// descriptor version for tcgen05, 128-byte swizzle.
+__device__ __forceinline__ uint32_t smem_desc_lo(uint32_t addr) { return ((addr >> 4) & 0x3FFFu) | (1u << 16); }
+// SW64: 64-byte rows and swizzle, groups 512 bytes apart.
+template <bool SW64 = false>
+__device__ __forceinline__ uint64_t smem_desc(uint32_t lo) {
+    constexpr uint32_t hi = SW64 ? (512u >> 4) | (1u << 14) | (4u << 29) : (1024u >> 4) | (1u << 14) | (2u << 29);
+    return ((uint64_t)hi << 32) | lo;
 }
+
+__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) { return smem_desc(smem_desc_lo(addr)); }
+
+// one lane of the (converged) warp
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(r));
+    return r != 0;
+}
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0); }
 
 // instruction descriptor of kind::tf32: D = F32, A = B = TF32, both K-major, M x N
 __host__ __device__ constexpr uint32_t idesc_tf32(int M, int N) {
@@ -141,6 +155,22 @@ template <bool H>
 __device__ __forceinline__ void mma_op(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
     if constexpr (H) mma_f16(dtmem, adesc, bdesc, idesc, acc);
     else mma_tf32(dtmem, adesc, bdesc, idesc, acc);
+}
+
+// The split product of one K chunk, NKS steps of 32 bytes: A_hi B_lo + A_lo B_hi + A_hi B_hi (small
+// cross terms first) into d; fresh: the first MMA overwrites d.  The operands are descriptor low
+// words.  The issuing warp runs its loops with all lanes on values that are the same in every lane,
+// and one elected lane issues: the operands of tcgen05.mma are uniform registers, and with a single
+// lane running the loops every one of them was moved there separately.
+template <bool H, int NKS, bool SW64 = false>
+__device__ __forceinline__ void mma_chunk(uint32_t d, uint32_t ah, uint32_t al, uint32_t bh, uint32_t bl,
+                                          uint32_t idesc, bool fresh) {
+#pragma unroll
+    for (int ks = 0; ks < NKS; ++ks) {
+        mma_op<H>(d, smem_desc<SW64>(ah + 2 * ks), smem_desc<SW64>(bl + 2 * ks), idesc, ks > 0 || !fresh);
+        mma_op<H>(d, smem_desc<SW64>(al + 2 * ks), smem_desc<SW64>(bh + 2 * ks), idesc, 1);
+        mma_op<H>(d, smem_desc<SW64>(ah + 2 * ks), smem_desc<SW64>(bh + 2 * ks), idesc, 1);
+    }
 }
 
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
@@ -264,10 +294,33 @@ struct Cfg {
     static_assert(ROWLEN % KSTEP == 0 && KSTEPS_LAST >= 1 && KSTEPS_LAST <= 4, "K steps");
 };
 
+// The harmonic M2L of uniform trees (k_tc_m2l): two octants' matrices side by side (N = 2 NP), K
+// chunks of 64 bytes (two MMA steps; a row of 96 F16 values is three whole chunks, in 128-byte ones
+// it would be two with a quarter of the bytes padding, and the ring would hold two stages instead
+// of five), and two accumulators of 2 NP columns.
+template <int P, bool H>
+struct CfgM2L {
+    using B = Cfg<P, H, true>;
+    static constexpr int NC = B::NC, NCP = B::NCP, NP = B::NP, NPL = B::NPL, ROWLEN = B::ROWLEN;
+    static constexpr int KPC = H ? 32 : 16;  // elements per 64-byte chunk
+    static constexpr int NKC = (ROWLEN + KPC - 1) / KPC;
+    static constexpr int KSTEPS_LAST = (ROWLEN - KPC * (NKC - 1)) / B::KSTEP;
+    static constexpr int A_PART = 128 * 64;              // hi or lo rows of a tile
+    static constexpr int B_ROWS = NPL * 64, B_PART = 2 * NP * 64;  // one matrix as loaded; both, NP rows apart
+    static constexpr int STAGE = 2 * A_PART + 2 * B_PART;
+    static constexpr int ROOM = (227 * 1024 - 2048) / STAGE;
+    static constexpr int STAGES = ROOM > 8 ? 8 : ROOM;
+    static constexpr int SMEM = STAGES * STAGE + 1024 /*align*/ + 512 /*barriers*/;
+    static constexpr uint32_t IDESC1 = B::IDESC, IDESC2 = H ? idesc_f16(128, 2 * NP) : idesc_tf32(128, 2 * NP);
+    static_assert(STAGES >= 3 && B::NHALF == 1 && 2 * NP <= 256 && NP % 8 == 0, "ring, MMA N");
+    static_assert(KSTEPS_LAST == 1 || KSTEPS_LAST == 2, "K steps");
+};
+
 // a work item of the uniform-tree kernel: level index, target octant, child octant (L2L),
 // tile origin in slab coordinates, output half
 struct WorkItem {
     int li, oct, c, px0, py0, pz0, half;
+    int part;  // harmonic M2L: this item's share of the tile's steps
 };
 
 // the terms of a work item, in a fixed order.  M2L: the displacements v_d in
@@ -323,6 +376,34 @@ struct Terms {
     }
 };
 
+
+// The steps of the harmonic M2L for the octants (0, oy, oz) and (1, oy, oz) of a tile.  With
+// d = o - v = 2 a + sc per axis (a: the source's parent offset, sc: its octant), the source rows
+// depend on d alone: one step per d in [-2, 3]^3 serves the displacements v = (0, oy, oz) - d and
+// (1, oy, oz) - d of the two octants, where they are well separated (mask bit 0 and 1).
+struct M2LSteps {
+    int oy, oz, g, g1, dx, dy, dz;
+    unsigned mask;
+    __device__ void init(int pair, int part, int nsplit) {
+        oy = pair & 1;
+        oz = pair >> 1;
+        g = 216 * part / nsplit - 1;
+        g1 = 216 * (part + 1) / nsplit;
+    }
+    __device__ bool next() {  // the next step that has a term; false at the end
+        while (++g < g1) {
+            dx = g % 6 - 2;
+            dy = g / 6 % 6 - 2;
+            dz = g / 36 - 2;
+            const bool far = abs(oy - dy) > 1 || abs(oz - dz) > 1;
+            mask = (far || abs(-dx) > 1 ? 1u : 0u) | (far || abs(1 - dx) > 1 ? 2u : 0u);
+            if (mask) return true;
+        }
+        return false;
+    }
+    __device__ int slab() const { return (dx & 1) | ((dy & 1) << 1) | ((dz & 1) << 2); }
+    __device__ int key(int e) const { return (e - dx + 3) * 49 + (oy - dy + 3) * 7 + (oz - dz + 3); }
+};
 
 // round to the nearest TF32 value (10 explicit mantissa bits) and clear the 13 low bits, so
 // that hi + lo reproduces the operand exactly as the tensor core reads it
@@ -474,17 +555,18 @@ inline PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
 
 
 // 3-D map (coef, row, matrix) over [nkey][npt][rowlen] elements (FP32, or F16 when f16) with
-// boxes of 128 bytes x np rows
+// boxes of `bytes` (128 or 64, swizzled likewise) x np rows
 inline bool encode_rows(PFN_cuTensorMapEncodeTiled_v12000 enc, CUtensorMap* map, const void* base, int rowlen, int npt,
-                        int nkey, int np, bool f16 = false) {
+                        int nkey, int np, bool f16 = false, int bytes = 128) {
     const cuuint64_t es_bytes = f16 ? 2 : 4;
     const cuuint64_t dims[3] = {(cuuint64_t)rowlen, (cuuint64_t)npt, (cuuint64_t)nkey};
     const cuuint64_t strides[2] = {(cuuint64_t)rowlen * es_bytes, (cuuint64_t)rowlen * es_bytes * npt};
-    const cuuint32_t box[3] = {(cuuint32_t)(128 / es_bytes), (cuuint32_t)np, 1};
+    const cuuint32_t box[3] = {(cuuint32_t)(bytes / es_bytes), (cuuint32_t)np, 1};
     const cuuint32_t es[3] = {1, 1, 1};
     return enc(map, f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base),
-               dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+               dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 

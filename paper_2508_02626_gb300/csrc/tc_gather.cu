@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(kTcgThreads, 1) k_tcg(const __grid_constant__ 
     uint64_t* drain = acc_empty + 2;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::STAGES; ++s) {
             mbar_init(smem_u32(&full[s]), 65);  // 2 x 32 gather lanes + the expect_tx arrival
@@ -236,8 +236,9 @@ __global__ void __launch_bounds__(kTcgThreads, 1) k_tcg(const __grid_constant__ 
             for (int s = 0; s < C::STAGES; ++s)
                 if (armed[s] >= 0) mbar_wait(smem_u32(&full[s]), (uint32_t)armed[s], prm.err, 42);
         __syncwarp();
-    } else if (warp == 1 && lane == 0) {
-        // ---------------- MMA issuer ----------------
+    } else if (warp == 1) {
+        // ---------------- MMA issuer (all lanes walk, one issues: mma_chunk) ----------------
+        const bool leader = elect_one();
         int stage = 0;
         uint32_t phase = 0;
         uint32_t acc_ph[2] = {0, 0};
@@ -250,39 +251,34 @@ __global__ void __launch_bounds__(kTcgThreads, 1) k_tcg(const __grid_constant__ 
             do {
                 if (!tm.valid()) continue;
                 const int buf = uses & 1;
-                ok = mbar_wait(smem_u32(&acc_empty[buf]), acc_ph[buf] ^ 1u, prm.err, 43);
+                ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&acc_empty[buf]), acc_ph[buf] ^ 1u, prm.err, 43));
                 if (!ok) break;
                 acc_ph[buf] ^= 1u;
                 fence_after_sync();
                 const uint32_t d = tmem_base + (uint32_t)(buf * C::NP);
-                uint32_t accum = 0;
                 for (int kc = 0; kc < C::NKC && ok; ++kc) {
-                    ok = mbar_wait(smem_u32(&full[stage]), phase, prm.err, 44);
+                    ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&full[stage]), phase, prm.err, 44));
                     if (!ok) break;
                     fence_after_sync();
                     const uint32_t st = smem_u32(base + stage * C::STAGE_BYTES);
-                    const int nks = (kc == C::NKC - 1) ? C::KSTEPS_LAST : 4;
-                    for (int ks = 0; ks < nks; ++ks) {
-                        const uint64_t ah = smem_desc_sw128(st + ks * 32);
-                        const uint64_t al = smem_desc_sw128(st + C::A_BYTES + ks * 32);
-                        const uint64_t bh = smem_desc_sw128(st + 2 * C::A_BYTES + ks * 32);
-                        const uint64_t bl = smem_desc_sw128(st + 2 * C::A_BYTES + C::B_BYTES + ks * 32);
-                        mma_op<H>(d, ah, bl, C::IDESC, accum);
-                        accum = 1;
-                        mma_op<H>(d, al, bh, C::IDESC, 1);
-                        mma_op<H>(d, ah, bh, C::IDESC, 1);
+                    const uint32_t ah = smem_desc_lo(st), al = smem_desc_lo(st + C::A_BYTES);
+                    const uint32_t bh = smem_desc_lo(st + 2 * C::A_BYTES), bl = smem_desc_lo(st + 2 * C::A_BYTES + C::B_BYTES);
+                    if (leader) {
+                        if (kc < C::NKC - 1) mma_chunk<H, 4>(d, ah, al, bh, bl, C::IDESC, kc == 0);
+                        else mma_chunk<H, C::KSTEPS_LAST>(d, ah, al, bh, bl, C::IDESC, kc == 0);
+                        mma_commit(smem_u32(&empty[stage]));
                     }
-                    mma_commit(smem_u32(&empty[stage]));
                     if (++stage == C::STAGES) {
                         stage = 0;
                         phase ^= 1u;
                     }
                 }
-                if (ok) mma_commit(smem_u32(&acc_full[buf]));
+                if (ok && leader) mma_commit(smem_u32(&acc_full[buf]));
                 ++uses;
             } while (tm.next() && ok);
         }
-        mma_commit(smem_u32(drain));
+        if (leader) mma_commit(smem_u32(drain));
+        __syncwarp();
         mbar_wait(smem_u32(drain), 0, prm.err, 45);
     } else if (warp >= 2 && warp <= 5) {
         // ---------------- epilogue ----------------

@@ -39,6 +39,7 @@ __device__ __forceinline__ WorkItem decode(const TCParams& prm, int w) {
     it.li = li;
     it.half = local % prm.nhalf;
     local /= prm.nhalf;
+    it.part = 0;
     it.oct = 0;
     it.c = 0;
     if (prm.mode == kTcM2L || prm.mode == kTcL2L) {
@@ -71,10 +72,10 @@ __device__ __forceinline__ int out_index(const TCParams& prm, const WorkItem& it
     return it.c * Pl * Pl * Pl + (cz * Pl + cy) * Pl + cx;
 }
 
-// ---- the kernel -----------------------------------------------------------------------------
-template <int P, bool H, bool R>
+// ---- the kernel of the full basis (M2L, M2M, L2L) ----------------------------------------------
+template <int P, bool H>
 __global__ void __launch_bounds__(192, 1) k_tc(const __grid_constant__ TCParams prm) {
-    using C = Cfg<P, H, R>;
+    using C = Cfg<P, H>;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // 1024-byte aligned stage ring, then barriers
     unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -86,7 +87,7 @@ __global__ void __launch_bounds__(192, 1) k_tc(const __grid_constant__ TCParams 
     uint64_t* drain = acc_empty + 2;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::STAGES; ++s) {
             mbar_init(smem_u32(&full[s]), 1);
@@ -154,8 +155,9 @@ __global__ void __launch_bounds__(192, 1) k_tc(const __grid_constant__ TCParams 
         // wait (bounded) until every copy this thread armed has landed before the block may exit
         for (int s = 0; s < C::STAGES; ++s)
             if (armed[s] >= 0) mbar_wait(smem_u32(&full[s]), (uint32_t)armed[s], prm.err, 12);
-    } else if (warp == 1 && lane == 0) {
-        // ---------------- MMA issuer ----------------
+    } else if (warp == 1) {
+        // ---------------- MMA issuer (all lanes walk, one issues: mma_chunk) ----------------
+        const bool leader = elect_one();
         // one fresh accumulator per term (alternating TMEM buffers): at most
         // 3 * ceil(ncoef/8) MMA accumulation steps land in one FP32 accumulator
         int stage = 0;
@@ -170,40 +172,35 @@ __global__ void __launch_bounds__(192, 1) k_tc(const __grid_constant__ TCParams 
             do {
                 if (!tm.valid()) continue;
                 const int buf = uses & 1;
-                ok = mbar_wait(smem_u32(&acc_empty[buf]), acc_ph[buf] ^ 1u, prm.err, 21);
+                ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&acc_empty[buf]), acc_ph[buf] ^ 1u, prm.err, 21));
                 if (!ok) break;
                 acc_ph[buf] ^= 1u;
                 fence_after_sync();
                 const uint32_t d = tmem_base + (uint32_t)(buf * C::NP);
-                uint32_t accum = 0;
                 for (int kc = 0; kc < C::NKC && ok; ++kc) {
-                    ok = mbar_wait(smem_u32(&full[stage]), phase, prm.err, 22);
+                    ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&full[stage]), phase, prm.err, 22));
                     if (!ok) break;
                     fence_after_sync();
                     const uint32_t st = smem_u32(base + stage * C::STAGE_BYTES);
-                    const int nks = (kc == C::NKC - 1) ? C::KSTEPS_LAST : 4;
-                    for (int ks = 0; ks < nks; ++ks) {
-                        const uint64_t ah = smem_desc_sw128(st + ks * 32);
-                        const uint64_t al = smem_desc_sw128(st + C::A_BYTES + ks * 32);
-                        const uint64_t bh = smem_desc_sw128(st + 2 * C::A_BYTES + ks * 32);
-                        const uint64_t bl = smem_desc_sw128(st + 2 * C::A_BYTES + C::B_BYTES + ks * 32);
-                        mma_op<H>(d, ah, bl, C::IDESC, accum);  // small cross terms first
-                        accum = 1;
-                        mma_op<H>(d, al, bh, C::IDESC, 1);
-                        mma_op<H>(d, ah, bh, C::IDESC, 1);
+                    const uint32_t ah = smem_desc_lo(st), al = smem_desc_lo(st + C::A_BYTES);
+                    const uint32_t bh = smem_desc_lo(st + 2 * C::A_BYTES), bl = smem_desc_lo(st + 2 * C::A_BYTES + C::B_BYTES);
+                    if (leader) {
+                        if (kc < C::NKC - 1) mma_chunk<H, 4>(d, ah, al, bh, bl, C::IDESC, kc == 0);
+                        else mma_chunk<H, C::KSTEPS_LAST>(d, ah, al, bh, bl, C::IDESC, kc == 0);
+                        mma_commit(smem_u32(&empty[stage]));
                     }
-                    mma_commit(smem_u32(&empty[stage]));
                     if (++stage == C::STAGES) {
                         stage = 0;
                         phase ^= 1u;
                     }
                 }
-                if (ok) mma_commit(smem_u32(&acc_full[buf]));
+                if (ok && leader) mma_commit(smem_u32(&acc_full[buf]));
                 ++uses;
             } while (tm.next() && ok);
         }
         // every MMA this thread issued has finished once the drain barrier flips
-        mma_commit(smem_u32(drain));
+        if (leader) mma_commit(smem_u32(drain));
+        __syncwarp();
         mbar_wait(smem_u32(drain), 0, prm.err, 23);
     } else if (warp >= 2) {
         // ---------------- epilogue ----------------
@@ -249,7 +246,7 @@ __global__ void __launch_bounds__(192, 1) k_tc(const __grid_constant__ TCParams 
                 accf_ph[buf] ^= 1u;
                 fence_after_sync();
                 const uint32_t tb = tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * C::NP);
-                fold_term<C::NP, H, R>(tb, f, S);
+                fold_term<C::NP, H, false>(tb, f, S);
                 ++uses;
                 have = tm.next_valid();
                 if (have) {
@@ -290,6 +287,249 @@ __global__ void __launch_bounds__(192, 1) k_tc(const __grid_constant__ TCParams 
         fence_after_sync();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(C::TMEM_COLS)
                      : "memory");
+    }
+}
+
+// ---- the harmonic M2L of uniform trees ---------------------------------------------------------
+// One persistent CTA per SM: a TMA producer warp, an MMA issuer warp and two groups of four epilogue
+// warps.  An item is a tile of 128 parents and two octants of their children, (0, oy, oz) and
+// (1, oy, oz): the sources of both at one offset d are the same rows (M2LSteps), so a step
+// multiplies them by two matrices side by side, N = 2 NP, into one accumulator.
+//   Why: the kernel is bound by shared memory, 128 bytes per clock.  At p = 8 (NP = 96) a term alone
+// takes 18 MMAs that read 4 KB of A and 3 KB of B each, and TMA writes 110 KB (the 96-column rows in
+// 128-byte chunks): 1870 cycles of shared memory against 1000 of tensor pipe, 2270 measured, the
+// tensor pipe 40 % busy.  Two octants to a step halve the A reads and writes (415 -> 324 us with
+// 128-byte chunks), and 64-byte chunks drop the padding and make the ring five stages deep (324 ->
+// 228 us).  (Other causes were ruled out by measurement: reusing A rows along a shared axis, which
+// cuts the traffic from L2 by a third, a second epilogue group, and alternating accumulators
+// gained nothing by themselves.)
+//   The epilogue groups take one octant each: a step's accumulator half scaled per row and added
+// in FP32 registers (one accumulator for all terms costs accuracy).  At depth 5 the items are as
+// many as the SMs: 4 x (32 + 4 + 1 + 1) = 152.
+// N = 1e6, depth 5, p = 8: FP32 (F16 operands) 415 -> 228 us, MIXED (TF32) 610 -> 505 us.
+struct PairItem {
+    int li, pair, part, px0, py0, pz0;
+};
+__device__ __forceinline__ PairItem decode_pair(const TCParams& prm, int w) {
+    PairItem it;
+    int li = 0;
+    while (li + 1 < prm.nlev && w >= prm.tile_base[li + 1]) ++li;
+    int local = w - prm.tile_base[li];
+    it.li = li;
+    it.part = local % prm.nsplit;
+    local /= prm.nsplit;
+    it.pair = local & 3;
+    local >>= 2;
+    const int nx = prm.S[li] / prm.bx[li], ny = prm.S[li] / prm.by[li];
+    it.px0 = (local % nx) * prm.bx[li];
+    it.py0 = ((local / nx) % ny) * prm.by[li];
+    it.pz0 = (local / (nx * ny)) * prm.bz[li];
+    return it;
+}
+
+template <int P, bool H>
+__global__ void __launch_bounds__(320, 1) k_tc_m2l(const __grid_constant__ TCParams prm) {
+    using C = CfgM2L<P, H>;
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint64_t* full = reinterpret_cast<uint64_t*>(base + C::STAGES * C::STAGE);
+    uint64_t* empty = full + C::STAGES;
+    uint64_t* acc_full = empty + C::STAGES;
+    uint64_t* acc_empty = acc_full + 2;
+    uint64_t* drain = acc_empty + 2;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+
+    const int warp = warp_index(), lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < C::STAGES; ++s) {
+            mbar_init(smem_u32(&full[s]), 1);
+            mbar_init(smem_u32(&empty[s]), 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(smem_u32(&acc_full[b]), 1);
+            mbar_init(smem_u32(&acc_empty[b]), 256);
+        }
+        mbar_init(smem_u32(drain), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "r"(512)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    fence_before_sync();
+    __syncthreads();
+    fence_after_sync();
+    const uint32_t tmem_base = *tmem_slot;
+
+    if (warp == 0 && lane == 0) {
+        // ---------------- TMA producer ----------------
+        for (int l = 0; l < prm.nlev; ++l) {
+            prefetch_map(&prm.a_hi[l]);
+            prefetch_map(&prm.a_lo[l]);
+        }
+        prefetch_map(&prm.b_hi);
+        prefetch_map(&prm.b_lo);
+        int stage = 0;
+        uint32_t phase = 0;
+        // which full barriers were armed, and the parities of their last phases (a bit per stage)
+        uint32_t armed = 0, parity = 0;
+        bool ok = true;
+        for (int w = blockIdx.x; w < prm.ntiles && ok; w += gridDim.x) {
+            const PairItem it = decode_pair(prm, w);
+            const uint32_t a_bytes = 2u * 64u * (uint32_t)(prm.bx[it.li] * prm.by[it.li] * prm.bz[it.li]);
+            M2LSteps st;
+            st.init(it.pair, it.part, prm.nsplit);
+            while (ok && st.next()) {
+                const int cx = it.px0 + (st.dx >> 1), cy = it.py0 + (st.dy >> 1), cz = it.pz0 + (st.dz >> 1),
+                          slab = st.slab();
+                for (int kc = 0; kc < C::NKC && ok; ++kc) {
+                    const int kx = kc * C::KPC;  // first element of the chunk (64-byte aligned)
+                    ok = mbar_wait(smem_u32(&empty[stage]), phase ^ 1u, prm.err, 11);
+                    if (!ok) break;
+                    const uint32_t sa = smem_u32(base + stage * C::STAGE), sb = sa + 2 * C::A_PART;
+                    const uint32_t fb = smem_u32(&full[stage]);
+                    mbar_expect_tx(fb, a_bytes + (st.mask == 3u ? 4u : 2u) * C::B_ROWS);
+                    armed |= 1u << stage;
+                    parity = (parity & ~(1u << stage)) | (phase << stage);
+                    tma_load_5d(sa, &prm.a_hi[it.li], fb, kx, cx, cy, cz, slab);
+                    tma_load_5d(sa + C::A_PART, &prm.a_lo[it.li], fb, kx, cx, cy, cz, slab);
+#pragma unroll
+                    for (int e = 0; e < 2; ++e)
+                        if (st.mask >> e & 1u) {
+                            const int key = st.key(e);
+                            tma_load_3d(sb + e * C::NP * 64, &prm.b_hi, fb, kx, 0, key);
+                            tma_load_3d(sb + C::B_PART + e * C::NP * 64, &prm.b_lo, fb, kx, 0, key);
+                        }
+                    if (++stage == C::STAGES) {
+                        stage = 0;
+                        phase ^= 1u;
+                    }
+                }
+            }
+        }
+        // wait (bounded) until every copy this thread armed has landed before the block may exit
+        for (int s = 0; s < C::STAGES; ++s)
+            if (armed >> s & 1u) mbar_wait(smem_u32(&full[s]), parity >> s & 1u, prm.err, 12);
+    } else if (warp == 1) {
+        // ---------------- MMA issuer (all lanes walk, one issues: mma_chunk) ----------------
+        const bool leader = elect_one();
+        int stage = 0, buf = 0;
+        uint32_t phase = 0, accph = 0;
+        bool ok = true;
+        for (int w = blockIdx.x; w < prm.ntiles && ok; w += gridDim.x) {
+            const PairItem it = decode_pair(prm, w);
+            M2LSteps st;
+            st.init(it.pair, it.part, prm.nsplit);
+            while (ok && st.next()) {
+                ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&acc_empty[buf]), accph ^ 1u, prm.err, 21));
+                // one octant alone: its half of the accumulator and of the matrices
+                const uint32_t half = st.mask == 2u ? 1u : 0u, idesc = st.mask == 3u ? C::IDESC2 : C::IDESC1;
+                const uint32_t d = tmem_base + (uint32_t)buf * 2u * C::NP + half * C::NP;
+                for (int kc = 0; kc < C::NKC && ok; ++kc) {
+                    ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&full[stage]), phase, prm.err, 22));
+                    if (!ok) break;
+                    fence_after_sync();
+                    const uint32_t ah = smem_desc_lo(smem_u32(base + stage * C::STAGE)), al = ah + (C::A_PART >> 4);
+                    const uint32_t bh = ah + (2 * C::A_PART >> 4) + half * (C::NP * 64u >> 4), bl = bh + (C::B_PART >> 4);
+                    if (leader) {
+                        if (kc < C::NKC - 1) mma_chunk<H, 2, true>(d, ah, al, bh, bl, idesc, kc == 0);
+                        else mma_chunk<H, C::KSTEPS_LAST, true>(d, ah, al, bh, bl, idesc, kc == 0);
+                        mma_commit(smem_u32(&empty[stage]));
+                        if (kc == C::NKC - 1) mma_commit(smem_u32(&acc_full[buf]));
+                    }
+                    if (++stage == C::STAGES) {
+                        stage = 0;
+                        phase ^= 1u;
+                    }
+                }
+                if (++buf == 2) {
+                    buf = 0;
+                    accph ^= 1u;
+                }
+            }
+        }
+        // every MMA the leader issued has finished once the drain barrier flips
+        if (leader) mma_commit(smem_u32(drain));
+        __syncwarp();
+        mbar_wait(smem_u32(drain), 0, prm.err, 23);
+    } else if (warp >= 2) {
+        // ---------------- epilogue ----------------
+        const int e = warp >= 6 ? 1 : 0;  // the octant of the pair
+        const int q = warp & 3;           // TMEM lane quarter of this warp
+        const int row = 32 * q + lane;    // accumulator row = box within the tile
+        const uint32_t tcol = tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(e * C::NP);
+        int buf = 0;
+        uint32_t accph = 0;
+        bool ok = true;
+        for (int w = blockIdx.x; w < prm.ntiles && ok; w += gridDim.x) {
+            const PairItem it = decode_pair(prm, w);
+            float S[C::NP];
+#pragma unroll
+            for (int j = 0; j < C::NP; ++j) S[j] = 0.f;
+            const int bx = prm.bx[it.li], by = prm.by[it.li], bz = prm.bz[it.li], SL = prm.S[it.li];
+            const bool valid = row < bx * by * bz;
+            const int px = it.px0 + row % bx, py = it.py0 + (row / bx) % by, pz = it.pz0 + row / (bx * by);
+            const float* __restrict__ a_inv = prm.a_inv[it.li];
+            M2LSteps st;
+            st.init(it.pair, it.part, prm.nsplit);
+            // F16 operands: a term's accumulator carries the source row's scale and the matrix's
+            // scalar; the factor undoing both (one per row and term) is looked up for the next step
+            // right after a step's accumulator is released, before waiting for the next one
+            auto factor = [&]() -> float {
+                if constexpr (H) {
+                    const int cx = px + (st.dx >> 1), cy = py + (st.dy >> 1), cz = pz + (st.dz >> 1);
+                    if (!valid || !(st.mask >> e & 1u) || cx < 0 || cy < 0 || cz < 0 || cx >= SL || cy >= SL || cz >= SL)
+                        return 0.f;
+                    return a_inv[((st.slab() * SL + cz) * SL + cy) * SL + cx] * prm.inv_c[st.key(e)];
+                } else {
+                    return 1.f;
+                }
+            };
+            bool have = st.next();
+            int held = -1;  // the last step's accumulator stays held until the rows are out
+            float f = have ? factor() : 0.f;
+            while (have) {
+                ok = mbar_wait(smem_u32(&acc_full[buf]), accph, prm.err, 31);
+                if (!ok) break;
+                fence_after_sync();
+                if (st.mask >> e & 1u) fold_term<C::NP, H, true>(tcol + (uint32_t)buf * 2u * C::NP, f, S);
+                const int done = buf;
+                if (++buf == 2) {
+                    buf = 0;
+                    accph ^= 1u;
+                }
+                have = st.next();
+                if (have) {
+                    fence_before_sync();
+                    mbar_arrive(smem_u32(&acc_empty[done]));
+                    f = factor();
+                } else {
+                    held = done;
+                }
+            }
+            if (!ok) break;
+            if (held < 0) continue;  // no step (does not occur: every share has one)
+            // the summed row into this group's half of the held accumulator, then out from there
+            const uint32_t tb = tcol + (uint32_t)held * 2u * C::NP;
+#pragma unroll
+            for (int c0 = 0; c0 < C::NP; c0 += 16) tmem_st16(tb + c0, S + c0);
+            tmem_wait_st();
+            float* orow = reinterpret_cast<float*>(prm.out[it.li]) + it.part * prm.split_stride[it.li];
+            if (valid) orow += ((((size_t)(e + 2 * it.pair) * SL + pz) * SL + py) * SL + px) * C::NCP;
+            store_row<C::NP, C::NC, C::NCP, H>(tb, valid, 0, prm.scale[it.li], (float)prm.scale[it.li], prm.inv_r, false,
+                                               true, orow, nullptr, nullptr);
+            fence_before_sync();
+            mbar_arrive(smem_u32(&acc_empty[held]));
+        }
+    }
+    fence_before_sync();
+    __syncthreads();
+    if (warp == 1) {
+        __syncwarp();
+        fence_after_sync();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
     }
 }
 
@@ -497,6 +737,7 @@ struct HarmSegments {
     float* lo[kTcMaxLevels];
     int first[kTcMaxLevels + 1];
     int nseg;
+    int nsplit;  // blocks of rows in red, summed in order
     int full_f32;
     int cst[kMaxOrder + 3];  // steps of z exponent c: [cst[c], cst[c + 1]), c = 2..p
 };
@@ -513,7 +754,12 @@ __global__ void __launch_bounds__(128) k_harm_expand(HarmSegments sg, const int4
     row -= sg.first[g];
     float* buf = sbuf[wi];
     const float* r = sg.red[g] + (size_t)row * nhp;
-    for (int k = lane; k < nh; k += 32) buf[harm_full_index(k)] = r[k];
+    const size_t stride = (size_t)(sg.first[g + 1] - sg.first[g]) * nhp;
+    for (int k = lane; k < nh; k += 32) {
+        float v = r[k];
+        for (int p1 = 1; p1 < sg.nsplit; ++p1) v += r[p1 * stride + k];
+        buf[harm_full_index(k)] = v;
+    }
     __syncwarp();
     for (int c = 2; c <= p; ++c) {
         for (int s = sg.cst[c] + lane; s < sg.cst[c + 1]; s += 32) {
@@ -615,11 +861,12 @@ cudaError_t tc_prepare_k16h(const double* K, int nkey, int p, const double* X, d
 
 cudaError_t tc_harm_expand(int p, int nseg, const float* const* red, void* const* full, float* const* hi,
                            float* const* lo, const int* nrows, bool full_f32, const int4* step, const float2* w,
-                           const int* cst, cudaStream_t s) {
-    if (nseg < 1 || nseg > kTcMaxLevels) return cudaErrorInvalidValue;
+                           const int* cst, int nsplit, cudaStream_t s) {
+    if (nseg < 1 || nseg > kTcMaxLevels || nsplit < 1) return cudaErrorInvalidValue;
     tc::HarmSegments sg;
     memset(&sg, 0, sizeof(sg));
     sg.nseg = nseg;
+    sg.nsplit = nsplit;
     sg.full_f32 = full_f32 ? 1 : 0;
     for (int g = 0; g < nseg; ++g) {
         sg.red[g] = red[g];
@@ -667,18 +914,32 @@ static void tile_shape(int S, int& bx, int& by, int& bz) {
 
 // 5-D map (coef, x, y, z, slab) over an octant-major level with S slab positions per axis
 static bool encode_level(PFN_cuTensorMapEncodeTiled_v12000 enc, CUtensorMap* map, const void* base, int rowlen, int S,
-                         int bx, int by, int bz, bool f16) {
+                         int bx, int by, int bz, bool f16, int bytes) {
     const cuuint64_t esz = f16 ? 2 : 4;
     const cuuint64_t dims[5] = {(cuuint64_t)rowlen, (cuuint64_t)S, (cuuint64_t)S, (cuuint64_t)S, 8};
     const cuuint64_t row = (cuuint64_t)rowlen * esz;
     const cuuint64_t strides[4] = {row, row * S, row * S * S, row * S * S * S};
-    const cuuint32_t box[5] = {(cuuint32_t)(128 / esz), (cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)bz, 1};
+    const cuuint32_t box[5] = {(cuuint32_t)(bytes / esz), (cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)bz, 1};
     const cuuint32_t es[5] = {1, 1, 1, 1, 1};
     return enc(map, f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, const_cast<void*>(base),
-               dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+               dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+int tc_m2l_split(int depth, int num_sms) {
+    int items = 0;
+    for (int l = 2; l <= depth; ++l) {
+        const int S = 1 << (l - 1);
+        int bx, by, bz;
+        tile_shape(S, bx, by, bz);
+        items += 4 * (S / bx) * (S / by) * (S / bz);
+    }
+    const int k = items > 0 ? num_sms / items : 1;
+    return k < 1 ? 1 : (k > 16 ? 16 : k);  // at least 13 steps per item
+}
+
+// R: the harmonic M2L (k_tc_m2l), else the full-basis kernel
 template <int P, bool H, bool R = false>
 static cudaError_t launch_tc(const TCArgs& a, cudaStream_t s) {
     using C = tc::Cfg<P, H, R>;
@@ -690,8 +951,11 @@ static cudaError_t launch_tc(const TCArgs& a, cudaStream_t s) {
     prm.nhalf = C::NHALF;
     prm.out_f32 = a.out_f32 ? 1 : 0;
     prm.err = a.err;
+    prm.nsplit = R && a.nsplit > 1 ? a.nsplit : 1;
+    if (R && (a.mode != kTcM2L || !a.out_f32)) return cudaErrorInvalidValue;
     int tiles = 0;
-    const int per_tile_groups = a.mode == kTcM2L ? 8 : (a.mode == kTcL2L ? 64 : 1);
+    const int kb = R ? 64 : 128;  // bytes of a K chunk
+    const int per_tile_groups = R ? 4 : (a.mode == kTcM2L ? 8 : (a.mode == kTcL2L ? 64 : 1));
     // finest level first: all work items of a launch cost about the same
     for (int l = a.lmax; l >= a.lmin; --l) {
         const int li = prm.nlev++;
@@ -707,10 +971,11 @@ static cudaError_t launch_tc(const TCArgs& a, cudaStream_t s) {
         prm.scale[li] = a.scale[l];
         prm.out_level[li] = a.mode == kTcM2M ? l - 1 : l;
         prm.tile_base[li] = tiles;
-        tiles += per_tile_groups * (S / bx) * (S / by) * (S / bz) * C::NHALF;
+        tiles += per_tile_groups * (S / bx) * (S / by) * (S / bz) * C::NHALF * prm.nsplit;
+        prm.split_stride[li] = prm.nsplit > 1 ? ((size_t)1 << (3 * l)) * C::NCP : 0;
         prm.a_inv[li] = a.a_inv[src];
-        if (!encode_level(enc, &prm.a_hi[li], a.a_hi[src], C::ROWLEN, S, bx, by, bz, H) ||
-            !encode_level(enc, &prm.a_lo[li], a.a_lo[src], C::ROWLEN, S, bx, by, bz, H))
+        if (!encode_level(enc, &prm.a_hi[li], a.a_hi[src], C::ROWLEN, S, bx, by, bz, H, kb) ||
+            !encode_level(enc, &prm.a_lo[li], a.a_lo[src], C::ROWLEN, S, bx, by, bz, H, kb))
             return cudaErrorInvalidValue;
     }
     prm.tile_base[prm.nlev] = tiles;
@@ -718,14 +983,22 @@ static cudaError_t launch_tc(const TCArgs& a, cudaStream_t s) {
     const int npt = C::NPT;
     prm.inv_r = a.inv_r;
     prm.inv_c = a.inv_c;
-    if (!encode_rows(enc, &prm.b_hi, a.b_hi, C::ROWLEN, npt, a.nkey, C::NPL, H) ||
-        !encode_rows(enc, &prm.b_lo, a.b_lo, C::ROWLEN, npt, a.nkey, C::NPL, H))
+    if (!encode_rows(enc, &prm.b_hi, a.b_hi, C::ROWLEN, npt, a.nkey, C::NPL, H, kb) ||
+        !encode_rows(enc, &prm.b_lo, a.b_lo, C::ROWLEN, npt, a.nkey, C::NPL, H, kb))
         return cudaErrorInvalidValue;
     if (tiles == 0) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(tc::k_tc<P, H, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
-    if (e != cudaSuccess) return e;
     const int grid = tiles < a.num_sms ? tiles : a.num_sms;
-    tc::k_tc<P, H, R><<<grid, 192, C::SMEM_BYTES, s>>>(prm);
+    if constexpr (R) {
+        constexpr int smem = tc::CfgM2L<P, H>::SMEM;
+        const cudaError_t e = cudaFuncSetAttribute(tc::k_tc_m2l<P, H>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        tc::k_tc_m2l<P, H><<<grid, 320, smem, s>>>(prm);
+    } else {
+        const cudaError_t e =
+            cudaFuncSetAttribute(tc::k_tc<P, H>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
+        if (e != cudaSuccess) return e;
+        tc::k_tc<P, H><<<grid, 192, C::SMEM_BYTES, s>>>(prm);
+    }
     return cudaGetLastError();
 }
 template <int P>

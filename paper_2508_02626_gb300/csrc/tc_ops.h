@@ -32,6 +32,10 @@ struct TCParams {
     const float* a_inv[kTcMaxLevels];
     const float* inv_r;
     const float* inv_c;
+    // harmonic M2L: the shares of a tile's steps, each an item of its own, whose output rows go to
+    // out + share * split_stride floats (tc_m2l_split)
+    int nsplit;
+    size_t split_stride[kTcMaxLevels];
     int nlev;
     int ntiles;
     int nhalf;
@@ -60,9 +64,17 @@ struct TCArgs {
     const float* inv_r;                          // F16: per-column factor of the matrices
     const float* inv_c;                          // F16: per-matrix factor
     int nkey;
+    int nsplit;                                  // (M2L, harm) shares of the terms: tc_m2l_split, or 1
     int* err;                                    // device error flag
     int num_sms;
 };
+
+// M2L of a uniform tree of this depth: over how many items a tile's steps are shared out.  A
+// depth-2 tree has 4 items (a tile, two octants each), a depth-3 tree 8, a depth-4 tree 24, each
+// walking its steps in series on one SM of 152; a depth-5 tree has 152.  The rows of the shares (FP32,
+// harmonic basis) lie one after another and are summed, in order, by the expansion
+// (tc_harm_expand).  N = 3001, depth 2, p = 4: the M2L 110 -> 10 us.
+int tc_m2l_split(int depth, int num_sms);
 
 // ---- gathered form (adaptive trees and forests) ----
 // Targets come in groups (boxes of one level and octant, contiguous in `tg`); the A rows of a
@@ -156,10 +168,10 @@ cudaError_t tc_split_tf32_harm(const double* src, size_t nrows, int p, float* hi
 // rows of free coefficients (FP32, nhp per row) of up to kTcMaxLevels arrays -> full rows (FP32
 // or FP64, ncp per row) by Laplace's equation: steps (i, i1, i2) with weights (w1, w2), those of
 // z exponent c at [cst[c], cst[c + 1]); hi / lo (optional, per array or null) receive the TF32
-// split of the written rows
+// split of the written rows; each red[g] holds nsplit blocks of nrows[g] rows, summed in order
 cudaError_t tc_harm_expand(int p, int nseg, const float* const* red, void* const* full, float* const* hi,
                            float* const* lo, const int* nrows, bool full_f32, const int4* step, const float2* w,
-                           const int* cst, cudaStream_t s);
+                           const int* cst, int nsplit, cudaStream_t s);
 cudaError_t tcg_launch(int p, const TCGArgs& a, cudaStream_t s);
 cudaError_t tc_split_tf32(const double* src, float* hi, float* lo, size_t n, cudaStream_t s);
 cudaError_t tc_split_rows(const double* src, int nkey, int p, float* hi, float* lo, cudaStream_t s);
