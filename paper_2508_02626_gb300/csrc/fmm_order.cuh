@@ -105,13 +105,83 @@ __device__ __forceinline__ void warp_row_to_f32(const double* __restrict__ row, 
     __syncwarp();
 }
 
+// The steps that restore the coefficients of z exponent >= 2 of a harmonic expansion from its free
+// ones by Laplace's equation (internal.h): V[i] = w1 V[i1] + w2 V[i2], those of z exponent c at
+// [cst[c], cst[c + 1]).
+struct HarmTab {
+    static constexpr int N = NC - nharm_of(P) > 0 ? NC - nharm_of(P) : 1;
+    int cst[P + 3];
+    unsigned short i[N], i1[N], i2[N];
+    float w1[N], w2[N], w1l[N], w2l[N];  // FP32, and its remainder (float-float)
+    double d1[N], d2[N];
+};
+constexpr HarmTab make_harm_tab() {
+    HarmTab t{};
+    int k = 0;
+    for (int c = 2; c <= P; ++c) {
+        t.cst[c] = k;
+        for (int n = c; n <= P; ++n)
+            for (int b = 0; b <= n - c; ++b, ++k) {
+                const int a = n - c - b;
+                t.i[k] = (unsigned short)da_index(a, b, c);
+                t.i1[k] = (unsigned short)da_index(a + 2, b, c - 2);
+                t.i2[k] = (unsigned short)da_index(a, b + 2, c - 2);
+                t.d1[k] = -(double)((a + 2) * (a + 1)) / (double)(c * (c - 1));
+                t.d2[k] = -(double)((b + 2) * (b + 1)) / (double)(c * (c - 1));
+                t.w1[k] = (float)t.d1[k];
+                t.w2[k] = (float)t.d2[k];
+                t.w1l[k] = (float)(t.d1[k] - (double)t.w1[k]);
+                t.w2l[k] = (float)(t.d2[k] - (double)t.w2[k]);
+            }
+    }
+    for (int c = P < 1 ? 2 : P + 1; c < P + 3; ++c) t.cst[c] = k;
+    return t;
+}
+__device__ const HarmTab harm_tab = make_harm_tab();
+
+__device__ __forceinline__ float harm_step(const float* V, int s) {
+    return fmaf(harm_tab.w1[s], V[harm_tab.i1[s]], harm_tab.w2[s] * V[harm_tab.i2[s]]);
+}
+__device__ __forceinline__ double harm_step(const double* V, int s) {
+    return fma(harm_tab.d1[s], V[harm_tab.i1[s]], harm_tab.d2[s] * V[harm_tab.i2[s]]);
+}
+__device__ __forceinline__ ff harm_step(const ff* V, int s) {
+    return ff_add(ff_mul(ff(harm_tab.w1[s], harm_tab.w1l[s]), V[harm_tab.i1[s]]),
+                  ff_mul(ff(harm_tab.w2[s], harm_tab.w2l[s]), V[harm_tab.i2[s]]));
+}
+// the warp restores V's coefficients of z exponent >= 2, exponent by exponent
+template <class R>
+__device__ __forceinline__ void harm_expand_warp(R* V, int lane) {
+#pragma unroll 1
+    for (int c = 2; c <= P; ++c) {
+        for (int s = harm_tab.cst[c] + lane; s < harm_tab.cst[c + 1]; s += 32) V[harm_tab.i[s]] = harm_step(V, s);
+        __syncwarp();
+    }
+}
+
 // ---- P2M ---------------------------------------------------------------------------------
+// the full FP64 row from a warp's free coefficients (acc[c]: coefficient 32 c + lane), by way of the
+// staging block sm
+template <class T, int NJ>
+__device__ __forceinline__ void p2m_row(const T (&acc)[NJ], T* sm, double* __restrict__ row, int lane) {
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < NJ; ++j)
+        if (lane + 32 * j < nharm_of(P)) sm[harm_full_index(lane + 32 * j)] = acc[j];
+    __syncwarp();
+    harm_expand_warp(sm, lane);
+    for (int k = lane; k < NC; k += 32) row[k] = (double)sm[k];
+}
+
 // rows32: the multipole rows are FP32 (NCP floats per leaf) instead of FP64.  The FP32 kernel
 // reads the particles' FP32 leaf-frame records, which hold exactly the values it would compute
 // from the FP64 coordinates ((x - c) / h rounded once to FP32), without FP64 arithmetic.
 // H: the harmonic basis -- the generated code emits only the (p + 1)^2 free coefficients
 // (z exponent <= 1), which are summed and written at their layout positions; the others are
-// not computed (the multipole's homogeneous parts are harmonic, Eq. 2, so they are implied).
+// not computed (the multipole's homogeneous parts are harmonic, Eq. 2, so they are implied).  FP64
+// and float-float (always H) restore them here, once per leaf, by Laplace's equation: the rows are
+// complete, with 0.4 times the arithmetic per particle at p = 8 (N = 200,003, depth 4: FP64 672 -> 315
+// us, float-float 493 -> 138 us).
 // f16 (H, FP32 rows): the row's F16 split as well, as tc_split_f16_multi makes it -- the warp
 // holds the whole row, so its largest magnitude is one warp reduction away.
 template <class T, bool H = false>
@@ -187,6 +257,10 @@ __global__ void k_p2m(TreeView tv, double* __restrict__ M, int rows32, F16Rows f
                 if (lane == 0) f16.inv[leaf] = ldexpf(1.f, e);
             }
         }
+        return;
+    }
+    if constexpr (H && sizeof(T) == 8) {
+        p2m_row(acc, sm, M + (size_t)leaf * NCP, lane);
         return;
     }
 #pragma unroll
@@ -566,60 +640,6 @@ __global__ void __launch_bounds__(256) k_m2l(const T* __restrict__ K, int l, con
             const int b = w + 8 * j;
             if (b < NC) L[(size_t)t * NCP + b] = (double)acc[j] * inv_h;
         }
-    }
-}
-
-// The steps that restore the coefficients of z exponent >= 2 of a harmonic expansion from its free
-// ones by Laplace's equation (internal.h): V[i] = w1 V[i1] + w2 V[i2], those of z exponent c at
-// [cst[c], cst[c + 1]).
-struct HarmTab {
-    static constexpr int N = NC - nharm_of(P) > 0 ? NC - nharm_of(P) : 1;
-    int cst[P + 3];
-    unsigned short i[N], i1[N], i2[N];
-    float w1[N], w2[N], w1l[N], w2l[N];  // FP32, and its remainder (float-float)
-    double d1[N], d2[N];
-};
-constexpr HarmTab make_harm_tab() {
-    HarmTab t{};
-    int k = 0;
-    for (int c = 2; c <= P; ++c) {
-        t.cst[c] = k;
-        for (int n = c; n <= P; ++n)
-            for (int b = 0; b <= n - c; ++b, ++k) {
-                const int a = n - c - b;
-                t.i[k] = (unsigned short)da_index(a, b, c);
-                t.i1[k] = (unsigned short)da_index(a + 2, b, c - 2);
-                t.i2[k] = (unsigned short)da_index(a, b + 2, c - 2);
-                t.d1[k] = -(double)((a + 2) * (a + 1)) / (double)(c * (c - 1));
-                t.d2[k] = -(double)((b + 2) * (b + 1)) / (double)(c * (c - 1));
-                t.w1[k] = (float)t.d1[k];
-                t.w2[k] = (float)t.d2[k];
-                t.w1l[k] = (float)(t.d1[k] - (double)t.w1[k]);
-                t.w2l[k] = (float)(t.d2[k] - (double)t.w2[k]);
-            }
-    }
-    for (int c = P < 1 ? 2 : P + 1; c < P + 3; ++c) t.cst[c] = k;
-    return t;
-}
-__device__ const HarmTab harm_tab = make_harm_tab();
-
-__device__ __forceinline__ float harm_step(const float* V, int s) {
-    return fmaf(harm_tab.w1[s], V[harm_tab.i1[s]], harm_tab.w2[s] * V[harm_tab.i2[s]]);
-}
-__device__ __forceinline__ double harm_step(const double* V, int s) {
-    return fma(harm_tab.d1[s], V[harm_tab.i1[s]], harm_tab.d2[s] * V[harm_tab.i2[s]]);
-}
-__device__ __forceinline__ ff harm_step(const ff* V, int s) {
-    return ff_add(ff_mul(ff(harm_tab.w1[s], harm_tab.w1l[s]), V[harm_tab.i1[s]]),
-                  ff_mul(ff(harm_tab.w2[s], harm_tab.w2l[s]), V[harm_tab.i2[s]]));
-}
-// the warp restores V's coefficients of z exponent >= 2, exponent by exponent
-template <class R>
-__device__ __forceinline__ void harm_expand_warp(R* V, int lane) {
-#pragma unroll 1
-    for (int c = 2; c <= P; ++c) {
-        for (int s = harm_tab.cst[c] + lane; s < harm_tab.cst[c + 1]; s += 32) V[harm_tab.i[s]] = harm_step(V, s);
-        __syncwarp();
     }
 }
 
@@ -1697,6 +1717,10 @@ __global__ void k_p2m_a(AdaptiveView av, const int* __restrict__ leaves, int nle
         if constexpr (H) gen::GEN(p2mh)<T>(x, y, z, q, sink);
         else gen::GEN(p2m)<T>(x, y, z, q, sink);
     }
+    if constexpr (H && sizeof(T) == 8) {
+        p2m_row(acc, sm, M + (size_t)b * NCP, lane);
+        return;
+    }
 #pragma unroll
     for (int j = 0; j < NJ; ++j) {
         const int k = lane + 32 * j;
@@ -2206,11 +2230,11 @@ static cudaError_t p2m_launch(const TreeView& tv, int prec, double* M, const F16
     dim3 blk(32, wpb), grd((tv.nleaf + wpb - 1) / wpb);
     cudaError_t e;
     if (f64) {
-        if ((e = set_smem(k_p2m<double>, smem)) != cudaSuccess) return e;
-        k_p2m<double><<<grd, blk, smem, s>>>(tv, M, 0, F16Rows{});
+        if ((e = set_smem(k_p2m<double, true>, smem)) != cudaSuccess) return e;
+        k_p2m<double, true><<<grd, blk, smem, s>>>(tv, M, 0, F16Rows{});
     } else if (fff) {
-        if ((e = set_smem(k_p2m<ff>, smem)) != cudaSuccess) return e;
-        k_p2m<ff><<<grd, blk, smem, s>>>(tv, M, 0, F16Rows{});
+        if ((e = set_smem(k_p2m<ff, true>, smem)) != cudaSuccess) return e;
+        k_p2m<ff, true><<<grd, blk, smem, s>>>(tv, M, 0, F16Rows{});
     } else if (harm) {
         if ((e = set_smem(k_p2m<float, true>, smem)) != cudaSuccess) return e;
         k_p2m<float, true><<<grd, blk, smem, s>>>(tv, M, rows32, fr);
@@ -2419,8 +2443,8 @@ static cudaError_t p2m_a_launch(const AdaptiveView& av, const int* leaves, int n
     dim3 blk(32, wpb), grd((nleaves + wpb - 1) / wpb);
     cudaError_t e;
     if (f64) {
-        if ((e = set_smem(k_p2m_a<double>, smem)) != cudaSuccess) return e;
-        k_p2m_a<double><<<grd, blk, smem, s>>>(av, leaves, nleaves, M);
+        if ((e = set_smem(k_p2m_a<double, true>, smem)) != cudaSuccess) return e;
+        k_p2m_a<double, true><<<grd, blk, smem, s>>>(av, leaves, nleaves, M);
     } else if (harm) {
         if ((e = set_smem(k_p2m_a<float, true>, smem)) != cudaSuccess) return e;
         k_p2m_a<float, true><<<grd, blk, smem, s>>>(av, leaves, nleaves, M);
