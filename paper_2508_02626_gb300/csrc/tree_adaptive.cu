@@ -115,11 +115,11 @@ __global__ void __launch_bounds__(256) k_bbox_roots(const double* __restrict__ x
     // a problem of 1e6 particles beside small ones, many blocks 20 us
     const int r = blockIdx.x;
     const int b = offs[r], e = offs[r + 1];
-    if (b + (int)(blockIdx.y * blockDim.x) >= e) return;
+    if (b + (int64_t)blockIdx.y * blockDim.x >= e) return;
     unsigned long long mn[3] = {~0ull, ~0ull, ~0ull}, mx[3] = {0ull, 0ull, 0ull};
-    for (int i = b + blockIdx.y * blockDim.x + threadIdx.x; i < e; i += gridDim.y * blockDim.x)
+    for (int64_t i = b + (int64_t)blockIdx.y * blockDim.x + threadIdx.x; i < e; i += gridDim.y * blockDim.x)
         for (int d = 0; d < 3; ++d) {
-            const unsigned long long u = ordered_bits(xyz[3 * (size_t)i + d]);
+            const unsigned long long u = ordered_bits(xyz[3 * i + d]);
             mn[d] = u < mn[d] ? u : mn[d];
             mx[d] = u > mx[d] ? u : mx[d];
         }
@@ -146,7 +146,7 @@ cudaError_t launch_bbox_roots(const double* xyz, const int* offs, int nroots, in
                               cudaStream_t s) {
     if (nroots == 0) return cudaSuccess;
     k_bbox_init<<<(6 * nroots + 255) / 256, 256, 0, s>>>(bb, nroots);
-    const int per = (max_n + 2047) / 2048;  // blocks of the largest problem: 8 particles per thread
+    const int per = (int)((max_n + (int64_t)2047) / 2048);  // blocks of the largest problem: 8 particles per thread
     k_bbox_roots<<<dim3(nroots, per < 1 ? 1 : (per > 608 ? 608 : per)), 256, 0, s>>>(xyz, offs, bb);
     return cudaGetLastError();
 }
@@ -351,10 +351,12 @@ __device__ inline bool touch(const AdaptiveBuild& ab, int a, int b) {
 
 // Colleague k of box b, at relative position (dx, dy, dz): one thread each.  Its parent is the
 // colleague of b's parent at offset floor((i_b + d) / 2) - floor(i_b / 2), its octant the parity.
-// (One thread per box tested all children of the parent's colleagues.)
+// (One thread per box tested all children of the parent's colleagues.)  A block takes whole boxes:
+// 27 times the boxes of a level may not fit an int.
+constexpr int kColleagueBoxes = 9;
+
 __global__ void k_colleagues(AdaptiveBuild ab, int lb, int le) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int b = lb + i / 27, k = i % 27;
+    const int b = lb + blockIdx.x * kColleagueBoxes + threadIdx.x / 27, k = threadIdx.x % 27;
     if (b >= le) return;
     int c = k == 13 ? b : -1;
     const int P = ab.parent[b];
@@ -369,7 +371,7 @@ __global__ void k_colleagues(AdaptiveBuild ab, int lb, int le) {
 
 cudaError_t launch_colleagues(AdaptiveBuild ab, int lb, int le, cudaStream_t s) {
     if (le <= lb) return cudaSuccess;
-    k_colleagues<<<(unsigned)(((size_t)(le - lb) * 27 + 255) / 256), 256, 0, s>>>(ab, lb, le);
+    k_colleagues<<<(le - lb + kColleagueBoxes - 1) / kColleagueBoxes, 27 * kColleagueBoxes, 0, s>>>(ab, lb, le);
     return cudaGetLastError();
 }
 
@@ -486,9 +488,11 @@ __device__ int v_count(const AdaptiveBuild& ab, int b, int lane) {
     return __reduce_add_sync(0xffffffffu, cv);
 }
 
+constexpr int kListBoxes = 4;  // boxes (warps) per block
+
 __global__ void k_list_count(AdaptiveBuild ab, int nbox, int* cu, int* cw, int* cx, unsigned long long* nv,
                              int* err) {
-    const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    const int b = blockIdx.x * kListBoxes + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     __shared__ unsigned long long sv;
     if (threadIdx.x == 0) sv = 0;
     __syncthreads();
@@ -509,7 +513,7 @@ __global__ void k_list_count(AdaptiveBuild ab, int nbox, int* cu, int* cw, int* 
 
 __global__ void k_list_fill(AdaptiveBuild ab, int nbox, const int* pu, const int* pw, const int* px, int* iu, int* iw,
                             int* ix, int* err) {
-    const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    const int b = blockIdx.x * kListBoxes + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (b >= nbox) return;
     int nu, nw, nx;
     box_lists<true>(ab, b, lane, nu, nw, nx, iu + pu[b], iw + pw[b], ix + px[b], err, pu[b + 1] - pu[b],
@@ -519,14 +523,14 @@ __global__ void k_list_fill(AdaptiveBuild ab, int nbox, const int* pu, const int
 cudaError_t launch_list_count(AdaptiveBuild ab, int nbox, int* cu, int* cw, int* cx, unsigned long long* nv, int* err,
                               cudaStream_t s) {
     if (nbox == 0) return cudaSuccess;
-    k_list_count<<<(unsigned)(((size_t)nbox * 32 + 127) / 128), 128, 0, s>>>(ab, nbox, cu, cw, cx, nv, err);
+    k_list_count<<<(nbox + kListBoxes - 1) / kListBoxes, 32 * kListBoxes, 0, s>>>(ab, nbox, cu, cw, cx, nv, err);
     return cudaGetLastError();
 }
 
 cudaError_t launch_list_fill(AdaptiveBuild ab, int nbox, const int* pu, const int* pw, const int* px, int* iu, int* iw,
                              int* ix, int* err, cudaStream_t s) {
     if (nbox == 0) return cudaSuccess;
-    k_list_fill<<<(unsigned)(((size_t)nbox * 32 + 127) / 128), 128, 0, s>>>(ab, nbox, pu, pw, px, iu, iw, ix, err);
+    k_list_fill<<<(nbox + kListBoxes - 1) / kListBoxes, 32 * kListBoxes, 0, s>>>(ab, nbox, pu, pw, px, iu, iw, ix, err);
     return cudaGetLastError();
 }
 
