@@ -21,11 +21,11 @@ namespace tc {
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32_t src_bytes) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+// the barrier counts this thread as arrived once all its copies so far have landed
+__device__ __forceinline__ void cp_async_arrive(uint32_t bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
 }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 struct GItem {
@@ -121,12 +121,11 @@ __global__ void __launch_bounds__(kTcgThreads, 1) k_tcg(const __grid_constant__ 
             prefetch_map(&prm.b_hi);
             prefetch_map(&prm.b_lo);
         }
+        // place of this lane's first row: row 64 pw + 4 k + lane / 8 of the tile, chunk lane % 8
+        // swizzled by row % 8 (for k odd row % 8 is 4 more: 512 bytes on and bit 6 the other way)
+        const uint32_t row0 = (uint32_t)(pw * 8192 + (lane >> 3) * 128 + (((lane & 7) ^ (lane >> 3)) << 4));
         int stage = 0;
         uint32_t phase = 0;
-        // the stage whose copies are committed but not yet signalled: it is signalled once the
-        // next stage's copies are issued (holding more stages back starves the MMAs while this
-        // warp issues)
-        int pend = -1;
         int armed[C::STAGES];
         for (int s = 0; s < C::STAGES; ++s) armed[s] = -1;
         bool ok = true;
@@ -168,16 +167,26 @@ __global__ void __launch_bounds__(kTcgThreads, 1) k_tcg(const __grid_constant__ 
 #pragma unroll
                 for (int i = 0; i < 2; ++i) qnn[i] = hnn ? colleague_of(prm, par[i], slot) : -1;
                 const int key = term_key(tm);
-                // Eight lanes per row, so that a copy instruction reads four whole 128-byte lines;
-                // the sources of a lane's 16 rows are fetched once per term, as the issue of the
-                // copies is what these two warps spend their time on.  With a row per lane an
-                // instruction touched 32 lines.  Clustered, 1e6 particles, 64 per leaf: F16 p = 4
-                // 689 -> 603 us, p = 8 1579 -> 1159, p = 10 1826 -> 1309; TF32 p = 4 903 -> 567,
-                // p = 8 2435 -> 1675, p = 10 3362 -> 2286.
-                int srow[16];
+                // Eight lanes per row, so that a copy instruction reads four whole 128-byte lines, and
+                // the addresses of a lane's 16 rows made once per term: the issue of the copies is
+                // much of what these two warps do (a row per lane touched 32 lines per
+                // instruction).  The copies signal their stage themselves, so that every stage of
+                // the ring may be in flight.  Clustered, 1e6 particles, 64 per leaf: F16 p = 4
+                // 689 -> 583 us, p = 8 1579 -> 1085, p = 10 1826 -> 1177; TF32 p = 4 903 -> 550,
+                // p = 8 2435 -> 1479, p = 10 3362 -> 2025.  What is left at low orders is a term's
+                // own chain (the source lookups, the handover of the accumulator).
+                const char* ph[16];
+                const char* pl[16];
+                uint32_t sz[16];
 #pragma unroll
-                for (int k = 0; k < 16; ++k)
-                    srow[k] = __shfl_sync(0xffffffffu, src[k >> 3], (4 * k + (lane >> 3)) & 31);
+                for (int k = 0; k < 16; ++k) {
+                    const int sr = __shfl_sync(0xffffffffu, src[k >> 3], (4 * k + (lane >> 3)) & 31);
+                    const size_t e = (sr >= 0 ? (size_t)sr * C::ROWLEN * ESZ : 0) + 16 * (lane & 7);
+                    ph[k] = static_cast<const char*>(prm.a_hi) + e;
+                    pl[k] = static_cast<const char*>(prm.a_lo) + e;
+                    sz[k] = sr >= 0 ? 16u : 0u;
+                }
+#pragma unroll
                 for (int kc = 0; kc < C::NKC; ++kc) {
                     int got = 1;
                     if (lane == 0) got = mbar_wait(smem_u32(&empty[stage]), phase ^ 1u, prm.err, 41) ? 1 : 0;
@@ -196,25 +205,17 @@ __global__ void __launch_bounds__(kTcgThreads, 1) k_tcg(const __grid_constant__ 
                                     it.half * C::NP, key);
                     }
                     const uint32_t sa = smem_u32(st);
-                    const char* ahi = static_cast<const char*>(prm.a_hi);
-                    const char* alo = static_cast<const char*>(prm.a_lo);
+                    const uint32_t d0 = sa + row0, d1 = (sa + row0 + 512) ^ 64;  // rows of k even, odd
+                    // the MMAs of a last, partial chunk read no further than the row's end
+                    if (kc * C::KPC + (lane & 7) * (16 / ESZ) < C::ROWLEN) {
 #pragma unroll
-                    for (int k = 0; k < 16; ++k) {
-                        const int r = 64 * pw + 4 * k + (lane >> 3), j = lane & 7;
-                        const int col = kc * C::KPC + j * (16 / ESZ);  // first element of the 16-byte chunk
-                        const bool hv = srow[k] >= 0 && col < C::ROWLEN;
-                        const size_t e = hv ? ((size_t)srow[k] * C::ROWLEN + col) * ESZ : 0;
-                        const uint32_t off = (uint32_t)((r >> 3) * 1024 + (r & 7) * 128 + ((j ^ (r & 7)) << 4));
-                        cp_async16(sa + off, ahi + e, hv ? 16u : 0u);
-                        cp_async16(sa + C::A_BYTES + off, alo + e, hv ? 16u : 0u);
+                        for (int k = 0; k < 16; ++k) {
+                            const uint32_t d = ((k & 1) ? d1 : d0) + (uint32_t)((k >> 1) * 1024);
+                            cp_async16(d, ph[k] + kc * 128, sz[k]);
+                            cp_async16(d + C::A_BYTES, pl[k] + kc * 128, sz[k]);
+                        }
                     }
-                    cp_async_commit();
-                    if (pend >= 0) {
-                        cp_async_wait<1>();
-                        fence_proxy_async_smem();
-                        mbar_arrive(smem_u32(&full[pend]));
-                    }
-                    pend = stage;
+                    cp_async_arrive(smem_u32(&full[stage]));
                     if (++stage == C::STAGES) {
                         stage = 0;
                         phase ^= 1u;
@@ -231,11 +232,7 @@ __global__ void __launch_bounds__(kTcgThreads, 1) k_tcg(const __grid_constant__ 
                 }
             }
         }
-        if (pend >= 0) {
-            cp_async_wait<0>();
-            fence_proxy_async_smem();
-            mbar_arrive(smem_u32(&full[pend]));
-        }
+        cp_async_wait_all();
         // every copy this warp armed must have landed before the block may exit
         if (warp == 0 && lane == 0)
             for (int s = 0; s < C::STAGES; ++s)
@@ -264,6 +261,7 @@ __global__ void __launch_bounds__(kTcgThreads, 1) k_tcg(const __grid_constant__ 
                 for (int kc = 0; kc < C::NKC && ok; ++kc) {
                     ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&full[stage]), phase, prm.err, 44));
                     if (!ok) break;
+                    fence_proxy_async_smem();  // the gathered rows (generic proxy) before the MMAs' reads
                     fence_after_sync();
                     const uint32_t st = smem_u32(base + stage * C::STAGE_BYTES);
                     const uint32_t ah = smem_desc_lo(st), al = smem_desc_lo(st + C::A_BYTES);
