@@ -201,8 +201,9 @@ int dafmm_last_phase_ms(dafmm_ctx* ctx, double* out10);
  *   faster one); the others run on the SIMT kernels. */
 #define DAFMM_OPT_TC_MASK 2
 /*   DAFMM_OPT_LEAF_WARPS: leaves per thread block of the adaptive near-field kernel (P2P,
- *   M2P, L2P), one warp each: 1, 2, 4 (default) or 8 -- the P2P tile the autotuner picks (FP32
- *   and MIXED; in FP64 several warps share a leaf whatever this says). */
+ *   M2P, L2P), one warp each: 1 (default), 2, 4 or 8 -- the P2P tile the autotuner picks (FP32
+ *   and MIXED; in FP64 several warps share a leaf whatever this says).  The results do not
+ *   depend on it. */
 #define DAFMM_OPT_LEAF_WARPS 3
 /*   DAFMM_OPT_M2L_F16: operands of the FP32 mode's tensor-core M2L: 1 (default) = F16 hi/lo
  *   splits with power-of-two scales per box, per matrix row and per matrix (twice the TF32

@@ -1178,7 +1178,7 @@ __device__ __forceinline__ void near_add(float2 ex, float2 ey, float2 ez, float2
 // FMA pipe 48 %); two targets halve the loads per interaction.  With the conflict-free staging:
 // uniform N = 1e6, p = 8: the kernel 0.80 -> 0.63 ms (5 or 6 blocks per SM; 4: 0.68); clustered
 // N = 4e6, p = 10: 10.5 -> 8.1 ms; 64-problem forest, p = 6: 2.74 -> 2.06 ms.  (The adaptive kernel
-// compiled for 24 warps per SM instead of 16: 7.4 and 2.04 ms.)
+// compiled for 24 warps per SM instead of 16: 7.4 and 2.04 ms, with one leaf per block 6.7 and 1.88.)
 template <bool GUARD>
 __device__ __forceinline__ void near_pairs(const float4* buf, int p0, int p1, const NearTarget (&t)[2],
                                            NearSums (&s)[2]) {
@@ -1916,6 +1916,12 @@ constexpr size_t kLeafWarpSmem = kNearSmem * sizeof(float4) + NCP * sizeof(float
 static_assert(2 * NCP * sizeof(float) <= 4 * kSegPairs * sizeof(float4), "two rows fit the segment");
 
 // leaves: P2P over the U list, M2P over the W list, L2P of the leaf's local expansion (FP32)
+// One warp per leaf, and one leaf per block unless the context says otherwise: the leaves' lists differ
+// in length, and a block holds its place on the SM until its longest leaf is done (with four leaves
+// 4.0 of the 6 warps per scheduler were there on average).  Four leaves per block against one:
+// clustered N = 4e6, p = 10: 7.46 -> 6.72 ms; 64-problem forest, p = 6: 2.02 -> 1.88 ms; Gaussian
+// N = 1e6, p = 4: 1.52 -> 1.49 ms.  Compiled for 16 or 32 warps per SM instead of 24: 7.88 and 6.73,
+// 2.16 and 2.02, 1.64 and 1.59 ms.
 __global__ void __launch_bounds__(256, 3) k_leaf_a(AdaptiveView av, const int* __restrict__ leaves, int nleaves,
                                                    const double* __restrict__ L, const double* __restrict__ M,
                                                    const float* __restrict__ Mf, double* __restrict__ phi,
