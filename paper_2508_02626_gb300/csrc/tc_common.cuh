@@ -320,7 +320,6 @@ struct CfgM2L {
 // tile origin in slab coordinates, output half
 struct WorkItem {
     int li, oct, c, px0, py0, pz0, half;
-    int part;  // harmonic M2L: this item's share of the tile's steps
 };
 
 // the terms of a work item, in a fixed order.  M2L: the displacements v_d in

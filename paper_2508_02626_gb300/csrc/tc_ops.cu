@@ -39,7 +39,6 @@ __device__ __forceinline__ WorkItem decode(const TCParams& prm, int w) {
     it.li = li;
     it.half = local % prm.nhalf;
     local /= prm.nhalf;
-    it.part = 0;
     it.oct = 0;
     it.c = 0;
     if (prm.mode == kTcM2L || prm.mode == kTcL2L) {
