@@ -517,8 +517,8 @@ def run_ours(args, rank, world):
         executed = tiles * 189 * 3 * 2.0 * 128 * npt * klen / m2l_s / 1e12
     roofline = {"bound": bound, "achieved": round(achieved, 3), "peak": round(peak, 3), "unit": "TFLOP/s",
                 "frac": round(achieved / peak, 4), "traffic": m2l_traffic(args.precision), "traffic_unit": "bytes per launch",
-                "kernel": ("M2L contraction (tcgen05 kind::f16 k_tc, all levels, one launch)" if f16 else
-                           "M2L contraction (tcgen05 kind::tf32 k_tc, all levels, one launch)") if bound == "tensor"
+                "kernel": ("M2L contraction (tcgen05 kind::f16 k_tc_m2l, all levels, one launch)" if f16 else
+                           "M2L contraction (tcgen05 kind::tf32 k_tc_m2l, all levels, one launch)") if bound == "tensor"
                 else ("M2L by rotation (k_m2l_rot, FP64 pipe, all levels)" if rot else
                       "M2L (SIMT FP64 k_m2l, all levels)"),
                 "algorithmic": ("2 x %d multiply-adds per well-separated pair (4 rotations + axial Eq. 5, "
