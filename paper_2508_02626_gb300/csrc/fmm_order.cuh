@@ -1812,7 +1812,7 @@ __global__ void __launch_bounds__(256) k_m2l_a(const T* __restrict__ K, Adaptive
 // 1/64 of the FP32 rate, and bound the kernel).
 // Measured against the full-basis form before (one launch per level, a leaf at a time, FP64
 // differences): 64-problem forest, p = 6 (FP32): 0.913 -> 0.296 ms; Gaussian N = 1e6, p = 4 (FP32):
-// 0.444 -> 0.159 ms; Gaussian N = 1e5, s = 256, p = 8 (FP64): 9.89 -> 2.91 ms.
+// 0.444 -> 0.159 ms; Gaussian N = 1e5, s = 256, p = 8 (FP64): 9.89 -> 2.44 ms.
 template <class T>
 __global__ void __launch_bounds__(128) k_p2l_a(AdaptiveView av, int lb, int le, double* __restrict__ L) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -2498,8 +2498,10 @@ static cudaError_t p2l_a_launch(const AdaptiveView& av, int prec, int lb, int le
     if (le <= lb) return cudaSuccess;
     const bool f64 = prec == DAFMM_FP64;
     const size_t per_warp = (size_t)32 * 33 * (f64 ? 8 : 4);
-    int wpb = (int)((96 * 1024) / per_warp);
-    wpb = wpb < 1 ? 1 : (wpb > 4 ? 4 : wpb);
+    // FP64: a box per block, as the X lists differ and a block stays until its longest is done
+    // (Gaussian N = 1e5, s = 256, p = 8: 2.90 ms with four warps, 2.68 with two, 2.44 with one); FP32
+    // does not care (clustered N = 4e6, p = 10: 2.44, 2.43 and 2.44 ms) and keeps the fewer blocks
+    const int wpb = f64 ? 1 : 4;
     const size_t smem = per_warp * wpb;
     dim3 blk(32, wpb), grd((le - lb + wpb - 1) / wpb);
     cudaError_t e;
