@@ -1283,7 +1283,9 @@ __device__ __forceinline__ CompSums near_join(float4* buf, int W, int tl) {
             }
         }
     }
-    if constexpr (NW > 1) __syncthreads();  // before the next pass starts from zero
+    // the other lanes' (and warps') sums are read: the next pass may start from zero (near_zero)
+    if constexpr (NW > 1) __syncthreads();
+    else __syncwarp();
     CompSums r;
     r.ph = k[0]; r.pl = k[1]; r.xh = k[2]; r.xl = k[3]; r.yh = k[4]; r.yl = k[5]; r.zh = k[6]; r.zl = k[7];
     return r;
