@@ -17,6 +17,7 @@
 
 #include "check.cuh"
 #include "internal.h"
+#include "launch_rules.h"
 #include "tree_adaptive.h"
 #include "tree_common.cuh"
 
@@ -146,8 +147,7 @@ cudaError_t launch_bbox_roots(const double* xyz, const int* offs, int nroots, in
                               cudaStream_t s) {
     if (nroots == 0) return cudaSuccess;
     k_bbox_init<<<(6 * nroots + 255) / 256, 256, 0, s>>>(bb, nroots);
-    const int per = (int)((max_n + (int64_t)2047) / 2048);  // blocks of the largest problem: 8 particles per thread
-    k_bbox_roots<<<dim3(nroots, per < 1 ? 1 : (per > 608 ? 608 : per)), 256, 0, s>>>(xyz, offs, bb);
+    k_bbox_roots<<<dim3(nroots, bbox_blocks(nroots, max_n)), 256, 0, s>>>(xyz, offs, bb);
     return cudaGetLastError();
 }
 

@@ -1,0 +1,4 @@
+// C entries to the launch rules, for tests/test_launch_rules.py
+#include "launch_rules.h"
+
+extern "C" int bbox_blocks(long long nroots, long long max_n) { return dafmm::bbox_blocks(nroots, max_n); }
