@@ -27,6 +27,7 @@
 #include "check.cuh"
 #include "ff.cuh"
 #include "internal.h"
+#include "launch_rules.h"
 #include "tree_adaptive.h"
 #include "tree_common.cuh"
 
@@ -1924,6 +1925,7 @@ static_assert(2 * NCP * sizeof(float) <= 4 * kSegPairs * sizeof(float4), "two ro
 // clustered N = 4e6, p = 10: 7.46 -> 6.72 ms; 64-problem forest, p = 6: 2.02 -> 1.88 ms; Gaussian
 // N = 1e6, p = 4: 1.52 -> 1.49 ms.  Compiled for 16 or 32 warps per SM instead of 24: 7.88 and 6.73,
 // 2.16 and 2.02, 1.64 and 1.59 ms.
+// Block (.., y) takes every gridDim.y-th pass of its leaves from the y-th on (leaf_a_split).
 __global__ void __launch_bounds__(256, 3) k_leaf_a(AdaptiveView av, const int* __restrict__ leaves, int nleaves,
                                                    const double* __restrict__ L, const double* __restrict__ M,
                                                    const float* __restrict__ Mf, double* __restrict__ phi,
@@ -1936,20 +1938,22 @@ __global__ void __launch_bounds__(256, 3) k_leaf_a(AdaptiveView av, const int* _
     float* lrow = reinterpret_cast<float*>(buf + kNearSmem);
     const int b = leaves[li];
     if (!DAFMM_IN(b, av.nbox, kChkBoxIndex)) return;
+    int i0 = av.pbeg[b], i1 = av.pend[b];
+    if (!DAFMM_RANGE(i0, i1, av.n, kChkBoxRange)) i0 = i1 = 0;
+    // the leaf's own records (its targets)
+    if (!DAFMM_RANGE(av.xq0[b], (long long)av.xq0[b] + (i1 - i0), av.nrec, kChkRecord)) i0 = i1 = 0;
+    const int base0 = i0 + 32 * (int)blockIdx.y;
+    if (base0 >= i1) return;
     double cx, cy, cz, h;
     abox_geom(av, b, cx, cy, cz, h);
     const double ih = 1.0 / h;
     const int lev = av.level[b];
     if (lev >= 2) warp_row_to_f32(L + (size_t)b * NCP, lrow, lane);
-    int i0 = av.pbeg[b], i1 = av.pend[b];
-    if (!DAFMM_RANGE(i0, i1, av.n, kChkBoxRange)) i0 = i1 = 0;
-    // the leaf's own records (its targets)
-    if (!DAFMM_RANGE(av.xq0[b], (long long)av.xq0[b] + (i1 - i0), av.nrec, kChkRecord)) i0 = i1 = 0;
     int u0 = av.u_ptr[b], u1 = av.u_ptr[b + 1];
     int w0 = av.w_ptr[b], w1 = av.w_ptr[b + 1];
     if (!DAFMM_RANGE(u0, u1, av.nu, kChkListPtr)) u0 = u1 = 0;
     if (!DAFMM_RANGE(w0, w1, av.nw, kChkListPtr)) w0 = w1 = 0;
-    for (int base = i0; base < i1; base += 32) {
+    for (int base = base0; base < i1; base += 32 * gridDim.y) {
         const int m = min(32, i1 - base);
         const int W = near_width(m), per = 2 * W;  // the lanes' split, see near_width
         const int tl = lane & (per - 1);
@@ -2529,7 +2533,7 @@ static cudaError_t leaf_a_launch(const AdaptiveView& av, const int* leaves, int 
                                  int max_leaf, cudaStream_t s) {
     if (nleaves == 0) return cudaSuccess;
     warps = warps < 1 ? 1 : (warps > 8 ? 8 : warps);
-    dim3 blk(32, warps), grd((nleaves + warps - 1) / warps);
+    dim3 blk(32, warps), grd((nleaves + warps - 1) / warps, leaf_a_split(nleaves, max_leaf));
     if (prec == DAFMM_FP64) {
         // blocks per leaf: one per pass of the largest leaf, up to 8
         const int ny = max_leaf < 32 ? 1 : (max_leaf > 8 * 32 ? 8 : (max_leaf + 31) / 32);

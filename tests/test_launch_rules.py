@@ -18,6 +18,7 @@ def lib():
                            "-o", so, os.path.join(ROOT, "tests", "launch_rules_check.cpp")])
     h = ctypes.CDLL(so)
     h.bbox_blocks.argtypes = [ctypes.c_longlong, ctypes.c_longlong]
+    h.leaf_a_split.argtypes = [ctypes.c_longlong, ctypes.c_int]
     return h
 
 
@@ -31,3 +32,18 @@ def test_bounding_boxes(lib, nroots, max_n):
     assert b == 1 or 0.5 * nroots * (b - 1) <= 2.2 * max_n
     if nroots == 1 and max_n:
         assert b == min(608, (max_n + 2047) // 2048)
+
+
+@pytest.mark.parametrize("nleaves", [1, 15, 200, 456, 457, 3648, 3649, 100_000])
+@pytest.mark.parametrize("max_leaf", [0, 1, 32, 33, 200, 1000, 1 << 30])
+def test_adaptive_leaves(lib, nleaves, max_leaf):
+    """Several blocks per leaf only where every one of them has a pass and a place on the GPU, and
+    then for every leaf too large for one: a lone warp on it was up to 1.44 times slower."""
+    s = lib.leaf_a_split(nleaves, max_leaf)
+    passes = -(-max_leaf // 32)
+    assert 1 <= s <= max(1, min(8, passes))
+    assert s == 1 or nleaves * s <= 24 * 152
+    if max_leaf > 32 and nleaves <= 24 * 152 // 2:
+        assert s >= 2
+    if nleaves == 1:
+        assert s == max(1, min(8, passes))
