@@ -16,8 +16,9 @@
 //                 k_m2l       L~_t = (1/h) sum_v K^_v M~_{t-v} over the 189 displacements of
 //                             the target's octant (SIMT, FP64 or FP32)
 //   L2L  (Eq. 7)  k_l2l       32 parents and 16 rows per block, 8 child tables by sign flips
-//   L2P + P2P     k_leaf      one warp per target leaf: pairwise sum over the 27 neighbour
-//                             leaves and the generated L2P of the leaf's local expansion
+//   L2P + P2P     k_leaf      one block per target leaf (8 warps in trees of few leaves, else one):
+//                 k_leaf64    pairwise sum over the 27 neighbour leaves and the generated L2P of the
+//                             leaf's local expansion
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -1355,8 +1356,8 @@ __device__ __forceinline__ ff ff_shfl_down(ff v, int d) {
 // leaves per block at 20 warps per SM, 0.61 with one, 0.60 with the sums in shared memory at 28
 // warps.  (More warps or independent pairs in flight do not help further, nor do scalar field
 // sums, although a packed FMA of three distinct registers takes 3.9 cycles in a loop of its own
-// and two scalar ones 2.3: 0.61-0.62 ms.)  A tree of few leaves gives each NW warps, which share
-// out the segments of its source list (leaf_launch): 64 leaves, N = 3001, p = 4: 91 -> 24 us.
+// and two scalar ones 2.3: 0.61-0.62 ms.)  A tree of few leaves gives each 8 warps, which share
+// out the segments of its source list (leaf_warps): 64 leaves, N = 3001, p = 4: 91 -> 24 us.
 constexpr int kLeafMinWarps = 28;
 
 // ---- FP64 near field ----
@@ -1602,8 +1603,7 @@ __global__ void __launch_bounds__(32 * NW, (std::is_same<T, float>::value ? kLea
 }
 
 // The same in FP64: a block of NW warps per leaf, the warps sharing out the sources of each pass.
-// NW grows as the leaves get fewer (leaf_launch), so that a tree of 64 or 512 leaves still gives
-// every SM its share.  Measured against one warp per leaf with passes of 32 and CUDA's rsqrt:
+// NW is 8 or 1 (leaf_warps), so that a tree of 64 or 512 leaves still gives every SM its share.  Measured against one warp per leaf with passes of 32 and CUDA's rsqrt:
 // uniform N = 200,003, depth 4, p = 8: 13.1 -> 9.6 ms; N = 1e4, depth 3, p = 6: the evaluation 2.57
 // -> 2.20 ms (this kernel 0.28).
 template <int NW>
@@ -2343,17 +2343,12 @@ static cudaError_t leaf_run(const TreeView& tv, const double* Lleaf, double* phi
 static cudaError_t leaf_launch(const TreeView& tv, int prec, const double* Lleaf, double* phi, double* field,
                                cudaStream_t s) {
     if (tv.nleaf == 0) return cudaSuccess;
-    if (prec == DAFMM_FP64) {
-        // about 16 warps per SM or more from 2432 leaves on; below, more warps per leaf
-        if (tv.nleaf >= 2432) k_leaf64<1><<<tv.nleaf, dim3(32, 1), 0, s>>>(tv, Lleaf, phi, field);
-        else if (tv.nleaf >= 1216) k_leaf64<2><<<tv.nleaf, dim3(32, 2), 0, s>>>(tv, Lleaf, phi, field);
-        else k_leaf64<8><<<tv.nleaf, dim3(32, 8), 0, s>>>(tv, Lleaf, phi, field);
-    } else if (prec == DAFMM_FF) {
-        return leaf_run<ff, 1>(tv, Lleaf, phi, field, s);
-    } else {  // one wave of warps needs 4256 leaves
-        if (tv.nleaf >= 2432) return leaf_run<float, 1>(tv, Lleaf, phi, field, s);
-        return tv.nleaf >= 608 ? leaf_run<float, 4>(tv, Lleaf, phi, field, s) : leaf_run<float, 8>(tv, Lleaf, phi, field, s);
-    }
+    if (prec == DAFMM_FF) return leaf_run<ff, 1>(tv, Lleaf, phi, field, s);
+    const bool f64 = prec == DAFMM_FP64;
+    const bool shared = leaf_warps(tv.nleaf) > 1;
+    if (!f64) return shared ? leaf_run<float, kLeafWarps>(tv, Lleaf, phi, field, s) : leaf_run<float, 1>(tv, Lleaf, phi, field, s);
+    if (shared) k_leaf64<kLeafWarps><<<tv.nleaf, dim3(32, kLeafWarps), 0, s>>>(tv, Lleaf, phi, field);
+    else k_leaf64<1><<<tv.nleaf, dim3(32, 1), 0, s>>>(tv, Lleaf, phi, field);
     return cudaGetLastError();
 }
 

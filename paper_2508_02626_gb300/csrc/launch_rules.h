@@ -23,6 +23,12 @@ inline int bbox_blocks(int64_t nroots, int64_t max_n) {
     return (int)std::max<int64_t>(1, std::min<int64_t>({fill, room, 4 * kSMs}));
 }
 
+// Near field of a uniform tree (FP32 and FP64): warps that share a leaf's sources.  Such a tree has 8^depth
+// leaves: from 4096 on, one warp each gives an SM the 24 or 28 warps that it holds; 512 leaves and
+// fewer do not fill the GPU, and take 8.
+constexpr int kLeafWarps = 8;
+inline int leaf_warps(int64_t nleaf) { return nleaf >= 16 * kSMs ? 1 : kLeafWarps; }
+
 // FP32 near field of an adaptive tree: blocks that share the passes (32 targets each) of a leaf, one
 // while the leaves alone fill the 24 warps that an SM holds, otherwise as many as the GPU has room
 // for, up to the passes of the largest leaf and 8.  A lone warp on a large leaf is bound by the latency

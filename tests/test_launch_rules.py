@@ -18,6 +18,7 @@ def lib():
                            "-o", so, os.path.join(ROOT, "tests", "launch_rules_check.cpp")])
     h = ctypes.CDLL(so)
     h.bbox_blocks.argtypes = [ctypes.c_longlong, ctypes.c_longlong]
+    h.leaf_warps.argtypes = [ctypes.c_longlong]
     h.leaf_a_split.argtypes = [ctypes.c_longlong, ctypes.c_int]
     return h
 
@@ -47,3 +48,10 @@ def test_adaptive_leaves(lib, nleaves, max_leaf):
         assert s >= 2
     if nleaves == 1:
         assert s == max(1, min(8, passes))
+
+
+def test_uniform_leaves(lib):
+    """The numbers of leaves that a uniform tree can have (8^depth, depth 0 to 7) reach both forms of the
+    near-field kernels, and the rule gives no other."""
+    assert [lib.leaf_warps(8 ** d) for d in range(8)] == [8, 8, 8, 8, 1, 1, 1, 1]
+    assert {lib.leaf_warps(n) for n in range(1, 5000)} == {8, 1}
