@@ -2345,7 +2345,7 @@ static cudaError_t leaf_launch(const TreeView& tv, int prec, const double* Lleaf
     if (tv.nleaf == 0) return cudaSuccess;
     if (prec == DAFMM_FF) return leaf_run<ff, 1>(tv, Lleaf, phi, field, s);
     const bool f64 = prec == DAFMM_FP64;
-    const bool shared = leaf_warps(tv.nleaf) > 1;
+    const bool shared = leaf_warps(tv.nleaf, tv.n, f64) > 1;
     if (!f64) return shared ? leaf_run<float, kLeafWarps>(tv, Lleaf, phi, field, s) : leaf_run<float, 1>(tv, Lleaf, phi, field, s);
     if (shared) k_leaf64<kLeafWarps><<<tv.nleaf, dim3(32, kLeafWarps), 0, s>>>(tv, Lleaf, phi, field);
     else k_leaf64<1><<<tv.nleaf, dim3(32, 1), 0, s>>>(tv, Lleaf, phi, field);

@@ -25,9 +25,14 @@ inline int bbox_blocks(int64_t nroots, int64_t max_n) {
 
 // Near field of a uniform tree (FP32 and FP64): warps that share a leaf's sources.  Such a tree has 8^depth
 // leaves: from 4096 on, one warp each gives an SM the 24 or 28 warps that it holds; 512 leaves and
-// fewer do not fill the GPU, and take 8.
+// fewer do not fill the GPU, and take 8.  In FP32 the warps share segments of 128 sources, so that a tree of
+// at most 128 particles has nothing to share: 8 warps only add their joining (2 particles, one
+// leaf: 7.5 us with one warp, 10.2 with 8).
 constexpr int kLeafWarps = 8;
-inline int leaf_warps(int64_t nleaf) { return nleaf >= 16 * kSMs ? 1 : kLeafWarps; }
+inline int leaf_warps(int64_t nleaf, int64_t n, bool f64) {
+    if (nleaf >= 16 * kSMs || (!f64 && n <= 128)) return 1;
+    return kLeafWarps;
+}
 
 // FP32 near field of an adaptive tree: blocks that share the passes (32 targets each) of a leaf, one
 // while the leaves alone fill the 24 warps that an SM holds, otherwise as many as the GPU has room

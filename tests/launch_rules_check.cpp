@@ -3,4 +3,4 @@
 
 extern "C" int bbox_blocks(long long nroots, long long max_n) { return dafmm::bbox_blocks(nroots, max_n); }
 extern "C" int leaf_a_split(long long nleaves, int max_leaf) { return dafmm::leaf_a_split(nleaves, max_leaf); }
-extern "C" int leaf_warps(long long nleaf) { return dafmm::leaf_warps(nleaf); }
+extern "C" int leaf_warps(long long nleaf, long long n, int f64) { return dafmm::leaf_warps(nleaf, n, f64 != 0); }

@@ -18,7 +18,7 @@ def lib():
                            "-o", so, os.path.join(ROOT, "tests", "launch_rules_check.cpp")])
     h = ctypes.CDLL(so)
     h.bbox_blocks.argtypes = [ctypes.c_longlong, ctypes.c_longlong]
-    h.leaf_warps.argtypes = [ctypes.c_longlong]
+    h.leaf_warps.argtypes = [ctypes.c_longlong, ctypes.c_longlong, ctypes.c_int]
     h.leaf_a_split.argtypes = [ctypes.c_longlong, ctypes.c_int]
     return h
 
@@ -50,8 +50,17 @@ def test_adaptive_leaves(lib, nleaves, max_leaf):
         assert s == max(1, min(8, passes))
 
 
-def test_uniform_leaves(lib):
+@pytest.mark.parametrize("f64", [0, 1])
+def test_uniform_leaves(lib, f64):
     """The numbers of leaves that a uniform tree can have (8^depth, depth 0 to 7) reach both forms of the
     near-field kernels, and the rule gives no other."""
-    assert [lib.leaf_warps(8 ** d) for d in range(8)] == [8, 8, 8, 8, 1, 1, 1, 1]
-    assert {lib.leaf_warps(n) for n in range(1, 5000)} == {8, 1}
+    assert [lib.leaf_warps(8 ** d, 10_000, f64) for d in range(8)] == [8, 8, 8, 8, 1, 1, 1, 1]
+    assert {lib.leaf_warps(k, 10_000, f64) for k in range(1, 5000)} == {8, 1}
+
+
+@pytest.mark.parametrize("depth", [0, 2, 3])
+def test_few_particles(lib, depth):
+    """At most one segment of 128 sources in all: nothing to share out in FP32 (FP64 shares single
+    sources)."""
+    assert [lib.leaf_warps(8 ** depth, n, 0) for n in (0, 1, 2, 128, 129, 1000)] == [1, 1, 1, 1, 8, 8]
+    assert [lib.leaf_warps(8 ** depth, n, 1) for n in (0, 2, 128, 129)] == [8, 8, 8, 8]
