@@ -880,10 +880,11 @@ constexpr size_t rot_smem(int nt) {
 // Measured against one warp per target reading the packed matrices: uniform N = 200,003, depth 4,
 // p = 8: FP64 9.7 -> 7.1 ms, float-float 9.7 -> 5.9 ms; N = 1e4, depth 3, p = 6, FP64: 1.84 -> 0.81
 // ms; Gaussian N = 100,003, p = 8, FP64 (all levels in one launch): 8.4 -> 2.8 ms.
-template <class R, bool HARM, int NT, class Fam>
-__global__ void __launch_bounds__(256, 2) k_m2l_rot(RotStream rs, const R* __restrict__ val, const R* __restrict__ ax,
-                                                    const __grid_constant__ Fam fam, RotRows m, double* __restrict__ L,
-                                                    int KS) {
+// MINB: blocks per SM it is compiled for (rot_targets).
+template <class R, bool HARM, int NT, int MINB, class Fam>
+__global__ void __launch_bounds__(256, MINB)
+    k_m2l_rot(RotStream rs, const R* __restrict__ val, const R* __restrict__ ax, const __grid_constant__ Fam fam, RotRows m,
+              double* __restrict__ L, int KS) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, sub = w % KS, oct = blockIdx.y;  // (adaptive: 8 (level - 2) + octant)
     if (fam.target(oct, (int)blockIdx.x * (8 / KS) * NT) < 0) return;  // beyond this group
@@ -2359,30 +2360,30 @@ static RotStream rot_stream(const OrderData& od, bool harm) {
 }
 
 // targets: the most in one group (octant); groups: blockIdx.y
-template <class R, bool HARM, int NT, class Fam>
+template <class R, bool HARM, int NT, int MINB = 2, class Fam>
 static cudaError_t rot_run(const OrderData& od, const R* val, const R* ax, const Fam& fam, const RotRows& m, double* L,
                            int targets, int groups, int KS, cudaStream_t s) {
     const size_t smem = rot_smem<R>(NT);
-    const cudaError_t e = set_smem(k_m2l_rot<R, HARM, NT, Fam>, smem);
+    const cudaError_t e = set_smem(k_m2l_rot<R, HARM, NT, MINB, Fam>, smem);
     if (e != cudaSuccess) return e;
     const int per = NT * (8 / KS);
-    k_m2l_rot<R, HARM, NT, Fam><<<dim3((targets + per - 1) / per, groups), 256, smem, s>>>(rot_stream(od, HARM), val, ax,
-                                                                                           fam, m, L, KS);
+    k_m2l_rot<R, HARM, NT, MINB, Fam>
+        <<<dim3((targets + per - 1) / per, groups), 256, smem, s>>>(rot_stream(od, HARM), val, ax, fam, m, L, KS);
     return cudaGetLastError();
 }
 
-// a uniform level: two targets per warp from 512 boxes on, the displacements shared out over up to
-// 8 warps while there are fewer than 2432 warps (16 per SM).  N = 200,003, depth 4, p = 8, against
-// one target per warp: FP64 7.1 -> 6.8 ms, float-float 5.9 -> 4.6 ms; N = 1e4, p = 6: 0.81 -> 0.78 ms.
+// a uniform level (rot_targets, rot_share)
 template <class R>
 static cudaError_t rot_uniform(const OrderData& od, const R* val, const R* ax, int l, const RotRows& m, double* L,
                                double inv_h, bool harm, cudaStream_t s) {
-    const int nbox = 1 << (3 * l), per = nbox / 8, nt = harm && nbox >= 512 ? 2 : 1;
+    const int nbox = 1 << (3 * l), per = nbox / 8, nt = rot_targets(nbox, harm, std::is_same<R, double>::value);
     const RotUniform fam{l, inv_h};
-    int KS = 1;
-    while (KS < 8 && nbox / nt * KS < 2432) KS *= 2;
+    const int KS = rot_share(nbox, nt);
     if (!harm) return rot_run<R, false, 1>(od, val, ax, fam, m, L, per, 8, KS, s);
     if (nt == 2) return rot_run<R, true, 2>(od, val, ax, fam, m, L, per, 8, KS, s);
+    if constexpr (std::is_same<R, double>::value) {
+        if (KS == 1) return rot_run<R, true, 1, 4>(od, val, ax, fam, m, L, per, 8, KS, s);
+    }
     return rot_run<R, true, 1>(od, val, ax, fam, m, L, per, 8, KS, s);
 }
 

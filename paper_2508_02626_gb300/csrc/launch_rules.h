@@ -34,6 +34,24 @@ inline int leaf_warps(int64_t nleaf, int64_t n, bool f64) {
     return kLeafWarps;
 }
 
+// M2L by rotation of a uniform level of nbox boxes: targets per warp.  Two from 512 boxes on (they share
+// the table reads: N = 200,003, depth 4, p = 8: FP64 7.1 -> 6.8 ms, float-float 5.9 -> 4.6 ms; N = 1e4, p = 6: 0.81
+// -> 0.78 ms), but in FP64 only while the level is about one wave: two targets need 96 registers, 16 warps
+// per SM, and from 32768 boxes on the warps in flight count for more.  One target compiled for 32
+// warps, finest level against two at 16: depth 5, p = 4, 6, 8, 10: 13.48, 21.49, 38.6, 68.6 -> 12.58, 20.27, 36.5, 65.3 ms;
+// depth 6, p = 4, 6: 109.5, 174.5 -> 102.9, 166.1 ms (one target at 24 warps, packed tables: 12.43, 20.15, 37.2,
+// 68.1; 103.5, 167.5).  Float-float (72 registers either way) keeps two.
+inline int rot_targets(int64_t nbox, bool harm, bool f64) {
+    return harm && nbox >= 512 && !(f64 && nbox >= 32768) ? 2 : 1;
+}
+// ... and warps that share the displacements of the same targets: up to 8 while there are fewer than 16
+// warps per SM
+inline int rot_share(int64_t nbox, int targets) {
+    int k = 1;
+    while (k < 8 && nbox / targets * k < 16 * kSMs) k *= 2;
+    return k;
+}
+
 // FP32 near field of an adaptive tree: blocks that share the passes (32 targets each) of a leaf, one
 // while the leaves alone fill the 24 warps that an SM holds, otherwise as many as the GPU has room
 // for, up to the passes of the largest leaf and 8.  A lone warp on a large leaf is bound by the latency

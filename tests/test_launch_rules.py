@@ -20,6 +20,8 @@ def lib():
     h.bbox_blocks.argtypes = [ctypes.c_longlong, ctypes.c_longlong]
     h.leaf_warps.argtypes = [ctypes.c_longlong, ctypes.c_longlong, ctypes.c_int]
     h.leaf_a_split.argtypes = [ctypes.c_longlong, ctypes.c_int]
+    h.rot_targets.argtypes = [ctypes.c_longlong, ctypes.c_int, ctypes.c_int]
+    h.rot_share.argtypes = [ctypes.c_longlong, ctypes.c_int]
     return h
 
 
@@ -64,3 +66,17 @@ def test_few_particles(lib, depth):
     sources)."""
     assert [lib.leaf_warps(8 ** depth, n, 0) for n in (0, 1, 2, 128, 129, 1000)] == [1, 1, 1, 1, 8, 8]
     assert [lib.leaf_warps(8 ** depth, n, 1) for n in (0, 2, 128, 129)] == [8, 8, 8, 8]
+
+
+def test_rotation(lib):
+    """Levels 2 to 7: two targets per warp between 512 boxes and one wave in FP64 (at 32768 boxes and more
+    they were up to 8 % slower than one), from 512 boxes on in float-float, never in the full basis; the
+    displacements shared out until the level has 16 warps per SM, or 8 warps per target."""
+    nbox = [8 ** l for l in range(2, 8)]
+    assert [lib.rot_targets(b, 1, 1) for b in nbox] == [1, 2, 2, 1, 1, 1]
+    assert [lib.rot_targets(b, 1, 0) for b in nbox] == [1, 2, 2, 2, 2, 2]
+    assert [lib.rot_targets(b, 0, f) for b in nbox for f in (0, 1)] == [1] * 12
+    for b in nbox:
+        for t in (1, 2):
+            k = lib.rot_share(b, t)
+            assert k in (1, 2, 4, 8) and (k == 8 or b // t * k >= 2432) and (k == 1 or b // t * (k // 2) < 2432)
