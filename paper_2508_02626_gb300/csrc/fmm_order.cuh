@@ -1362,9 +1362,13 @@ __device__ __forceinline__ ff ff_shfl_down(ff v, int d) {
 constexpr int kLeafMinWarps = 28;
 
 // ---- FP64 near field ----
-// 1/sqrt(x) for x well inside the normal range: the PTX approximation rsqrt.approx.ftz.f64 y and
-// the binomial series of (1 - e)^(-1/2) in its residual e = 1 - x y^2 up to e^2 (the next term is
-// 5/16 e^3, far below an FP64 rounding for a seed good to 2^-19): five FP64 instructions.
+// 1/sqrt(x) for x well inside the normal range: the PTX approximation y (rsqrt.approx.ftz.f64, which works on
+// the upper 32 bits of x and fills those of y: 20 explicit significand bits) and the binomial series of
+// (1 - e)^(-1/2) in its residual e = 1 - x y^2 up to e^2: five FP64 instructions.  y y is exact, so that e
+// carries no error to speak of, and with a seed good to 2^-19 (the two truncations leave 2^-21 + 2^-20;
+// PTX states no bound) |e| <= 2^-18 and the first term left out is 5/16 e^3 <= 5/32 2^-53 of the result.  Measured
+// on 300,000 arguments over the whole range: at most 1.003 2^-53 (one rounding alone: 1), every result
+// equal to CUDA's rsqrt.
 __device__ __forceinline__ double rsqrt_series(double x) {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
@@ -1397,9 +1401,9 @@ __device__ __forceinline__ int pass_width(int rem) {
 // bound, so everything else is spent to feed it: every lane has a target or a share of the
 // sources (the list position of a source is a search in the prefix sums), 1/r takes five FP64
 // instructions, and a pair takes 18 (20 with CUDA's rsqrt and an FP64 comparison).  r^2 outside
-// the safe range -- zero for the target itself and coincident particles, which add nothing,
-// denormal, infinite or NaN -- is seen in the exponent by an integer comparison and takes CUDA's
-// rsqrt.
+// the series' window (2^-991 to 2^977) is seen in the exponent by an integer comparison: positive it takes
+// CUDA's rsqrt (an infinite one adds 1/inf = 0); zero -- the target itself and coincident particles --
+// and NaN add nothing.
 __device__ __forceinline__ void near64_list(const double* __restrict__ x, const double* __restrict__ y,
                                             const double* __restrict__ z, const double* __restrict__ q, int cnt,
                                             int first, int G, int g, int lane, double xt, double yt, double zt,
