@@ -8,8 +8,10 @@ On the GPU the balance is different -- P2P runs at FP32 ALU rate, M2L on the ten
 pipes -- so the tuner times candidate values around the paper's choice on the actual
 workload (a forest of the problems to solve) together with the near-field kernel's tile
 (leaves per thread block, DAFMM_OPT_LEAF_WARPS), and caches the winner as JSON keyed by the
-GPU, order, precision and a size class of the workload.
+GPU, the library's sources, order, precision and a size class of the workload.
 """
+import functools
+import hashlib
 import json
 import math
 import os
@@ -18,17 +20,27 @@ import time
 
 import numpy as np
 
+from . import _build
 from . import binding as B
 
 # fastest leaf size of the paper's CPU sweep for large N, per order (Table 10)
 PAPER_LEAF_SIZE = {2: 64, 4: 128, 6: 256, 8: 256, 10: 512}
-LEAF_WARPS = (2, 4, 8)
+# near-field tiles of the FP32 and MIXED modes; one leaf per block, the default, is usually the fastest
+# (64-problem forest, p = 6: 1.88 ms, four leaves per block 2.02)
+LEAF_WARPS = (1, 2, 4, 8)
 
 
 def paper_leaf_size(order):
     """The paper's leaf size for `order` (odd orders take the next even order's value)."""
     o = min(10, max(2, order + (order & 1)))
     return PAPER_LEAF_SIZE[o]
+
+
+def tile_candidates(precision):
+    """The tiles worth timing: in FP64 (and float-float, which a forest evaluates in FP64) the kernel
+    does not have any."""
+    prec = B.PRECISIONS[precision] if isinstance(precision, str) else int(precision)
+    return LEAF_WARPS if prec in (B.DAFMM_FP32, B.DAFMM_MIXED) else (1,)
 
 
 def leaf_candidates(order):
@@ -74,8 +86,22 @@ class Cache:
         os.replace(tmp, self.path)
 
 
-def make_key(device_name, order, precision, n_total, n_trees):
-    return "%s|p%d|%s|%s" % (device_name, order, precision, size_class(n_total, n_trees))
+@functools.lru_cache(maxsize=None)
+def library_stamp():
+    """Names the library's sources and build flags: what was the fastest for other kernels says nothing
+    about these."""
+    h = hashlib.sha256(" ".join(_build.NVCC_FLAGS + _build._extra_flags()).encode())
+    for name in sorted(os.listdir(_build.CSRC)):
+        path = os.path.join(_build.CSRC, name)
+        if os.path.isfile(path):
+            with open(path, "rb") as f:
+                h.update(name.encode() + f.read())
+    return h.hexdigest()[:12]
+
+
+def make_key(device_name, order, precision, n_total, n_trees, library=None):
+    return "%s|%s|p%d|%s|%s" % (device_name, library or library_stamp(), order, precision,
+                                size_class(n_total, n_trees))
 
 
 def tune_forest(ctx, xyz, q, offsets, order, precision="fp32", cache=None, reps=2, force=False):
@@ -103,7 +129,7 @@ def tune_forest(ctx, xyz, q, offsets, order, precision="fp32", cache=None, reps=
         f = ctx.build_forest(xyz, q, offsets, max_leaf=s)
         torch.cuda.synchronize()
         build_ms = (time.perf_counter() - t0) * 1e3
-        for w in LEAF_WARPS:
+        for w in tile_candidates(precision):
             B.dafmm_set_option(ctx.h, B.DAFMM_OPT_LEAF_WARPS, w)
             f.eval(order, phi, E, precision=precision)  # warm (tables, expansions)
             ms = []
