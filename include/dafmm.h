@@ -303,9 +303,12 @@ int dafmm_eval_noalloc(dafmm_tree* tree, int order, double* phi, double* field, 
 #define DAFMM_PEAK_MMA_F16 5
 int dafmm_probe_peak(int device, int kind, double* rate, double* ms);
 
-/* Device bytes an evaluation of a tree with these parameters needs (an upper estimate; for a
- * uniform tree it includes the build's scratch and the staging of host input arrays, which a
- * pooled context's asynchronous build keeps until the build has completed). */
+/* Device bytes that a tree with these parameters and its first evaluation need in a context of its own
+ * with the default options: the build with its scratch and the staging of host arrays (a pooled
+ * context's asynchronous uniform build keeps them until it has completed), the expansions, and the
+ * order's tables for this precision with the scratch of their making.  An upper estimate for uniform
+ * trees; for adaptive ones it assumes 16 n / max_leaf boxes (a split box's particles spread over its
+ * children; steeply graded point sets may need more). */
 size_t dafmm_footprint(int64_t n, int order, int uniform_depth, int max_leaf, int precision);
 
 /* ---- single-operator batches (the paper's per-operator verification, Sec. 3) --------

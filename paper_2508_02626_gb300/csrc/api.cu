@@ -15,6 +15,7 @@
 #include "check.cuh"
 #include "da_common.cuh"
 #include "internal.h"
+#include "launch_rules.h"
 #include "rot_lists.h"
 #include "tc_ops.h"
 #include "tree_common.cuh"
@@ -1509,6 +1510,101 @@ int tree_ready(dafmm_tree* t, cudaStream_t s) {
     return q == cudaSuccess ? DAFMM_OK : cuda_fail(c, q, "tree build");
 }
 
+// ---- estimates of device memory -------------------------------------------------------------------
+namespace {
+struct ByteSum {
+    size_t total = 0;
+    void add(size_t bytes) { total += (bytes + 255) / 256 * 256; }  // as dev_alloc rounds
+};
+
+// the sizes of the rotation M2L's tables (rot_lists.h), found once per order
+struct RotSizes {
+    size_t tasks, xz, axial, nnz;  // task words, and of them those of the substitutions and the axial step
+};
+const RotSizes& rot_sizes(int p) {
+    static std::once_flag once[kMaxOrder + 1];
+    static RotSizes sizes[kMaxOrder + 1];
+    std::call_once(once[p], [p] {
+        const RotStructure r = rot_structure(p, true);
+        const size_t xz = 32 * (size_t)(r.len[0] + r.len[1]), a = 32 * (size_t)r.len[2];
+        sizes[p] = RotSizes{xz + a, xz, a, r.col.size()};
+    });
+    return sizes[p];
+}
+
+// the tables of an order that an evaluation with the context's default options makes
+// (ensure_order; f32: ensure_k16h; f64: ensure_rotation and its float-float copies), the scratch of
+// their making included; far: a far field (the M2L's tables)
+size_t order_table_bytes(int p, bool far, bool f32, bool f64) {
+    const OrderOps* ops = order_ops(p);
+    const size_t nc = ncoef_of(p), ncp = ncp_of(p), nh = nharm_of(p), K = kNumKeys;
+    ByteSum b;
+    for (const HostShiftTable* t : {&ops->m2m, &ops->l2l, &ops->m2mh}) {
+        for (size_t width : {2, 1, 8, 4}) b.add((size_t)t->nnz * width);
+        b.add((nc + 1) * 4);
+        b.add((8 * nc + 1) * 4);
+    }
+    size_t pairs = 1;  // products of two coefficients of total degree up to p: C(p + 6, 6)
+    for (int k = 1; k <= 6; ++k) pairs = pairs * (p + k) / k;
+    b.add((nc + 1) * 4);
+    b.add(pairs * 4);
+    b.add(3 * nc * 2);
+    if (!far) return b.total;
+    b.add(K * nc * ncp * 8);
+    b.add(K * nc * ncp * 4);
+    b.add(256 * 6 + 12 * nc + 16 * K);  // (the symmetry tables)
+    if (p >= 2) {
+        const size_t npt = tc_npt(p);
+        for (int k = 0; k < 2; ++k) b.add(K * npt * ncp * 4);
+        for (int k = 0; k < 4; ++k) b.add(8 * npt * ncp * 4);
+        b.add(8 * nc * ncp * 8);
+    }
+    if (f32 && p >= 2) {
+        const size_t npt = tc_npt_h(p), row = tc_rowlen16h(p), nhp = harm_row(p), steps = std::max<size_t>(nc - nh, 1);
+        for (int k = 0; k < 2; ++k) b.add(K * npt * row * 2);
+        for (int k = 0; k < 2; ++k) b.add(K * npt * nhp * 4);
+        for (int k = 0; k < 2; ++k) b.add((npt + K) * 4);
+        b.add(npt * 4);
+        for (size_t width : {16, 8, 16}) b.add(steps * width);
+        b.add(nc * nh * 8);
+        b.add(K * nh * nhp * 8);
+    }
+    if (f64 && p >= 2) {
+        const RotSizes& rs = rot_sizes(p);
+        const size_t lengths = 15;  // distinct |v| of the 316 displacements
+        b.add(K * 4 * ops->rot_tsz * 8);
+        b.add(lengths * rs.nnz * 8);
+        b.add(K * 4);
+        b.add((nc + 1) * 4);
+        b.add(rs.nnz * 2);
+        b.add(lengths * 24);
+        b.add(lengths * nc * ncp * 8);
+        b.add(rs.tasks * 4);
+        b.add(rs.tasks * 8);
+        for (int k = 0; k < 2; ++k) b.add(2 * K * rs.xz * 8);
+        for (int k = 0; k < 2; ++k) b.add(lengths * rs.axial * 8);
+    }
+    return b.total;
+}
+}  // namespace
+
+namespace dafmm {
+// an adaptive tree or forest of n particles, its expansions and build scratch, and the dense M2L
+// matrices of its order.  (The server admits requests by differences of it.)
+size_t forest_estimate(int64_t n, int order, int max_leaf) {
+    const size_t ncp = ncp_of(order), nc = ncoef_of(order);
+    size_t b = tree_bytes(n, 0);
+    // about 16 n / max_leaf boxes; per box its hierarchy record, list entries (U, W and X, about 64
+    // on average), its first FP32 record, a padding record (with its remainder record), its place in
+    // the list of parents and the expansions
+    const size_t nbox = 2 + (size_t)(16 * n) / (size_t)(max_leaf > 0 ? max_leaf : 1);
+    b += nbox * (kBoxInts * 4 + 64 * 4 + 24 + 32 + 4 + ncp * (8 + 8 + 4));
+    b += (size_t)kNumKeys * nc * ncp * 12;
+    b += (size_t)n * 12 + radix_sort_temp_bytes(n) + radix_sort_temp_bytes((int64_t)nbox);
+    return b;
+}
+}  // namespace dafmm
+
 // ================================ C ABI =======================================================
 extern "C" {
 
@@ -2351,28 +2447,37 @@ int dafmm_last_phase_ms(dafmm_ctx* c, double* out) {
 }
 
 size_t dafmm_footprint(int64_t n, int order, int uniform_depth, int max_leaf, int precision) {
-    (void)precision;
     if (order < 0 || order > kMaxOrder || n < 0) return 0;
-    const int depth = uniform_depth < 0 ? 0 : uniform_depth;
-    size_t b = tree_bytes(n, depth);
-    const size_t ncp = ncp_of(order), nc = ncoef_of(order);
+    const size_t ncp = ncp_of(order);
+    const bool f32 = precision != DAFMM_FP64 && precision != DAFMM_FF;  // (an unknown mode: every table)
+    const bool f64 = precision != DAFMM_FP32 && precision != DAFMM_MIXED;
+    const bool far = uniform_depth < 0 || uniform_depth >= 2;
+    ByteSum b;
+    b.total = (size_t)1 << 16;  // rounding of the single arrays, flags, small lists
+    b.total += order_table_bytes(order, far, far && f32, far && f64);
+    b.add((size_t)n * 32);  // outputs, when the caller's are host arrays
     if (uniform_depth < 0) {
-        // adaptive: about 16 n / max_leaf boxes; per box its hierarchy record, list entries
-        // (U, W and X, about 64 on average), its first FP32 record, a padding record (with its
-        // remainder record), its place in the list of parents and the expansions
-        const size_t nbox = 2 + (size_t)(16 * n) / (size_t)(max_leaf > 0 ? max_leaf : 1);
-        b += nbox * (kBoxInts * 4 + 64 * 4 + 24 + 32 + 4 + ncp * (8 + 8 + 4));
-        b += (size_t)kNumKeys * nc * ncp * 12;
-        b += (size_t)n * 12 + radix_sort_temp_bytes(n) + radix_sort_temp_bytes((int64_t)nbox);
-        return b;
+        b.total += forest_estimate(n, order, max_leaf);
+        b.add((size_t)n * 32);               // staged host inputs
+        b.add(1024 * kBoxInts * 4);          // (the box arrays start at 1024 boxes)
+        b.add(1024 * 64);
+        return b.total;
     }
-    for (int l = 2; l <= depth; ++l) b += level_boxes(l) * ncp * (8 + 8 + 4);
-    b += (size_t)kNumKeys * nc * ncp * 12;
-    b += (size_t)n * 12 + radix_sort_temp_bytes(n);  // build-time scratch
+    const int depth = uniform_depth;
+    b.add(tree_bytes(n, depth));
+    b.add((size_t)n * 8);  // build-time scratch
+    b.add(radix_sort_temp_bytes(n));
     // the staging of host input arrays (xyz and q): a pooled context's asynchronous build holds
     // it, with the scratch above, until the build has completed
-    b += (size_t)n * 32;
-    return b;
+    b.add((size_t)n * 32);
+    for (int l = 2; l <= depth; ++l) {
+        const size_t nb = level_boxes(l);
+        b.add(nb * ncp * (2 * sizeof(double) + 5 * sizeof(float)));  // ensure_expansions
+        if (!f32) continue;
+        b.add(nb * (tc_rowlen16(order) * 4 + sizeof(float)));  // ensure_f16_levels
+        b.add(nb * harm_row(order) * sizeof(float) * tc_m2l_split(depth, kSMs));  // ensure_lh_levels
+    }
+    return b.total;
 }
 
 // ---- single-operator batches -------------------------------------------------------------------

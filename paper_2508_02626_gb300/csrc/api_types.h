@@ -144,6 +144,8 @@ namespace dafmm {
 // device allocation through a context (its budget or pool); used by other runtime units
 int ctx_alloc(dafmm_ctx* c, void** p, size_t bytes, const char* what);
 void ctx_free(dafmm_ctx* c, void* p, size_t bytes);
+// device bytes of an adaptive tree or forest with its order's dense M2L matrices (an estimate)
+size_t forest_estimate(int64_t n, int order, int max_leaf);
 }  // namespace dafmm
 
 // the uniform tree's build (if still asynchronous) ordered before work on stream s; the build's

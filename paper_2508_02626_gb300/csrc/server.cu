@@ -100,15 +100,15 @@ void CUDART_CB on_job_done(void* arg) {
 // device bytes of one request inside a job: its share of the tree and expansions plus the
 // job's staging buffers (the per-order tables are counted once, by the admission)
 size_t request_estimate(const SReq* r) {
-    const size_t with = dafmm_footprint(r->n, r->order, -1, r->max_leaf, r->precision);
-    const size_t without = dafmm_footprint(0, r->order, -1, r->max_leaf, r->precision);
+    const size_t with = forest_estimate(r->n, r->order, r->max_leaf);
+    const size_t without = forest_estimate(0, r->order, r->max_leaf);
     return (with > without ? with - without : 0) + (size_t)r->n * 64 + ((size_t)1 << 20);
 }
 
 // the per-order tables (M2L matrices and their splits), when the order is not loaded yet
 size_t tables_estimate(const dafmm_ctx* c, const SReq* r) {
     if (c->ord[r->order].k_ready) return 0;
-    return 2 * dafmm_footprint(0, r->order, -1, r->max_leaf, r->precision);
+    return 2 * forest_estimate(0, r->order, r->max_leaf);
 }
 
 // launch one job on its slot's stream; returns a DAFMM code (the job is not running on error)
