@@ -4,7 +4,9 @@ One step = one dafmm_eval (P2M -> M2M -> M2L -> L2L -> L2P + P2P, the whole hot 
 the resident tree of the workload: N = 1,000,000 particles uniform in the unit cube,
 charges U[-1,1], uniform octree of depth 5, expansion order p = 8, seed 2002.
 
-Prints one JSON line (rank 0).  Under torchrun every rank runs an independent replica of
+Prints one JSON line (rank 0): the headline, its end-to-end and roofline figures and a summary of the
+other workloads.  The whole record (every mode, phase, operator and sweep; some 20 KB) goes to the
+standard error as one JSON line, or with --record FILE to a file.  Under torchrun every rank runs an independent replica of
 the workload on its own GPU (independent solves shard with no data exchange); the value
 is the total particles of all ranks divided by the slowest rank's time.
 
@@ -1188,6 +1190,26 @@ def cpu_baseline(x, q, dom, cfg, phi_gpu, E_gpu, phi_by_order=None, mode_results
     return cpu, acc
 
 
+# keys of the whole record that the printed line keeps as they are
+HEADLINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+                 "vs_baseline", "dtype", "data", "config", "phases_ms", "gpu_launches", "roofline", "roofline_m2l",
+                 "clocks", "e2e", "cpu_baseline")
+
+
+def headline(out):
+    """The printed line: a few KB whatever the workloads report (readers of a log's tail, or with a limit
+    on a line's length, lose a line of 20 KB)."""
+    line = {k: out[k] for k in HEADLINE_KEYS if k in out}
+    line["modes"] = {m: {"value": r["value"], "ms_per_step": r["ms_per_step"]} for m, r in out.get("modes", {}).items()}
+    if "serving" in out:
+        line["served"] = dict(out["serving"]["saturated"],
+                              rates=[{k: r[k] for k in ("load", "solves_per_s", "p50_ms", "p99_ms")}
+                                     for r in out["serving"]["rates"]])
+    if "accuracy" in out:
+        line["accuracy"] = {k: v for k, v in out["accuracy"].items() if not isinstance(v, dict)}
+    return line
+
+
 def run_reference(args, rank, world):
     """CPU oracle arm: every step, warm-up steps included, is one full oracle FMM solve of the
     workload (all particles, all host cores); the rate is particles over the mean step time."""
@@ -1241,6 +1263,7 @@ def main():
     ap.add_argument("--sections", default="adaptive,batch,serving,operators,leafsize,paper",
                     help="comma-separated extra workloads at N = 1: adaptive, batch, serving, operators, leafsize, "
                          "paper")
+    ap.add_argument("--record", default="", help="file for the whole record (default: one line on the standard error)")
     args = ap.parse_args()
     rank = int(os.environ.get("RANK", 0))
     world = int(os.environ.get("WORLD_SIZE", 1))
@@ -1256,7 +1279,12 @@ def main():
         dist.init_process_group("nccl")
     out = run_ours(args, rank, world)
     if rank == 0:
-        print(json.dumps(out))
+        if args.record:
+            with open(args.record, "w") as f:
+                json.dump(out, f)
+        else:
+            print(json.dumps(out), file=sys.stderr)
+        print(json.dumps(headline(out)))
     if world > 1:
         import torch.distributed as dist
         dist.destroy_process_group()
