@@ -321,7 +321,7 @@ struct ShiftAdaptive {
     int n;
     __device__ __forceinline__ int parent(int i) const { return list[i]; }
     __device__ __forceinline__ int child(int i, int c) const {
-        const int ch = av.child[8 * list[i] + c];
+        const int ch = av.child[8 * (size_t)list[i] + c];
         return ch >= 0 && DAFMM_IN(ch, av.nbox, kChkBoxIndex) ? ch : -1;
     }
 };
@@ -1768,9 +1768,9 @@ __global__ void __launch_bounds__(256) k_m2l_a(const T* __restrict__ K, Adaptive
                         const int dx = ox - vx, dy = oy - vy, dz = oz - vz;  // = 2a + sc
                         const int scx = dx & 1, scy = dy & 1, scz = dz & 1;
                         const int ax = (dx - scx) >> 1, ay = (dy - scy) >> 1, az = (dz - scz) >> 1;
-                        const int Q = av.colleague[27 * P + (ax + 1) * 9 + (ay + 1) * 3 + (az + 1)];
+                        const int Q = av.colleague[27 * (size_t)P + (ax + 1) * 9 + (ay + 1) * 3 + (az + 1)];
                         if (Q >= 0 && DAFMM_IN(Q, av.nbox, kChkBoxIndex))
-                            sbox = av.child[8 * Q + (scx | (scy << 1) | (scz << 2))];
+                            sbox = av.child[8 * (size_t)Q + (scx | (scy << 1) | (scz << 2))];
                         if (sbox >= 0 && !DAFMM_IN(sbox, av.nbox, kChkBoxIndex)) sbox = -1;
                     }
                     sidx[threadIdx.x] = sbox;

@@ -62,10 +62,10 @@ __device__ __forceinline__ void term_slot(const Terms& tm, int& slot, int& sc) {
 }
 // the two dependent loads of that lookup, for a target whose parent is `par` (-1: none)
 __device__ __forceinline__ int colleague_of(const TCGParams& prm, int par, int slot) {
-    return par >= 0 && DAFMM_IN(par, prm.nbox, kChkGatherSource) ? prm.colleague[27 * par + slot] : -1;
+    return par >= 0 && DAFMM_IN(par, prm.nbox, kChkGatherSource) ? prm.colleague[27 * (size_t)par + slot] : -1;
 }
 __device__ __forceinline__ int child_of(const TCGParams& prm, int Q, int sc) {
-    const int s = Q >= 0 && DAFMM_IN(Q, prm.nbox, kChkGatherSource) ? prm.child[8 * Q + sc] : -1;
+    const int s = Q >= 0 && DAFMM_IN(Q, prm.nbox, kChkGatherSource) ? prm.child[8 * (size_t)Q + sc] : -1;
     return s < 0 || DAFMM_IN(s, prm.nbox, kChkGatherSource) ? s : -1;
 }
 __device__ __forceinline__ int term_key(const Terms& tm) {

@@ -158,8 +158,8 @@ __global__ void k_box_geometry(const int* __restrict__ root, const int* __restri
     if (b >= nbox) return;
     const double* d = rootdom + 4 * root[b];
     const double h = ldexp(d[3], -level[b]);
-    geom[b] = make_double4(d[0] + ((double)ijk[3 * b] + 0.5) * h, d[1] + ((double)ijk[3 * b + 1] + 0.5) * h,
-                           d[2] + ((double)ijk[3 * b + 2] + 0.5) * h, h);
+    geom[b] = make_double4(d[0] + ((double)ijk[3 * (size_t)b] + 0.5) * h, d[1] + ((double)ijk[3 * (size_t)b + 1] + 0.5) * h,
+                           d[2] + ((double)ijk[3 * (size_t)b + 2] + 0.5) * h, h);
 }
 
 cudaError_t launch_box_geometry(const int* root, const int* level, const int* ijk, const double* rootdom, int nbox,
@@ -191,31 +191,31 @@ __device__ inline void child_range(const AdaptiveBuild& ab, int b, int level, bo
 
 // per box of level l: number of non-empty children when it splits
 __global__ void k_split_count(AdaptiveBuild ab, int lb, int le, int level, int max_leaf, int max_depth, int* nch) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x, c = i & 7;
-    const int b = min(lb + (i >> 3), le - 1);
+    const int c = threadIdx.x & 7, own = lb + (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 3);
+    const int b = min(own, le - 1);
     int s, e;
     child_range(ab, b, level, ab.pend[b] - ab.pbeg[b] > max_leaf && level < max_depth, c, s, e);
     const unsigned any = __ballot_sync(0xffffffffu, e > s);
-    if (c == 0 && lb + (i >> 3) < le) nch[b - lb] = __popc((any >> (threadIdx.x & 24)) & 0xffu);
+    if (c == 0 && own < le) nch[b - lb] = __popc((any >> (threadIdx.x & 24)) & 0xffu);
 }
 
 __global__ void k_split_fill(AdaptiveBuild ab, int lb, int le, int level, const int* offs, int first_new) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x, c = i & 7;
-    const int b = min(lb + (i >> 3), le - 1);
+    const int c = threadIdx.x & 7, own = lb + (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 3);
+    const int b = min(own, le - 1);
     const int k0 = offs[b - lb], k1 = offs[b - lb + 1];
     int s, e;
     child_range(ab, b, level, k1 > k0, c, s, e);
     const unsigned any = (__ballot_sync(0xffffffffu, e > s) >> (threadIdx.x & 24)) & 0xffu;
-    if (lb + (i >> 3) >= le) return;
+    if (own >= le) return;
     int k = -1;
     if (e > s) {
         k = first_new + k0 + __popc(any & ((1u << c) - 1u));
         if (DAFMM_IN(k, ab.cap, kChkSplitChild)) {
             ab.root[k] = ab.root[b];
             ab.level[k] = level + 1;
-            ab.ijk[3 * k] = 2 * ab.ijk[3 * b] + (c & 1);
-            ab.ijk[3 * k + 1] = 2 * ab.ijk[3 * b + 1] + ((c >> 1) & 1);
-            ab.ijk[3 * k + 2] = 2 * ab.ijk[3 * b + 2] + ((c >> 2) & 1);
+            ab.ijk[3 * (size_t)k] = 2 * ab.ijk[3 * (size_t)b] + (c & 1);
+            ab.ijk[3 * (size_t)k + 1] = 2 * ab.ijk[3 * (size_t)b + 1] + ((c >> 1) & 1);
+            ab.ijk[3 * (size_t)k + 2] = 2 * ab.ijk[3 * (size_t)b + 2] + ((c >> 2) & 1);
             ab.parent[k] = b;
             ab.pbeg[k] = s;
             ab.pend[k] = e;
@@ -223,13 +223,13 @@ __global__ void k_split_fill(AdaptiveBuild ab, int lb, int le, int level, const 
             k = -1;
         }
     }
-    ab.child[8 * b + c] = k;
+    ab.child[8 * (size_t)b + c] = k;
 }
 
 __global__ void k_leaf_children_init(int* child, int b0, int b1) {
     const int b = b0 + blockIdx.x * blockDim.x + threadIdx.x;
     if (b < b1)
-        for (int c = 0; c < 8; ++c) child[8 * b + c] = -1;
+        for (int c = 0; c < 8; ++c) child[8 * (size_t)b + c] = -1;
 }
 
 cudaError_t launch_split(AdaptiveBuild ab, int lb, int le, int level, int max_leaf, int max_depth, int* nch,
@@ -330,7 +330,7 @@ cudaError_t launch_scan(const int* in, int* out, int n, int* temp, cudaStream_t 
 // ---- colleagues ---------------------------------------------------------------------------
 __device__ inline bool same_level_adjacent(const int* ijk, int a, int b) {
     for (int d = 0; d < 3; ++d) {
-        const int df = ijk[3 * a + d] - ijk[3 * b + d];
+        const int df = ijk[3 * (size_t)a + d] - ijk[3 * (size_t)b + d];
         if (df < -1 || df > 1) return false;
     }
     return true;
@@ -342,8 +342,8 @@ __device__ inline bool touch(const AdaptiveBuild& ab, int a, int b) {
     const int L = la > lb ? la : lb;
     for (int d = 0; d < 3; ++d) {
         // (levels up to 20: everything below 2^21)
-        const int alo = ab.ijk[3 * a + d] << (L - la), ahi = (ab.ijk[3 * a + d] + 1) << (L - la);
-        const int blo = ab.ijk[3 * b + d] << (L - lb), bhi = (ab.ijk[3 * b + d] + 1) << (L - lb);
+        const int alo = ab.ijk[3 * (size_t)a + d] << (L - la), ahi = (ab.ijk[3 * (size_t)a + d] + 1) << (L - la);
+        const int blo = ab.ijk[3 * (size_t)b + d] << (L - lb), bhi = (ab.ijk[3 * (size_t)b + d] + 1) << (L - lb);
         if (alo > bhi || blo > ahi) return false;
     }
     return true;
@@ -361,8 +361,8 @@ __global__ void k_colleagues(AdaptiveBuild ab, int lb, int le) {
     int c = k == 13 ? b : -1;
     const int P = ab.parent[b];
     if (P >= 0 && k != 13) {
-        const int nx = (ab.ijk[3 * b] & 1) + k / 9 - 1, ny = (ab.ijk[3 * b + 1] & 1) + (k / 3) % 3 - 1,
-                  nz = (ab.ijk[3 * b + 2] & 1) + k % 3 - 1;  // in [-1, 2]: parent offset n >> 1, parity n & 1
+        const int nx = (ab.ijk[3 * (size_t)b] & 1) + k / 9 - 1, ny = (ab.ijk[3 * (size_t)b + 1] & 1) + (k / 3) % 3 - 1,
+                  nz = (ab.ijk[3 * (size_t)b + 2] & 1) + k % 3 - 1;  // in [-1, 2]: parent offset n >> 1, parity n & 1
         const int Q = ab.colleague[27 * (size_t)P + ((nx >> 1) + 1) * 9 + ((ny >> 1) + 1) * 3 + ((nz >> 1) + 1)];
         if (Q >= 0) c = ab.child[8 * (size_t)Q + ((nx & 1) | ((ny & 1) << 1) | ((nz & 1) << 2))];
     }
@@ -550,7 +550,7 @@ __global__ void k_gather_adaptive(const double* __restrict__ xyz, const double* 
     for (int t = ab.pbeg[b] + threadIdx.x; t < ab.pend[b]; t += blockDim.x) {
         const int i = perm[t];
         if (!DAFMM_IN(i, n, kChkPerm)) continue;
-        const double px = xyz[3 * i], py = xyz[3 * i + 1], pz = xyz[3 * i + 2], pq = q[i];
+        const double px = xyz[3 * (size_t)i], py = xyz[3 * (size_t)i + 1], pz = xyz[3 * (size_t)i + 2], pq = q[i];
         x[t] = px; y[t] = py; z[t] = pz; qs[t] = pq;
         const double ox = (px - cx) * ih, oy = (py - cy) * ih, oz = (pz - cz) * ih;
         const float hx = (float)ox, hy = (float)oy, hz = (float)oz;
@@ -603,7 +603,7 @@ __global__ void k_leaf_flags(const int* __restrict__ child, int nbox, int* flags
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= nbox) return;
     bool leaf = true;
-    for (int j = 0; j < 8; ++j) leaf = leaf && child[8 * b + j] < 0;
+    for (int j = 0; j < 8; ++j) leaf = leaf && child[8 * (size_t)b + j] < 0;
     flags[b] = leaf ? 1 : 0;
 }
 
@@ -631,7 +631,7 @@ __global__ void k_group_keys(const int* __restrict__ level, const int* __restric
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= nbox) return;
     const int l = level[b];
-    const int oct = (ijk[3 * b] & 1) | ((ijk[3 * b + 1] & 1) << 1) | ((ijk[3 * b + 2] & 1) << 2);
+    const int oct = (ijk[3 * (size_t)b] & 1) | ((ijk[3 * (size_t)b + 1] & 1) << 1) | ((ijk[3 * (size_t)b + 2] & 1) << 2);
     keys[b] = l >= 2 ? (uint64_t)(l * 8 + oct) : 0xffu;
     vals[b] = b;
 }

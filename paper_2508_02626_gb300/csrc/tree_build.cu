@@ -235,7 +235,7 @@ __global__ void k_gather_uniform(const double* __restrict__ xyz, const double* _
     if (t >= n) return;
     const int i = perm[t];
     if (!DAFMM_IN(i, n, kChkPerm) || !DAFMM_IN(keys[t], tv.nleaf, kChkLeafKey)) return;
-    const double px = xyz[3 * i], py = xyz[3 * i + 1], pz = xyz[3 * i + 2], pq = q[i];
+    const double px = xyz[3 * (size_t)i], py = xyz[3 * (size_t)i + 1], pz = xyz[3 * (size_t)i + 2], pq = q[i];
     x[t] = px; y[t] = py; z[t] = pz; qs[t] = pq;
     int a, b, c;
     octmajor_decode(tv.depth, (int)keys[t], a, b, c);
@@ -290,7 +290,7 @@ __global__ void k_scatter_out(const double* __restrict__ ps, const double* __res
     if (!DAFMM_IN(i, n, kChkPerm)) return;
     if (phi) phi[i] = ps[t];
     if (field)
-        for (int d = 0; d < 3; ++d) field[3 * i + d] = fs[3 * t + d];
+        for (int d = 0; d < 3; ++d) field[3 * (size_t)i + d] = fs[3 * t + d];
 }
 
 cudaError_t launch_scatter_outputs(const double* phi_sorted, const double* field_sorted, const int* perm,
