@@ -99,8 +99,8 @@ size_t dafmm_bytes_in_use(const dafmm_ctx* ctx);
  * flight on `stream`; every later call on the tree (on any stream) is ordered after it.
  * Otherwise the call returns with the tree built. 
  * Errors: DAFMM_ERR_INVALID_ARG for n < 0, missing arrays, max_leaf < 1 on an adaptive
- * tree, depth > 7 or a bad domain; DAFMM_ERR_OVER_BUDGET when the context's budget or the
- * device runs out of memory. */
+ * tree, depth > 7, a bad domain or n and the leaves together above 2^31 - 4;
+ * DAFMM_ERR_OVER_BUDGET when the context's budget or the device runs out of memory. */
 int dafmm_build_tree(dafmm_ctx* ctx, const double* xyz, const double* q, int64_t n,
                      const double* domain, int uniform_depth, int max_leaf, void* stream,
                      dafmm_tree** tree);

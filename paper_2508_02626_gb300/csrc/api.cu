@@ -1141,6 +1141,10 @@ int build_adaptive(dafmm_ctx* c, dafmm_tree* t, const double* dxyz, const double
     // padding record per leaf)
     dev_free(c, t->xq, 2 * t->xq_n4 * sizeof(float4));
     t->xq = nullptr;
+    if (xq_records(t->n, nl) > (size_t)INT32_MAX) {  // (indexed by int)
+        t->xq_n4 = 0;
+        return fail(c, DAFMM_ERR_INVALID_ARG, "particles and leaves above 2^31");
+    }
     t->xq_n4 = xq_records(t->n, nl);
     if ((rc = dev_alloc(c, (void**)&t->xq, 2 * t->xq_n4 * sizeof(float4), "particles"))) {
         t->xq_n4 = 0;
@@ -1685,6 +1689,9 @@ int dafmm_build_tree(dafmm_ctx* c, const double* xyz, const double* q, int64_t n
     if (uniform_depth < 0 && max_leaf < 1) return fail(c, DAFMM_ERR_INVALID_ARG, "max_leaf must be >= 1");
     if (uniform_depth > kMaxUniformDepth)
         return fail(c, DAFMM_ERR_INVALID_ARG, "uniform depth above " + std::to_string(kMaxUniformDepth));
+    // the FP32 records (one per particle and a padding one per leaf) are indexed by int
+    if (uniform_depth >= 0 && xq_records(n, (int64_t)level_boxes(uniform_depth)) > (size_t)INT32_MAX)
+        return fail(c, DAFMM_ERR_INVALID_ARG, "particles and leaves above 2^31");
     if (domain && !(domain[3] > 0.0 && isfinite(domain[0]) && isfinite(domain[1]) && isfinite(domain[2]) &&
                     isfinite(domain[3])))
         return fail(c, DAFMM_ERR_INVALID_ARG, "domain");
