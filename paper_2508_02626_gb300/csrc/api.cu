@@ -1374,10 +1374,11 @@ int eval_adaptive(dafmm_tree* t, int order, int precision, double* dphi, double*
                 for (int g = l0 * 8; g < (l1 + 1) * 8; ++g) mx = std::max(mx, t->grp_ptr_h[g + 1] - t->grp_ptr_h[g]);
                 return mx;
             };
-            // by rotation: every level in one launch; dense: level by level
-            for (int l = 2; l <= t->maxlev; l = rot ? t->maxlev + 1 : l + 1) {
-                if (rot || l == t->maxlev) mark(4);
-                const int le = rot ? t->maxlev : l;
+            // by rotation: every level in one launch (the finest by itself when phases are timed); dense:
+            // level by level
+            for (int l = 2, le; l <= t->maxlev; l = le + 1) {
+                le = !rot ? l : (c->profile && l < t->maxlev ? t->maxlev - 1 : t->maxlev);
+                if (le == t->maxlev) mark(4);
                 CK(c, ops->m2l_a(od, av, precision | rflags, t->grp_tg, t->grp_ptr, l * 8, (le - l + 1) * 8,
                                  largest(l, le), t->aM, t->aMf, t->aL, s),
                    "M2L");
