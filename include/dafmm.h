@@ -187,7 +187,8 @@ int dafmm_server_destroy(dafmm_server* server);
 /* Per-phase device time of the last dafmm_eval on this context, measured with CUDA events
  * recorded on that call's stream while profiling is enabled (dafmm_set_profiling).
  * out10 = {P2M, M2M, M2L (all levels), M2L finest level, L2L, L2P+P2P, conversions,
- * total, kernel launches, 0}; times in milliseconds.  Waits for the recorded events. */
+ * total, kernel launches, 0}; times in milliseconds.  The tensor-core M2L takes every level in
+ * one launch and counts whole as the finest level's; the P2L of adaptive trees counts with the M2L.  Waits for the recorded events. */
 int dafmm_set_profiling(dafmm_ctx* ctx, int enable);
 int dafmm_last_phase_ms(dafmm_ctx* ctx, double* out10);
 
@@ -218,15 +219,18 @@ int dafmm_last_phase_ms(dafmm_ctx* ctx, double* out10);
  *   (the V-list pairs of a level have the same 316 box displacements). */
 #define DAFMM_OPT_M2L_ROTATION 5
 /*   DAFMM_OPT_M2L_HARMONIC: the tensor-core M2L of the FP32 (F16 operands) and MIXED (TF32)
- *   modes, uniform and adaptive trees and forests: 1 (default) = in the harmonic basis.  The homogeneous parts of the multipole expansions
+ *   modes and the M2L by rotation (FP64, float-float), uniform and adaptive trees and forests:
+ *   1 (default) = in the harmonic basis.  The homogeneous parts of the multipole expansions
  *   (Eq. 2: the Legendre generating function) and of the local expansions (Taylor polynomials
  *   of a harmonic potential) are harmonic polynomials, each fixed by its coefficients of z
  *   exponent <= 1; the M2L contracts those (p + 1)^2 coefficients against K^_v restricted and
  *   composed accordingly (81 instead of 165 at p = 8) and restores the others by Laplace's
  *   equation -- the same result up to rounding with about a quarter of the multiply-adds.
- *   The P2M and the M2M then compute the multipoles' free coefficients only (the M2M by its
- *   table composed with that expansion; adaptive trees fill in the rest for the M2P).
- *   0 = all ncoef coefficients. */
+ *   The P2M and the M2M of FP32 and MIXED then compute the multipoles' free coefficients only (the M2M
+ *   by its table composed with that expansion; adaptive trees fill in the rest for the M2P); the
+ *   rotation's steps compute only those of their outputs and restore the others where a step reads
+ *   them.  0 = all ncoef coefficients.  (The P2M of FP64 and float-float and every P2L sum the free
+ *   coefficients and restore the others either way.) */
 #define DAFMM_OPT_M2L_HARMONIC 6
 int dafmm_set_option(dafmm_ctx* ctx, int option, int64_t value);
 

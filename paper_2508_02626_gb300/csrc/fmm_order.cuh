@@ -15,6 +15,8 @@
 //                             generated transfer map (one block per v)
 //                 k_m2l       L~_t = (1/h) sum_v K^_v M~_{t-v} over the 189 displacements of
 //                             the target's octant (SIMT, FP64 or FP32)
+//                 k_m2l_rot   the same by rotation (Sec. 3.4), FP64 and float-float: one or two
+//                             targets per warp (the FP32 and MIXED M2L: tc_ops.cu, tc_gather.cu)
 //   L2L  (Eq. 7)  k_l2l       32 parents and 16 rows per block, 8 child tables by sign flips
 //   L2P + P2P     k_leaf      one block per target leaf (8 warps in trees of few leaves, else one):
 //                 k_leaf64    pairwise sum over the 27 neighbour leaves and the generated L2P of the

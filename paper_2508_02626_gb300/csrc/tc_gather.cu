@@ -13,11 +13,14 @@ namespace tc {
 // Same pipeline as k_tc, but the A rows (source multipoles) of a 128-target tile are gathered
 // one 16-byte chunk at a time with cp.async into the 128-byte-swizzled K-major layout that a
 // TMA box would produce (chunk j of row r at (r / 8) * 1024 + (r % 8) * 128 + (j ^ r % 8) * 16),
-// zero-filled for missing sources and for columns past ncp.  Two producer warps gather, half the
-// rows each (one warp issuing all of a stage's copies paced the kernel); lane 0 of the first
-// also loads the K^_v tile by TMA.  A stage is signalled full once the TMA bytes have landed and
-// every producer lane has seen its own copies complete, fenced them for the async proxy and
-// arrived (65 arrivals: 2 x 32 lanes + the expect_tx arrival).
+// zero-filled for missing sources; chunks past the row's end are not copied (the MMAs of the last K
+// chunk read no further than the row).  Two producer warps gather, half the rows each (one warp
+// issuing all of a stage's copies paced the kernel); lane 0 of the first also loads the K^_v tile by
+// TMA.  The copies signal their stage themselves: every producer lane leaves an arrival on the
+// stage's barrier that fires when its copies so far have landed (cp.async.mbarrier.arrive.noinc), and a
+// stage is full after 65 arrivals (2 x 32 lanes and the expect_tx arrival) and the TMA bytes.  Nothing
+// on the producers' side orders the gathered rows (generic proxy) before the tensor core's reads (async
+// proxy): the issuing warp does, by fence.proxy.async between its wait for the stage and its MMAs.
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32_t src_bytes) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
 }
