@@ -1610,9 +1610,9 @@ __global__ void __launch_bounds__(32 * NW, (std::is_same<T, float>::value ? kLea
 }
 
 // The same in FP64: a block of NW warps per leaf, the warps sharing out the sources of each pass.
-// NW is 8 or 1 (leaf_warps), so that a tree of 64 or 512 leaves still gives every SM its share.  Measured against one warp per leaf with passes of 32 and CUDA's rsqrt:
-// uniform N = 200,003, depth 4, p = 8: 13.1 -> 9.6 ms; N = 1e4, depth 3, p = 6: the evaluation 2.57
-// -> 2.20 ms (this kernel 0.28).
+// NW is 8 or 1 (leaf_warps), so that a tree of 64 or 512 leaves still gives every SM its share.
+// Measured against one warp per leaf with passes of 32 and CUDA's rsqrt: uniform N = 200,003, depth 4,
+// p = 8: 13.1 -> 9.6 ms; N = 1e4, depth 3, p = 6: the evaluation 2.57 -> 2.20 ms (this kernel 0.28).
 template <int NW>
 __global__ void __launch_bounds__(32 * NW, 24 / NW) k_leaf64(TreeView tv, const double* __restrict__ Lleaf,
                                                              double* __restrict__ phi, double* __restrict__ field) {
