@@ -1945,17 +1945,17 @@ __global__ void __launch_bounds__(256, 3) k_leaf_a(AdaptiveView av, const int* _
     float* lrow = reinterpret_cast<float*>(buf + kNearSmem);
     const int b = leaves[li];
     if (!DAFMM_IN(b, av.nbox, kChkBoxIndex)) return;
+    double cx, cy, cz, h;
+    abox_geom(av, b, cx, cy, cz, h);
+    const double ih = 1.0 / h;
+    const int lev = av.level[b];
+    if (lev >= 2) warp_row_to_f32(L + (size_t)b * NCP, lrow, lane);
     int i0 = av.pbeg[b], i1 = av.pend[b];
     if (!DAFMM_RANGE(i0, i1, av.n, kChkBoxRange)) i0 = i1 = 0;
     // the leaf's own records (its targets)
     if (!DAFMM_RANGE(av.xq0[b], (long long)av.xq0[b] + (i1 - i0), av.nrec, kChkRecord)) i0 = i1 = 0;
     const int base0 = i0 + 32 * (int)blockIdx.y;
     if (base0 >= i1) return;
-    double cx, cy, cz, h;
-    abox_geom(av, b, cx, cy, cz, h);
-    const double ih = 1.0 / h;
-    const int lev = av.level[b];
-    if (lev >= 2) warp_row_to_f32(L + (size_t)b * NCP, lrow, lane);
     int u0 = av.u_ptr[b], u1 = av.u_ptr[b + 1];
     int w0 = av.w_ptr[b], w1 = av.w_ptr[b + 1];
     if (!DAFMM_RANGE(u0, u1, av.nu, kChkListPtr)) u0 = u1 = 0;
